@@ -359,7 +359,15 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->dfs_items = w.take<SymItem>(c->dfs_n_items);
     c->dfs_row_nk = w.take<int>(std::max<long long>(1, c->sym_n_tiles));
     c->dfs_part_i = w.take<double4_32a>((long long)c->dfs_kmax * NBL);
-    c->dfs_part_j = w.take<double4_32a>(std::max<long long>(1, c->sym_n_jslots) * GDC_SYM_TILE);
+    // source-side slots of the double-float and the FP64 kernel: one product at a time uses them
+    c->dfs_part_j = w.take<double4_32a>(std::max<long long>(
+        1, std::max(c->sym_n_jslots * GDC_SYM_TILE, c->h_p64_jbase.back() * c->p64_tile)));
+    c->p64_part_j = c->dfs_part_j;
+    c->p64_items = w.take<P64Item>((long long)c->h_p64_items.size());
+    c->p64_row_nk = w.take<int>((long long)c->h_p64_row_nk.size());
+    c->p64_tile_base = w.take<long long>(S + 1);
+    c->p64_jbase = w.take<long long>(S + 1);
+    c->p64_part_i = w.take<double4_32a>((long long)c->p64_kmax * NBL);
     c->h_near_items.clear();
     for (int s = 0; s < c->S; ++s) {
         const long long ns = c->h_blob_off[s + 1] - c->h_blob_off[s];
@@ -439,6 +447,10 @@ static gdc_status upload_layout(gdc_ctx* c, const double* tmpl_xyz_centred) {
     chk(up(c, c->mv_nk, c->h_mv_nk.data(), S));
     chk(up(c, c->dfs_items, c->h_dfs_items.data(), c->h_dfs_items.size()));
     chk(up(c, c->dfs_row_nk, c->h_dfs_row_nk.data(), c->h_dfs_row_nk.size()));
+    chk(up(c, c->p64_items, c->h_p64_items.data(), c->h_p64_items.size()));
+    chk(up(c, c->p64_row_nk, c->h_p64_row_nk.data(), c->h_p64_row_nk.size()));
+    chk(up(c, c->p64_tile_base, c->h_p64_tile_base.data(), S + 1));
+    chk(up(c, c->p64_jbase, c->h_p64_jbase.data(), S + 1));
     if (c->p.wall) {
         chk(up(c, c->blk_off, c->h_blk_off.data(), NB + 1));
         chk(up(c, c->wall_items, c->h_wall_items.data(), c->h_wall_items.size()));

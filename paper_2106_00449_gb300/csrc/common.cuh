@@ -36,6 +36,7 @@
 #ifndef GDC_DFS_WIDTH
 #define GDC_DFS_WIDTH 2          // source tiles per item of the symmetric double-float kernel
 #endif
+#define GDC_P64_WIDE 16384       // FP64 pair kernel: 512-blob tiles for suspensions above this, 128-blob ones up to it
 #define GDC_CELL_MIN_BLOBS 16384 // GDC_FORCES_CHOOSE: the cell list from this many blobs on
 #define GDC_WAIT_POLLS 400000    // default bound of a pair kernel's wait for a tile copy (polls)
 
@@ -51,6 +52,12 @@ struct MvItem {      // one block of the pair kernels: targets [t0, t0+tile) x s
 
 struct SymItem {     // one block of the symmetric pair kernel: target tile I x source tiles [J0, J1) of suspension s
     int s, I, J0, J1;
+    int k;           // target-side partial-sum slot (the item's index within row I)
+    int pad[3];
+};
+
+struct P64Item {     // one block of the symmetric FP64 pair kernel: target tile I x sources [j0, j1) of suspension s
+    int s, I, j0, j1;
     int k;           // target-side partial-sum slot (the item's index within row I)
     int pad[3];
 };
@@ -239,6 +246,15 @@ struct gdc_ctx {
     std::vector<int> h_dfs_row_nk;
     double4_32a *dfs_part_i = 0, *dfs_part_j = 0;
     std::vector<long long> h_sym_tile_base, h_sym_jbase;
+    // symmetric FP64 kernel (pair64.cu): its tile size, work list, slots
+    int p64_tile = 128, p64_kmax = 1;
+    gdc::P64Item* p64_items = 0;
+    int* p64_row_nk = 0;                      // target-side slots per tile row
+    long long *p64_tile_base = 0, *p64_jbase = 0;
+    double4_32a *p64_part_i = 0, *p64_part_j = 0;
+    std::vector<gdc::P64Item> h_p64_items;
+    std::vector<int> h_p64_row_nk;
+    std::vector<long long> h_p64_tile_base, h_p64_jbase;
 
     // pairs closer than 2a (self pair excluded) of the loaded configuration, for the FP32
     // products' corrections: per blob a count and up to GDC_NEAR_CAP blob indices
@@ -362,7 +378,7 @@ void launch_scatter_solution(gdc_ctx* c, const double* x, double* V, double* lam
 
 // rpy.cu
 void launch_pack_lambda(gdc_ctx* c, int prec, const double* x, int gm_layout);
-void launch_rpy(gdc_ctx* c, int prec);
+void launch_rpy(gdc_ctx* c, int prec, const double* x, int gm_layout);
 void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout,
                          bool same_body = true);   // same_body = false: blocks between different bodies only (FP32)
 void launch_forces_pair(gdc_ctx* c, int prec, double* fblob);
@@ -381,6 +397,10 @@ void launch_near_build(gdc_ctx* c);
 // sym.cu
 void build_sym_items(gdc_ctx* c, int width);
 void build_sym_list(const gdc_ctx* c, int width, std::vector<SymItem>& items, std::vector<int>& row_nk, int& kmax);
+// pair64.cu
+void build_p64_list(gdc_ctx* c);
+void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout);
+void launch_p64_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout);
 // dfsym.cu
 gdc_status dfsym_init_attributes(gdc_ctx* c);
 long long lz_q_doubles(int kmax);   // krylov.cu

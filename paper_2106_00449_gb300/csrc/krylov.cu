@@ -240,7 +240,7 @@ gdc_status rpy_op(gdc_ctx* c, int prec, const double* lam, double* u) {
         return st == GDC_OK ? st : fail(c, st, std::string("FCM: ") + gdc_fcm_last_error(c->fcm));
     }
     launch_pack_lambda(c, prec, lam, 0);
-    launch_rpy(c, prec);
+    launch_rpy(c, prec, lam, 0);
     launch_rpy_epilogue(c, prec, lam, u, 0);
     if (c->p.wall) launch_wall_apply(c, prec, lam, u, 0);   // + the wall correction of every pair
     return GDC_OK;
@@ -255,7 +255,7 @@ gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y) {
         return GDC_OK;
     }
     launch_pack_lambda(c, prec, x, 1);
-    launch_rpy(c, prec);
+    launch_rpy(c, prec, x, 1);
     launch_rpy_epilogue(c, prec, x, y, 1);
     if (c->p.wall) launch_wall_apply(c, prec, x, y, 1);
     launch_body_KT(c, x, 1, y, 1, -1.0);
@@ -277,7 +277,7 @@ static void lz_operator(gdc_ctx* c, int prec, const double* x, double* w) {
         // the factor products in FP32 too: the coupling term they feed carries FP32 rounding
         launch_body_tri(c, TRI_LINV_T, x, nullptr, c->lz_z, true);
         launch_pack_lambda(c, prec, c->lz_z, 0);
-        launch_rpy(c, prec);
+        launch_rpy(c, prec, c->lz_z, 0);
         launch_rpy_epilogue(c, prec, c->lz_z, c->lz_u, 0, false);
         launch_body_tri(c, TRI_LINV, c->lz_u, x, w, true);
     } else {

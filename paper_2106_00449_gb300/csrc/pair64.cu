@@ -1,0 +1,332 @@
+// Symmetric FP64 RPY product: every unordered pair of blobs evaluated once for both of its
+// blobs (M_ij = M_ji, even in d = r_j - r_i).
+//
+// What bounds it: the FP64 pipe.  GB300 issues 2 FP64 lanes per clock per SM (a warp
+// instruction takes 16 clocks), so loads, shuffles and integer work are free beside it and
+// the count of FP64 instructions is everything.  A pair costs 16 of them (difference 3, r^2 3,
+// reciprocal square root 5, coefficients 5) plus 10 per side (d . lambda 3, scale 1,
+// accumulate 6): 36 per unordered pair against 2 x 33 for the ordered form that this kernel
+// replaced.  The comparison with (2a)^2 is made on the bit patterns (integer pipe; both are
+// positive), and the reciprocal square root is refined from the hardware's approximation by
+// the series y (1 + e/2 + 3 e^2/8), e = 1 - r^2 y^2 (the binomial series of (1 - e)^(-1/2)
+// cut after e^2: with |e| below 4e-6 the next term is below 2e-17).
+//
+// Work split.  A suspension is cut into tiles of TS = 128 TPL blobs (TPL targets per lane).  An
+// item is a target tile I against a range [j0, j1) of sources, j0 >= I TS; ranges of one row
+// of tiles do not overlap.  Sources of tile I itself are taken ordered (target side only),
+// sources of later tiles symmetrically: W sources (32, or a smaller power of two when the
+// range is shorter) are swept in W steps in which lane l reads source (l + step) mod W, and
+// the source-side sums travel with their source, one lane per step by shuffles.  The four
+// warps' sums of a source meet in shared memory, are added in warp order and go to the one
+// slot of (I, J): every slot is written once, all sums run in a fixed order (deterministic).
+// Because the pipe is so slow one target per lane already hides every latency, and short
+// ranges spread a small suspension over all SMs: 1,560 blobs take 1,360 items of 8 sources.
+// Above GDC_P64_WIDE blobs TPL = 4 keeps the slot arrays at n^2/1024 entries.
+//
+// Measured against the ordered kernel that it replaced (128 or 256 or 512 targets per block
+// against source chunks of at least 512): one product of 9,126 blobs 4.81 -> 2.85 ms (83% of
+// the pipe's 2.38 ms for 36 instructions per pair); 13 products of 1,560 blobs in a Brownian
+// velocity 14.2 -> 3.7 ms, 28 blocks before; a gDC step of 48 blobs 4.46 -> 2.04 ms, where the
+// ordered kernel ran on one block.
+#include <algorithm>
+#include <cstring>
+
+#include "common.cuh"
+
+namespace gdc {
+
+constexpr int P64_STAGE = 128;   // sources staged in shared memory at a time
+
+struct Rpy64K {
+    double c23, c2, cA, c9, cB;
+    long long four_a2_bits;
+};
+
+// 1/sqrt(x) for positive normal x
+__device__ __forceinline__ double rsqrt_series(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(fma(0.375, e, 0.5), y * e, y);
+}
+
+// RPY coefficients A, B (units of 1/(8 pi eta)) of a pair at squared distance r2
+__device__ __forceinline__ void rpy64_coeff(double r2, const Rpy64K& k, double& A, double& B) {
+    const double ri = rsqrt_series(r2);
+    if (__double_as_longlong(r2) >= k.four_a2_bits) {
+        const double ri2 = ri * ri, ri3 = ri2 * ri;
+        A = fma(k.c23, ri3, ri);
+        B = ri3 * fma(-k.c2, ri2, 1.0);
+    } else if (r2 > 1e-290) {   // overlapping blobs
+        A = k.cA * fma(-k.c9, r2 * ri, 1.0);
+        B = k.cB * ri;
+    } else {                    // the self pair (or coincident blobs: B d d^T vanishes with r)
+        A = k.cA;
+        B = 0.0;
+    }
+}
+
+template <int TPL>
+__global__ void __launch_bounds__(128, TPL == 1 ? 5 : 3) k_rpy64_sym(
+    const P64Item* __restrict__ items, const int* __restrict__ active, const long long* __restrict__ susp_blob_off,
+    const long long* __restrict__ jbase, const double4_32a* __restrict__ spos, const double* __restrict__ x,
+    const int* __restrict__ map, double4_32a* __restrict__ part_i, double4_32a* __restrict__ part_j, int NBL, Rpy64K k) {
+    constexpr int TS = 128 * TPL;
+    __shared__ double src[6][P64_STAGE];
+    __shared__ double red[2][4][3][32];
+    const P64Item it = items[blockIdx.x];
+    const long long b0 = susp_blob_off[it.s];
+    const int ns = (int)(susp_blob_off[it.s + 1] - b0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tbase = it.I * TS;
+    if (active && !active[it.s]) {
+        // a suspension whose Krylov loop has stopped: its product is not used; leave zeros
+        const double4_32a z = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+        for (int t = threadIdx.x; t < TS && tbase + t < ns; t += 128) part_i[(long long)it.k * NBL + b0 + tbase + t] = z;
+        for (int j = max(it.j0, tbase + TS) + (int)threadIdx.x; j < it.j1; j += 128) {
+            const int J = j / TS;
+            part_j[(jbase[it.s] + (long long)J * (J - 1) / 2 + it.I) * TS + j - J * TS] = z;
+        }
+        return;
+    }
+    // targets tbase + threadIdx.x + 128 m; one past the end sits on the last blob with lambda =
+    // 0 (it adds nothing to a source and its own sums are not written)
+    double xt[TPL], yt[TPL], zt[TPL], lxt[TPL], lyt[TPL], lzt[TPL], ux[TPL], uy[TPL], uz[TPL];
+#pragma unroll
+    for (int m = 0; m < TPL; ++m) {
+        const int t = tbase + (int)threadIdx.x + 128 * m;
+        const long long g = b0 + min(t, ns - 1);
+        const double4_32a p = spos[g];
+        const long long o = map ? (long long)map[g] : 3 * g;
+        xt[m] = p.x;
+        yt[m] = p.y;
+        zt[m] = p.z;
+        lxt[m] = t < ns ? x[o] : 0.0;
+        lyt[m] = t < ns ? x[o + 1] : 0.0;
+        lzt[m] = t < ns ? x[o + 2] : 0.0;
+        ux[m] = uy[m] = uz[m] = 0.0;
+    }
+    const int range = it.j1 - it.j0;
+    int W = 32;   // sources per sweep: a power of two, at least the range when that is short
+    while (W > 1 && (W >> 1) >= range) W >>= 1;
+    int buf = 0;
+    for (int c0 = it.j0; c0 < it.j1; c0 += P64_STAGE) {
+        const int n = min(P64_STAGE, it.j1 - c0);
+        const int nr = (n + W - 1) & ~(W - 1);
+        __syncthreads();   // the previous sources are no longer read
+        if ((int)threadIdx.x < nr) {
+            const bool in = (int)threadIdx.x < n;   // past the range: the last blob of it with lambda = 0
+            const long long g = b0 + c0 + min((int)threadIdx.x, n - 1);
+            const double4_32a p = spos[g];
+            const long long o = map ? (long long)map[g] : 3 * g;
+            src[0][threadIdx.x] = p.x;
+            src[1][threadIdx.x] = p.y;
+            src[2][threadIdx.x] = p.z;
+            src[3][threadIdx.x] = in ? x[o] : 0.0;
+            src[4][threadIdx.x] = in ? x[o + 1] : 0.0;
+            src[5][threadIdx.x] = in ? x[o + 2] : 0.0;
+        }
+        __syncthreads();
+        for (int jc = 0; jc < n; jc += W) {
+            const int J = (c0 + jc) / TS;
+            if (J == it.I) {
+                // the tile itself: every ordered pair, target side only
+                for (int j = jc; j < min(jc + W, n); ++j) {
+                    const double xs = src[0][j], ys = src[1][j], zs = src[2][j];
+                    const double lx = src[3][j], ly = src[4][j], lz = src[5][j];
+#pragma unroll
+                    for (int m = 0; m < TPL; ++m) {
+                        if (tbase + 32 * warp + 128 * m >= ns) continue;   // no target in this warp
+                        const double dx = xs - xt[m], dy = ys - yt[m], dz = zs - zt[m];
+                        double A, B;
+                        rpy64_coeff(fma(dx, dx, fma(dy, dy, dz * dz)), k, A, B);
+                        const double s = B * fma(dx, lx, fma(dy, ly, dz * lz));
+                        ux[m] = fma(A, lx, fma(s, dx, ux[m]));
+                        uy[m] = fma(A, ly, fma(s, dy, uy[m]));
+                        uz[m] = fma(A, lz, fma(s, dz, uz[m]));
+                    }
+                }
+                continue;
+            }
+            double jx = 0.0, jy = 0.0, jz = 0.0;   // sums of the source this lane holds
+            for (int st = 0; st < W; ++st) {
+                const int j = jc + ((lane + st) & (W - 1));
+                const double xs = src[0][j], ys = src[1][j], zs = src[2][j];
+                const double lx = src[3][j], ly = src[4][j], lz = src[5][j];
+#pragma unroll
+                for (int m = 0; m < TPL; ++m) {
+                    if (tbase + 32 * warp + 128 * m >= ns) continue;
+                    const double dx = xs - xt[m], dy = ys - yt[m], dz = zs - zt[m];
+                    double A, B;
+                    rpy64_coeff(fma(dx, dx, fma(dy, dy, dz * dz)), k, A, B);
+                    const double s = B * fma(dx, lx, fma(dy, ly, dz * lz));          // M lambda_j
+                    ux[m] = fma(A, lx, fma(s, dx, ux[m]));
+                    uy[m] = fma(A, ly, fma(s, dy, uy[m]));
+                    uz[m] = fma(A, lz, fma(s, dz, uz[m]));
+                    const double w = B * fma(dx, lxt[m], fma(dy, lyt[m], dz * lzt[m]));   // M lambda_i
+                    jx = fma(A, lxt[m], fma(w, dx, jx));
+                    jy = fma(A, lyt[m], fma(w, dy, jy));
+                    jz = fma(A, lzt[m], fma(w, dz, jz));
+                }
+                const int from = (lane + 1) & 31;   // the source of lane l + 1 is lane l's next
+                jx = __shfl_sync(0xffffffffu, jx, from);
+                jy = __shfl_sync(0xffffffffu, jy, from);
+                jz = __shfl_sync(0xffffffffu, jz, from);
+            }
+            // W < 32: the 32/W lanes with the same remainder mod W hold parts of one source
+            for (int o = W; o < 32; o <<= 1) {
+                jx += __shfl_xor_sync(0xffffffffu, jx, o);
+                jy += __shfl_xor_sync(0xffffffffu, jy, o);
+                jz += __shfl_xor_sync(0xffffffffu, jz, o);
+            }
+            // the buffer this sweep writes was last read before the previous sweep's barrier
+            red[buf][warp][0][lane] = jx;
+            red[buf][warp][1][lane] = jy;
+            red[buf][warp][2][lane] = jz;
+            __syncthreads();
+            if (warp == 0 && lane < W && jc + lane < n) {   // in warp order
+                double v[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    v[c] = ((red[buf][0][c][lane] + red[buf][1][c][lane]) + red[buf][2][c][lane]) + red[buf][3][c][lane];
+                const long long slot = jbase[it.s] + (long long)J * (J - 1) / 2 + it.I;
+                part_j[slot * TS + (c0 + jc + lane) - J * TS] = make_double4_32a(v[0], v[1], v[2], 0.0);
+            }
+            buf ^= 1;
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < TPL; ++m) {
+        const int t = tbase + (int)threadIdx.x + 128 * m;
+        if (t < ns) part_i[(long long)it.k * NBL + b0 + t] = make_double4_32a(ux[m], uy[m], uz[m], 0.0);
+    }
+}
+
+// u_i = c0 (target-side slots of the blob's tile row + source-side slots of the tiles before
+// it) [- K V].  Four threads per blob, each taking every fourth slot, added in a fixed order:
+// the slots are latency-bound L2 reads, and one thread per blob left small suspensions with
+// a few warps.
+__global__ void __launch_bounds__(128) k_p64_epilogue(
+    int NBL, int TS, const double4_32a* __restrict__ part_i, const double4_32a* __restrict__ part_j,
+    const int* __restrict__ blob_susp, const long long* __restrict__ susp_blob_off, const int* __restrict__ row_nk,
+    const long long* __restrict__ tile_base, const long long* __restrict__ jbase, double c0, const double* __restrict__ x,
+    double* __restrict__ y, int gm_layout, const int* __restrict__ blob_gm, const int* __restrict__ body_gm,
+    const int* __restrict__ blob_body, const double* __restrict__ r, const double* __restrict__ Yc) {
+    const int sub = threadIdx.x & 3;
+    const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 2);
+    double ux = 0.0, uy = 0.0, uz = 0.0;
+    if (i < NBL) {
+        const int s = blob_susp[i];
+        const int loc = (int)(i - susp_blob_off[s]);
+        const int J = loc / TS, e = loc - J * TS;
+        const int n = row_nk[tile_base[s] + J];
+#pragma unroll 4
+        for (int q = sub; q < n; q += 4) {
+            const double4_32a v = part_i[(long long)q * NBL + i];
+            ux += v.x;
+            uy += v.y;
+            uz += v.z;
+        }
+        const long long s0 = jbase[s] + (long long)J * (J - 1) / 2;
+#pragma unroll 4
+        for (int I = sub; I < J; I += 4) {
+            const double4_32a v = part_j[(s0 + I) * TS + e];
+            ux += v.x;
+            uy += v.y;
+            uz += v.z;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        ux += __shfl_xor_sync(0xffffffffu, ux, o);
+        uy += __shfl_xor_sync(0xffffffffu, uy, o);
+        uz += __shfl_xor_sync(0xffffffffu, uz, o);
+    }
+    if (i >= NBL || sub != 0) return;
+    ux *= c0;
+    uy *= c0;
+    uz *= c0;
+    if (!gm_layout) {
+        y[3LL * i] = ux;
+        y[3LL * i + 1] = uy;
+        y[3LL * i + 2] = uz;
+        return;
+    }
+    // saddle operator: M lambda - K V, K V = U_p + Omega_p x (r_i - Y_p)  (Eq. rigid_body_cond)
+    const int p = blob_body[i];
+    const double* V = x + body_gm[p];
+    const double dx = r[3LL * i] - Yc[3 * p], dy = r[3LL * i + 1] - Yc[3 * p + 1], dz = r[3LL * i + 2] - Yc[3 * p + 2];
+    const long long o = blob_gm[i];
+    y[o] = ux - (V[0] + (V[4] * dz - V[5] * dy));
+    y[o + 1] = uy - (V[1] + (V[5] * dx - V[3] * dz));
+    y[o + 2] = uz - (V[2] + (V[3] * dy - V[4] * dx));
+}
+
+// Work list: tiles of 128 blobs, or 512 when a suspension is larger than GDC_P64_WIDE; source
+// ranges as long as possible while a launch still has 8 items per SM (all of them resident
+// together, so an SM's share differs from the mean by at most an eighth), longest first.
+void build_p64_list(gdc_ctx* c) {
+    long long nmax = 0;
+    for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
+    const int TS = c->p64_tile = nmax > GDC_P64_WIDE ? 512 : 128;
+    c->h_p64_tile_base.assign(c->S + 1, 0);
+    c->h_p64_jbase.assign(c->S + 1, 0);
+    for (int s = 0; s < c->S; ++s) {
+        const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s], T = (n + TS - 1) / TS;
+        c->h_p64_tile_base[s + 1] = c->h_p64_tile_base[s] + T;
+        c->h_p64_jbase[s + 1] = c->h_p64_jbase[s] + T * (T - 1) / 2;
+    }
+    const long long want = 8LL * c->num_sms;
+    int w = 2 * TS;
+    for (; w > 4; w >>= 1) {
+        long long items = 0;
+        for (int s = 0; s < c->S && items < want; ++s) {
+            const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
+            for (long long t0 = 0; t0 < n && items < want; t0 += TS) items += (n - t0 + w - 1) / w;
+        }
+        if (items >= want) break;
+    }
+    c->h_p64_items.clear();
+    c->h_p64_row_nk.clear();
+    c->p64_kmax = 1;
+    for (int s = 0; s < c->S; ++s) {
+        const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
+        for (int I = 0; (long long)I * TS < n; ++I) {
+            int k = 0;
+            const long long left = n - (long long)I * TS;
+            // very large suspensions: at most 128 slots per row, ranges of whole tiles
+            const long long step = w == 2 * TS ? std::max<long long>(w, ((left + 127) / 128 + TS - 1) / TS * TS) : w;
+            for (long long j0 = (long long)I * TS; j0 < n; j0 += step, ++k)
+                c->h_p64_items.push_back(P64Item{s, I, (int)j0, (int)std::min(n, j0 + step), k, {0, 0, 0}});
+            c->h_p64_row_nk.push_back(k);
+            c->p64_kmax = std::max(c->p64_kmax, k);
+        }
+    }
+    std::stable_sort(c->h_p64_items.begin(), c->h_p64_items.end(),
+                     [](const P64Item& a, const P64Item& b) { return a.j1 - a.j0 > b.j1 - b.j0; });
+}
+
+void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout) {
+    const double a = c->p.a, four_a2 = 4.0 * a * a;
+    Rpy64K k{2.0 * a * a / 3.0, 2.0 * a * a, 4.0 / (3.0 * a), 9.0 / (32.0 * a), 1.0 / (8.0 * a * a), 0};
+    static_assert(sizeof(four_a2) == sizeof(k.four_a2_bits), "bit pattern of a double");
+    memcpy(&k.four_a2_bits, &four_a2, sizeof(four_a2));
+    const int* map = gm_layout ? c->blob_gm : nullptr;
+    const unsigned n = (unsigned)c->h_p64_items.size();
+    ++c->n_launch;
+    if (c->p64_tile == 128)
+        k_rpy64_sym<1><<<n, 128, 0, c->stream>>>(c->p64_items, c->mv_active, c->susp_blob_off, c->p64_jbase, c->spos64, x,
+                                                 map, c->p64_part_i, c->p64_part_j, c->NBL, k);
+    else
+        k_rpy64_sym<4><<<n, 128, 0, c->stream>>>(c->p64_items, c->mv_active, c->susp_blob_off, c->p64_jbase, c->spos64, x,
+                                                 map, c->p64_part_i, c->p64_part_j, c->NBL, k);
+}
+
+void launch_p64_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout) {
+    ++c->n_launch, k_p64_epilogue<<<ceil_div(4LL * c->NBL, 128), 128, 0, c->stream>>>(
+        c->NBL, c->p64_tile, c->p64_part_i, c->p64_part_j, c->blob_susp, c->susp_blob_off, c->p64_row_nk,
+        c->p64_tile_base, c->p64_jbase, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm,
+        c->body_gm, c->blob_body, c->r, c->Yc);
+}
+
+}  // namespace gdc

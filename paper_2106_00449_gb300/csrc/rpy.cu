@@ -51,7 +51,7 @@ void launch_pack_lambda(gdc_ctx* c, int prec, const double* x, int gm_layout) {
     const int* map = gm_layout ? c->blob_gm : nullptr;
     if (prec == GDC_FP32_MIXED)
         ++c->n_launch, k_pack_lam32<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(c->NBL, map, x, c->spos, c->sdup);
-    else
+    else if (prec == GDC_PREC_DF64)
         ++c->n_launch, k_pack_lam64<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(c->NBL, map, x, c->slam64);
 }
 
@@ -269,80 +269,8 @@ __global__ void __launch_bounds__(128) k_rpy_df(const MvItem* __restrict__ items
     }
 }
 
-template <int TPT>
-__global__ void __launch_bounds__(128) k_rpy64(const MvItem* __restrict__ items, const int* __restrict__ active,
-                                               const long long* __restrict__ susp_blob_off,
-                                               const double4_32a* __restrict__ spos, const double4_32a* __restrict__ slam,
-                                               double4_32a* __restrict__ part, int NBL, double a) {
-    __shared__ double4_32a sp[MV_TILE];
-    __shared__ double4_32a sl[MV_TILE];
-    const MvItem it = items[blockIdx.x];
-    const long long b0 = susp_blob_off[it.s];
-    const int ns = (int)(susp_blob_off[it.s + 1] - b0);
-    if (active && !active[it.s]) {   // stopped Krylov loop: product unused, leave zeros
-        for (int t = threadIdx.x; t < 128 * TPT && it.t0 + t < ns; t += 128)
-            part[(long long)it.k * NBL + b0 + it.t0 + t] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-        return;
-    }
-    const double c23 = 2.0 * a * a / 3.0, c2 = 2.0 * a * a, four_a2 = 4.0 * a * a;
-    const double cA = 4.0 / (3.0 * a), c9 = 9.0 / (32.0 * a), cB = 1.0 / (8.0 * a * a);
-    double xt[TPT], yt[TPT], zt[TPT], ax[TPT], ay[TPT], az[TPT];
-#pragma unroll
-    for (int t = 0; t < TPT; ++t) {
-        const int ti = it.t0 + threadIdx.x + t * 128;
-        const double4_32a p = spos[b0 + min(ti, ns - 1)];
-        xt[t] = p.x;
-        yt[t] = p.y;
-        zt[t] = p.z;
-        ax[t] = ay[t] = az[t] = 0.0;
-    }
-    for (int j0 = it.j0; j0 < it.j1; j0 += MV_TILE) {
-        const int n = min(MV_TILE, it.j1 - j0);
-        __syncthreads();
-        for (int e = threadIdx.x; e < n; e += 128) {
-            sp[e] = spos[b0 + j0 + e];
-            sl[e] = slam[b0 + j0 + e];
-        }
-        __syncthreads();
-        for (int j = 0; j < n; ++j) {
-            const double4_32a ps = sp[j];
-            const double4_32a ls = sl[j];
-#pragma unroll
-            for (int t = 0; t < TPT; ++t) {
-                const double dx = ps.x - xt[t], dy = ps.y - yt[t], dz = ps.z - zt[t];
-                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                double A, B;
-                if (r2 < four_a2) {
-                    if (r2 > 0.0) {
-                        const double r = sqrt(r2);
-                        A = cA * fma(-c9, r, 1.0);
-                        B = cB / r;
-                    } else {
-                        A = cA;
-                        B = 0.0;
-                    }
-                } else {
-                    const double ri = rsqrt(r2);
-                    const double ri2 = ri * ri, ri3 = ri2 * ri;
-                    A = fma(c23, ri3, ri);
-                    B = ri3 * fma(-c2, ri2, 1.0);
-                }
-                const double dl = fma(dx, ls.x, fma(dy, ls.y, dz * ls.z));
-                const double s = B * dl;
-                ax[t] = fma(A, ls.x, fma(s, dx, ax[t]));
-                ay[t] = fma(A, ls.y, fma(s, dy, ay[t]));
-                az[t] = fma(A, ls.z, fma(s, dz, az[t]));
-            }
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < TPT; ++t) {
-        const int ti = it.t0 + threadIdx.x + t * 128;
-        if (ti < ns) part[(long long)it.k * NBL + b0 + ti] = make_double4_32a(ax[t], ay[t], az[t], 0.0);
-    }
-}
-
-void launch_rpy(gdc_ctx* c, int prec) {
+// x, gm_layout: the vector launch_pack_lambda was given (the FP64 kernel reads it unpacked)
+void launch_rpy(gdc_ctx* c, int prec, const double* x, int gm_layout) {
     const int pe = prof_begin(c, prec == GDC_FP32_MIXED ? 0 : (prec == GDC_PREC_DF64 ? 3 : 1));
     if (prec == GDC_FP32_MIXED) {
         const double a = c->p.a;
@@ -380,15 +308,7 @@ void launch_rpy(gdc_ctx* c, int prec) {
             ++c->n_launch, k_rpy_df<2><<<c->mv_n_items, 128, 0, c->stream>>>(c->mv_items, c->susp_blob_off, c->spos64,
                                                                              c->slam64, (double4_32a*)c->mv_part, c->NBL, k);
     } else {
-        if (c->mv_tpt == 1)
-            ++c->n_launch, k_rpy64<1><<<c->mv_n_items, 128, 0, c->stream>>>(c->mv_items, c->mv_active, c->susp_blob_off, c->spos64, c->slam64,
-                                                             (double4_32a*)c->mv_part, c->NBL, c->p.a);
-        else if (c->mv_tpt == 4)
-            ++c->n_launch, k_rpy64<4><<<c->mv_n_items, 128, 0, c->stream>>>(c->mv_items, c->mv_active, c->susp_blob_off, c->spos64, c->slam64,
-                                                             (double4_32a*)c->mv_part, c->NBL, c->p.a);
-        else
-            ++c->n_launch, k_rpy64<2><<<c->mv_n_items, 128, 0, c->stream>>>(c->mv_items, c->mv_active, c->susp_blob_off, c->spos64, c->slam64,
-                                                             (double4_32a*)c->mv_part, c->NBL, c->p.a);
+        launch_rpy64_sym(c, x, gm_layout);   // its epilogue runs in launch_rpy_epilogue
     }
     prof_end(c, pe);
 }
@@ -606,6 +526,8 @@ static void launch_epilogue(gdc_ctx* c, int prec, double c0, const double* x, do
 void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout, bool same_body) {
     if (prec == GDC_PREC_DF64 && c->dfs_minb)
         launch_rpy_df_sym_epilogue(c, x, y, gm_layout);
+    else if (prec == GDC_FP64)
+        launch_p64_epilogue(c, x, y, gm_layout);
     else
         launch_epilogue(c, prec, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, prec == GDC_FP32_MIXED);
     // same-body blocks from the template: the df64 pair kernel leaves those pairs out and the
@@ -908,6 +830,7 @@ void plan_mv_capacity(gdc_ctx* c) {
         tmax = std::max(tmax, (int)((c->h_blob_off[s + 1] - c->h_blob_off[s] + GDC_SYM_TILE - 1) / GDC_SYM_TILE));
     build_sym_list(c, std::max(GDC_DFS_WIDTH, (tmax + 63) / 64), c->h_dfs_items, c->h_dfs_row_nk, c->dfs_kmax);
     c->dfs_n_items = (int)c->h_dfs_items.size();
+    build_p64_list(c);
 }
 
 static gdc_status upload_items(gdc_ctx* c) {
@@ -934,9 +857,9 @@ gdc_status autotune_pair_kernel(gdc_ctx* c) {
     int bt = 2, bsym = 0, bwid = 4;
     double bw = 8.0;
     auto time3 = [&](float& ms) -> gdc_status {
-        launch_rpy(c, GDC_FP32_MIXED);  // warm-up
+        launch_rpy(c, GDC_FP32_MIXED, c->W, 0);  // warm-up
         cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < 3; ++r) launch_rpy(c, GDC_FP32_MIXED);
+        for (int r = 0; r < 3; ++r) launch_rpy(c, GDC_FP32_MIXED, c->W, 0);
         cudaEventRecord(e1, c->stream);
         gdc_status s2 = cuda_check(c, cudaEventSynchronize(e1), "autotune");
         if (s2 == GDC_OK) cudaEventElapsedTime(&ms, e0, e1);
@@ -1006,9 +929,9 @@ gdc_status autotune_pair_kernel(gdc_ctx* c) {
             if (mb == 0 && only == 2) continue;
             c->dfs_minb = mb;
             float ms = 0.f;
-            launch_rpy(c, GDC_PREC_DF64);   // warm-up
+            launch_rpy(c, GDC_PREC_DF64, c->W, 0);   // warm-up
             cudaEventRecord(e0, c->stream);
-            launch_rpy(c, GDC_PREC_DF64);
+            launch_rpy(c, GDC_PREC_DF64, c->W, 0);
             cudaEventRecord(e1, c->stream);
             if ((st = cuda_check(c, cudaEventSynchronize(e1), "autotune")) != GDC_OK) break;
             cudaEventElapsedTime(&ms, e0, e1);
