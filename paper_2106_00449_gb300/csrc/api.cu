@@ -989,6 +989,7 @@ gdc_status gdc_init(gdc_ctx** out, const gdc_params* params, int n_templates, co
     if ((st = sym_init_attributes(c)) != GDC_OK) return st;
     if ((st = dfsym_init_attributes(c)) != GDC_OK) return st;
     if (c->p.wall) {   // every blob must start above z = a
+        if ((st = wall_init_attributes(c)) != GDC_OK) return st;
         load_at(c, c->Y, c->q);
         if ((st = read_status(c)) != GDC_OK) return st;
     }

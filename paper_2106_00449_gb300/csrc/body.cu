@@ -934,143 +934,268 @@ void launch_template_setup(gdc_ctx* c, const double* Mext) {
 // M_pp^-1 = X^T X, G = M_pp^-1 K_p (K_p from d), N = (K_p^T G)^+, and LT = L^T, X, XT = X^T
 // stored for k_body_tri<LAB>.  A blob at or below z = a (overlapping the wall, where the
 // correction is not a mobility) sets status[2]; a block that is not positive definite sets
-// status[0] = 1.  Shared memory: 3n doubles.
+// status[0] = 1.
+//
+// Bound by the FP64 pipe and by the serial chain of pivots (a suspension above a wall holds
+// few bodies, so one block per body leaves the chip mostly idle and the latency of one
+// body counts).  The lower triangle lives in shared memory when it fits (bodies of up to 55
+// blobs), and factor and inverse come out of one elimination in place, one barrier per
+// column: at column k, row i > k is reduced by f_i = a_ik / d_k times the pivot row, whose
+// entries left of the diagonal already hold the inverse of the unit factor and right of it
+// the remaining matrix (column k by symmetry); entry (i, k) becomes -f_i.  Rows are dealt to
+// warps, columns to lanes; the warp that finishes the next pivot forms its reciprocal root
+// while the others still update.  M is assembled once per blob pair i >= j (one set of
+// coefficients for the nine entries).  The 6 x 6 inverse is a Gauss-Jordan elimination on
+// one warp, with the serial Jacobi pseudo-inverse only when the spectrum may reach below the
+// pseudo-inverse's cut (a collinear body).  36 bodies of 15 blobs: 138 us, against
+// 782 us with the matrices in global memory, an entry-wise assembly, separate Cholesky and
+// inverse and a serial Jacobi.
+
+// P = A^-1 for symmetric positive definite A (row-major 6 x 6) on one warp, by Gauss-Jordan
+// elimination without pivoting, lane r < 6 holding row r of [A | P].  Returns (on every lane)
+// whether all eigenvalues are sure to lie above rel_tol times the largest, so that P is also
+// the pseudo-inverse pinv6 forms: |A|_F bounds the largest, 1/|P|_F the smallest.
+__device__ bool spd_inverse6(const double* A, double* P, double rel_tol) {
+    const int lane = threadIdx.x & 31, row = lane < 6 ? lane : 0;
+    double a[6], b[6];
+    double na = 0.0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        a[c] = A[6 * row + c];
+        b[c] = c == row ? 1.0 : 0.0;
+        na = fma(a[c], a[c], na);
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const double piv = __shfl_sync(0xffffffffu, a[k], k);
+        ok = ok && piv > 0.0;
+        const double inv = 1.0 / piv;
+        const double f = a[k] * inv;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const double ak = __shfl_sync(0xffffffffu, a[c], k), bk = __shfl_sync(0xffffffffu, b[c], k);
+            a[c] = row == k ? ak * inv : fma(-f, ak, a[c]);
+            b[c] = row == k ? bk * inv : fma(-f, bk, b[c]);
+        }
+    }
+    double nb = 0.0;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) nb = fma(b[c], b[c], nb);
+    if (lane >= 6) na = nb = 0.0;
+    na = warp_sum(na);
+    nb = warp_sum(nb);
+    if (lane < 6)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) P[6 * lane + c] = b[c];
+    __syncwarp();
+    return ok && sqrt(na) * sqrt(nb) * rel_tol < 1.0;   // false for NaN
+}
+
+// doubles of shared memory beside the triangle: d, two columns, pivots' reciprocal roots,
+// G (6 per row) and the 6 x 6 matrix
+__host__ __device__ inline int wall_block_doubles(int n3) { return 10 * n3 + 36 + 2; }
+
+template <bool SMEM>   // the triangle in shared memory (row stride n3 | 1), else in global memory
 __global__ void __launch_bounds__(256) k_wall_blocks(const long long* __restrict__ body_blob_off,
                                                      const long long* __restrict__ blk_off, const double* __restrict__ r,
-                                                     const double* __restrict__ Yc, double a, double eta,
-                                                     double* __restrict__ work, double* __restrict__ Minv,
-                                                     double* __restrict__ Gb, double* __restrict__ Nb,
-                                                     double* __restrict__ LT, double* __restrict__ Xo,
-                                                     double* __restrict__ XT, int* __restrict__ status) {
+                                                     const double* __restrict__ Yc, double a, double eta, double* work,
+                                                     double* __restrict__ Minv, double* __restrict__ Gb,
+                                                     double* __restrict__ Nb, double* __restrict__ LT,
+                                                     double* __restrict__ Xo, double* __restrict__ XT,
+                                                     int* __restrict__ status) {
     extern __shared__ double dsh[];
     const int p = blockIdx.x;
     const long long i0 = body_blob_off[p];
     const int n = (int)(body_blob_off[p + 1] - i0), n3 = 3 * n;
-    double* d = dsh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const long long mo = blk_off[p];
+    double* d = dsh;               // blob offsets
+    double* col = d + n3;          // [2][n3]: column k of the remaining matrix, double-buffered
+    double* rs = col + 2 * n3;     // 1 / L_kk
+    double* G = rs + n3;           // [row][6]
+    double* A6 = G + 6 * n3;       // 36
+    double* M = SMEM ? A6 + 38 : work + 2 * mo;
+    const int ld = SMEM ? (n3 | 1) : n3;
     const double zc = Yc[3 * p + 2];
     for (int e = threadIdx.x; e < n3; e += blockDim.x) d[e] = r[3 * i0 + e] - Yc[3 * p + e % 3];
     for (int b = threadIdx.x; b < n; b += blockDim.x)
         if (!(r[3 * (i0 + b) + 2] > a)) atomicExch(status + 2, 1);
     __syncthreads();
-    const long long mo = blk_off[p];
-    double* L = work + 2 * mo;
-    double* X = L + (long long)n3 * n3;
     const double c0 = 1.0 / (8.0 * 3.141592653589793 * eta);
-    // 1. M_pp row-major in L: RPY entry (units of 1/(8 pi eta)) + wall correction of column be
-    for (long long e = threadIdx.x; e < (long long)n3 * n3; e += blockDim.x) {
-        const int row = (int)(e / n3), col = (int)(e % n3);
-        const int i = row / 3, al = row % 3, j = col / 3, be = col % 3;
-        const double dx = d[3 * j] - d[3 * i], dy = d[3 * j + 1] - d[3 * i + 1], dz = d[3 * j + 2] - d[3 * i + 2];
-        const double dd[3] = {dx, dy, dz};
-        const double r2 = dx * dx + dy * dy + dz * dz;
+    // 1. M_pp, blob pairs i >= j: RPY block + wall correction
+    for (int e = threadIdx.x; e < n * (n + 1) / 2; e += blockDim.x) {
+        int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);   // e = i (i + 1)/2 + j
+        while (i * (i + 1) / 2 > e) --i;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        const int j = e - i * (i + 1) / 2;
+        const double dd[3] = {d[3 * j] - d[3 * i], d[3 * j + 1] - d[3 * i + 1], d[3 * j + 2] - d[3 * i + 2]};
+        const double r2 = dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2];
         double A, B;
-        if (r2 == 0.0) {
+        if (i == j || r2 == 0.0) {
             A = 4.0 / (3.0 * a);
             B = 0.0;
-        } else if (r2 < 4.0 * a * a) {
-            const double rr = sqrt(r2);
-            A = 4.0 / (3.0 * a) * (1.0 - 9.0 * rr / (32.0 * a));
-            B = 1.0 / (8.0 * a * a * rr);
         } else {
-            const double rr = sqrt(r2);
-            A = 1.0 / rr + 2.0 * a * a / (3.0 * rr * r2);
-            B = (1.0 - 2.0 * a * a / r2) / (rr * r2);
-        }
-        double w[3] = {0.0, 0.0, 0.0};
-        wall_pair<double>(d[3 * i] - d[3 * j], d[3 * i + 1] - d[3 * j + 1], d[3 * i + 2] + d[3 * j + 2] + 2.0 * zc,
-                          d[3 * j + 2] + zc, a * a, be == 0 ? 1.0 : 0.0, be == 1 ? 1.0 : 0.0, be == 2 ? 1.0 : 0.0,
-                          w[0], w[1], w[2]);
-        L[e] = c0 * ((al == be ? A : 0.0) + B * dd[al] * dd[be] + w[al]);
-    }
-    __syncthreads();
-    // 2. Cholesky M = L L^T (right-looking; lower triangle of L overwritten)
-    for (int k = 0; k < n3; ++k) {
-        if (threadIdx.x == 0) {
-            const double dkk = L[(long long)k * n3 + k];
-            if (!(dkk > 0.0)) atomicExch(status, 1);
-            L[(long long)k * n3 + k] = sqrt(fmax(dkk, 1e-300));
-        }
-        __syncthreads();
-        const double lkk = L[(long long)k * n3 + k];
-        for (int i = k + 1 + threadIdx.x; i < n3; i += blockDim.x) L[(long long)i * n3 + k] /= lkk;
-        __syncthreads();
-        const int m = n3 - k - 1;
-        for (long long e = threadIdx.x; e < (long long)m * m; e += blockDim.x) {
-            const int i = k + 1 + (int)(e / m), j = k + 1 + (int)(e % m);
-            if (j <= i) L[(long long)i * n3 + j] -= L[(long long)i * n3 + k] * L[(long long)j * n3 + k];
-        }
-        __syncthreads();
-    }
-    // 3. X = L^-1 (forward substitution per column), M^-1 = X^T X and the factor layouts
-    for (int col = threadIdx.x; col < n3; col += blockDim.x) {
-        for (int i = 0; i < n3; ++i) X[(long long)i * n3 + col] = 0.0;
-        for (int i = col; i < n3; ++i) {
-            double acc = (i == col) ? 1.0 : 0.0;
-            for (int k = col; k < i; ++k) acc -= L[(long long)i * n3 + k] * X[(long long)k * n3 + col];
-            X[(long long)i * n3 + col] = acc / L[(long long)i * n3 + i];
-        }
-    }
-    __syncthreads();
-    for (long long e = threadIdx.x; e < (long long)n3 * n3; e += blockDim.x) {
-        const int i = (int)(e / n3), j = (int)(e % n3);
-        double acc = 0.0;
-        for (int k = max(i, j); k < n3; ++k) acc += X[(long long)k * n3 + i] * X[(long long)k * n3 + j];
-        Minv[mo + e] = acc;
-        LT[mo + e] = j >= i ? L[(long long)j * n3 + i] : 0.0;
-        Xo[mo + e] = X[e];
-        XT[mo + e] = X[(long long)j * n3 + i];
-    }
-    __syncthreads();
-    // 4. G = M^-1 K (3n x 6), K columns: unit translations and e_c x d_i
-    double* G = Gb + 18LL * i0;
-    for (long long e = threadIdx.x; e < 6LL * n3; e += blockDim.x) {
-        const int row = (int)(e / 6), col = (int)(e % 6);
-        double acc = 0.0;
-        for (int i = 0; i < n; ++i) {
-            double kc[3];
-            if (col < 3) {
-                kc[0] = col == 0;
-                kc[1] = col == 1;
-                kc[2] = col == 2;
+            const double ri = rsqrt_series(r2);
+            if (r2 < 4.0 * a * a) {
+                A = 4.0 / (3.0 * a) * (1.0 - 9.0 * r2 * ri / (32.0 * a));
+                B = 1.0 / (8.0 * a * a) * ri;
             } else {
-                const int bb = col - 3;
-                const double e3[3] = {(double)(bb == 0), (double)(bb == 1), (double)(bb == 2)};
-                kc[0] = e3[1] * d[3 * i + 2] - e3[2] * d[3 * i + 1];
-                kc[1] = e3[2] * d[3 * i] - e3[0] * d[3 * i + 2];
-                kc[2] = e3[0] * d[3 * i + 1] - e3[1] * d[3 * i];
+                const double ri2 = ri * ri, ri3 = ri2 * ri;
+                A = ri + 2.0 * a * a / 3.0 * ri3;
+                B = ri3 * (1.0 - 2.0 * a * a * ri2);
             }
-            for (int al = 0; al < 3; ++al) acc += Minv[mo + (long long)row * n3 + 3 * i + al] * kc[al];
         }
-        G[e] = acc;
+        const double R[3] = {-dd[0], -dd[1], d[3 * i + 2] + d[3 * j + 2] + 2.0 * zc};
+        const WallCoeff<double> w = wall_coeff<double>(R[0], R[1], R[2], d[3 * j + 2] + zc, a * a);
+#pragma unroll
+        for (int be = 0; be < 3; ++be) {
+            const double P2 = be == 2 ? -2.0 : 2.0;   // twice the mirror's sign
+#pragma unroll
+            for (int al = 0; al < 3; ++al) {
+                double v = B * dd[al] * dd[be] + R[al] * R[be] * (w.be0 + P2 * w.be);
+                if (al == be) v += A + w.al0 + P2 * w.al;
+                if (al == 2) v += P2 * w.ga * R[be];
+                if (be == 2) v += P2 * w.ep * R[al];
+                if (al == 2 && be == 2) v += P2 * w.ze;
+                M[(long long)(3 * i + al) * ld + 3 * j + be] = c0 * v;
+            }
+        }
     }
     __syncthreads();
-    // 5. N = (K^T G)^+ (symmetrised, pseudo-inverse for collinear bodies)
+    // 2. L and the inverse of its unit form
+    for (int i = threadIdx.x; i < n3; i += blockDim.x) col[i] = M[(long long)i * ld];
     if (threadIdx.x == 0) {
-        double A6[36];
-        for (int k = 0; k < 36; ++k) A6[k] = 0.0;
-        for (int i = 0; i < n; ++i) {
-            const double bx = d[3 * i], by = d[3 * i + 1], bz = d[3 * i + 2];
-            double Kc[6][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {0, -bz, by}, {bz, 0, -bx}, {-by, bx, 0}};
-            for (int u = 0; u < 6; ++u)
-                for (int v = 0; v < 6; ++v) {
-                    double s1 = 0.0;
-                    for (int al = 0; al < 3; ++al) s1 += Kc[u][al] * G[6LL * (3 * i + al) + v];
-                    A6[6 * u + v] += s1;
-                }
-        }
-        for (int u = 0; u < 6; ++u)
-            for (int v = u + 1; v < 6; ++v) {
-                const double m = 0.5 * (A6[6 * u + v] + A6[6 * v + u]);
-                A6[6 * u + v] = A6[6 * v + u] = m;
-            }
-        pinv6(A6, Nb + 36LL * p, 1e-10);
+        if (!(M[0] > 0.0)) atomicExch(status, 1);
+        rs[0] = rsqrt_series(fmax(M[0], 1e-300));
     }
+    for (int k = 0; k < n3; ++k) {
+        __syncthreads();   // column k, its pivot's root and every row of the previous step
+        const double* ck = col + (k & 1) * n3;
+        double* cn = col + ((k + 1) & 1) * n3;
+        const double rk = rs[k], inv = rk * rk;
+        for (int i = threadIdx.x; i < n3; i += blockDim.x) LT[mo + (long long)k * n3 + i] = i >= k ? ck[i] * rk : 0.0;
+        const double* Mk = M + (long long)k * ld;
+        for (int first = k + 1 + warp; first < n3; first += 32 * nw) {   // up to 32 rows of this warp at a time
+            const int mine = first + nw * lane;
+            const double fl = mine < n3 ? ck[mine] * inv : 0.0;
+            for (int t = 0; t < 32 && first + nw * t < n3; ++t) {
+                const int i = first + nw * t;
+                const double f = __shfl_sync(0xffffffffu, fl, t);
+                double* Mi = M + (long long)i * ld;
+                for (int c = lane; c <= i; c += 32) {
+                    double v;
+                    if (c == k)
+                        v = -f;
+                    else
+                        v = fma(-f, c < k ? Mk[c] : ck[c], Mi[c]);
+                    Mi[c] = v;
+                    if (c == k + 1) {
+                        cn[i] = v;
+                        if (i == k + 1) {
+                            if (!(v > 0.0)) atomicExch(status, 1);
+                            rs[i] = rsqrt_series(fmax(v, 1e-300));
+                        }
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    // 3. X = L^-1 (rows scaled by 1 / L_ii), M^-1 = X^T X and the factor layouts
+    for (int i = warp; i < n3; i += nw) {
+        const double ri = rs[i];
+        double* Mi = M + (long long)i * ld;
+        for (int c = lane; c < n3; c += 32) {
+            const double v = c < i ? Mi[c] * ri : (c == i ? ri : 0.0);
+            if (c <= i) Mi[c] = v;
+            Xo[mo + (long long)i * n3 + c] = v;
+        }
+    }
+    __syncthreads();
+    for (int i = warp; i < n3; i += nw)
+        for (int j = lane; j < n3; j += 32) {
+            XT[mo + (long long)i * n3 + j] = j >= i ? M[(long long)j * ld + i] : 0.0;
+            if (j > i) continue;
+            double s0 = 0.0, s1 = 0.0;
+            int k = i;
+            for (; k + 1 < n3; k += 2) {
+                s0 = fma(M[(long long)k * ld + i], M[(long long)k * ld + j], s0);
+                s1 = fma(M[(long long)(k + 1) * ld + i], M[(long long)(k + 1) * ld + j], s1);
+            }
+            if (k < n3) s0 = fma(M[(long long)k * ld + i], M[(long long)k * ld + j], s0);
+            Minv[mo + (long long)i * n3 + j] = Minv[mo + (long long)j * n3 + i] = s0 + s1;
+        }
+    __syncthreads();
+    // 4. G = M^-1 K (3n x 6), K columns: unit translations and e_c x d_i (M^-1 is symmetric:
+    // read down its columns, coalesced over rows)
+    for (int e = threadIdx.x; e < 6 * n3; e += blockDim.x) {
+        const int c = e / n3, row = e - c * n3;
+        const double* Mc = Minv + mo + row;
+        double s0 = 0.0, s1 = 0.0;
+        if (c < 3) {
+            for (int i = 0; i < n; ++i) s0 += Mc[(long long)(3 * i + c) * n3];
+        } else {   // (e_c x d): component c + 2 is d_(c+1), component c + 1 is -d_(c+2) (cyclic)
+            const int u = (c + 1) % 3, v = (c + 2) % 3;
+            for (int i = 0; i < n; ++i) {
+                s0 = fma(Mc[(long long)(3 * i + v) * n3], d[3 * i + u], s0);
+                s1 = fma(Mc[(long long)(3 * i + u) * n3], d[3 * i + v], s1);
+            }
+        }
+        G[6 * row + c] = s0 - s1;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 6 * n3; e += blockDim.x) Gb[18LL * i0 + e] = G[e];
+    // 5. N = (K^T G)^+ (symmetrised, pseudo-inverse for collinear bodies)
+    if (threadIdx.x < 36) {
+        const int u = threadIdx.x / 6, v = threadIdx.x % 6;
+        double s0 = 0.0, s1 = 0.0;
+        if (u < 3) {
+            for (int i = 0; i < n; ++i) s0 += G[6 * (3 * i + u) + v];
+        } else {
+            const int w = (u + 1) % 3, z = (u + 2) % 3;
+            for (int i = 0; i < n; ++i) {
+                s0 = fma(d[3 * i + w], G[6 * (3 * i + z) + v], s0);
+                s1 = fma(d[3 * i + z], G[6 * (3 * i + w) + v], s1);
+            }
+        }
+        A6[threadIdx.x] = s0 - s1;
+    }
+    __syncthreads();
+    double sym = 0.0;
+    if (threadIdx.x < 36) sym = 0.5 * (A6[threadIdx.x] + A6[6 * (threadIdx.x % 6) + threadIdx.x / 6]);
+    __syncthreads();
+    if (threadIdx.x < 36) A6[threadIdx.x] = sym;
+    __syncthreads();
+    if (warp == 0 && !spd_inverse6(A6, Nb + 36LL * p, 1e-10) && lane == 0) pinv6(A6, Nb + 36LL * p, 1e-10);
+}
+
+// the largest body whose triangle fits the 227 KB of shared memory a block may have
+static size_t wall_block_smem(int n3, bool tri) {
+    return (size_t)(wall_block_doubles(n3) + (tri ? n3 * (n3 | 1) : 0)) * sizeof(double);
 }
 
 void launch_wall_blocks(gdc_ctx* c) {
-    ++c->n_launch, k_wall_blocks<<<c->NB, 256, (size_t)3 * c->max_body_blobs * sizeof(double), c->stream>>>(
-        c->body_blob_off, c->blk_off, c->r, c->Yc, c->p.a, c->p.eta, c->blk_work, c->blk_Minv, c->blk_G, c->blk_N,
-        c->blk_LT, c->blk_X, c->blk_XT, c->dev_status);
+    const int n3 = 3 * c->max_body_blobs, th = n3 <= 64 ? 128 : 256;
+    const bool tri = wall_block_smem(n3, true) <= 227 * 1024;
+    const size_t smem = wall_block_smem(n3, tri);
+    ++c->n_launch;
+    if (tri)
+        k_wall_blocks<true><<<c->NB, th, smem, c->stream>>>(c->body_blob_off, c->blk_off, c->r, c->Yc, c->p.a, c->p.eta,
+                                                            c->blk_work, c->blk_Minv, c->blk_G, c->blk_N, c->blk_LT,
+                                                            c->blk_X, c->blk_XT, c->dev_status);
+    else
+        k_wall_blocks<false><<<c->NB, th, smem, c->stream>>>(c->body_blob_off, c->blk_off, c->r, c->Yc, c->p.a, c->p.eta,
+                                                             c->blk_work, c->blk_Minv, c->blk_G, c->blk_N, c->blk_LT,
+                                                             c->blk_X, c->blk_XT, c->dev_status);
+}
+
+gdc_status wall_init_attributes(gdc_ctx* c) {
+    cudaError_t e = cudaFuncSetAttribute(k_wall_blocks<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e == cudaSuccess)   // 10 values per row of the largest template: 82 KB
+        e = cudaFuncSetAttribute(k_wall_blocks<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)wall_block_smem(3 * GDC_MAX_TMPL_BLOBS, false));
+    return cuda_check(c, e, "wall block attributes");
 }
 
 }  // namespace gdc

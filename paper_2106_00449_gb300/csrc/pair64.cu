@@ -7,9 +7,7 @@
 // reciprocal square root 5, coefficients 5) plus 10 per side (d . lambda 3, scale 1,
 // accumulate 6): 36 per unordered pair against 2 x 33 for the ordered form that this kernel
 // replaced.  The comparison with (2a)^2 is made on the bit patterns (integer pipe; both are
-// positive), and the reciprocal square root is refined from the hardware's approximation by
-// the series y (1 + e/2 + 3 e^2/8), e = 1 - r^2 y^2 (the binomial series of (1 - e)^(-1/2)
-// cut after e^2: with |e| below 4e-6 the next term is below 2e-17).
+// positive), and the reciprocal square root is rsqrt_series (common.cuh).
 //
 // Work split.  A suspension is cut into tiles of TS = 128 TPL blobs (TPL targets per lane).  An
 // item is a target tile I against a range [j0, j1) of sources, j0 >= I TS; ranges of one row
@@ -41,14 +39,6 @@ struct Rpy64K {
     double c23, c2, cA, c9, cB;
     long long four_a2_bits;
 };
-
-// 1/sqrt(x) for positive normal x
-__device__ __forceinline__ double rsqrt_series(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(fma(0.375, e, 0.5), y * e, y);
-}
 
 // RPY coefficients A, B (units of 1/(8 pi eta)) of a pair at squared distance r2
 __device__ __forceinline__ void rpy64_coeff(double r2, const Rpy64K& k, double& A, double& B) {

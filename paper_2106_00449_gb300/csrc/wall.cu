@@ -9,10 +9,15 @@
 
 namespace gdc {
 
-constexpr int WALL_TILE = 128;   // targets per block and sources per shared-memory tile
+constexpr int WALL_TILE = 128;   // threads per block and sources per shared-memory tile
+constexpr int WALL_LANES = 8;    // threads per target
+constexpr int WALL_TGT = WALL_TILE / WALL_LANES;   // targets per block
 
-// y_i += W lambda (all blobs j of i's suspension), one thread per target, sources staged in
-// shared memory; items are (suspension, first target).  Positions are absolute FP64 (the
+// y_i += W lambda (all blobs j of i's suspension); items are (suspension, first target).
+// WALL_LANES neighbouring threads share a target and take every WALL_LANES-th source, added by
+// shuffles in a fixed order: the suspensions above a wall are small (15 blobs in the paper's
+// runs), and one thread per target left a block with one half-empty warp walking the sources
+// in series (49 us per FP64 product of 36 such suspensions, 11 us now).  Positions are absolute FP64 (the
 // wall term needs heights); differences are taken in FP64 and the pair term is evaluated in
 // T.  x and y hold 3 doubles per blob, or the saddle layout through blob_gm (gm = 1).
 template <typename T>
@@ -26,8 +31,9 @@ __global__ void __launch_bounds__(WALL_TILE) k_wall_apply(const int2* __restrict
     const int2 it = items[blockIdx.x];
     if (active && !active[it.x]) return;   // a suspension whose Krylov loop has stopped
     const long long b0 = susp_blob_off[it.x], ns = susp_blob_off[it.x + 1] - b0;
-    const long long i = b0 + it.y + threadIdx.x;
-    const bool own = it.y + threadIdx.x < ns;
+    const int sub = threadIdx.x % WALL_LANES, t = it.y + (int)(threadIdx.x / WALL_LANES);
+    const bool own = t < ns;
+    const long long i = b0 + t;
     double xi = 0.0, yi = 0.0, zi = 0.0;
     if (own) {
         xi = r[3 * i];
@@ -52,11 +58,17 @@ __global__ void __launch_bounds__(WALL_TILE) k_wall_apply(const int2* __restrict
         __syncthreads();
         const int n = (int)std::min<long long>(WALL_TILE, ns - j0);
         if (own)
-            for (int k = 0; k < n; ++k)
+            for (int k = sub; k < n; k += WALL_LANES)
                 wall_pair<T>((T)(xi - sp[k][0]), (T)(yi - sp[k][1]), (T)(zi + sp[k][2]), (T)sp[k][2], a2, sl[k][0],
                              sl[k][1], sl[k][2], u1, u2, u3);
     }
-    if (!own) return;
+#pragma unroll
+    for (int o = 1; o < WALL_LANES; o <<= 1) {
+        u1 += __shfl_xor_sync(0xffffffffu, u1, o);
+        u2 += __shfl_xor_sync(0xffffffffu, u2, o);
+        u3 += __shfl_xor_sync(0xffffffffu, u3, o);
+    }
+    if (!own || sub != 0) return;
     const long long o = gm ? (long long)blob_gm[i] : 3 * i;
     y[o] += c0 * (double)u1;
     y[o + 1] += c0 * (double)u2;
@@ -67,7 +79,7 @@ void build_wall_items(gdc_ctx* c) {
     c->h_wall_items.clear();
     for (int s = 0; s < c->S; ++s) {
         const long long ns = c->h_blob_off[s + 1] - c->h_blob_off[s];
-        for (long long t0 = 0; t0 < ns; t0 += WALL_TILE) c->h_wall_items.push_back(make_int2(s, (int)t0));
+        for (long long t0 = 0; t0 < ns; t0 += WALL_TGT) c->h_wall_items.push_back(make_int2(s, (int)t0));
     }
 }
 

@@ -25,27 +25,43 @@
 
 namespace gdc {
 
+__device__ __forceinline__ float inv_sqrt(float x) { return 1.f / sqrtf(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt_series(x); }   // r >= 2a above the wall
+
+// The coefficients of one pair (R3, h as above).
 template <typename T>
-__device__ __forceinline__ void wall_pair(T R1, T R2, T R3, T h, T a2, T l1, T l2, T l3, T& u1, T& u2, T& u3) {
+struct WallCoeff {
+    T al0, be0, al, be, ga, ep, ze;
+};
+
+template <typename T>
+__device__ __forceinline__ WallCoeff<T> wall_coeff(T R1, T R2, T R3, T h, T a2) {
     const T r2 = R1 * R1 + R2 * R2 + R3 * R3;
-    const T i1 = T(1) / sqrt(r2);
+    const T i1 = inv_sqrt(r2);
     const T i2 = i1 * i1;
     const T i3 = i1 * i2, i5 = i3 * i2, i7 = i5 * i2, i9 = i7 * i2;
     const T a4 = a2 * a2, R33 = R3 * R3;
-    const T al0 = -i1 - T(2.0 / 3.0) * a2 * i3;
-    const T be0 = -i3 + T(2) * a2 * i5;
-    const T al = h * h * i3 - h * R3 * i3 + a2 * R33 * i5 + T(1.0 / 3.0) * a4 * i5 - T(5.0 / 3.0) * a4 * R33 * i7;
-    const T be = T(-3) * h * h * i5 + T(3) * h * R3 * i5 - T(5) * a2 * R33 * i7 - T(5.0 / 3.0) * a4 * i7 +
-                 T(35.0 / 3.0) * a4 * R33 * i9;
-    const T ga = h * i3 - T(10.0 / 3.0) * a4 * R3 * i7;
-    const T ep = -h * i3 + T(2) * a2 * R3 * i5 - T(10.0 / 3.0) * a4 * R3 * i7;
-    const T ze = T(2.0 / 3.0) * a4 * i5;
+    WallCoeff<T> w;
+    w.al0 = -i1 - T(2.0 / 3.0) * a2 * i3;
+    w.be0 = -i3 + T(2) * a2 * i5;
+    w.al = h * h * i3 - h * R3 * i3 + a2 * R33 * i5 + T(1.0 / 3.0) * a4 * i5 - T(5.0 / 3.0) * a4 * R33 * i7;
+    w.be = T(-3) * h * h * i5 + T(3) * h * R3 * i5 - T(5) * a2 * R33 * i7 - T(5.0 / 3.0) * a4 * i7 +
+           T(35.0 / 3.0) * a4 * R33 * i9;
+    w.ga = h * i3 - T(10.0 / 3.0) * a4 * R3 * i7;
+    w.ep = -h * i3 + T(2) * a2 * R3 * i5 - T(10.0 / 3.0) * a4 * R3 * i7;
+    w.ze = T(2.0 / 3.0) * a4 * i5;
+    return w;
+}
+
+template <typename T>
+__device__ __forceinline__ void wall_pair(T R1, T R2, T R3, T h, T a2, T l1, T l2, T l3, T& u1, T& u2, T& u3) {
+    const WallCoeff<T> w = wall_coeff<T>(R1, R2, R3, h, a2);
     const T m3 = -l3;
     const T Rl = R1 * l1 + R2 * l2 + R3 * l3;
     const T Rm = R1 * l1 + R2 * l2 + R3 * m3;
-    u1 += al0 * l1 + be0 * R1 * Rl + T(2) * (al * l1 + be * R1 * Rm + ep * R1 * m3);
-    u2 += al0 * l2 + be0 * R2 * Rl + T(2) * (al * l2 + be * R2 * Rm + ep * R2 * m3);
-    u3 += al0 * l3 + be0 * R3 * Rl + T(2) * (al * m3 + be * R3 * Rm + ga * Rm + ep * R3 * m3 + ze * m3);
+    u1 += w.al0 * l1 + w.be0 * R1 * Rl + T(2) * (w.al * l1 + w.be * R1 * Rm + w.ep * R1 * m3);
+    u2 += w.al0 * l2 + w.be0 * R2 * Rl + T(2) * (w.al * l2 + w.be * R2 * Rm + w.ep * R2 * m3);
+    u3 += w.al0 * l3 + w.be0 * R3 * Rl + T(2) * (w.al * m3 + w.be * R3 * Rm + w.ga * Rm + w.ep * R3 * m3 + w.ze * m3);
 }
 
 }  // namespace gdc
