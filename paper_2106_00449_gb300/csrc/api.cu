@@ -369,11 +369,22 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->p64_jbase = w.take<long long>(S + 1);
     c->p64_part_i = w.take<double4_32a>((long long)c->p64_kmax * NBL);
     c->h_near_items.clear();
+    // search blocks of 256 targets x near_src sources: as few sources as keep the list within
+    // 64 blocks per SM (2,560 blobs at 2,048 sources ran 20 blocks for 103 us)
+    int near_src = GDC_NEAR_SRC_MIN;
+    for (; near_src < GDC_NEAR_SRC_MAX; near_src *= 2) {
+        long long items = 0;
+        for (int s = 0; s < c->S; ++s) {
+            const long long ns = c->h_blob_off[s + 1] - c->h_blob_off[s];
+            items += ((ns + 255) / 256) * ((ns + near_src - 1) / near_src);
+        }
+        if (items <= 64LL * c->num_sms) break;
+    }
     for (int s = 0; s < c->S; ++s) {
         const long long ns = c->h_blob_off[s + 1] - c->h_blob_off[s];
         for (long long t0 = 0; t0 < ns; t0 += 256)
-            for (long long j0 = 0; j0 < ns; j0 += GDC_NEAR_SRC)
-                c->h_near_items.push_back(make_int4(s, (int)t0, (int)j0, (int)std::min(ns, j0 + GDC_NEAR_SRC)));
+            for (long long j0 = 0; j0 < ns; j0 += near_src)
+                c->h_near_items.push_back(make_int4(s, (int)t0, (int)j0, (int)std::min(ns, j0 + near_src)));
     }
     c->n_near_items = (int)c->h_near_items.size();
     c->near_items = w.take<int4>(c->n_near_items);
@@ -541,10 +552,13 @@ static gdc_status fcm_template_blocks(gdc_ctx* c) {
 
 // ---- the steps -------------------------------------------------------------------------
 
-static void load_at(gdc_ctx* c, const double* Y, const double* q) {
+// near: the configuration's near-pair lists too, which FP32 products correct their pairs with
+static void load_at(gdc_ctx* c, const double* Y, const double* q, bool near) {
     launch_ref(c, Y);
-    load_config(c, Y, q);
+    load_config(c, Y, q, near);
 }
+
+static bool mixed(const gdc_ctx* c) { return c->p.precision == GDC_FP32_MIXED; }
 
 static gdc_status forces_at_loaded(gdc_ctx* c, double* FT) {
     if (forces_on(c->p) || c->p.wall) {
@@ -594,7 +608,7 @@ static gdc_status one_step(gdc_ctx* c, gdc_step_info* info) {
     launch_normals(c, c->step, 1, c->Wt);
     if (c->p.scheme == GDC_SCHEME_EM) {
         // App. D: one full solve at x^n, then x^(n+1) = x^n + dt V^n
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, mixed(c));
         forces_at_loaded(c, c->FT);
         if ((st = slip_at_loaded(c, c->W, c->vb_m, 0, &inf.lanczos_iters[2], &inf.lanczos_err)) != GDC_OK) return st;
         launch_rhs(c, c->vb_m, c->FT, c->gm_b);
@@ -606,14 +620,14 @@ static gdc_status one_step(gdc_ctx* c, gdc_step_info* info) {
         matvecs = inf.lanczos_iters[2] + inf.solve.matvecs_fp32 + inf.solve.matvecs_fp64;
     } else {
         // step 2 at x^n
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, mixed(c));
         if ((st = slip_at_loaded(c, c->W, c->vb_n, 0, &inf.lanczos_iters[0], &inf.lanczos_err)) != GDC_OK) return st;
         launch_lsq(c, c->vb_n, c->calV);
         // step 3: divergence of calV
         double e2 = 0.0;
         if (c->p.divmode == GDC_DIV_RFD) {
             launch_perturb(c, c->Y, c->q, c->Wt, c->p.rfd_delta, c->Yt, c->qt);
-            load_config(c, c->Yt, c->qt);  // same reference point as x^n
+            load_config(c, c->Yt, c->qt, mixed(c));  // same reference point as x^n
             cudaMemcpyAsync(c->lz_fix, c->lz_k, sizeof(int) * c->S, cudaMemcpyDeviceToDevice, c->stream);
             if ((st = slip_at_loaded(c, c->W, c->vb_t, 1, &inf.lanczos_iters[1], &e2)) != GDC_OK) return st;
             launch_lsq(c, c->vb_t, c->calVt);
@@ -625,7 +639,7 @@ static gdc_status one_step(gdc_ctx* c, gdc_step_info* info) {
             for (int pl = 0; pl < maxn; ++pl)
                 for (int coord = 0; coord < 6; ++coord) {
                     launch_perturb_one(c, c->Y, c->q, pl, coord, c->p.rfd_delta, c->Yt, c->qt);
-                    load_config(c, c->Yt, c->qt);
+                    load_config(c, c->Yt, c->qt, mixed(c));
                     int it = 0;
                     if ((st = slip_at_loaded(c, c->W, c->vb_t, 1, &it, &e2)) != GDC_OK) return st;
                     inf.lanczos_iters[1] += it;
@@ -637,7 +651,7 @@ static gdc_status one_step(gdc_ctx* c, gdc_step_info* info) {
         // step 4: mid-step
         launch_advance(c, c->Y, c->q, c->calV, 0.5 * dt, nullptr, c->Ym, c->qm);
         // step 5: forces and the full mobility solve at the mid-step, same W
-        load_at(c, c->Ym, c->qm);
+        load_at(c, c->Ym, c->qm, mixed(c));
         forces_at_loaded(c, c->FT);
         double e3 = 0.0;
         if ((st = slip_at_loaded(c, c->W, c->vb_m, 0, &inf.lanczos_iters[2], &e3)) != GDC_OK) return st;
@@ -761,7 +775,7 @@ static void enqueue_step_graph(gdc_ctx* c) {
     launch_normals(c, 0, 1, c->Wt, sd);
     const bool gdc_scheme = c->p.scheme != GDC_SCHEME_EM;
     if (!gdc_scheme) {
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, mixed(c));
         forces_at_loaded(c, c->FT);
         graph_slip(c, c->W, c->vb_m, 0, 2);
         launch_rhs(c, c->vb_m, c->FT, c->gm_b);
@@ -770,17 +784,17 @@ static void enqueue_step_graph(gdc_ctx* c) {
         ++c->n_launch, k_step_ok<<<1, 1, 0, c->stream>>>(c->rep, c->dev_status);
         launch_advance(c, c->Y, c->q, c->Vm, dt, nullptr, c->Y, c->q, &c->rep->ok);
     } else {
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, mixed(c));
         graph_slip(c, c->W, c->vb_n, 0, 0);
         launch_lsq(c, c->vb_n, c->calV);
         launch_perturb(c, c->Y, c->q, c->Wt, c->p.rfd_delta, c->Yt, c->qt);
-        load_config(c, c->Yt, c->qt);
+        load_config(c, c->Yt, c->qt, mixed(c));
         cudaMemcpyAsync(c->lz_fix, c->lz_k, sizeof(int) * c->S, cudaMemcpyDeviceToDevice, c->stream);
         graph_slip(c, c->W, c->vb_t, 1, 1);
         launch_lsq(c, c->vb_t, c->calVt);
         launch_rfd_div(c, c->Wt, c->calV, c->calVt, c->p.rfd_delta, dt, c->nu);
         launch_advance(c, c->Y, c->q, c->calV, 0.5 * dt, nullptr, c->Ym, c->qm);
-        load_at(c, c->Ym, c->qm);
+        load_at(c, c->Ym, c->qm, mixed(c));
         forces_at_loaded(c, c->FT);
         graph_slip(c, c->W, c->vb_m, 0, 2);
         launch_rhs(c, c->vb_m, c->FT, c->gm_b);
@@ -990,11 +1004,11 @@ gdc_status gdc_init(gdc_ctx** out, const gdc_params* params, int n_templates, co
     if ((st = dfsym_init_attributes(c)) != GDC_OK) return st;
     if (c->p.wall) {   // every blob must start above z = a
         if ((st = wall_init_attributes(c)) != GDC_OK) return st;
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, false);
         if ((st = read_status(c)) != GDC_OK) return st;
     }
     if (c->p.autotune && c->p.mobility == GDC_MOB_RPY) {   // the RPY pair kernels only
-        load_at(c, c->Y, c->q);
+        load_at(c, c->Y, c->q, false);
         if ((st = autotune_pair_kernel(c)) != GDC_OK) return st;
     } else if ((st = default_pair_kernel(c)) != GDC_OK) {
         return st;
@@ -1090,7 +1104,7 @@ gdc_status gdc_mobility_solve(gdc_ctx* c, const double* FT, const double* vbrev,
                               gdc_solve_info* info) {
     if (!c) return GDC_ERR_INVALID_ARG;
     if (!FT || !V) return fail(c, GDC_ERR_INVALID_ARG, "FT and V are required");
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, mixed(c));
     launch_rhs(c, vbrev, FT, c->gm_b);
     gdc_solve_info inf{};
     gdc_status st = gmres_solve(c, c->gm_b, c->gm_x, &inf);
@@ -1147,7 +1161,7 @@ gdc_status gdc_set_state(gdc_ctx* c, const double* Y, const double* q, unsigned 
 
 gdc_status gdc_blob_positions(gdc_ctx* c, double* r) {
     if (!c || !r) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL output") : GDC_ERR_INVALID_ARG;
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, false);
     cudaMemcpyAsync(r, c->r, sizeof(double) * 3 * c->NBL, cudaMemcpyDeviceToDevice, c->stream);
     return cuda_check(c, cudaStreamSynchronize(c->stream), "blob positions");
 }
@@ -1156,7 +1170,7 @@ gdc_status gdc_rpy_apply(gdc_ctx* c, int precision, const double* lam, double* u
     if (!c || !lam || !u) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
     if (precision != GDC_FP64 && precision != GDC_FP32_MIXED && precision != GDC_DF64_RESIDUAL)
         return fail(c, GDC_ERR_INVALID_ARG, "unknown precision");
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, precision == GDC_FP32_MIXED);
     rpy_op(c, precision, lam, u);
     gdc_status st = cuda_check(c, cudaStreamSynchronize(c->stream), "rpy apply");
     return st != GDC_OK ? st : read_status(c);
@@ -1166,7 +1180,7 @@ gdc_status gdc_saddle_apply(gdc_ctx* c, int precision, const double* x, double* 
     if (!c || !x || !y) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
     if (precision != GDC_FP64 && precision != GDC_FP32_MIXED && precision != GDC_DF64_RESIDUAL)
         return fail(c, GDC_ERR_INVALID_ARG, "unknown precision");
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, precision == GDC_FP32_MIXED);
     saddle_op(c, precision, x, y);
     gdc_status st = cuda_check(c, cudaStreamSynchronize(c->stream), "saddle apply");
     return st != GDC_OK ? st : read_status(c);
@@ -1174,14 +1188,14 @@ gdc_status gdc_saddle_apply(gdc_ctx* c, int precision, const double* x, double* 
 
 gdc_status gdc_precond_apply(gdc_ctx* c, const double* r, double* z) {
     if (!c || !r || !z) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, false);
     launch_precond(c, r, z);
     return cuda_check(c, cudaStreamSynchronize(c->stream), "precond apply");
 }
 
 gdc_status gdc_brownian_slip(gdc_ctx* c, const double* W, double* vbrev, int* iters, double* err) {
     if (!c || !W || !vbrev) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, mixed(c));
     gdc_status st = slip_at_loaded(c, W, vbrev, 0, iters, err);
     const gdc_status e2 = cuda_check(c, cudaStreamSynchronize(c->stream), "brownian slip");
     return e2 != GDC_OK ? e2 : settle(c, st);
@@ -1189,14 +1203,14 @@ gdc_status gdc_brownian_slip(gdc_ctx* c, const double* W, double* vbrev, int* it
 
 gdc_status gdc_lsq_velocity(gdc_ctx* c, const double* vbrev, double* calV) {
     if (!c || !vbrev || !calV) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, false);
     launch_lsq(c, vbrev, calV);
     return cuda_check(c, cudaStreamSynchronize(c->stream), "lsq velocity");
 }
 
 gdc_status gdc_forces(gdc_ctx* c, double* FT) {
     if (!c || !FT) return c ? fail(c, GDC_ERR_INVALID_ARG, "NULL pointer") : GDC_ERR_INVALID_ARG;
-    load_at(c, c->Y, c->q);
+    load_at(c, c->Y, c->q, false);
     forces_at_loaded(c, FT);
     return cuda_check(c, cudaStreamSynchronize(c->stream), "forces");
 }

@@ -31,7 +31,9 @@
 #define GDC_MAX_TMPL_BLOBS 340   // 3n <= 1020 rows of a template block
 #define GDC_TB_MAX 8             // bodies of one template per block in the factor products
 #define GDC_NEAR_CAP 32          // blobs closer than 2a listed per blob (beyond: a search of the suspension)
-#define GDC_NEAR_SRC 2048        // sources per block of the near-pair search
+#define GDC_EPI_WIDE 32768       // FP32 product epilogue: 8 threads per blob up to this many blobs, one above
+#define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
+#define GDC_NEAR_SRC_MAX 2048
 #define GDC_SYM_TILE 512         // blobs per tile of the symmetric FP32 pair kernel
 #ifndef GDC_DFS_WIDTH
 #define GDC_DFS_WIDTH 2          // source tiles per item of the symmetric double-float kernel
@@ -368,7 +370,7 @@ void prof_flush(gdc_ctx* c);
 
 // ---- kernels launched across translation units ----------------------------
 // geometry.cu
-void load_config(gdc_ctx* c, const double* Y, const double* q);
+void load_config(gdc_ctx* c, const double* Y, const double* q, bool near);   // near: the near-pair lists too
 void launch_ref(gdc_ctx* c, const double* Y);
 void launch_normals(gdc_ctx* c, unsigned long long step, int stream, double* out,
                     const unsigned long long* step_dev = nullptr);

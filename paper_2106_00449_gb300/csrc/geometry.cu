@@ -47,12 +47,12 @@ __global__ void k_blob_pos(int NBL, const int* __restrict__ blob_body, const int
     spos64[i] = make_double4_32a(rx, ry, rz, (double)p);
 }
 
-void load_config(gdc_ctx* c, const double* Y, const double* q) {
+void load_config(gdc_ctx* c, const double* Y, const double* q, bool near) {
     ++c->n_launch, k_body_rot<<<ceil_div(c->NB, 128), 128, 0, c->stream>>>(c->NB, Y, q, c->Rb, c->Yc);
     ++c->n_launch, k_blob_pos<<<ceil_div(c->NBL, 128), 128, 0, c->stream>>>(
         c->NBL, c->blob_body, c->blob_susp, c->body_tmpl, c->body_blob_off, c->tmpl_off, c->tmpl_xyz,
         Y, c->Rb, c->ref, c->r, c->spos, c->spos64);
-    launch_near_build(c);   // pairs closer than 2a, corrected after every FP32 product
+    if (near) launch_near_build(c);   // pairs closer than 2a, corrected after every FP32 product
     if (c->p.wall) launch_wall_blocks(c);   // a wall: per-body blocks depend on the configuration
 }
 

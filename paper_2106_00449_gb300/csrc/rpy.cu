@@ -337,15 +337,16 @@ __device__ inline void near_delta(float a, float r, float& dA, float& dB) {
 // pairs with blobs of other bodies closer than 2a: from the list when it holds them all, else
 // by a search of the suspension's blobs [so, se) (FP64 distances; blob_body given: skip
 // same-body blobs, else only j = i).  x holds lambda, 3 per blob, or in the saddle layout
-// through gm (blob -> offset) when gm is given.
+// through gm (blob -> offset) when gm is given.  Entries sub, sub + nsub, ... are taken.
 __device__ inline void near_pair_correction(long long i, long long so, long long se, const int* __restrict__ near_cnt,
                                             const int* __restrict__ near_idx, const int* __restrict__ blob_body,
                                             const double* __restrict__ r, const double* __restrict__ x,
-                                            const int* __restrict__ gm, double a, double& ux, double& uy, double& uz) {
+                                            const int* __restrict__ gm, double a, int sub, int nsub, double& ux,
+                                            double& uy, double& uz) {
     const int m = near_cnt[i];
     const double four_a2 = 4.0 * a * a;
     const long long cnt = m <= GDC_NEAR_CAP ? m : se - so;
-    for (long long q = 0; q < cnt; ++q) {
+    for (long long q = sub; q < cnt; q += nsub) {
         const long long j = m <= GDC_NEAR_CAP ? (long long)near_idx[i * GDC_NEAR_CAP + q] : so + q;
         if (j == i || (blob_body && blob_body[j] == blob_body[i])) continue;
         const double dx = r[3 * j] - r[3 * i], dy = r[3 * j + 1] - r[3 * i + 1], dz = r[3 * j + 2] - r[3 * i + 2];
@@ -362,21 +363,39 @@ __device__ inline void near_pair_correction(long long i, long long so, long long
     }
 }
 
-// Subtracts from (ux, uy, uz) the terms the FP32 pair kernel added for blob i's own body
-// [j0, j1) (self pair included), recomputed from the same FP32 operands with the same
-// operations, so that the FP32 rounding of those near-field terms cancels; the intra-body
-// kernel then adds the same-body block of the body's template.
-__device__ inline void same_body_subtract(const float4 pt, long long j0, long long j1, const float4* __restrict__ sdup,
-                                          const RpyConst32& k, double& ux, double& uy, double& uz) {
-    // summed in FP32 with compensation (FP64 adds are slow on GB300), subtracted once
-    float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
-    auto kahan = [](float& sum, float& comp, float v) {
+// A sum in FP32 with compensation (FP64 adds are slow on GB300): sum - comp is the value.
+struct Kahan {
+    float sum = 0.f, comp = 0.f;
+    __device__ __forceinline__ void add(float v) {
         const float y = __fsub_rn(v, comp);
         const float t = __fadd_rn(sum, y);
         comp = __fsub_rn(__fsub_rn(t, sum), y);
         sum = t;
-    };
-    for (long long j = j0; j < j1; ++j) {
+    }
+    // the sum over a group of EPI neighbouring lanes, on every lane: exact two-sums of the
+    // leading parts, their errors joined with the compensations
+    template <int EPI>
+    __device__ __forceinline__ void group() {
+#pragma unroll
+        for (int o = 1; o < EPI; o <<= 1) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, sum, o), c2 = __shfl_xor_sync(0xffffffffu, comp, o);
+            const float t = __fadd_rn(sum, s2), bb = __fsub_rn(t, sum);
+            const float err = __fadd_rn(__fsub_rn(sum, __fsub_rn(t, bb)), __fsub_rn(s2, bb));
+            comp = __fsub_rn(__fadd_rn(comp, c2), err);
+            sum = t;
+        }
+    }
+    __device__ __forceinline__ double value() const { return (double)sum - (double)comp; }
+};
+
+// Subtracts from (sx, sy, sz) the terms the FP32 pair kernel added for blob i's own body
+// [j0, j1) (self pair included), recomputed from the same FP32 operands with the same
+// operations, so that the FP32 rounding of those near-field terms cancels; the intra-body
+// kernel then adds the same-body block of the body's template.  Blobs j0 + sub, j0 + sub +
+// nsub, ... are taken.
+__device__ inline void same_body_subtract(const float4 pt, long long j0, long long j1, const float4* __restrict__ sdup,
+                                          const RpyConst32& k, int sub, int nsub, Kahan& sx, Kahan& sy, Kahan& sz) {
+    for (long long j = j0 + sub; j < j1; j += nsub) {
         const float4 s0 = sdup[3 * j], s1 = sdup[3 * j + 1], s2 = sdup[3 * j + 2];
         const float dx = __fsub_rn(s0.x, pt.x), dy = __fsub_rn(s0.z, pt.y), dz = __fsub_rn(s1.x, pt.z);
         const float lx = s1.z, ly = s2.x, lz = s2.z;
@@ -386,21 +405,24 @@ __device__ inline void same_body_subtract(const float4 pt, long long j0, long lo
         const float A = __fmaf_rn(k.c23, ri3, ri);
         const float B = __fmul_rn(ri3, __fmaf_rn(-k.c2, ri2, 1.f));
         const float sj = __fmul_rn(B, __fmaf_rn(dx, lx, __fmaf_rn(dy, ly, __fmul_rn(dz, lz))));
-        kahan(sx, cx, __fmaf_rn(A, lx, __fmul_rn(sj, dx)));
-        kahan(sy, cy, __fmaf_rn(A, ly, __fmul_rn(sj, dy)));
-        kahan(sz, cz, __fmaf_rn(A, lz, __fmul_rn(sj, dz)));
+        sx.add(-__fmaf_rn(A, lx, __fmul_rn(sj, dx)));
+        sy.add(-__fmaf_rn(A, ly, __fmul_rn(sj, dy)));
+        sz.add(-__fmaf_rn(A, lz, __fmul_rn(sj, dz)));
     }
-    ux -= (double)sx - (double)cx;
-    uy -= (double)sy - (double)cy;
-    uz -= (double)sz - (double)cz;
 }
 
 // u_i = c0 (sum of the chunk partial sums [+ near-pair corrections]) [- K V]
 //
 // near_cnt != 0 (FP32 products): corrects the pairs of other bodies closer than 2a and takes
 // out the pair kernel's same-body terms (the intra-body kernel adds the template's block).
-template <typename P>
-__global__ void k_rpy_epilogue(int NBL, const P* __restrict__ part, const int* __restrict__ blob_susp,
+//
+// EPI neighbouring threads share a blob: they take every EPI-th slot, same-body blob and near
+// pair, joined by shuffles in a fixed order.  8 threads up to GDC_EPI_WIDE blobs, where the
+// chain of dependent loads of one thread is what the launch waits for (2,560 blobs: 12.9 us
+// at one thread per blob); one thread above it, where the FP64 tail (2 lanes per clock per
+// SM, paid per warp) would cost more than the chain.
+template <typename P, int EPI>
+__global__ void __launch_bounds__(256) k_rpy_epilogue(int NBL, const P* __restrict__ part, const int* __restrict__ blob_susp,
                                const int* __restrict__ nk, double c0, const double* __restrict__ x,
                                double* __restrict__ y, int gm_layout, const int* __restrict__ blob_gm,
                                const int* __restrict__ body_gm, const int* __restrict__ blob_body,
@@ -410,45 +432,39 @@ __global__ void k_rpy_epilogue(int NBL, const P* __restrict__ part, const int* _
                                const float4* __restrict__ spos, const float4* __restrict__ sdup, RpyConst32 k32,
                                const float4* __restrict__ sym_part_j, const int* __restrict__ sym_row_nk,
                                const long long* __restrict__ sym_tile_base, const long long* __restrict__ sym_jbase) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NBL) return;
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int sub = (int)(tid % EPI);
+    const bool in = tid / EPI < NBL;
+    const int i = in ? (int)(tid / EPI) : NBL - 1;   // whole warps reach the shuffles
     double ux = 0.0, uy = 0.0, uz = 0.0;
+    Kahan sx, sy, sz;
     if (sym_part_j) {
         // symmetric kernel: the target-side slots of the blob's tile row, then the source-side
         // slots (I, J) of every tile I before the blob's tile J, in order.  FP32 partials are
-        // added with compensation in FP32 (GB300 adds in FP64 at a small fraction of the FP32
-        // rate), then converted once.
+        // added with compensation in FP32, then converted once.
         const int s = blob_susp[i];
         const long long loc = i - susp_blob_off[s];
         const int J = (int)(loc / GDC_SYM_TILE), e = (int)(loc % GDC_SYM_TILE);
         const int n = sym_row_nk[sym_tile_base[s] + J];
         const float4* pi = reinterpret_cast<const float4*>(part);
-        float sx = 0.f, sy = 0.f, sz = 0.f, kx = 0.f, ky = 0.f, kz = 0.f;
-        auto kahan = [](float& sum, float& comp, float v) {
-            const float y = __fsub_rn(v, comp);
-            const float t = __fadd_rn(sum, y);
-            comp = __fsub_rn(__fsub_rn(t, sum), y);
-            sum = t;
-        };
-        for (int k = 0; k < n; ++k) {
+#pragma unroll 4
+        for (int k = sub; k < n; k += EPI) {
             const float4 v = pi[(long long)k * NBL + i];
-            kahan(sx, kx, v.x);
-            kahan(sy, ky, v.y);
-            kahan(sz, kz, v.z);
+            sx.add(v.x);
+            sy.add(v.y);
+            sz.add(v.z);
         }
         const long long s0 = sym_jbase[s] + (long long)J * (J - 1) / 2;
-        for (int I = 0; I < J; ++I) {
+#pragma unroll 4
+        for (int I = sub; I < J; I += EPI) {
             const float4 v = sym_part_j[(s0 + I) * GDC_SYM_TILE + e];
-            kahan(sx, kx, v.x);
-            kahan(sy, ky, v.y);
-            kahan(sz, kz, v.z);
+            sx.add(v.x);
+            sy.add(v.y);
+            sz.add(v.z);
         }
-        ux = (double)sx - (double)kx;
-        uy = (double)sy - (double)ky;
-        uz = (double)sz - (double)kz;
     } else {
         const int n = nk[blob_susp[i]];
-        for (int k = 0; k < n; ++k) {
+        for (int k = sub; k < n; k += EPI) {
             double a0, b, cc;
             load_part(part, (long long)k * NBL + i, a0, b, cc);
             ux += a0;
@@ -456,12 +472,31 @@ __global__ void k_rpy_epilogue(int NBL, const P* __restrict__ part, const int* _
             uz += cc;
         }
     }
+    bool join64 = true;   // FP64 parts to join
     if (near_cnt) {
-        const long long so = susp_blob_off[blob_susp[i]], se = susp_blob_off[blob_susp[i] + 1];
-        near_pair_correction(i, so, se, near_cnt, near_idx, blob_body, r, x, gm_layout ? blob_gm : nullptr, a, ux, uy,
-                             uz);
         const int p = blob_body[i];
-        same_body_subtract(spos[i], body_blob_off[p], body_blob_off[p + 1], sdup, k32, ux, uy, uz);
+        same_body_subtract(spos[i], body_blob_off[p], body_blob_off[p + 1], sdup, k32, sub, EPI, sx, sy, sz);
+        sx.group<EPI>();
+        sy.group<EPI>();
+        sz.group<EPI>();
+        const long long so = susp_blob_off[blob_susp[i]], se = susp_blob_off[blob_susp[i] + 1];
+        near_pair_correction(i, so, se, near_cnt, near_idx, blob_body, r, x, gm_layout ? blob_gm : nullptr, a, sub, EPI,
+                             ux, uy, uz);
+        join64 = !sym_part_j || __any_sync(0xffffffffu, near_cnt[i] != 0);
+    }
+    if (EPI > 1 && join64) {
+#pragma unroll
+        for (int o = 1; o < EPI; o <<= 1) {
+            ux += __shfl_xor_sync(0xffffffffu, ux, o);
+            uy += __shfl_xor_sync(0xffffffffu, uy, o);
+            uz += __shfl_xor_sync(0xffffffffu, uz, o);
+        }
+    }
+    if (!in || sub != 0) return;
+    if (near_cnt) {
+        ux += sx.value();
+        uy += sy.value();
+        uz += sz.value();
     }
     ux *= c0;
     uy *= c0;
@@ -507,20 +542,30 @@ void launch_fcm_saddle_rows(gdc_ctx* c, const double* x, double* y) {
         c->NBL, c->fcm_u, x, y, c->blob_gm, c->body_gm, c->blob_body, c->r, c->Yc);
 }
 
+template <typename P, int EPI>
+static void launch_epilogue_t(gdc_ctx* c, const P* part, bool sym, double c0, const double* x, double* y, int gm_layout,
+                              bool near) {
+    ++c->n_launch, k_rpy_epilogue<P, EPI><<<ceil_div((long long)EPI * c->NBL, 256), 256, 0, c->stream>>>(
+        c->NBL, part, c->blob_susp, c->mv_nk, c0, x, y, gm_layout, c->blob_gm, c->body_gm, c->blob_body, c->r, c->Yc,
+        near ? c->near_cnt : nullptr, c->near_idx, c->p.a, c->susp_blob_off, c->body_blob_off, c->spos, c->sdup,
+        rpy_const32(c->p.a), sym ? c->sym_part_j : nullptr, c->sym_row_nk, c->sym_tile_base, c->sym_jbase);
+}
+
 static void launch_epilogue(gdc_ctx* c, int prec, double c0, const double* x, double* y, int gm_layout,
                             bool near) {
     const bool sym = prec == GDC_FP32_MIXED && near && c->use_sym;   // RPY products only, not forces
-    if (prec == GDC_FP32_MIXED)
-        ++c->n_launch, k_rpy_epilogue<float4><<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(
-            c->NBL, sym ? c->sym_part_i : (const float4*)c->mv_part, c->blob_susp, c->mv_nk, c0, x, y, gm_layout,
-            c->blob_gm, c->body_gm, c->blob_body, c->r, c->Yc, near ? c->near_cnt : nullptr, c->near_idx, c->p.a,
-            c->susp_blob_off, c->body_blob_off, c->spos, c->sdup, rpy_const32(c->p.a), sym ? c->sym_part_j : nullptr,
-            c->sym_row_nk, c->sym_tile_base, c->sym_jbase);
-    else
-        ++c->n_launch, k_rpy_epilogue<double4_32a><<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(
-            c->NBL, (const double4_32a*)c->mv_part, c->blob_susp, c->mv_nk, c0, x, y, gm_layout, c->blob_gm, c->body_gm,
-            c->blob_body, c->r, c->Yc, nullptr, nullptr, c->p.a, c->susp_blob_off, c->body_blob_off, c->spos, c->sdup,
-            rpy_const32(c->p.a), nullptr, nullptr, nullptr, nullptr);
+    const bool wide = c->NBL > GDC_EPI_WIDE;
+    if (prec == GDC_FP32_MIXED) {
+        const float4* part = sym ? c->sym_part_i : (const float4*)c->mv_part;
+        if (wide)
+            launch_epilogue_t<float4, 1>(c, part, sym, c0, x, y, gm_layout, near);
+        else
+            launch_epilogue_t<float4, 8>(c, part, sym, c0, x, y, gm_layout, near);
+    } else if (wide) {
+        launch_epilogue_t<double4_32a, 1>(c, (const double4_32a*)c->mv_part, false, c0, x, y, gm_layout, false);
+    } else {
+        launch_epilogue_t<double4_32a, 8>(c, (const double4_32a*)c->mv_part, false, c0, x, y, gm_layout, false);
+    }
 }
 
 void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout, bool same_body) {
@@ -545,11 +590,19 @@ void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int g
 // suspension, two targets per thread in packed arithmetic; a found pair takes the next slot
 // of its target's list (near_cnt starts at zero), and k_near_sort then orders every list so
 // that the corrections are summed in a fixed order.
-__global__ void __launch_bounds__(128) k_near_build(const int4* __restrict__ items, const long long* __restrict__ susp_blob_off,
+// items = nullptr: one suspension, blocks in rows of `chunks` chunks of `src` sources.
+__global__ void __launch_bounds__(128) k_near_build(const int4* __restrict__ items, int chunks, int src,
+                                                   const long long* __restrict__ susp_blob_off,
                                                    const float4* __restrict__ spos, float four_a2,
                                                    int* __restrict__ near_cnt, int* __restrict__ near_idx) {
     __shared__ float4 sh[2 * 256];
-    const int4 it = items[blockIdx.x];   // (suspension, first target, first source, end source)
+    int4 it;   // (suspension, first target, first source, end source)
+    if (items) {
+        it = items[blockIdx.x];
+    } else {
+        const int n = (int)susp_blob_off[1], j0 = (int)(blockIdx.x % chunks) * src;
+        it = make_int4(0, (int)(blockIdx.x / chunks) * 256, j0, min(n, j0 + src));
+    }
     const long long b0 = susp_blob_off[it.x];
     const int ns = (int)(susp_blob_off[it.x + 1] - b0);
     const int ta = it.y + (int)threadIdx.x, tb = ta + 128;
@@ -611,7 +664,7 @@ void launch_near_build(gdc_ctx* c) {
         launch_near_cell(c);   // the same lists from a cell list, O(N_b)
     } else {
         cudaMemsetAsync(c->near_cnt, 0, sizeof(int) * c->NBL, c->stream);
-        ++c->n_launch, k_near_build<<<c->n_near_items, 128, 0, c->stream>>>(c->near_items, c->susp_blob_off, c->spos,
+        ++c->n_launch, k_near_build<<<c->n_near_items, 128, 0, c->stream>>>(c->near_items, 0, 0, c->susp_blob_off, c->spos,
                                                                             (float)(4.0 * c->p.a * c->p.a), c->near_cnt,
                                                                             c->near_idx);
     }
@@ -969,17 +1022,18 @@ gdc_status default_pair_kernel(gdc_ctx* c) {
 
 #include <mutex>
 
-#define GDC_NOALLOC_MAX_CHUNKS 16
+#define GDC_NOALLOC_SLOTS (16 * GDC_NOALLOC_MAX_BLOBS)   // partial sums: chunks x blobs of a call
 #define GDC_NOALLOC_TILE 256   // targets per work item (two per thread)
+#define GDC_NOALLOC_ITEMS 2048 // work items of a call
+#define GDC_NOALLOC_EPI 8      // threads per blob of the epilogue
 
 namespace gdc {
 
 struct NoallocScratch {
     float4 spos[GDC_NOALLOC_MAX_BLOBS];
     float4 sdup[3 * GDC_NOALLOC_MAX_BLOBS];
-    float4 part[GDC_NOALLOC_MAX_CHUNKS * GDC_NOALLOC_MAX_BLOBS];
-    MvItem items[(GDC_NOALLOC_MAX_BLOBS / GDC_NOALLOC_TILE) * GDC_NOALLOC_MAX_CHUNKS];
-    int4 near_items[(GDC_NOALLOC_MAX_BLOBS / 256) * (GDC_NOALLOC_MAX_BLOBS / GDC_NEAR_SRC)];
+    float4 part[GDC_NOALLOC_SLOTS];
+    MvItem items[GDC_NOALLOC_ITEMS];
     int near_cnt[GDC_NOALLOC_MAX_BLOBS];
     int near_idx[GDC_NOALLOC_MAX_BLOBS * GDC_NEAR_CAP];
     long long susp_blob_off[2];
@@ -990,21 +1044,24 @@ struct NoallocScratch {
 static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 
 // Start of a call: the blob centroid (one block; per-thread strided sums added in a fixed
-// tree order, so the result does not depend on timing) and the status words cleared.
-__global__ void __launch_bounds__(256) k_noalloc_begin(NoallocScratch* __restrict__ sc, const double* __restrict__ r,
-                                                       int n) {
-    __shared__ double part[3][256];
+// order, so the result does not depend on timing) and the status words cleared.
+__global__ void __launch_bounds__(1024) k_noalloc_begin(NoallocScratch* __restrict__ sc, const double* __restrict__ r,
+                                                        int n) {
+    __shared__ double part[3][32];
     double acc[3] = {0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < n; i += 256)
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += 1024)
         for (int d = 0; d < 3; ++d) acc[d] += r[3 * i + d];
-    for (int d = 0; d < 3; ++d) part[d][threadIdx.x] = acc[d];
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h)
-            for (int d = 0; d < 3; ++d) part[d][threadIdx.x] += part[d][threadIdx.x + h];
-        __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int d = 0; d < 3; ++d) {
+        const double v = warp_sum(acc[d]);
+        if (lane == 0) part[d][warp] = v;
     }
-    if (threadIdx.x < 3) sc->cen[threadIdx.x] = part[threadIdx.x][0] / n;
+    __syncthreads();
+    if (warp < 3) {
+        const double v = warp_sum(part[warp][lane]);
+        if (lane == 0) sc->cen[warp] = v / n;
+    }
     if (threadIdx.x < 4) sc->status[threadIdx.x] = 0;
 }
 
@@ -1014,10 +1071,6 @@ __global__ void k_noalloc_prepare(NoallocScratch* __restrict__ sc, const double*
     const double c0 = sc->cen[0], c1 = sc->cen[1], c2 = sc->cen[2];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         sc->near_cnt[i] = 0;
-        if (i % 256 == 0)   // near-pair blocks: 256 targets x source chunks of GDC_NEAR_SRC
-            for (int j0 = 0, q = 0; j0 < n; j0 += GDC_NEAR_SRC, ++q)
-                sc->near_items[(i / 256) * ((n + GDC_NEAR_SRC - 1) / GDC_NEAR_SRC) + q] =
-                    make_int4(0, i, j0, min(n, j0 + GDC_NEAR_SRC));
         const float x = (float)(r[3 * i] - c0), y = (float)(r[3 * i + 1] - c1), z = (float)(r[3 * i + 2] - c2);
         const float lx = (float)lam[3 * i], ly = (float)lam[3 * i + 1], lz = (float)lam[3 * i + 2];
         sc->spos[i] = make_float4(x, y, z, __int_as_float(i));
@@ -1041,29 +1094,43 @@ __global__ void k_noalloc_prepare(NoallocScratch* __restrict__ sc, const double*
     }
 }
 
-// u_i = c0 (sum of chunk partials + self-pair and near-pair corrections)
-__global__ void k_noalloc_epilogue(const NoallocScratch* __restrict__ sc, const double* __restrict__ r,
-                                   const double* __restrict__ lam, int n, int nk, double c0, double a,
-                                   double* __restrict__ u) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (sc->status[1] != 0) {   // a tile copy of the pair kernel timed out: u would be incomplete
-        u[3 * i] = u[3 * i + 1] = u[3 * i + 2] = __longlong_as_double(0x7ff8000000000000LL);
-        return;
-    }
+// u_i = c0 (sum of chunk partials + self-pair and near-pair corrections), GDC_NOALLOC_EPI
+// neighbouring threads per blob (at most 16,384 blobs: the chain of one thread's dependent loads
+// is what a launch waits for)
+__global__ void __launch_bounds__(256) k_noalloc_epilogue(const NoallocScratch* __restrict__ sc,
+                                                          const double* __restrict__ r, const double* __restrict__ lam,
+                                                          int n, int nk, double c0, double a, double* __restrict__ u) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int sub = tid % GDC_NOALLOC_EPI;
+    const bool in = tid / GDC_NOALLOC_EPI < n;
+    const int i = in ? tid / GDC_NOALLOC_EPI : n - 1;   // whole warps reach the shuffles
     double x = 0.0, y = 0.0, z = 0.0;
-    for (int k = 0; k < nk; ++k) {
-        const float4 v = sc->part[(long long)k * GDC_NOALLOC_MAX_BLOBS + i];
+#pragma unroll 4
+    for (int k = sub; k < nk; k += GDC_NOALLOC_EPI) {
+        const float4 v = sc->part[(long long)k * n + i];
         x += v.x;
         y += v.y;
         z += v.z;
     }
-    // self pair: exact 4/(3a), clamped far field 7/(12a) (d = 0, so FP32 leaves only the rsqrt rounding)
-    const double cs = 4.0 / (3.0 * a) - 7.0 / (12.0 * a);
-    x += cs * lam[3 * i];
-    y += cs * lam[3 * i + 1];
-    z += cs * lam[3 * i + 2];
-    near_pair_correction(i, 0, n, sc->near_cnt, sc->near_idx, nullptr, r, lam, nullptr, a, x, y, z);
+    if (sub == 0) {
+        // self pair: exact 4/(3a), clamped far field 7/(12a) (d = 0, so FP32 leaves only the rsqrt rounding)
+        const double cs = 4.0 / (3.0 * a) - 7.0 / (12.0 * a);
+        x += cs * lam[3 * i];
+        y += cs * lam[3 * i + 1];
+        z += cs * lam[3 * i + 2];
+    }
+    near_pair_correction(i, 0, n, sc->near_cnt, sc->near_idx, nullptr, r, lam, nullptr, a, sub, GDC_NOALLOC_EPI, x, y, z);
+#pragma unroll
+    for (int o = 1; o < GDC_NOALLOC_EPI; o <<= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+        z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    if (!in || sub != 0) return;
+    if (sc->status[1] != 0) {   // a tile copy of the pair kernel timed out: u would be incomplete
+        u[3 * i] = u[3 * i + 1] = u[3 * i + 2] = __longlong_as_double(0x7ff8000000000000LL);
+        return;
+    }
     u[3 * i] = c0 * x;
     u[3 * i + 1] = c0 * y;
     u[3 * i + 2] = c0 * z;
@@ -1117,23 +1184,26 @@ extern "C" gdc_status gdc_rpy_apply_noalloc(const double* r, const double* lambd
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int ntile = (n_blobs + GDC_NOALLOC_TILE - 1) / GDC_NOALLOC_TILE;
-    int nk = std::max(1, std::min(GDC_NOALLOC_MAX_CHUNKS, (8 * sms + ntile - 1) / ntile));
-    nk = std::min(nk, std::max(1, (n_blobs + 255) / 256));
+    // source chunks: 6 blocks per SM (the pair kernel's resident blocks), at least 32 sources
+    // each, within the scratch for partial sums and items (64 tiles at most, so 32 chunks fit)
+    int nk = std::max(1, (6 * sms + ntile - 1) / ntile);
+    nk = std::min(nk, std::min(GDC_NOALLOC_SLOTS / n_blobs, GDC_NOALLOC_ITEMS / ntile));
+    nk = std::min(nk, std::max(1, (n_blobs + 31) / 32));
     int csz = (n_blobs + nk - 1) / nk;
     csz = (csz + 31) / 32 * 32;
     nk = (n_blobs + csz - 1) / csz;
-    k_noalloc_begin<<<1, 256, 0, st>>>(sc, r, n_blobs);
+    k_noalloc_begin<<<1, 1024, 0, st>>>(sc, r, n_blobs);
     k_noalloc_prepare<<<std::min(1024, (n_blobs + 255) / 256 + 1), 256, 0, st>>>(sc, r, lambda, n_blobs, nk, csz);
     RpyConst32 k{(float)(2.0 * a * a / 3.0), (float)(2.0 * a * a), (float)(4.0 * a * a), (float)(4.0 / (3.0 * a)),
                  (float)(9.0 / (32.0 * a)), (float)(1.0 / (8.0 * a * a))};
-    // the pair kernel addresses partial sums as part[k * NBL + i]: pass the array's row length
-    const int near_chunks = (n_blobs + GDC_NEAR_SRC - 1) / GDC_NEAR_SRC;
-    k_near_build<<<((n_blobs + 255) / 256) * near_chunks, 128, 0, st>>>(sc->near_items, sc->susp_blob_off, sc->spos,
-                                                                       (float)(4.0 * a * a), sc->near_cnt, sc->near_idx);
+    const int near_chunks = (n_blobs + GDC_NEAR_SRC_MIN - 1) / GDC_NEAR_SRC_MIN;
+    k_near_build<<<((n_blobs + 255) / 256) * near_chunks, 128, 0, st>>>(nullptr, near_chunks, GDC_NEAR_SRC_MIN,
+                                                                       sc->susp_blob_off, sc->spos, (float)(4.0 * a * a),
+                                                                       sc->near_cnt, sc->near_idx);
     k_near_sort<<<(n_blobs + 255) / 256, 256, 0, st>>>(n_blobs, sc->near_cnt, sc->near_idx);
     k_rpy32<1, 6><<<ntile * nk, 128, 0, st>>>(sc->items, nullptr, sc->susp_blob_off, sc->spos, sc->sdup, sc->part,
-                                             GDC_NOALLOC_MAX_BLOBS, k, sc->status, first_wait_polls());
-    k_noalloc_epilogue<<<(n_blobs + 255) / 256, 256, 0, st>>>(sc, r, lambda, n_blobs, nk,
+                                             n_blobs, k, sc->status, first_wait_polls());
+    k_noalloc_epilogue<<<(GDC_NOALLOC_EPI * n_blobs + 255) / 256, 256, 0, st>>>(sc, r, lambda, n_blobs, nk,
                                                               1.0 / (8.0 * 3.141592653589793 * eta), a, u);
     e = cudaGetLastError();
     if (e != cudaSuccess)
