@@ -113,11 +113,13 @@ typedef struct {
     double rep_b;          /* soft repulsion range b (Eq. soft_sphere_potential)                          */
     double shear_rate;     /* background flow u = (shear_rate * y, 0, 0); 0 = off      */
     unsigned long long seed; /* Philox4x32-10 key of the W and W-tilde draws            */
-    int    autotune;       /* 1: gdc_init times the FP32 pair kernels' candidates at the
-                              initial configuration and keeps the fastest: kernel, work-
-                              item shape and the resident blocks per SM it is compiled for;
-                              then the double-float residual kernels (ordered, symmetric
-                              at 3 or 4 blocks per SM) the same way                      */
+    int    autotune;       /* 1: gdc_init times candidates of the FP32 pair kernel at the
+                              initial configuration and keeps the fastest (sources per work
+                              item and the resident blocks per SM it is compiled for), then
+                              the double-float residual kernel the same way (3 or 4 blocks
+                              per SM), on contexts of at least 2^28 ordered blob pairs per
+                              product; smaller ones take their sizes' rule, so that two
+                              contexts of one suspension round alike                     */
     int    graph;          /* 1: gdc_step captures one step as a CUDA graph at its first
                               call and replays it; the Lanczos and GMRES loops are
                               conditional WHILE nodes whose conditions the loop kernels
@@ -126,11 +128,9 @@ typedef struct {
                               (host-driven loops).  Used for the RFD divergence and for
                               Euler-Maruyama, not while gdc_profile is on.              */
     int    pair_kernel;    /* FP32 RPY pair kernel, fixed at init: 1 ordered (every ordered
-                              pair, target-side sums), 2 symmetric (every unordered pair
-                              once, both sides), 0 the faster of the two as timed by the
-                              autotuner (symmetric when autotune = 0).  The double-float
-                              residual kernel is ordered for 1, symmetric for 2, and for
-                              0 the autotuner's pick (symmetric when autotune = 0)        */
+                              pair, target-side sums), 2 or 0 symmetric (every unordered pair
+                              once, both sides).  The double-float residual kernel is
+                              ordered for 1, symmetric otherwise                         */
     int    potential;      /* gdc_potential                                            */
     double well_A;         /* well amplitude A_w, energy units (Sec. 6.4: 5 kT); 0 = no wells */
     double well_lambda;    /* well width lambda, a length (Sec. 6.4: 0.5 a)            */
@@ -390,13 +390,14 @@ typedef struct {
     unsigned long long rpydf_launches;  /* double-float residual pair-kernel launches     */
     double rpydf_ms;                    /* their summed CUDA-event durations              */
     int    pair_kernel;                 /* FP32 pair kernel in use: 1 ordered, 2 symmetric */
-    int    sym_width;                   /* source tiles per work item (symmetric kernel)  */
+    int    sym_width;                   /* source tiles per work item (symmetric kernel; 1
+                                           also for items of less than a tile)            */
     double unique_pairs_per_product;    /* unordered pairs incl. self, sum n (n + 1) / 2  */
     int    min_blocks_per_sm;           /* resident blocks per SM the FP32 pair kernel in use
-                                           was compiled for (chosen by the autotuner)     */
+                                           was compiled for                               */
     int    df_kernel;                   /* double-float residual kernel in use: 0 ordered,
                                            else the resident blocks per SM (3 or 4) of the
-                                           symmetric one (chosen by the autotuner)        */
+                                           symmetric one                                  */
 } gdc_profile_info;
 
 /* FP32 FMA throughput probe (the measured denominator of the pair kernels' FP32 roofline):

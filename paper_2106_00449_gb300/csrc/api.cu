@@ -350,20 +350,20 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->mv_nk = w.take<int>(S);
     c->mv_part = (void*)w.take<double4_32a>((long long)c->mv_cap_kmax * NBL);
     c->dev_status = w.take<int>(4);
-    c->sym_items = w.take<SymItem>(c->sym_cap_items);
+    c->sym_items = w.take<PairItem>(c->sym_cap_items);
     c->sym_row_nk = w.take<int>(std::max<long long>(1, c->sym_n_tiles));
     c->sym_tile_base = w.take<long long>(S + 1);
     c->sym_jbase = w.take<long long>(S + 1);
     c->sym_part_i = w.take<float4>((long long)c->sym_cap_kmax * NBL);
     c->sym_part_j = w.take<float4>(std::max<long long>(1, c->sym_n_jslots) * GDC_SYM_TILE);
-    c->dfs_items = w.take<SymItem>(c->dfs_n_items);
+    c->dfs_items = w.take<PairItem>(c->dfs_n_items);
     c->dfs_row_nk = w.take<int>(std::max<long long>(1, c->sym_n_tiles));
     c->dfs_part_i = w.take<double4_32a>((long long)c->dfs_kmax * NBL);
     // source-side slots of the double-float and the FP64 kernel: one product at a time uses them
     c->dfs_part_j = w.take<double4_32a>(std::max<long long>(
         1, std::max(c->sym_n_jslots * GDC_SYM_TILE, c->h_p64_jbase.back() * c->p64_tile)));
     c->p64_part_j = c->dfs_part_j;
-    c->p64_items = w.take<P64Item>((long long)c->h_p64_items.size());
+    c->p64_items = w.take<PairItem>((long long)c->h_p64_items.size());
     c->p64_row_nk = w.take<int>((long long)c->h_p64_row_nk.size());
     c->p64_tile_base = w.take<long long>(S + 1);
     c->p64_jbase = w.take<long long>(S + 1);
@@ -1008,7 +1008,7 @@ gdc_status gdc_init(gdc_ctx** out, const gdc_params* params, int n_templates, co
         if ((st = read_status(c)) != GDC_OK) return st;
     }
     if (c->p.autotune && c->p.mobility == GDC_MOB_RPY) {   // the RPY pair kernels only
-        load_at(c, c->Y, c->q, false);
+        load_at(c, c->Y, c->q, true);
         if ((st = autotune_pair_kernel(c)) != GDC_OK) return st;
     } else if ((st = default_pair_kernel(c)) != GDC_OK) {
         return st;
@@ -1065,7 +1065,7 @@ gdc_status gdc_profile_read(gdc_ctx* c, gdc_profile_info* out) {
     out->work_waves = c->mv_waves;
     out->autotune_ms = c->autotune_ms;
     out->pair_kernel = c->use_sym ? 2 : 1;
-    out->sym_width = c->sym_width;
+    out->sym_width = std::max(1, c->sym_width / GDC_SYM_TILE);
     out->min_blocks_per_sm = c->use_sym ? c->sym_minb : c->mv_minb;
     out->df_kernel = c->dfs_minb;
     double up = 0.0;

@@ -35,10 +35,8 @@
 #define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
 #define GDC_NEAR_SRC_MAX 2048
 #define GDC_SYM_TILE 512         // blobs per tile of the symmetric FP32 pair kernel
-#ifndef GDC_DFS_WIDTH
-#define GDC_DFS_WIDTH 2          // source tiles per item of the symmetric double-float kernel
-#endif
 #define GDC_P64_WIDE 16384       // FP64 pair kernel: 512-blob tiles for suspensions above this, 128-blob ones up to it
+#define GDC_TUNE_PAIRS 268435456.0   // ordered pairs per product (16,384^2) from which the autotuner times candidates
 #define GDC_CELL_MIN_BLOBS 16384 // GDC_FORCES_CHOOSE: the cell list from this many blobs on
 #define GDC_WAIT_POLLS 400000    // default bound of a pair kernel's wait for a tile copy (polls)
 
@@ -52,14 +50,8 @@ struct MvItem {      // one block of the pair kernels: targets [t0, t0+tile) x s
     int pad[3];
 };
 
-struct SymItem {     // one block of the symmetric pair kernel: target tile I x source tiles [J0, J1) of suspension s
-    int s, I, J0, J1;
-    int k;           // target-side partial-sum slot (the item's index within row I)
-    int pad[3];
-};
-
-struct P64Item {     // one block of the symmetric FP64 pair kernel: target tile I x sources [j0, j1) of suspension s
-    int s, I, j0, j1;
+struct PairItem {    // one block of the symmetric pair kernels: target tile I x sources [j0, j1) of suspension s,
+    int s, I, j0, j1;    // j0 at or after the tile's first blob; positions local to the suspension
     int k;           // target-side partial-sum slot (the item's index within row I)
     int pad[3];
 };
@@ -228,33 +220,34 @@ struct gdc_ctx {
     void* mv_part = 0;            // mv_kmax x NBL x (float4 | double4_32a)
     const int* mv_active = 0;     // when set, suspensions flagged 0 are skipped by the pair kernels
 
-    // symmetric FP32 pair kernel (each unordered pair once) and its work list
-    int use_sym = 0, sym_width = 4, sym_n_items = 0, sym_kmax = 1;
-    int sym_minb = 2;                         // resident blocks per SM the kernel was compiled for (2, 3, 4)
+    // symmetric FP32 pair kernel (each unordered pair once) and its work list (sym_width
+    // sources per item)
+    int use_sym = 0, sym_width = 2048, sym_n_items = 0, sym_kmax = 1;
+    int sym_minb = 3;                         // resident blocks per SM the kernel was compiled for (2, 3, 4)
     int sym_cap_items = 0, sym_cap_kmax = 1;
     long long sym_n_jslots = 0, sym_n_tiles = 0;
-    gdc::SymItem* sym_items = 0;
+    gdc::PairItem* sym_items = 0;
     int* sym_row_nk = 0;                      // target-side slots per tile row
     long long *sym_tile_base = 0, *sym_jbase = 0;   // per suspension: first tile, first source-side slot
     float4 *sym_part_i = 0, *sym_part_j = 0;  // target-side [slot][blob], source-side [slot][GDC_SYM_TILE]
-    std::vector<gdc::SymItem> h_sym_items;
+    std::vector<gdc::PairItem> h_sym_items;
     std::vector<int> h_sym_row_nk;
     // symmetric double-float residual kernel (dfsym.cu): its own work list (wider items), FP64 slots
-    gdc::SymItem* dfs_items = 0;
-    int dfs_n_items = 0, dfs_kmax = 1;
+    gdc::PairItem* dfs_items = 0;
+    int dfs_n_items = 0, dfs_kmax = 1, dfs_width = 1024;   // sources per item
     int dfs_minb = 4;   // 0: the ordered double-float kernel; 3 or 4: symmetric, blocks per SM
     int* dfs_row_nk = 0;
-    std::vector<gdc::SymItem> h_dfs_items;
+    std::vector<gdc::PairItem> h_dfs_items;
     std::vector<int> h_dfs_row_nk;
     double4_32a *dfs_part_i = 0, *dfs_part_j = 0;
     std::vector<long long> h_sym_tile_base, h_sym_jbase;
     // symmetric FP64 kernel (pair64.cu): its tile size, work list, slots
     int p64_tile = 128, p64_kmax = 1;
-    gdc::P64Item* p64_items = 0;
+    gdc::PairItem* p64_items = 0;
     int* p64_row_nk = 0;                      // target-side slots per tile row
     long long *p64_tile_base = 0, *p64_jbase = 0;
     double4_32a *p64_part_i = 0, *p64_part_j = 0;
-    std::vector<gdc::P64Item> h_p64_items;
+    std::vector<gdc::PairItem> h_p64_items;
     std::vector<int> h_p64_row_nk;
     std::vector<long long> h_p64_tile_base, h_p64_jbase;
 
@@ -408,16 +401,18 @@ __global__ void k_cell_sort(int H, const int* __restrict__ cnt, const int* __res
 void launch_near_build(gdc_ctx* c);
 // sym.cu
 void build_sym_items(gdc_ctx* c, int width);
-void build_sym_list(const gdc_ctx* c, int width, std::vector<SymItem>& items, std::vector<int>& row_nk, int& kmax);
+void build_pair_list(const gdc_ctx* c, int TS, long long width, std::vector<PairItem>& items, std::vector<int>& row_nk,
+                     int& kmax);
+long long pair_list_items(const gdc_ctx* c, int TS, long long width);   // items that list has
 // pair64.cu
 void build_p64_list(gdc_ctx* c);
 void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout);
-void launch_p64_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout);
+void launch_p64_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout);
 // dfsym.cu
 gdc_status dfsym_init_attributes(gdc_ctx* c);
 long long lz_q_doubles(int kmax);   // krylov.cu
 void launch_rpy_df_sym_pairs(gdc_ctx* c);
-void launch_rpy_df_sym_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout);
+void build_dfs_list(gdc_ctx* c);
 gdc_status sym_upload(gdc_ctx* c);
 gdc_status sym_init_attributes(gdc_ctx* c);
 void launch_rpy32_sym(gdc_ctx* c);

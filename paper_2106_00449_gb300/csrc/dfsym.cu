@@ -5,10 +5,11 @@
 // two products with lambda_j and lambda_i remain per side.
 //
 // Layout as in the symmetric FP32 kernel (sym.cu): tiles of 512 blobs; a block takes target
-// tile I against source tiles J0..J1-1 (J >= I), the diagonal tile J = I ordered.  For J > I
-// each warp holds 128 targets (four per lane); a 32-source sub-chunk is swept in 32 steps in
-// which lane l takes source (l + step) mod 32, and the source-side sums (double-float) move
-// one lane per step by shuffles, back at their source's lane after 32 steps.  At the end of
+// tile I against a range of sources, those of the tile itself ordered.  For later tiles J > I
+// each warp holds 128 targets (four per lane); W sources (32, or 16 when the range is
+// shorter) are swept in W steps in which lane l takes source (l + step) mod W, and the
+// source-side sums (double-float) move one lane per step by shuffles, back at their source's
+// lane after W steps; for W = 16 the two lanes of a source are then added.  At the end of
 // each sub-chunk the four warps' source-side sums meet in shared memory (double-buffered, one
 // barrier per sub-chunk) and warp 0 adds them in warp order into the tile pair's FP64 slot
 // (deterministic).
@@ -68,8 +69,9 @@ __device__ __forceinline__ df shfl_df(df v, int src) {
 
 // MINB: resident blocks per SM the register allocator is asked to allow, 3 (162 registers) or
 // 4 (128); the autotuner times both against the ordered double-float kernel.
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restrict__ items,
+// FULL: every range is whole tiles, as in the symmetric FP32 kernel.
+template <int MINB, bool FULL>
+__global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const PairItem* __restrict__ items,
                                                        const long long* __restrict__ susp_blob_off,
                                                        const long long* __restrict__ jbase,
                                                        const double4_32a* __restrict__ spos,
@@ -79,7 +81,7 @@ __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restr
     extern __shared__ __align__(16) unsigned char dfs_smem[];
     float4* sh = reinterpret_cast<float4*>(dfs_smem);                       // [plane][source]
     double* ws = reinterpret_cast<double*>(dfs_smem + DFS_TILE * 4 * 16);  // [buffer][warp][3][32]
-    const SymItem it = items[blockIdx.x];
+    const PairItem it = items[blockIdx.x];
     const long long b0 = susp_blob_off[it.s];
     const int ns = (int)(susp_blob_off[it.s + 1] - b0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -103,10 +105,14 @@ __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restr
         bt[m] = in ? (float)p.w : -1.f;
         ux[m] = uy[m] = uz[m] = df{0.f, 0.f};
     }
-    for (int J = it.J0; J < it.J1; ++J) {
-        const int j0 = J * DFS_TILE;
-        const int n = min(DFS_TILE, ns - j0);
-        const int nr = (n + 31) & ~31;
+    int W = 32;   // sources per sweep
+    if (!FULL && it.j1 - it.j0 <= 16) W = 16;
+    int buf = 0;
+    const int J1 = (it.j1 + DFS_TILE - 1) / DFS_TILE;
+    for (int J = it.j0 / DFS_TILE; J < J1; ++J) {   // the part of the range in source tile J
+        const int j0 = FULL ? J * DFS_TILE : max(it.j0, J * DFS_TILE);
+        const int n = FULL ? min(DFS_TILE, ns - j0) : min((J + 1) * DFS_TILE, it.j1) - j0;
+        const int nr = (n + W - 1) & ~(W - 1);
         __syncthreads();   // the previous tile's sources and sums are no longer read
         for (int e = threadIdx.x; e < nr; e += 128) {
             if (e < n) {
@@ -137,10 +143,10 @@ __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restr
             }
         } else {
             const long long slot = jbase[it.s] + (long long)J * (J - 1) / 2 + it.I;
-            for (int jc = 0; jc < nr; jc += 32) {
+            for (int jc = 0; jc < nr; jc += W) {
                 df jx{0.f, 0.f}, jy{0.f, 0.f}, jz{0.f, 0.f};   // sums of the source this lane holds
-                for (int st = 0; st < 32; ++st) {
-                    const int j = jc + ((lane + st) & 31);
+                for (int st = 0; st < W; ++st) {
+                    const int j = jc + ((lane + st) & (W - 1));
                     const float4 s0 = sh[j], s1 = sh[DFS_TILE + j], s2 = sh[2 * DFS_TILE + j], s3 = sh[3 * DFS_TILE + j];
                     const df xs{s0.x, s1.x}, ys{s0.y, s1.y}, zs{s0.z, s1.z};
                     const df lx{s2.x, s3.x}, ly{s2.y, s3.y}, lz{s2.z, s3.z};
@@ -157,20 +163,23 @@ __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restr
                     jy = shfl_df(jy, from);
                     jz = shfl_df(jz, from);
                 }
-                // after 32 passes the sums of source jc + lane are back at lane; the buffer this
-                // sub-chunk writes was last read by warp 0 before the previous barrier
-                double* wb = ws + ((jc >> 5) & 1) * (4 * 3 * 32);
-                wb[(warp * 3 + 0) * 32 + lane] = df_to(jx);
-                wb[(warp * 3 + 1) * 32 + lane] = df_to(jy);
-                wb[(warp * 3 + 2) * 32 + lane] = df_to(jz);
+                // after W steps the sums of source jc + (lane mod W) are back at lane; the buffer
+                // this sweep writes was last read by warp 0 before the previous barrier
+                double v[3] = {df_to(jx), df_to(jy), df_to(jz)};
+                if (!FULL && W == 16)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], 16);
+                double* wb = ws + buf * (4 * 3 * 32);
+                buf ^= 1;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) wb[(warp * 3 + c) * 32 + lane] = v[c];
                 __syncthreads();
-                if (warp == 0 && jc + lane < n) {   // the four warps' sums, in warp order
-                    double v[3];
+                if (warp == 0 && lane < W && jc + lane < n) {   // the four warps' sums, in warp order
 #pragma unroll
                     for (int c = 0; c < 3; ++c)
                         v[c] = ((wb[(0 * 3 + c) * 32 + lane] + wb[(1 * 3 + c) * 32 + lane]) +
                                 wb[(2 * 3 + c) * 32 + lane]) + wb[(3 * 3 + c) * 32 + lane];
-                    part_j[slot * DFS_TILE + jc + lane] = make_double4_32a(v[0], v[1], v[2], 0.0);
+                    part_j[slot * DFS_TILE + (j0 - J * DFS_TILE) + jc + lane] = make_double4_32a(v[0], v[1], v[2], 0.0);
                 }
             }
         }
@@ -183,80 +192,48 @@ __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const SymItem* __restr
     }
 }
 
-// u_i = c0 (target-side slots of the blob's tile row + source-side slots of the tiles before
-// it, added in FP64 in a fixed order) [- K V]; the same-body blocks are added afterwards.
-__global__ void k_rpy_df_sym_epilogue(int NBL, const double4_32a* __restrict__ part_i,
-                                      const double4_32a* __restrict__ part_j, const int* __restrict__ blob_susp,
-                                      const long long* __restrict__ susp_blob_off, const int* __restrict__ row_nk,
-                                      const long long* __restrict__ tile_base, const long long* __restrict__ jbase,
-                                      double c0, const double* __restrict__ x, double* __restrict__ y, int gm_layout,
-                                      const int* __restrict__ blob_gm, const int* __restrict__ body_gm,
-                                      const int* __restrict__ blob_body, const double* __restrict__ r,
-                                      const double* __restrict__ Yc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NBL) return;
-    const int s = blob_susp[i];
-    const long long loc = i - susp_blob_off[s];
-    const int J = (int)(loc / DFS_TILE), e = (int)(loc % DFS_TILE);
-    const int n = row_nk[tile_base[s] + J];
-    double ux = 0.0, uy = 0.0, uz = 0.0;
-    for (int kk = 0; kk < n; ++kk) {
-        const double4_32a v = part_i[(long long)kk * NBL + i];
-        ux += v.x;
-        uy += v.y;
-        uz += v.z;
-    }
-    const long long s0 = jbase[s] + (long long)J * (J - 1) / 2;
-    for (int I = 0; I < J; ++I) {
-        const double4_32a v = part_j[(s0 + I) * DFS_TILE + e];
-        ux += v.x;
-        uy += v.y;
-        uz += v.z;
-    }
-    ux *= c0;
-    uy *= c0;
-    uz *= c0;
-    if (!gm_layout) {
-        y[3LL * i] = ux;
-        y[3LL * i + 1] = uy;
-        y[3LL * i + 2] = uz;
-        return;
-    }
-    // saddle operator: M lambda - K V, K V = U_p + Omega_p x (r_i - Y_p)  (Eq. rigid_body_cond)
-    const int p = blob_body[i];
-    const double* V = x + body_gm[p];
-    const double dx = r[3LL * i] - Yc[3 * p], dy = r[3LL * i + 1] - Yc[3 * p + 1], dz = r[3LL * i + 2] - Yc[3 * p + 2];
-    const long long o = blob_gm[i];
-    y[o] = ux - (V[0] + (V[4] * dz - V[5] * dy));
-    y[o + 1] = uy - (V[1] + (V[5] * dx - V[3] * dz));
-    y[o + 2] = uz - (V[2] + (V[3] * dy - V[4] * dx));
+template <int MINB, bool FULL>
+static cudaError_t dfsym_attribute() {
+    return cudaFuncSetAttribute(k_rpy_df_sym<MINB, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, DFS_SMEM);
 }
 
 gdc_status dfsym_init_attributes(gdc_ctx* c) {
-    cudaError_t e = cudaFuncSetAttribute(k_rpy_df_sym<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, DFS_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rpy_df_sym<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, DFS_SMEM);
-    return cuda_check(c, e, "symmetric double-float kernel attributes");
+    for (cudaError_t e : {dfsym_attribute<3, true>(), dfsym_attribute<4, true>(), dfsym_attribute<3, false>(),
+                          dfsym_attribute<4, false>()})
+        if (e != cudaSuccess) return cuda_check(c, e, "symmetric double-float kernel attributes");
+    return GDC_OK;
 }
 
 // The symmetric double-float pair kernel alone (same-body blocks excluded).
 void launch_rpy_df_sym_pairs(gdc_ctx* c) {
+#define GDC_DFS_LAUNCH(MB, FULL)                                                                                \
+    k_rpy_df_sym<MB, FULL><<<c->dfs_n_items, 128, DFS_SMEM, c->stream>>>(                                       \
+        c->dfs_items, c->susp_blob_off, c->sym_jbase, c->spos64, c->slam64, c->dfs_part_i, c->dfs_part_j, c->NBL, \
+        df_constants(c->p.a))
     ++c->n_launch;
-    if (c->dfs_minb == 3)
-        k_rpy_df_sym<3><<<c->dfs_n_items, 128, DFS_SMEM, c->stream>>>(c->dfs_items, c->susp_blob_off, c->sym_jbase,
-                                                                       c->spos64, c->slam64, c->dfs_part_i,
-                                                                       c->dfs_part_j, c->NBL, df_constants(c->p.a));
-    else
-        k_rpy_df_sym<4><<<c->dfs_n_items, 128, DFS_SMEM, c->stream>>>(c->dfs_items, c->susp_blob_off, c->sym_jbase,
-                                                                       c->spos64, c->slam64, c->dfs_part_i,
-                                                                       c->dfs_part_j, c->NBL, df_constants(c->p.a));
+    const bool full = c->dfs_width >= DFS_TILE;
+    if (c->dfs_minb == 3) {
+        if (full) GDC_DFS_LAUNCH(3, true); else GDC_DFS_LAUNCH(3, false);
+    } else {
+        if (full) GDC_DFS_LAUNCH(4, true); else GDC_DFS_LAUNCH(4, false);
+    }
+#undef GDC_DFS_LAUNCH
 }
 
-// Its epilogue: the slots into y (same-body blocks excluded; they are added afterwards).
-void launch_rpy_df_sym_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout) {
-    ++c->n_launch, k_rpy_df_sym_epilogue<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(
-        c->NBL, c->dfs_part_i, c->dfs_part_j, c->blob_susp, c->susp_blob_off, c->dfs_row_nk, c->sym_tile_base,
-        c->sym_jbase, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm, c->body_gm,
-        c->blob_body, c->r, c->Yc);
+// Work list: the longest ranges (16 to 1,024 sources; longer in suspensions above 65,536
+// blobs, so that a row has at most 64 target-side slots) that give 24 items per SM.  us per
+// launch by that rule, and as items of two whole tiles before: 2,560 blobs 98 / 2,067, 7,800
+// blobs 543 / 2,159, 20,202 blobs 3,144 / 3,813, 48 suspensions of 63,702 blobs 1,196 / 2,624,
+// 65,520 blobs 30,660 / 30,640.
+void build_dfs_list(gdc_ctx* c) {
+    long long nmax = 1;
+    for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
+    long long w = 1024;
+    while (w < (nmax + 63) / 64) w *= 2;
+    while (w > 16 && pair_list_items(c, DFS_TILE, w) < 24LL * c->num_sms) w >>= 1;
+    build_pair_list(c, DFS_TILE, w, c->h_dfs_items, c->h_dfs_row_nk, c->dfs_kmax);
+    c->dfs_width = (int)w;
+    c->dfs_n_items = (int)c->h_dfs_items.size();
 }
 
 }  // namespace gdc

@@ -58,13 +58,13 @@ __device__ __forceinline__ void rpy64_coeff(double r2, const Rpy64K& k, double& 
 
 template <int TPL>
 __global__ void __launch_bounds__(128, TPL == 1 ? 5 : 3) k_rpy64_sym(
-    const P64Item* __restrict__ items, const int* __restrict__ active, const long long* __restrict__ susp_blob_off,
+    const PairItem* __restrict__ items, const int* __restrict__ active, const long long* __restrict__ susp_blob_off,
     const long long* __restrict__ jbase, const double4_32a* __restrict__ spos, const double* __restrict__ x,
     const int* __restrict__ map, double4_32a* __restrict__ part_i, double4_32a* __restrict__ part_j, int NBL, Rpy64K k) {
     constexpr int TS = 128 * TPL;
     __shared__ double src[6][P64_STAGE];
     __shared__ double red[2][4][3][32];
-    const P64Item it = items[blockIdx.x];
+    const PairItem it = items[blockIdx.x];
     const long long b0 = susp_blob_off[it.s];
     const int ns = (int)(susp_blob_off[it.s + 1] - b0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(128, TPL == 1 ? 5 : 3) k_rpy64_sym(
 }
 
 // u_i = c0 (target-side slots of the blob's tile row + source-side slots of the tiles before
-// it) [- K V].  Four threads per blob, each taking every fourth slot, added in a fixed order:
+// it) [- K V], for this kernel and the symmetric double-float one (dfsym.cu; its same-body
+// blocks are added afterwards).  Four threads per blob, each taking every fourth slot, added in a fixed order:
 // the slots are latency-bound L2 reads, and one thread per blob left small suspensions with
 // a few warps.
 __global__ void __launch_bounds__(128) k_p64_epilogue(
@@ -267,33 +268,11 @@ void build_p64_list(gdc_ctx* c) {
         c->h_p64_jbase[s + 1] = c->h_p64_jbase[s] + T * (T - 1) / 2;
     }
     const long long want = 8LL * c->num_sms;
-    int w = 2 * TS;
-    for (; w > 4; w >>= 1) {
-        long long items = 0;
-        for (int s = 0; s < c->S && items < want; ++s) {
-            const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
-            for (long long t0 = 0; t0 < n && items < want; t0 += TS) items += (n - t0 + w - 1) / w;
-        }
-        if (items >= want) break;
-    }
-    c->h_p64_items.clear();
-    c->h_p64_row_nk.clear();
-    c->p64_kmax = 1;
-    for (int s = 0; s < c->S; ++s) {
-        const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
-        for (int I = 0; (long long)I * TS < n; ++I) {
-            int k = 0;
-            const long long left = n - (long long)I * TS;
-            // very large suspensions: at most 128 slots per row, ranges of whole tiles
-            const long long step = w == 2 * TS ? std::max<long long>(w, ((left + 127) / 128 + TS - 1) / TS * TS) : w;
-            for (long long j0 = (long long)I * TS; j0 < n; j0 += step, ++k)
-                c->h_p64_items.push_back(P64Item{s, I, (int)j0, (int)std::min(n, j0 + step), k, {0, 0, 0}});
-            c->h_p64_row_nk.push_back(k);
-            c->p64_kmax = std::max(c->p64_kmax, k);
-        }
-    }
-    std::stable_sort(c->h_p64_items.begin(), c->h_p64_items.end(),
-                     [](const P64Item& a, const P64Item& b) { return a.j1 - a.j0 > b.j1 - b.j0; });
+    long long w = 2 * TS;
+    while (w > 4 && pair_list_items(c, TS, w) < want) w >>= 1;
+    // very large suspensions: at most 128 target-side slots per row, ranges of whole tiles
+    if (w == 2 * TS) w = std::max<long long>(w, ((nmax + 127) / 128 + TS - 1) / TS * TS);
+    build_pair_list(c, TS, w, c->h_p64_items, c->h_p64_row_nk, c->p64_kmax);
 }
 
 void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout) {
@@ -312,10 +291,12 @@ void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout) {
                                                  map, c->p64_part_i, c->p64_part_j, c->NBL, k);
 }
 
-void launch_p64_epilogue(gdc_ctx* c, const double* x, double* y, int gm_layout) {
+void launch_p64_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout) {
+    const bool df = prec == GDC_PREC_DF64;   // the double-float kernel's slots
     ++c->n_launch, k_p64_epilogue<<<ceil_div(4LL * c->NBL, 128), 128, 0, c->stream>>>(
-        c->NBL, c->p64_tile, c->p64_part_i, c->p64_part_j, c->blob_susp, c->susp_blob_off, c->p64_row_nk,
-        c->p64_tile_base, c->p64_jbase, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm,
+        c->NBL, df ? GDC_SYM_TILE : c->p64_tile, df ? c->dfs_part_i : c->p64_part_i, df ? c->dfs_part_j : c->p64_part_j,
+        c->blob_susp, c->susp_blob_off, df ? c->dfs_row_nk : c->p64_row_nk, df ? c->sym_tile_base : c->p64_tile_base,
+        df ? c->sym_jbase : c->p64_jbase, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm,
         c->body_gm, c->blob_body, c->r, c->Yc);
 }
 

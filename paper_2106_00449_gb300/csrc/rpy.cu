@@ -569,10 +569,8 @@ static void launch_epilogue(gdc_ctx* c, int prec, double c0, const double* x, do
 }
 
 void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout, bool same_body) {
-    if (prec == GDC_PREC_DF64 && c->dfs_minb)
-        launch_rpy_df_sym_epilogue(c, x, y, gm_layout);
-    else if (prec == GDC_FP64)
-        launch_p64_epilogue(c, x, y, gm_layout);
+    if (prec == GDC_FP64 || (prec == GDC_PREC_DF64 && c->dfs_minb))
+        launch_p64_epilogue(c, prec, x, y, gm_layout);
     else
         launch_epilogue(c, prec, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, prec == GDC_FP32_MIXED);
     // same-body blocks from the template: the df64 pair kernel leaves those pairs out and the
@@ -812,7 +810,7 @@ void build_mv_items(gdc_ctx* c, int tpt, double waves) {
         const long long n = ns[s];
         const int nt = ceil_div(n, tile_targets);
         int nk = (int)std::lround(target_items * (double)n * (double)n / std::max(P, 1.0) / std::max(nt, 1));
-        nk = std::max(1, std::min(nk, std::max(1, ceil_div(n, 512))));
+        nk = std::max(1, std::min(nk, std::max(1, ceil_div(n, 32))));
         nk = std::min(nk, 64);
         long long csz = (n + nk - 1) / nk;
         csz = ((csz + 31) / 32) * 32;
@@ -847,10 +845,29 @@ namespace gdc {
 // Candidate tilings of the pair kernels: targets per thread x work items per launch.
 static const int kTpt[2] = {2, 4};
 static const double kWaves[3] = {4.0, 8.0, 16.0};
-static const int kSymWidth[3] = {2, 4, 8};   // source tiles per item of the symmetric kernel
 static const int kSymMinBlocks[3] = {2, 3, 4};   // resident blocks per SM of the symmetric kernel
 static const int kMvMinBlocks[2] = {4, 6};       // resident blocks per SM of the ordered kernel
-static const int kDfsMinBlocks[3] = {0, 3, 4};   // double-float kernel: ordered, symmetric at 3 or 4 per SM
+static const int kDfsMinBlocks[2] = {3, 4};      // resident blocks per SM of the symmetric double-float kernel
+
+// Sources per item of the symmetric FP32 kernel: the longest range (a power of two, 32 to
+// 2,048) that gives at least 6 items per SM and at most 1/48 of the largest suspension.
+// Swept over 32..2,048 sources with 2, 3 and 4 resident blocks per SM (us per launch, this
+// rule's width first, then the best): 2,560 blobs 12.2 / 12.2 (widths 32 / 32), 7,800 blobs
+// 46.4 / 46.4 (64), 20,202 blobs 249 / 241 (256 / 128; whole product 438 / 431), 65,520 blobs
+// 2,346 / 2,343 (1,024 / 256), 48 suspensions of 63,702 blobs 81.8 / 81.6 (128 / 64).  Items
+// of whole tiles (1,024 sources at least) took 99, 119, 281, 2,325 and 133 us.
+static int sym_default_width(const gdc_ctx* c) {
+    long long nmax = 1;
+    for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
+    int w = 2048;
+    while (w > 32 && (w > nmax / 48 || pair_list_items(c, GDC_SYM_TILE, w) < 6LL * c->num_sms)) w /= 2;
+    return w;
+}
+
+// The tuner times half, once and twice that width from GDC_TUNE_PAIRS ordered pairs per product
+// on; below, the rule stands (timings of a few microseconds would pick differently from one
+// context to the next, and the product's rounding with them).
+static bool tuned(const gdc_ctx* c) { return c->p.autotune && c->pair_evals_per_matvec >= GDC_TUNE_PAIRS; }
 
 void plan_mv_capacity(gdc_ctx* c) {
     int cap_items = 0, cap_k = 1;
@@ -863,8 +880,10 @@ void plan_mv_capacity(gdc_ctx* c) {
     c->mv_cap_items = cap_items;
     c->mv_cap_kmax = cap_k;
     build_mv_items(c, 2, 8.0);
+    const int w0 = sym_default_width(c);
     int scap = 0, sk = 1;
-    for (int w : kSymWidth) {
+    for (int w : {w0 / 2, w0, 2 * w0}) {
+        if (w < 32 || (w != w0 && !tuned(c))) continue;
         build_sym_items(c, w);
         scap = std::max(scap, c->sym_n_items);
         sk = std::max(sk, c->sym_kmax);
@@ -873,16 +892,8 @@ void plan_mv_capacity(gdc_ctx* c) {
     c->sym_cap_kmax = sk;
     c->sym_n_tiles = c->h_sym_tile_base.back();
     c->sym_n_jslots = c->h_sym_jbase.back();
-    build_sym_items(c, 4);
-    // the symmetric double-float kernel: items of GDC_DFS_WIDTH source tiles, so that with 3
-    // or 4 resident blocks per SM the last wave of long items stays full; wider in
-    // suspensions of more than 64 x GDC_DFS_WIDTH tiles, which keeps the target-side slots
-    // at 64 per blob (each wave is then a small part of the launch anyway)
-    int tmax = 1;
-    for (int s = 0; s < c->S; ++s)
-        tmax = std::max(tmax, (int)((c->h_blob_off[s + 1] - c->h_blob_off[s] + GDC_SYM_TILE - 1) / GDC_SYM_TILE));
-    build_sym_list(c, std::max(GDC_DFS_WIDTH, (tmax + 63) / 64), c->h_dfs_items, c->h_dfs_row_nk, c->dfs_kmax);
-    c->dfs_n_items = (int)c->h_dfs_items.size();
+    build_sym_items(c, w0);
+    build_dfs_list(c);
     build_p64_list(c);
 }
 
@@ -895,32 +906,38 @@ static gdc_status upload_items(gdc_ctx* c) {
     return cuda_check(c, e, "work-list upload");
 }
 
-// Times three launches of the FP32 RPY kernel per candidate at the loaded configuration
-// (lambda = the current W buffer) and keeps the fastest tiling; then one launch of each
-// double-float residual kernel.
+// At the loaded configuration (lambda = the current W buffer), three FP32 RPY products (pair
+// kernel and epilogue: more items leave more partial sums to add) per candidate, and the
+// fastest is kept: the symmetric kernel's item width and resident blocks per SM, or with
+// pair_kernel = 1 the ordered kernel's tiling (the ordered kernel took 1.2 to 1.9 times as
+// long at every size measured); then one launch of each double-float residual kernel.
 gdc_status autotune_pair_kernel(gdc_ctx* c) {
+    if (!tuned(c)) return default_pair_kernel(c);
     cudaEvent_t e0, e1;
     gdc_status st = cuda_check(c, cudaEventCreate(&e0), "event");
     if (st != GDC_OK) return st;
     if ((st = cuda_check(c, cudaEventCreate(&e1), "event")) != GDC_OK) return st;
     launch_normals(c, 0, 0, c->W);
     launch_pack_lambda(c, GDC_FP32_MIXED, c->W, 0);
-    const int only = c->p.pair_kernel;   // 0: both kernels, 1: ordered, 2: symmetric
+    const bool ordered = c->p.pair_kernel == 1;
     float best = 1e30f;
-    int bt = 2, bsym = 0, bwid = 4;
-    double bw = 8.0;
+    auto product = [&] {
+        launch_rpy(c, GDC_FP32_MIXED, c->W, 0);
+        launch_rpy_epilogue(c, GDC_FP32_MIXED, c->W, c->lz_u, 0, false);
+    };
     auto time3 = [&](float& ms) -> gdc_status {
-        launch_rpy(c, GDC_FP32_MIXED, c->W, 0);  // warm-up
+        product();  // warm-up
         cudaEventRecord(e0, c->stream);
-        for (int r = 0; r < 3; ++r) launch_rpy(c, GDC_FP32_MIXED, c->W, 0);
+        for (int r = 0; r < 3; ++r) product();
         cudaEventRecord(e1, c->stream);
         gdc_status s2 = cuda_check(c, cudaEventSynchronize(e1), "autotune");
         if (s2 == GDC_OK) cudaEventElapsedTime(&ms, e0, e1);
         return s2;
     };
-    int bmv_minb = 6;
-    if (only != 2) {
-        c->use_sym = 0;
+    c->use_sym = !ordered;
+    if (ordered) {
+        int bt = 2, bminb = 6;
+        double bw = 8.0;
         for (int a = 0; a < 2 && st == GDC_OK; ++a)
             for (int b = 0; b < 3 && st == GDC_OK; ++b) {
                 build_mv_items(c, kTpt[a], kWaves[b]);
@@ -933,16 +950,17 @@ gdc_status autotune_pair_kernel(gdc_ctx* c) {
                         best = ms;
                         bt = kTpt[a];
                         bw = kWaves[b];
-                        bmv_minb = mb;
-                        bsym = 0;
+                        bminb = mb;
                     }
                 }
             }
-    }
-    int bminb = 2;
-    if (only != 1 && st == GDC_OK) {
-        c->use_sym = 1;
-        for (int w : kSymWidth) {
+        build_mv_items(c, bt, bw);
+        c->mv_minb = bminb;
+    } else {
+        const int w0 = sym_default_width(c);
+        int bwid = w0, bminb = 3;
+        for (int w : {w0 / 2, w0, 2 * w0}) {
+            if (w < 32 || st != GDC_OK) continue;
             build_sym_items(c, w);
             if ((st = sym_upload(c)) != GDC_OK) break;
             for (int mb : kSymMinBlocks) {
@@ -953,33 +971,27 @@ gdc_status autotune_pair_kernel(gdc_ctx* c) {
                     best = ms;
                     bwid = w;
                     bminb = mb;
-                    bsym = 1;
                 }
             }
-            if (st != GDC_OK) break;
         }
+        build_sym_items(c, bwid);
+        c->sym_minb = bminb;
     }
     if (st == GDC_OK) {
-        build_mv_items(c, bt, bw);
-        build_sym_items(c, bwid);
-        c->use_sym = bsym;
-        c->sym_minb = bminb;
-        c->mv_minb = bmv_minb;
         c->autotune_ms = best / 3.0;
         st = upload_items(c);
         if (st == GDC_OK) st = sym_upload(c);
     }
     // the double-float residual kernel, one timed launch each after a warm-up (about 40 ms
-    // per product at 65k blobs): ordered unless the FP32 kernel is pinned to symmetric
-    c->dfs_minb = only == 1 ? 0 : 4;
+    // per product at 65k blobs)
+    c->dfs_minb = ordered ? 0 : 4;
     if (c->p.df_kernel) {
         c->dfs_minb = c->p.df_kernel == 1 ? 0 : c->p.df_kernel;
-    } else if (only != 1 && st == GDC_OK) {
+    } else if (!ordered && st == GDC_OK) {
         launch_pack_lambda(c, GDC_PREC_DF64, c->W, 0);
         float dbest = 1e30f;
         int bdf = 4;
         for (int mb : kDfsMinBlocks) {
-            if (mb == 0 && only == 2) continue;
             c->dfs_minb = mb;
             float ms = 0.f;
             launch_rpy(c, GDC_PREC_DF64, c->W, 0);   // warm-up
@@ -1000,8 +1012,8 @@ gdc_status autotune_pair_kernel(gdc_ctx* c) {
     return st;
 }
 
-// Without the autotuner: the kernel params.pair_kernel names (symmetric for 0 and 2) with
-// the default work lists, and the double-float kernel of the same kind.
+// Untuned: the kernel params.pair_kernel names (symmetric for 0 and 2) with the default work
+// lists, and the double-float kernel of the same kind.
 gdc_status default_pair_kernel(gdc_ctx* c) {
     c->use_sym = c->p.pair_kernel != 1;
     c->dfs_minb = c->p.df_kernel ? (c->p.df_kernel == 1 ? 0 : c->p.df_kernel) : (c->use_sym ? 4 : 0);

@@ -4,9 +4,9 @@
 // unordered pair the distance and the coefficients A, B are shared and only the two
 // products with lambda_j and lambda_i remain.
 //
-// A suspension's blobs are cut into tiles of SYM_TILE.  A block takes target tile I against
-// source tiles J0..J1-1 (J >= I).  The diagonal tile J = I is evaluated ordered (every
-// ordered pair, i-side only).  For J > I each warp holds 128 targets (four per lane, two
+// A suspension's blobs are cut into tiles of SYM_TILE.  A block takes target tile I against a
+// range of sources (whole sub-chunks of 32, from the tile's first blob on).  Sources of the
+// tile itself (J = I) are evaluated ordered (every ordered pair, i-side only).  For J > I each warp holds 128 targets (four per lane, two
 // packed pairs); a 32-source sub-chunk is swept in 32 steps in which lane l reads source
 // (l + step) mod 32 from shared memory, so that the 32 lanes hold 32 different sources, and
 // the source-side sum travels with its source: after every step the lanes pass their
@@ -34,8 +34,11 @@ __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restrict__ items,
+// FULL: every range is whole tiles (item widths of a tile and more), whose bounds are then simple
+// enough for the compiler to keep the sweep's registers as they are (2.325 against 2.35 ms at
+// 65,520 blobs).
+template <int MINB, bool FULL>
+__global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const PairItem* __restrict__ items,
                                                                  const int* __restrict__ active,
                                                                  const long long* __restrict__ susp_blob_off,
                                                                  const long long* __restrict__ jbase,
@@ -50,7 +53,7 @@ __global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restri
     float* jsy = jsx + 4 * SYM_TILE;
     float* jsz = jsy + 4 * SYM_TILE;
     unsigned long long* mbar = reinterpret_cast<unsigned long long*>(jsz + 4 * SYM_TILE);
-    const SymItem it = items[blockIdx.x];
+    const PairItem it = items[blockIdx.x];
     const long long b0 = susp_blob_off[it.s];
     const int ns = (int)(susp_blob_off[it.s + 1] - b0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -59,10 +62,10 @@ __global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restri
         // a suspension whose Krylov loop has stopped: its product is not used; leave zeros
         for (int t = threadIdx.x; t < SYM_TILE && tbase + t < ns; t += 128)
             part_i[(long long)it.k * NBL + b0 + tbase + t] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int J = max(it.J0, it.I + 1); J < it.J1; ++J) {
-            const long long slot = jbase[it.s] + (long long)J * (J - 1) / 2 + it.I;
-            for (int e = threadIdx.x; e < SYM_TILE; e += 128)
-                part_j[slot * SYM_TILE + e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = max(it.j0, tbase + SYM_TILE) + (int)threadIdx.x; j < it.j1; j += 128) {
+            const int J = j / SYM_TILE;
+            part_j[(jbase[it.s] + (long long)J * (J - 1) / 2 + it.I) * SYM_TILE + j - J * SYM_TILE] =
+                make_float4(0.f, 0.f, 0.f, 0.f);
         }
         return;
     }
@@ -93,9 +96,10 @@ __global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restri
     }
     __syncthreads();
     unsigned phase = 0;
-    for (int J = it.J0; J < it.J1; ++J) {
-        const int j0 = J * SYM_TILE;
-        const int n = min(SYM_TILE, ns - j0);
+    const int J1 = (it.j1 + SYM_TILE - 1) / SYM_TILE;
+    for (int J = it.j0 / SYM_TILE; J < J1; ++J) {   // the part of the range in source tile J
+        const int j0 = FULL ? J * SYM_TILE : max(it.j0, J * SYM_TILE);
+        const int n = FULL ? min(SYM_TILE, ns - j0) : min((J + 1) * SYM_TILE, it.j1) - j0;
         const int nr = (n + 31) & ~31;
         if (threadIdx.x == 0) {
             // the previous tile's generic-proxy reads and writes of sh are ordered before this copy
@@ -205,7 +209,7 @@ __global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restri
                 const float sx = ((jsx[e] + jsx[SYM_TILE + e]) + jsx[2 * SYM_TILE + e]) + jsx[3 * SYM_TILE + e];
                 const float sy = ((jsy[e] + jsy[SYM_TILE + e]) + jsy[2 * SYM_TILE + e]) + jsy[3 * SYM_TILE + e];
                 const float sz = ((jsz[e] + jsz[SYM_TILE + e]) + jsz[2 * SYM_TILE + e]) + jsz[3 * SYM_TILE + e];
-                part_j[slot * SYM_TILE + e] = make_float4(sx, sy, sz, 0.f);
+                part_j[slot * SYM_TILE + (FULL ? 0 : j0 - J * SYM_TILE) + e] = make_float4(sx, sy, sz, 0.f);
             }
         }
         __syncthreads();   // sh and the sums are rewritten for the next tile
@@ -219,25 +223,25 @@ __global__ void __launch_bounds__(128, MINB) k_rpy32_sym(const SymItem* __restri
     }
 }
 
-// Work list: per suspension, T = ceil(n / SYM_TILE) tiles; row I holds tiles I..T-1, cut
-// into items of at most `width` tiles (the first of a row holds the diagonal).  Fills the
-// per-tile item counts (i-side slots), the per-suspension first j-side slot, and orders
-// the items largest first.
-void build_sym_list(const gdc_ctx* c, int width, std::vector<SymItem>& items, std::vector<int>& row_nk, int& kmax) {
+// Work list of a symmetric pair kernel with tiles of TS blobs: row I of a suspension (targets of
+// tile I) takes the sources from the tile's first blob to the end in ranges of `width` (a
+// power of two that divides TS, or a multiple of TS), longest first.  Fills the per-row item
+// counts (target-side slots).
+void build_pair_list(const gdc_ctx* c, int TS, long long width, std::vector<PairItem>& items, std::vector<int>& row_nk,
+                     int& kmax) {
     items.clear();
     row_nk.clear();
     kmax = 1;
     for (int s = 0; s < c->S; ++s) {
         const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
-        const int T = (int)((n + SYM_TILE - 1) / SYM_TILE);
-        for (int I = 0; I < T; ++I) {
+        for (int I = 0; (long long)I * TS < n; ++I) {
             int kk = 0;
-            for (int J0 = I; J0 < T; J0 += width, ++kk) {
-                SymItem it{};
+            for (long long j0 = (long long)I * TS; j0 < n; j0 += width, ++kk) {
+                PairItem it{};
                 it.s = s;
                 it.I = I;
-                it.J0 = J0;
-                it.J1 = std::min(T, J0 + width);
+                it.j0 = (int)j0;
+                it.j1 = (int)std::min(n, j0 + width);
                 it.k = kk;
                 items.push_back(it);
             }
@@ -246,12 +250,21 @@ void build_sym_list(const gdc_ctx* c, int width, std::vector<SymItem>& items, st
         }
     }
     std::stable_sort(items.begin(), items.end(),
-                     [](const SymItem& x, const SymItem& y) { return x.J1 - x.J0 > y.J1 - y.J0; });
+                     [](const PairItem& x, const PairItem& y) { return x.j1 - x.j0 > y.j1 - y.j0; });
+}
+
+long long pair_list_items(const gdc_ctx* c, int TS, long long width) {
+    long long items = 0;
+    for (int s = 0; s < c->S; ++s) {
+        const long long n = c->h_blob_off[s + 1] - c->h_blob_off[s];
+        for (long long t0 = 0; t0 < n; t0 += TS) items += (n - t0 + width - 1) / width;
+    }
+    return items;
 }
 
 void build_sym_items(gdc_ctx* c, int width) {
     c->sym_width = width;
-    build_sym_list(c, width, c->h_sym_items, c->h_sym_row_nk, c->sym_kmax);
+    build_pair_list(c, SYM_TILE, width, c->h_sym_items, c->h_sym_row_nk, c->sym_kmax);
     c->h_sym_tile_base.assign(c->S + 1, 0);
     c->h_sym_jbase.assign(c->S + 1, 0);
     for (int s = 0; s < c->S; ++s) {
@@ -264,7 +277,7 @@ void build_sym_items(gdc_ctx* c, int width) {
 }
 
 gdc_status sym_upload(gdc_ctx* c) {
-    cudaError_t e = cudaMemcpyAsync(c->sym_items, c->h_sym_items.data(), sizeof(SymItem) * c->h_sym_items.size(),
+    cudaError_t e = cudaMemcpyAsync(c->sym_items, c->h_sym_items.data(), sizeof(PairItem) * c->h_sym_items.size(),
                                     cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->sym_row_nk, c->h_sym_row_nk.data(), sizeof(int) * c->h_sym_row_nk.size(),
@@ -279,26 +292,32 @@ gdc_status sym_upload(gdc_ctx* c) {
     return cuda_check(c, e, "upload of the symmetric work list");
 }
 
+template <int MINB, bool FULL>
+static cudaError_t sym_attribute() {
+    return cudaFuncSetAttribute(k_rpy32_sym<MINB, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, SYM_SMEM);
+}
+
 gdc_status sym_init_attributes(gdc_ctx* c) {
-    cudaError_t e = cudaFuncSetAttribute(k_rpy32_sym<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SYM_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rpy32_sym<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, SYM_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rpy32_sym<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SYM_SMEM);
-    return cuda_check(c, e, "symmetric pair kernel attributes");
+    for (cudaError_t e : {sym_attribute<2, true>(), sym_attribute<3, true>(), sym_attribute<4, true>(),
+                          sym_attribute<2, false>(), sym_attribute<3, false>(), sym_attribute<4, false>()})
+        if (e != cudaSuccess) return cuda_check(c, e, "symmetric pair kernel attributes");
+    return GDC_OK;
 }
 
 void launch_rpy32_sym(gdc_ctx* c) {
-#define GDC_SYM_LAUNCH(MB)                                                                                         \
-    k_rpy32_sym<MB><<<c->sym_n_items, 128, SYM_SMEM, c->stream>>>(c->sym_items, c->mv_active, c->susp_blob_off,     \
-                                                                  c->sym_jbase, c->spos, c->sdup, c->sym_part_i,   \
-                                                                  c->sym_part_j, c->NBL, rpy_const32(c->p.a),      \
-                                                                  c->dev_status, first_wait_polls())
+#define GDC_SYM_LAUNCH(MB, FULL)                                                                                   \
+    k_rpy32_sym<MB, FULL><<<c->sym_n_items, 128, SYM_SMEM, c->stream>>>(                                           \
+        c->sym_items, c->mv_active, c->susp_blob_off, c->sym_jbase, c->spos, c->sdup, c->sym_part_i, c->sym_part_j, \
+        c->NBL, rpy_const32(c->p.a), c->dev_status, first_wait_polls())
     ++c->n_launch;
-    if (c->sym_minb == 3)
-        GDC_SYM_LAUNCH(3);
-    else if (c->sym_minb == 4)
-        GDC_SYM_LAUNCH(4);
-    else
-        GDC_SYM_LAUNCH(2);
+    const bool full = c->sym_width >= SYM_TILE;
+    if (c->sym_minb == 3) {
+        if (full) GDC_SYM_LAUNCH(3, true); else GDC_SYM_LAUNCH(3, false);
+    } else if (c->sym_minb == 4) {
+        if (full) GDC_SYM_LAUNCH(4, true); else GDC_SYM_LAUNCH(4, false);
+    } else {
+        if (full) GDC_SYM_LAUNCH(2, true); else GDC_SYM_LAUNCH(2, false);
+    }
 #undef GDC_SYM_LAUNCH
 }
 
