@@ -234,6 +234,7 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->susp_body_off = w.take<long long>(S + 1);
     c->susp_blob_off = w.take<long long>(S + 1);
     c->susp_gm_off = w.take<long long>(S + 1);
+    c->susp_lz_off = w.take<long long>(S + 1);
     c->body_blob_off = w.take<long long>(NB + 1);
     c->minv_off = w.take<long long>(T + 1);
     c->body_tmpl = w.take<int>(NB);
@@ -343,6 +344,7 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->seg_gm.chunks = w.take<Chunk>(c->seg_gm.n_chunks);
     c->seg_gm.seg_chunk_off = w.take<int>(S + 1);
     c->seg_gm.off = c->susp_gm_off;
+    c->seg_lz.off = c->susp_lz_off;
     c->seg_lz.chunks = w.take<Chunk>(c->seg_lz.n_chunks);
     c->seg_lz.seg_chunk_off = w.take<int>(S + 1);
     c->red_part = w.take<double>((long long)std::max(c->seg_gm.n_chunks, c->seg_lz.n_chunks) * cols);
@@ -434,6 +436,7 @@ static gdc_status upload_layout(gdc_ctx* c, const double* tmpl_xyz_centred) {
     chk(up(c, c->susp_body_off, c->h_body_off.data(), S + 1));
     chk(up(c, c->susp_blob_off, c->h_blob_off.data(), S + 1));
     chk(up(c, c->susp_gm_off, c->h_gm_off.data(), S + 1));
+    chk(up(c, c->susp_lz_off, c->seg_lz.h_off.data(), S + 1));
     chk(up(c, c->body_blob_off, c->h_body_blob_off.data(), NB + 1));
     chk(up(c, c->minv_off, c->h_minv_off.data(), T + 1));
     chk(up(c, c->body_tmpl, c->h_body_tmpl.data(), NB));

@@ -30,6 +30,7 @@
 #define GDC_MAX_LANCZOS 128
 #define GDC_MAX_TMPL_BLOBS 340   // 3n <= 1020 rows of a template block
 #define GDC_TB_MAX 8             // bodies of one template per block in the factor products
+#define GDC_ORTH_SLICE 4096      // elements per block of the fused orthogonalisation (8 blocks per suspension at most)
 #define GDC_NEAR_CAP 32          // blobs closer than 2a listed per blob (beyond: a search of the suspension)
 #define GDC_EPI_WIDE 32768       // FP32 product epilogue: 8 threads per blob up to this many blobs, one above
 #define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
@@ -136,7 +137,7 @@ struct gdc_ctx {
     std::vector<double> h_tmpl_xyz, h_tmpl_L;
 
     // device layout tables
-    long long *susp_body_off = 0, *susp_blob_off = 0, *susp_gm_off = 0, *body_blob_off = 0;
+    long long *susp_body_off = 0, *susp_blob_off = 0, *susp_gm_off = 0, *susp_lz_off = 0, *body_blob_off = 0;
     long long *minv_off = 0;
     int *body_tmpl = 0, *body_susp = 0, *blob_body = 0, *blob_susp = 0, *tmpl_n = 0, *tmpl_off = 0;
     int *blob_gm = 0, *body_gm = 0;

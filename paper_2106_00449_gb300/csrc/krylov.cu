@@ -11,6 +11,8 @@
 // GDC_FP32_MIXED mode the operator inside the Krylov loop uses the FP32 pair kernel; each
 // GMRES cycle ends with an accurate residual (double-float pairs, FP64 same-body blocks),
 // and the solver restarts from it until that residual meets gmres_tol (iterative refinement).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -386,6 +388,236 @@ __global__ void k_gm_backsolve(int S, int m, const double* __restrict__ H, const
     for (int i = k; i < cols; ++i) ys[i] = 0.0;
 }
 
+// ---- one iteration's orthogonalisation in one launch -----------------------------------
+//
+// w is orthogonalised against V_0..V_j (classical Gram-Schmidt, twice), normalised into
+// V_(j+1), and for GMRES the Hessenberg column is rotated (k_gm_arnoldi's work).  As separate
+// kernels this is eleven launches of 2 to 13 us for suspensions of a few thousand blobs,
+// each waiting for a handful of warps; here a cluster of up to 8 blocks per suspension keeps
+// its part of w in shared memory, and the partial inner products meet through distributed
+// shared memory (every block adds all of them in block order, so each holds the same sums;
+// deterministic).
+//
+// Bound by the FP64 pipes of the cluster's SMs: 4 (j + 1) n FMAs at 2 per clock per SM.  Eight
+// SMs take 8 us for n = 9,216 at j = 6; at n = 32,768 (GDC_ORTH_SLICE elements per block) the
+// whole chip's separate kernels become as fast, and beyond it they are used.
+
+namespace cg = cooperative_groups;
+
+constexpr int ORTH_TH = 256;
+constexpr int ORTH_PART = GDC_MAX_LANCZOS + 8;
+
+struct OrthGm {   // the rotation of a GMRES column (see k_gm_arnoldi); H null for Lanczos
+    int m;
+    double *H, *cs, *sn, *g;
+    const double* bnorm;
+    double inner_tol;
+    double* est;
+    int *active, *jcount;
+};
+
+struct OrthLz {   // what k_lz_tridiag reads (h null for GMRES), and the exhaustion test's inputs
+    double *h, *wn2;
+    const double* alpha;
+    int cols, kmax;
+    const long long* susp_blob_off;
+};
+
+__global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __restrict__ off, double* V, long long ld,
+                                                  const double* __restrict__ w, int j, const int* __restrict__ jdev,
+                                                  const int* active, double* __restrict__ vcur, OrthGm gm, OrthLz lz) {
+    extern __shared__ double ws[];   // this block's part of w
+    __shared__ double part[3][ORTH_PART];   // this block's partial sums: two passes, the norm
+    __shared__ double hs[ORTH_PART], hsum[ORTH_PART];
+    __shared__ double norm[2];   // beta and 1 / beta (0 when the space is exhausted)
+    cg::cluster_group cl = cg::this_cluster();
+    const int s = blockIdx.x / C, rank = blockIdx.x % C;
+    if (jdev) j = *jdev;
+    const int k = j + 1;
+    const long long o0 = off[s], n = off[s + 1] - o0;
+    const int per = (int)((n + C - 1) / C);
+    const long long lo = o0 + (long long)rank * per;
+    const int m = (int)max(0LL, min((long long)per, o0 + n - lo));
+    double* Vn = V + (long long)k * ld + lo;
+    if (!active[s]) {   // a stopped loop: zeros, as its scale factor was
+        for (int e = threadIdx.x; e < m; e += ORTH_TH) {
+            Vn[e] = 0.0;
+            if (vcur) vcur[lo + e] = 0.0;
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < m; e += ORTH_TH) ws[e] = w[lo + e];
+    if (threadIdx.x < k) hsum[threadIdx.x] = 0.0;
+    // few columns: G warps share one, each a contiguous piece of the block's part
+    const int G = k >= 8 ? 1 : (k >= 4 ? 2 : (k >= 2 ? 4 : 8));
+    const int piece = (m + G - 1) / G;
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int u = warp; u < k * G; u += ORTH_TH / 32) {
+            const int i = u / G, e0 = (u % G) * piece, e1 = min(m, e0 + piece);
+            const double* Vi = V + (long long)i * ld + lo;
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+            int e = e0 + lane;
+            for (; e + 96 < e1; e += 128) {
+                const double v0 = Vi[e], v1 = Vi[e + 32], v2 = Vi[e + 64], v3 = Vi[e + 96];
+                a0 = fma(v0, ws[e], a0);
+                a1 = fma(v1, ws[e + 32], a1);
+                a2 = fma(v2, ws[e + 64], a2);
+                a3 = fma(v3, ws[e + 96], a3);
+            }
+            for (; e < e1; e += 32) a0 = fma(Vi[e], ws[e], a0);
+            const double acc = warp_sum((a0 + a1) + (a2 + a3));
+            if (lane == 0) part[pass][u] = acc;
+        }
+        cl.sync();
+        if (threadIdx.x < k) {
+            double h = 0.0;
+            for (int c = 0; c < C; ++c) {
+                const double* p = cl.map_shared_rank(part[pass], c);
+                for (int g = 0; g < G; ++g) h += p[threadIdx.x * G + g];
+            }
+            hs[threadIdx.x] = h;
+            hsum[threadIdx.x] += h;
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < m; e += ORTH_TH) {
+            const double* Ve = V + lo + e;
+            double a0 = ws[e], a1 = 0.0;
+            int i = 0;
+#pragma unroll 4
+            for (; i + 1 < k; i += 2) {
+                a0 = fma(-hs[i], Ve[(long long)i * ld], a0);
+                a1 = fma(-hs[i + 1], Ve[(long long)(i + 1) * ld], a1);
+            }
+            if (i < k) a0 = fma(-hs[i], Ve[(long long)i * ld], a0);
+            ws[e] = a0 + a1;
+        }
+        __syncthreads();
+    }
+    double q = 0.0;
+    for (int e = threadIdx.x; e < m; e += ORTH_TH) q = fma(ws[e], ws[e], q);
+    q = warp_sum(q);
+    if (lane == 0) part[2][warp] = q;
+    __syncthreads();
+    if (warp == 0) {
+        q = warp_sum(lane < ORTH_TH / 32 ? part[2][lane] : 0.0);
+        if (lane == 0) part[2][ORTH_TH / 32] = q;
+    }
+    cl.sync();
+    if (warp == 0) {   // one warp: FP64 instructions cost the same whichever lanes need them
+        const double wn2 = warp_sum(lane < C ? *cl.map_shared_rank(&part[2][ORTH_TH / 32], lane) : 0.0);
+        double beta = sqrt(fmax(wn2, 0.0));
+        if (lz.h) {   // Krylov space exhausted or numerically invariant, as k_lz_tridiag decides
+            const double aj = hsum[j], a0 = j == 0 ? aj : lz.alpha[(long long)s * lz.kmax];
+            const long long dim = 3 * (lz.susp_blob_off[s + 1] - lz.susp_blob_off[s]);
+            if (k >= dim || beta <= 1e-14 * fmax(fabs(a0), fabs(aj))) beta = 0.0;
+            if (rank == 0 && lane == 0) lz.wn2[(long long)s * lz.cols] = wn2;
+        }
+        if (lane == 0) {
+            norm[0] = beta;
+            norm[1] = beta > 0.0 ? 1.0 / beta : 0.0;
+        }
+    }
+    __syncthreads();
+    const double scal = norm[1];
+    for (int e = threadIdx.x; e < m; e += ORTH_TH) {
+        const double v = ws[e] * scal;
+        Vn[e] = v;
+        if (vcur) vcur[lo + e] = v;
+    }
+    if (rank == 0) {
+        if (lz.h && threadIdx.x < k) lz.h[(long long)s * lz.cols + threadIdx.x] = hsum[threadIdx.x];
+        if (gm.H && threadIdx.x < j) {   // the previous rotations into shared memory for the chain below
+            part[0][threadIdx.x] = gm.cs[(long long)s * gm.m + threadIdx.x];
+            part[1][threadIdx.x] = gm.sn[(long long)s * gm.m + threadIdx.x];
+        }
+    }
+    cl.sync();   // every block has read the others' norms before any leaves
+    if (gm.H && rank == 0 && threadIdx.x == 0) {
+        double* Hs = gm.H + (long long)s * (gm.m + 1) * gm.m;
+        double* gs = gm.g + (long long)s * (gm.m + 1);
+        double a = hsum[0];
+        for (int i = 0; i < j; ++i) {
+            const double c = part[0][i], t = part[1][i], b = hsum[i + 1];
+            Hs[i * gm.m + j] = c * a + t * b;
+            a = -t * a + c * b;
+        }
+        const double beta = norm[0], rr = hypot(a, beta);
+        const double cc = rr > 0.0 ? a / rr : 1.0, ss = rr > 0.0 ? beta / rr : 0.0;
+        gm.cs[(long long)s * gm.m + j] = cc;
+        gm.sn[(long long)s * gm.m + j] = ss;
+        Hs[j * gm.m + j] = rr;
+        Hs[(j + 1) * gm.m + j] = 0.0;
+        const double gj = gs[j];
+        gs[j + 1] = -ss * gj;
+        gs[j] = cc * gj;
+        const double e = fabs(ss * gj) / gm.bnorm[s];
+        gm.est[s] = e;
+        gm.jcount[s] = j + 1;
+        if (!(e > gm.inner_tol) || beta == 0.0 || j + 1 == gm.m) gm.active[s] = 0;
+    }
+}
+
+static long long longest_segment(const gdc::Seg& sg) {
+    long long n = 1;
+    for (size_t s = 0; s + 1 < sg.h_off.size(); ++s) n = std::max(n, sg.h_off[s + 1] - sg.h_off[s]);
+    return n;
+}
+
+// Blocks per cluster of the fused orthogonalisation of a segmented space, 0: the separate
+// kernels (a suspension longer than 8 parts).  Parts of at most 1,024 elements while the
+// cluster can grow, so that a suspension spreads over more FP64 pipes.
+static int orth_cluster(const gdc::Seg& sg) {
+    const long long n = longest_segment(sg);
+    if (n > 8LL * GDC_ORTH_SLICE) return 0;
+    int C = 1;
+    while (C < 8 && n > 1024LL * C) C *= 2;
+    return C;
+}
+
+static void launch_orth(gdc_ctx* c, const gdc::Seg& sg, int C, double* V, long long ld, const double* w, int j,
+                        const int* jdev, const int* active, double* vcur, const OrthGm& gm, const OrthLz& lz) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(c->S * C));
+    cfg.blockDim = dim3(ORTH_TH);
+    cfg.dynamicSmemBytes = sizeof(double) * (size_t)((longest_segment(sg) + C - 1) / C);
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ++c->n_launch;
+    cudaLaunchKernelEx(&cfg, k_orth, C, sg.off, V, ld, w, j, jdev, active, vcur, gm, lz);
+}
+
+// A GMRES iteration's orthogonalisation of gm_w against V_0..V_j, and its column of H
+static void gm_orthogonalise(gdc_ctx* c, int j, const int* jd, double inner_tol, double* vcur) {
+    const gdc::Seg& sg = c->seg_gm;
+    const long long n = c->ngm;
+    const int m = c->m, cols = c->red_cols, cap = jd ? m : 0, k = jd ? 1 : j + 1;
+    if (const int C = orth_cluster(sg)) {
+        const OrthGm gm{m, c->gm_H, c->gm_cs, c->gm_sn, c->gm_g, c->gm_bnorm, inner_tol, c->gm_res + c->S, c->gm_active,
+                        c->gm_j};
+        launch_orth(c, sg, C, c->gm_V, n, c->gm_w, j, jd, c->gm_active, vcur, gm, OrthLz{});
+        return;
+    }
+    seg_mdot(c, sg, c->gm_V, n, k, c->gm_w, c->gm_h, cols, jd, cap);
+    ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, k, jd, c->gm_h, cols, c->gm_w);
+    seg_mdot(c, sg, c->gm_V, n, k, c->gm_w, c->gm_h2, cols, jd, cap);
+    ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, k, jd, c->gm_h2, cols, c->gm_w);
+    ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(k, jd, c->gm_h, c->gm_h2, cols);
+    // ||w||: the column of wn2 lives after the h coefficients
+    seg_mdot(c, sg, c->gm_w, 0, 1, c->gm_w, c->gm_h2, cols);
+    ++c->n_launch, k_gm_arnoldi<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(
+        c->S, j, jd, m, c->gm_h, cols, c->gm_h2, c->gm_H, c->gm_cs, c->gm_sn, c->gm_g, c->gm_bnorm, inner_tol,
+        c->gm_res + c->S, c->gm_active, c->gm_j, c->gm_scal);
+    ++c->n_launch, k_seg_scale_slot<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_w, c->gm_scal, c->gm_V, n, jd,
+                                                                        jd ? 1 : j + 1, vcur);
+}
+
 gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* info) {
     // FCM: one operator whatever the precision, so no refinement against a second product
     const int prec = c->fcm ? GDC_FP64 : c->p.precision;
@@ -446,19 +678,7 @@ gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* i
             saddle_op(c, prec, c->gm_z, c->gm_w);
             c->mv_active = nullptr;
             if (prec == GDC_FP32_MIXED) inf.matvecs_fp32++; else inf.matvecs_fp64++;
-            // classical Gram-Schmidt, twice
-            seg_mdot(c, sg, c->gm_V, n, j + 1, c->gm_w, c->gm_h, cols);
-            ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, j + 1, nullptr, c->gm_h, cols, c->gm_w);
-            seg_mdot(c, sg, c->gm_V, n, j + 1, c->gm_w, c->gm_h2, cols);
-            ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, j + 1, nullptr, c->gm_h2, cols, c->gm_w);
-            ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(j + 1, nullptr, c->gm_h, c->gm_h2, cols);
-            // ||w||: the column of wn2 lives after the h coefficients
-            seg_mdot(c, sg, c->gm_w, 0, 1, c->gm_w, c->gm_h2, cols);
-            ++c->n_launch, k_gm_arnoldi<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(c->S, j, nullptr, m, c->gm_h, cols, c->gm_h2, c->gm_H,
-                                                                     c->gm_cs, c->gm_sn, c->gm_g, c->gm_bnorm,
-                                                                     inner_tol, c->gm_res + c->S, c->gm_active,
-                                                                     c->gm_j, c->gm_scal);
-            ++c->n_launch, k_seg_scale<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_w, c->gm_scal, c->gm_V + (long long)(j + 1) * n);
+            gm_orthogonalise(c, j, nullptr, inner_tol, nullptr);
             ++total;
             if ((st = sync_read(c, c->gm_active, act.data(), sizeof(int) * c->S)) != GDC_OK) return st;
             bool still = false;
@@ -907,6 +1127,33 @@ void krylov_init_attributes() {
                          (int)lz_tridiag_smem(GDC_MAX_LANCZOS));
 }
 
+// A Lanczos iteration's full reorthogonalisation of lz_w against v_0..v_j, the eigen-step and
+// v_(j+1)
+static void lz_orthogonalise(gdc_ctx* c, int j, const int* jd, int fixed_mode, double* vcur) {
+    const gdc::Seg& sg = c->seg_lz;
+    const long long n = 3LL * c->NBL;
+    const int cols = c->red_cols, kmax = c->kmax, cap = jd ? kmax : 0, k = jd ? 1 : j + 1;
+    const int C = orth_cluster(sg);
+    if (C) {
+        launch_orth(c, sg, C, c->lz_V, n, c->lz_w, j, jd, c->lz_active, vcur, OrthGm{},
+                    OrthLz{c->lz_h, c->gm_h2, c->lz_alpha, cols, kmax, c->susp_blob_off});
+    } else {
+        seg_mdot(c, sg, c->lz_V, n, k, c->lz_w, c->lz_h, cols, jd, cap);
+        ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, k, jd, c->lz_h, cols, c->lz_w);
+        seg_mdot(c, sg, c->lz_V, n, k, c->lz_w, c->gm_h2, cols, jd, cap);
+        ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, k, jd, c->gm_h2, cols, c->lz_w);
+        ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(k, jd, c->lz_h, c->gm_h2, cols);
+        seg_mdot(c, sg, c->lz_w, 0, 1, c->lz_w, c->gm_h2, cols);
+    }
+    ++c->n_launch, k_lz_tridiag<<<c->S, 32, lz_launch_smem(c), c->stream>>>(
+        c->S, j, jd, c->lz_h, cols, c->gm_h2, c->lz_alpha, c->lz_beta, c->lz_Wnorm, c->lz_c, c->lz_err, c->lz_active,
+        c->lz_k, c->lz_lastk, c->lz_scal, c->p.lanczos_tol, fixed_mode ? c->lz_fix : nullptr, c->lz_hint, kmax,
+        c->susp_blob_off, c->dev_status, c->lz_qbuf_on ? c->lz_qbuf : nullptr);
+    if (!C)
+        ++c->n_launch, k_seg_scale_slot<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_w, c->lz_scal, c->lz_V, n,
+                                                                            jd, jd ? 1 : j + 1, vcur);
+}
+
 gdc_status lanczos_sqrt(gdc_ctx* c, const double* W, double* out, double scale, int fixed_mode,
                         int* iters_out, double* err_out) {
     const int prec = c->p.precision;
@@ -927,19 +1174,7 @@ gdc_status lanczos_sqrt(gdc_ctx* c, const double* W, double* out, double scale, 
         c->mv_active = c->lz_active;   // suspensions that have stopped need no product
         lz_operator(c, prec, Vj, c->lz_w);
         c->mv_active = nullptr;
-        // w = M v_j orthogonalised against v_0..v_j twice (full reorthogonalisation)
-        seg_mdot(c, sg, c->lz_V, n, j + 1, c->lz_w, c->lz_h, cols);
-        ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, j + 1, nullptr, c->lz_h, cols, c->lz_w);
-        seg_mdot(c, sg, c->lz_V, n, j + 1, c->lz_w, c->gm_h2, cols);
-        ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, j + 1, nullptr, c->gm_h2, cols, c->lz_w);
-        ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(j + 1, nullptr, c->lz_h, c->gm_h2, cols);
-        seg_mdot(c, sg, c->lz_w, 0, 1, c->lz_w, c->gm_h2, cols);
-        ++c->n_launch, k_lz_tridiag<<<c->S, 32, lz_launch_smem(c), c->stream>>>(
-            c->S, j, nullptr, c->lz_h, cols, c->gm_h2, c->lz_alpha, c->lz_beta, c->lz_Wnorm, c->lz_c, c->lz_err, c->lz_active,
-            c->lz_k, c->lz_lastk, c->lz_scal, c->p.lanczos_tol, fixed_mode ? c->lz_fix : nullptr, c->lz_hint, kmax, c->susp_blob_off,
-            c->dev_status, c->lz_qbuf_on ? c->lz_qbuf : nullptr);
-        ++c->n_launch, k_seg_scale<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_w, c->lz_scal,
-                                                                       c->lz_V + (long long)(j + 1) * n);
+        lz_orthogonalise(c, j, nullptr, fixed_mode, nullptr);
         if ((st = sync_read(c, c->lz_active, act.data(), sizeof(int) * c->S)) != GDC_OK) return st;
         bool still = false;
         for (int s = 0; s < c->S; ++s) still = still || act[s];
@@ -1211,18 +1446,7 @@ void lanczos_sqrt_graph(gdc_ctx* c, const double* W, double* out, double scale, 
     c->mv_active = c->lz_active;
     lz_operator(c, prec, c->lz_vcur, c->lz_w);
     c->mv_active = nullptr;
-    seg_mdot(c, sg, c->lz_V, n, 1, c->lz_w, c->lz_h, cols, jd, kmax);
-    ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, 1, jd, c->lz_h, cols, c->lz_w);
-    seg_mdot(c, sg, c->lz_V, n, 1, c->lz_w, c->gm_h2, cols, jd, kmax);
-    ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_V, n, 1, jd, c->gm_h2, cols, c->lz_w);
-    ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(1, jd, c->lz_h, c->gm_h2, cols);
-    seg_mdot(c, sg, c->lz_w, 0, 1, c->lz_w, c->gm_h2, cols);
-    ++c->n_launch, k_lz_tridiag<<<c->S, 32, lz_launch_smem(c), c->stream>>>(
-        c->S, 0, jd, c->lz_h, cols, c->gm_h2, c->lz_alpha, c->lz_beta, c->lz_Wnorm, c->lz_c, c->lz_err, c->lz_active,
-        c->lz_k, c->lz_lastk, c->lz_scal, c->p.lanczos_tol, fixed_mode ? c->lz_fix : nullptr, c->lz_hint, kmax,
-        c->susp_blob_off, c->dev_status, c->lz_qbuf_on ? c->lz_qbuf : nullptr);
-    ++c->n_launch, k_seg_scale_slot<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->lz_w, c->lz_scal, c->lz_V, n, jd,
-                                                                        1, c->lz_vcur);
+    lz_orthogonalise(c, 0, jd, fixed_mode, c->lz_vcur);
     ++c->n_launch, k_lz_next<<<1, 32, 0, c->stream>>>(c->S, c->lz_active, c->ctl, kmax, h);
     cap_while_end(c, REP_LZ0 + run, before);
     lz_result(c, scale, out);
@@ -1269,17 +1493,7 @@ void gmres_solve_graph(gdc_ctx* c, const double* b, double* x) {
             c->mv_active = c->gm_active;
             saddle_op(c, prec, c->gm_z, c->gm_w);
             c->mv_active = nullptr;
-            seg_mdot(c, sg, c->gm_V, n, 1, c->gm_w, c->gm_h, cols, jd, m);
-            ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, 1, jd, c->gm_h, cols, c->gm_w);
-            seg_mdot(c, sg, c->gm_V, n, 1, c->gm_w, c->gm_h2, cols, jd, m);
-            ++c->n_launch, k_mupdate<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, 1, jd, c->gm_h2, cols, c->gm_w);
-            ++c->n_launch, k_add_cols<<<c->S, 128, 0, c->stream>>>(1, jd, c->gm_h, c->gm_h2, cols);
-            seg_mdot(c, sg, c->gm_w, 0, 1, c->gm_w, c->gm_h2, cols);
-            ++c->n_launch, k_gm_arnoldi<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(
-                c->S, 0, jd, m, c->gm_h, cols, c->gm_h2, c->gm_H, c->gm_cs, c->gm_sn, c->gm_g, c->gm_bnorm, inner_tol,
-                c->gm_res + c->S, c->gm_active, c->gm_j, c->gm_scal);
-            ++c->n_launch, k_seg_scale_slot<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_w, c->gm_scal, c->gm_V,
-                                                                                n, jd, 1, c->gm_vcur);
+            gm_orthogonalise(c, 0, jd, inner_tol, c->gm_vcur);
             ++c->n_launch, k_gm_inner_next<<<1, 32, 0, c->stream>>>(c->S, c->gm_active, c->ctl, max_iter, hi);
         }
         cap_while_end(c, REP_GM_TOTAL, before_i);
