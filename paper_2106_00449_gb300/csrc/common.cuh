@@ -36,6 +36,7 @@
 #define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
 #define GDC_NEAR_SRC_MAX 2048
 #define GDC_SYM_TILE 512         // blobs per tile of the symmetric FP32 pair kernel
+#define GDC_P64_EPI_WIDE 8192    // its epilogue: 16 threads per blob up to this many blobs, 4 above
 #define GDC_P64_WIDE 16384       // FP64 pair kernel: 512-blob tiles for suspensions above this, 128-blob ones up to it
 #define GDC_TUNE_PAIRS 268435456.0   // ordered pairs per product (16,384^2) from which the autotuner times candidates
 #define GDC_CELL_MIN_BLOBS 16384 // GDC_FORCES_CHOOSE: the cell list from this many blobs on

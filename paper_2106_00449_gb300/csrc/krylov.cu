@@ -399,12 +399,13 @@ __global__ void k_gm_backsolve(int S, int m, const double* __restrict__ H, const
 // deterministic).
 //
 // Bound by the FP64 pipes of the cluster's SMs: 4 (j + 1) n FMAs at 2 per clock per SM.  Eight
-// SMs take 8 us for n = 9,216 at j = 6; at n = 32,768 (GDC_ORTH_SLICE elements per block) the
+// SMs need 8 us for n = 9,216 at j = 6 (30 us measured, 46% FP64 pipe: the rest is the latency of
+// the passes, kept down by 16 warps and 8 loads in flight per thread); at n = 32,768 (GDC_ORTH_SLICE elements per block) the
 // whole chip's separate kernels become as fast, and beyond it they are used.
 
 namespace cg = cooperative_groups;
 
-constexpr int ORTH_TH = 256;
+constexpr int ORTH_TH = 512;
 constexpr int ORTH_PART = GDC_MAX_LANCZOS + 8;
 
 struct OrthGm {   // the rotation of a GMRES column (see k_gm_arnoldi); H null for Lanczos
@@ -450,24 +451,26 @@ __global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __rest
     for (int e = threadIdx.x; e < m; e += ORTH_TH) ws[e] = w[lo + e];
     if (threadIdx.x < k) hsum[threadIdx.x] = 0.0;
     // few columns: G warps share one, each a contiguous piece of the block's part
-    const int G = k >= 8 ? 1 : (k >= 4 ? 2 : (k >= 2 ? 4 : 8));
+    const int G = k >= 9 ? 1 : (k >= 5 ? 2 : (k >= 3 ? 4 : 8));
     const int piece = (m + G - 1) / G;
     __syncthreads();
     for (int pass = 0; pass < 2; ++pass) {
         for (int u = warp; u < k * G; u += ORTH_TH / 32) {
             const int i = u / G, e0 = (u % G) * piece, e1 = min(m, e0 + piece);
             const double* Vi = V + (long long)i * ld + lo;
-            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-            int e = e0 + lane;
-            for (; e + 96 < e1; e += 128) {
-                const double v0 = Vi[e], v1 = Vi[e + 32], v2 = Vi[e + 64], v3 = Vi[e + 96];
-                a0 = fma(v0, ws[e], a0);
-                a1 = fma(v1, ws[e + 32], a1);
-                a2 = fma(v2, ws[e + 64], a2);
-                a3 = fma(v3, ws[e + 96], a3);
+            // eight loads in flight per lane: the first pass waits for L2
+            double a0 = 0.0, a1 = 0.0;
+            for (int e = e0 + lane; e < e1; e += 256) {
+                double v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = e + 32 * q < e1 ? Vi[e + 32 * q] : 0.0;
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    if (e + 32 * q < e1) a0 = fma(v[q], ws[e + 32 * q], a0);
+                    if (e + 32 * q + 32 < e1) a1 = fma(v[q + 1], ws[e + 32 * q + 32], a1);
+                }
             }
-            for (; e < e1; e += 32) a0 = fma(Vi[e], ws[e], a0);
-            const double acc = warp_sum((a0 + a1) + (a2 + a3));
+            const double acc = warp_sum(a0 + a1);
             if (lane == 0) part[pass][u] = acc;
         }
         cl.sync();
@@ -485,12 +488,18 @@ __global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __rest
             const double* Ve = V + lo + e;
             double a0 = ws[e], a1 = 0.0;
             int i = 0;
-#pragma unroll 4
-            for (; i + 1 < k; i += 2) {
-                a0 = fma(-hs[i], Ve[(long long)i * ld], a0);
-                a1 = fma(-hs[i + 1], Ve[(long long)(i + 1) * ld], a1);
+            for (; i + 7 < k; i += 8) {
+                double v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = Ve[(long long)(i + q) * ld];
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    a0 = fma(-hs[i + q], v[q], a0);
+                    a1 = fma(-hs[i + q + 1], v[q + 1], a1);
+                }
             }
-            if (i < k) a0 = fma(-hs[i], Ve[(long long)i * ld], a0);
+#pragma unroll 4
+            for (; i < k; ++i) a0 = fma(-hs[i], Ve[(long long)i * ld], a0);
             ws[e] = a0 + a1;
         }
         __syncthreads();

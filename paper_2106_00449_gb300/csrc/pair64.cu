@@ -194,17 +194,19 @@ __global__ void __launch_bounds__(128, TPL == 1 ? 5 : 3) k_rpy64_sym(
 
 // u_i = c0 (target-side slots of the blob's tile row + source-side slots of the tiles before
 // it) [- K V], for this kernel and the symmetric double-float one (dfsym.cu; its same-body
-// blocks are added afterwards).  Four threads per blob, each taking every fourth slot, added in a fixed order:
-// the slots are latency-bound L2 reads, and one thread per blob left small suspensions with
-// a few warps.
+// blocks are added afterwards).  EPI threads per blob, each taking every EPI-th slot, joined in
+// a fixed order: the slots are latency-bound L2 reads, and the short ranges of small
+// suspensions leave up to 200 of them per blob.  16 threads up to GDC_P64_EPI_WIDE blobs, 4
+// above, where the FP64 shuffle sums would cost more than the chain.
+template <int EPI>
 __global__ void __launch_bounds__(128) k_p64_epilogue(
     int NBL, int TS, const double4_32a* __restrict__ part_i, const double4_32a* __restrict__ part_j,
     const int* __restrict__ blob_susp, const long long* __restrict__ susp_blob_off, const int* __restrict__ row_nk,
     const long long* __restrict__ tile_base, const long long* __restrict__ jbase, double c0, const double* __restrict__ x,
     double* __restrict__ y, int gm_layout, const int* __restrict__ blob_gm, const int* __restrict__ body_gm,
     const int* __restrict__ blob_body, const double* __restrict__ r, const double* __restrict__ Yc) {
-    const int sub = threadIdx.x & 3;
-    const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 2);
+    const int sub = threadIdx.x % EPI;
+    const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / EPI);
     double ux = 0.0, uy = 0.0, uz = 0.0;
     if (i < NBL) {
         const int s = blob_susp[i];
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(128) k_p64_epilogue(
         const int J = loc / TS, e = loc - J * TS;
         const int n = row_nk[tile_base[s] + J];
 #pragma unroll 4
-        for (int q = sub; q < n; q += 4) {
+        for (int q = sub; q < n; q += EPI) {
             const double4_32a v = part_i[(long long)q * NBL + i];
             ux += v.x;
             uy += v.y;
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(128) k_p64_epilogue(
         }
         const long long s0 = jbase[s] + (long long)J * (J - 1) / 2;
 #pragma unroll 4
-        for (int I = sub; I < J; I += 4) {
+        for (int I = sub; I < J; I += EPI) {
             const double4_32a v = part_j[(s0 + I) * TS + e];
             ux += v.x;
             uy += v.y;
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(128) k_p64_epilogue(
         }
     }
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
+    for (int o = 1; o < EPI; o <<= 1) {
         ux += __shfl_xor_sync(0xffffffffu, ux, o);
         uy += __shfl_xor_sync(0xffffffffu, uy, o);
         uz += __shfl_xor_sync(0xffffffffu, uz, o);
@@ -293,11 +295,18 @@ void launch_rpy64_sym(gdc_ctx* c, const double* x, int gm_layout) {
 
 void launch_p64_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int gm_layout) {
     const bool df = prec == GDC_PREC_DF64;   // the double-float kernel's slots
-    ++c->n_launch, k_p64_epilogue<<<ceil_div(4LL * c->NBL, 128), 128, 0, c->stream>>>(
-        c->NBL, df ? GDC_SYM_TILE : c->p64_tile, df ? c->dfs_part_i : c->p64_part_i, df ? c->dfs_part_j : c->p64_part_j,
-        c->blob_susp, c->susp_blob_off, df ? c->dfs_row_nk : c->p64_row_nk, df ? c->sym_tile_base : c->p64_tile_base,
-        df ? c->sym_jbase : c->p64_jbase, 1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm,
-        c->body_gm, c->blob_body, c->r, c->Yc);
+#define GDC_P64_EPI(EPI)                                                                                          \
+    k_p64_epilogue<EPI><<<ceil_div((long long)EPI * c->NBL, 128), 128, 0, c->stream>>>(                           \
+        c->NBL, df ? GDC_SYM_TILE : c->p64_tile, df ? c->dfs_part_i : c->p64_part_i,                              \
+        df ? c->dfs_part_j : c->p64_part_j, c->blob_susp, c->susp_blob_off, df ? c->dfs_row_nk : c->p64_row_nk,    \
+        df ? c->sym_tile_base : c->p64_tile_base, df ? c->sym_jbase : c->p64_jbase,                               \
+        1.0 / (8.0 * 3.141592653589793 * c->p.eta), x, y, gm_layout, c->blob_gm, c->body_gm, c->blob_body, c->r, c->Yc)
+    ++c->n_launch;
+    if (c->NBL <= GDC_P64_EPI_WIDE)
+        GDC_P64_EPI(16);
+    else
+        GDC_P64_EPI(4);
+#undef GDC_P64_EPI
 }
 
 }  // namespace gdc
