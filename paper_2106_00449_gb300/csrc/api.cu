@@ -172,31 +172,20 @@ static const char* build_host_layout(gdc_ctx* c, const gdc_params* p, int n_temp
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 152;
     c->device = dev;
     c->num_sms = sms;
-    // bodies per block of the factor products: as many as keep 8 blocks per SM busy (at most
-    // GDC_TB_MAX), fewer for large templates (at most 2,048 rows per block: 40 KB of shared
-    // memory in the factor products, 41 KB in the preconditioner); below 4 per
-    // block the products keep one block per body (measured faster there: 2,520 bodies)
+    // bodies of one template per block of the per-body products (body.cu)
     {
-        int B = 1;
-        while (B < GDC_TB_MAX && NB >= 2LL * B * 8 * sms) B *= 2;
-        c->tb_use = B >= 4;
+        int B = NB >= 40LL * sms ? 8 : (NB >= 512 ? 4 : 1);
+        if (3 * c->max_body_blobs > 256) B = 1;
+        c->tb_group = B;
         c->lz_qbuf_on = n_susp > sms;   // the eigen-step's scratch: see krylov.cu
         std::vector<std::vector<int>> by_t(n_templates);
         for (long long b = 0; b < NB; ++b) by_t[body_tmpl[b]].push_back((int)b);
         c->h_tb_items.clear();
         c->h_tb_bodies.clear();
-        c->tb_smem = 0;
-        c->tb_precond_smem = 0;
         for (int t = 0; t < n_templates; ++t) {
-            const int n3 = 3 * tmpl_nblobs[t];
-            const int bt = std::max(1, std::min(B, 2048 / n3));
-            for (size_t i = 0; i < by_t[t].size(); i += bt) {
-                const int cnt = (int)std::min<size_t>(bt, by_t[t].size() - i);
-                c->h_tb_items.push_back(make_int4(t, (int)c->h_tb_bodies.size() + (int)i, cnt, 0));
-                c->tb_smem = std::max(c->tb_smem, (size_t)cnt * n3 * 2 * sizeof(double));
-                c->tb_precond_smem = std::max(c->tb_precond_smem,
-                                              (size_t)cnt * ((2 * n3 + 16) * sizeof(double) + n3 * sizeof(float)));
-            }
+            for (size_t i = 0; i < by_t[t].size(); i += B)
+                c->h_tb_items.push_back(make_int4(t, (int)c->h_tb_bodies.size() + (int)i,
+                                                  (int)std::min<size_t>(B, by_t[t].size() - i), 0));
             c->h_tb_bodies.insert(c->h_tb_bodies.end(), by_t[t].begin(), by_t[t].end());
         }
         c->tb_n_items = (int)c->h_tb_items.size();

@@ -16,49 +16,54 @@
 
 namespace gdc {
 
-// ---- K^T: [sum lambda_i; sum (r_i - Y_p) x lambda_i] per body, one warp per body ----
+// ---- K^T: [sum lambda_i; sum (r_i - Y_p) x lambda_i] per body, eight lanes per body ----
+//
+// Bound by the FP64 pipe, which charges a warp instruction the same whichever lanes need it:
+// a warp per body spends 30 adds on the six shuffle sums of each body, eight lanes per body 18
+// on those of four (2,987 bodies: 18.5 us a warp each).
 
-__global__ void k_body_KT(int NB, const long long* __restrict__ body_blob_off, const int* __restrict__ blob_gm,
-                          const int* __restrict__ body_gm, const double* __restrict__ x, int x_gm,
-                          double* __restrict__ y, int y_gm, double scale, const double* __restrict__ r,
-                          const double* __restrict__ Yc) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= NB) return;
-    const int p = warp;
+constexpr int KT_LANES = 8;
+
+// the sum of each of six values over the KT_LANES lanes of a body, on every lane
+__device__ __forceinline__ void body_sum6(double* g) {
+#pragma unroll
+    for (int o = 1; o < KT_LANES; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) g[k] += __shfl_xor_sync(0xffffffffu, g[k], o);
+}
+
+__device__ __forceinline__ void kt_add(double* g, double d0, double d1, double d2, double l0, double l1, double l2) {
+    g[0] += l0;
+    g[1] += l1;
+    g[2] += l2;
+    g[3] += d1 * l2 - d2 * l1;
+    g[4] += d2 * l0 - d0 * l2;
+    g[5] += d0 * l1 - d1 * l0;
+}
+
+__global__ void __launch_bounds__(128) k_body_KT(int NB, const long long* __restrict__ body_blob_off,
+                                                 const int* __restrict__ blob_gm, const int* __restrict__ body_gm,
+                                                 const double* __restrict__ x, int x_gm, double* __restrict__ y, int y_gm,
+                                                 double scale, const double* __restrict__ r, const double* __restrict__ Yc) {
+    const int sub = threadIdx.x % KT_LANES;
+    const int p0 = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / KT_LANES);
+    const int p = min(p0, NB - 1);   // whole warps reach the shuffles
     const double Y0 = Yc[3 * p], Y1 = Yc[3 * p + 1], Y2 = Yc[3 * p + 2];
-    double f0 = 0, f1 = 0, f2 = 0, t0 = 0, t1 = 0, t2 = 0;
-    for (long long i = body_blob_off[p] + lane; i < body_blob_off[p + 1]; i += 32) {
+    double g[6] = {0, 0, 0, 0, 0, 0};
+    for (long long i = body_blob_off[p] + sub; i < body_blob_off[p + 1]; i += KT_LANES) {
         const long long o = x_gm ? (long long)blob_gm[i] : 3 * i;
-        const double l0 = x[o], l1 = x[o + 1], l2 = x[o + 2];
-        const double d0 = r[3 * i] - Y0, d1 = r[3 * i + 1] - Y1, d2 = r[3 * i + 2] - Y2;
-        f0 += l0;
-        f1 += l1;
-        f2 += l2;
-        t0 += d1 * l2 - d2 * l1;
-        t1 += d2 * l0 - d0 * l2;
-        t2 += d0 * l1 - d1 * l0;
+        kt_add(g, r[3 * i] - Y0, r[3 * i + 1] - Y1, r[3 * i + 2] - Y2, x[o], x[o + 1], x[o + 2]);
     }
-    f0 = warp_sum(f0);
-    f1 = warp_sum(f1);
-    f2 = warp_sum(f2);
-    t0 = warp_sum(t0);
-    t1 = warp_sum(t1);
-    t2 = warp_sum(t2);
-    if (lane == 0) {
-        const long long o = y_gm ? (long long)body_gm[p] : 6LL * p;
-        y[o] = scale * f0;
-        y[o + 1] = scale * f1;
-        y[o + 2] = scale * f2;
-        y[o + 3] = scale * t0;
-        y[o + 4] = scale * t1;
-        y[o + 5] = scale * t2;
+    body_sum6(g);
+    if (p0 < NB && sub < 6) {
+        const double v = sub == 0 ? g[0] : sub == 1 ? g[1] : sub == 2 ? g[2] : sub == 3 ? g[3] : sub == 4 ? g[4] : g[5];
+        y[(y_gm ? (long long)body_gm[p] : 6LL * p) + sub] = scale * v;
     }
 }
 
 void launch_body_KT(gdc_ctx* c, const double* x, int x_gm, double* y, int y_gm, double scale) {
-    ++c->n_launch, k_body_KT<<<ceil_div(32LL * c->NB, 256), 256, 0, c->stream>>>(c->NB, c->body_blob_off, c->blob_gm, c->body_gm, x,
-                                                                  x_gm, y, y_gm, scale, c->r, c->Yc);
+    ++c->n_launch, k_body_KT<<<ceil_div((long long)KT_LANES * c->NB, 128), 128, 0, c->stream>>>(
+        c->NB, c->body_blob_off, c->blob_gm, c->body_gm, x, x_gm, y, y_gm, scale, c->r, c->Yc);
 }
 
 // ---- step 2: calV_p = (K^T K)_p^+ K_p^T vbrev ----------------------------------------
@@ -75,463 +80,364 @@ __device__ inline void rot(const double* R, const double* v, double* o) {  // o 
     o[2] = R[6] * v[0] + R[7] * v[1] + R[8] * v[2];
 }
 
-__global__ void k_lsq(int NB, const long long* __restrict__ body_blob_off, const int* __restrict__ body_tmpl,
-                      const double* __restrict__ KtKp, const double* __restrict__ vb, const double* __restrict__ r,
-                      const double* __restrict__ Yc, const double* __restrict__ Rb, double* __restrict__ calV) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= NB) return;
-    const int p = warp;
+// eight lanes per body; lane a < 6 forms row a of the 6 x 6 product
+__global__ void __launch_bounds__(128) k_lsq(int NB, const long long* __restrict__ body_blob_off,
+                                             const int* __restrict__ body_tmpl, const double* __restrict__ KtKp,
+                                             const double* __restrict__ vb, const double* __restrict__ r,
+                                             const double* __restrict__ Yc, const double* __restrict__ Rb,
+                                             double* __restrict__ calV) {
+    const int sub = threadIdx.x % KT_LANES, lane = threadIdx.x & 31;
+    const int p0 = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) / KT_LANES);
+    const int p = min(p0, NB - 1);
     const double Y0 = Yc[3 * p], Y1 = Yc[3 * p + 1], Y2 = Yc[3 * p + 2];
     double g[6] = {0, 0, 0, 0, 0, 0};
-    for (long long i = body_blob_off[p] + lane; i < body_blob_off[p + 1]; i += 32) {
-        const double l0 = vb[3 * i], l1 = vb[3 * i + 1], l2 = vb[3 * i + 2];
-        const double d0 = r[3 * i] - Y0, d1 = r[3 * i + 1] - Y1, d2 = r[3 * i + 2] - Y2;
-        g[0] += l0;
-        g[1] += l1;
-        g[2] += l2;
-        g[3] += d1 * l2 - d2 * l1;
-        g[4] += d2 * l0 - d0 * l2;
-        g[5] += d0 * l1 - d1 * l0;
-    }
+    for (long long i = body_blob_off[p] + sub; i < body_blob_off[p + 1]; i += KT_LANES)
+        kt_add(g, r[3 * i] - Y0, r[3 * i + 1] - Y1, r[3 * i + 2] - Y2, vb[3 * i], vb[3 * i + 1], vb[3 * i + 2]);
+    body_sum6(g);
+    const double* R = Rb + 9 * p;
+    double gb[6];
+    rotT(R, g, gb);
+    rotT(R, g + 3, gb + 3);
+    const int a = min(sub, 5);
+    const double* A = KtKp + 36 * body_tmpl[p] + 6 * a;
+    double v = 0.0;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) g[k] = warp_sum(g[k]);
-    if (lane == 0) {
-        const double* R = Rb + 9 * p;
-        double gb[6], vbody[6], out[6];
-        rotT(R, g, gb);
-        rotT(R, g + 3, gb + 3);
-        const double* A = KtKp + 36 * body_tmpl[p];
-        for (int a = 0; a < 6; ++a) {
-            double acc = 0.0;
-            for (int b = 0; b < 6; ++b) acc += A[6 * a + b] * gb[b];
-            vbody[a] = acc;
-        }
-        rot(R, vbody, out);
-        rot(R, vbody + 3, out + 3);
-        for (int k = 0; k < 6; ++k) calV[6 * p + k] = out[k];
-    }
+    for (int b = 0; b < 6; ++b) v = fma(A[b], gb[b], v);
+    // rotate back: component a of R v (translation, rotation)
+    const int first = (lane & ~(KT_LANES - 1)) + (a >= 3 ? 3 : 0);
+    double o = 0.0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) o = fma(R[3 * (a % 3) + b], __shfl_sync(0xffffffffu, v, first + b), o);
+    if (p0 < NB && sub < 6) calV[6 * p + sub] = o;
 }
 
 void launch_lsq(gdc_ctx* c, const double* vbrev, double* calV) {
-    ++c->n_launch, k_lsq<<<ceil_div(32LL * c->NB, 256), 256, 0, c->stream>>>(c->NB, c->body_blob_off, c->body_tmpl, c->tmpl_KtKp,
-                                                              vbrev, c->r, c->Yc, c->Rb, calV);
+    ++c->n_launch, k_lsq<<<ceil_div((long long)KT_LANES * c->NB, 128), 128, 0, c->stream>>>(
+        c->NB, c->body_blob_off, c->body_tmpl, c->tmpl_KtKp, vbrev, c->r, c->Yc, c->Rb, calV);
 }
 
-// ---- block-diagonal preconditioner, one block per body ---------------------------------
+// ---- per-body products, bodies of one template grouped per block -------------------------
+//
+// The block preconditioner, the same-body block of a product and the factor products of the
+// preconditioned Lanczos operator all apply a (3n)^2 matrix of the body's template to rotated
+// blob vectors.  A block takes up to GB bodies of one template (tb_items): each matrix element
+// is read once for all of them.  Rows are dealt to threads and, when a block has more threads
+// than rows, the columns of a row to KS threads whose partial sums meet in shared memory (a
+// 30-row product walks 4 columns per thread instead of 30).
+//
+// Bound by the L2 latency of the matrix elements (eight in flight per thread) and, in the rest,
+// by the FP64 pipe: its cost is per warp instruction, so the rotations, the sums K^T and the
+// 6 x 6 products run flat over (body, blob) or (body, row) items of the whole block and leave no
+// lanes idle.  One 128-thread block per body spent 200 FP64 warp instructions per body in the
+// preconditioner (68% of the pipe), mostly on one lane's 6 x 6 product and 30 shuffle adds.
+//
+// GB, the bodies per block, in FP32: 8 from 40 bodies per SM on, 4 from 512 bodies on, 1 below and
+// with templates above 85 blobs.  us per launch with GB = 1 / 4 / 8 (preconditioner; same-body
+// block with K^T; factor products): 777 bodies 16.6 / 14.2 / 18.5; 15.1 / 12.3 / 16.3; 23.8 /
+// 27.5 / 24.8.  2,520 bodies 39.9 / 21.1 / 22.8; 40.2 / 18.1 / 20.7; 50.2 / 40.0 / 32.6.  12,082
+// bodies 140 / 70 / 60; 129 / 57 / 66; 154 / 95 / 77.  One block per body took 40.0, 36.0
+// (two launches) and 34.8 at 2,520 bodies.  In FP64 one body per block is as fast or faster up
+// to 3,000 bodies (same-body block 57.6 / 54.1 / 65.1, factor 34.9 / 36.6 / 46.3) and always used.
+
+constexpr int GP_TH = 256;
+
+// The columns k0..k1 of row i that a product takes: all, or a triangle's.
+enum { GP_FULL = 0, GP_FROM_DIAG = 1, GP_TO_DIAG = 2 };
+
+// Threads per row of an n3-row product and the doubles of shared memory its partial sums take.
+__host__ __device__ inline int gp_split(int n3) {
+    const int R = (n3 + 31) & ~31;
+    return R >= GP_TH ? 1 : GP_TH / R;
+}
+
+// out[u n3 + i] = sum_k M[k n3 + i] in[k GB + u] over the columns SHAPE leaves row i, u < GB (in
+// padded with zeros): sums of type T over at most n3 / KS columns, the KS partial sums added
+// in FP64.  part: KS GB n3 values of T (unused for KS = 1).  Ends with a barrier.
+template <int GB, int SHAPE, typename T>
+__device__ __forceinline__ void group_product(const T* __restrict__ M, int n3, const T* in_, T* part, double* out) {
+    // 16-byte aligned by the callers' layouts for GB >= 4, so a column's entries are vector loads
+    const T* in = GB >= 4 ? (const T*)__builtin_assume_aligned(in_, 16) : in_;
+    const int R = (n3 + 31) & ~31, KS = gp_split(n3);
+    const int ks = KS == 1 ? 0 : (int)threadIdx.x / R;
+    const int chunk = (n3 + KS - 1) / KS;
+    for (int row = KS == 1 ? (int)threadIdx.x : (int)threadIdx.x % R; row < n3 && ks < KS; row += GP_TH) {
+        int k0 = ks * chunk, k1 = min(n3, k0 + chunk);
+        if (SHAPE == GP_FROM_DIAG) k0 = max(k0, row);
+        if (SHAPE == GP_TO_DIAG) k1 = min(k1, row + 1);
+        T a[GB], b[GB];
+#pragma unroll
+        for (int u = 0; u < GB; ++u) a[u] = b[u] = T(0);
+        int k = k0;
+        const T* Mr = M + row;
+        for (; k + 7 < k1; k += 8) {   // eight elements in flight: the matrix comes from L2
+            T f[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = Mr[(long long)(k + q) * n3];
+#pragma unroll
+            for (int q = 0; q < 8; q += 2)
+#pragma unroll
+                for (int u = 0; u < GB; ++u) {
+                    a[u] = fma(f[q], in[(k + q) * GB + u], a[u]);
+                    b[u] = fma(f[q + 1], in[(k + q + 1) * GB + u], b[u]);
+                }
+        }
+#pragma unroll 2
+        for (; k + 1 < k1; k += 2) {
+            const T f = Mr[(long long)k * n3], g = Mr[(long long)(k + 1) * n3];
+#pragma unroll
+            for (int u = 0; u < GB; ++u) {
+                a[u] = fma(f, in[k * GB + u], a[u]);
+                b[u] = fma(g, in[(k + 1) * GB + u], b[u]);
+            }
+        }
+        if (k < k1) {
+            const T f = M[(long long)k * n3 + row];
+#pragma unroll
+            for (int u = 0; u < GB; ++u) a[u] = fma(f, in[k * GB + u], a[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < GB; ++u) {
+            if (KS == 1)
+                out[u * n3 + row] = (double)a[u] + (double)b[u];
+            else
+                part[(ks * GB + u) * n3 + row] = a[u] + b[u];
+        }
+    }
+    __syncthreads();
+    if (KS > 1) {
+        for (int e = threadIdx.x; e < GB * n3; e += GP_TH) {
+            double s = (double)part[e];
+            for (int q = 1; q < KS; ++q) s += (double)part[q * GB * n3 + e];
+            out[e] = s;
+        }
+        __syncthreads();
+    }
+}
+
+// Bytes of group_product's arrays: in (T), part (T), out (double)
+static size_t gp_bytes(int GB, int n3, size_t t) {
+    const int KS = gp_split(n3);
+    return (size_t)GB * n3 * (sizeof(double) + t + (KS > 1 ? KS * t : 0));
+}
+
+// K^T of the group's body-frame vectors v (double, [u][n3]) with blob offsets b: four threads per
+// (body, component), added by shuffles; thread with sub = 0 hands the sum to store(u, c, value).
+template <typename F>
+__device__ __forceinline__ void group_KT(int cnt, int n, const double* b, const double* v, F store) {
+    const int n3 = 3 * n, total = cnt * 24;
+    for (int it = threadIdx.x; it < ((total + 31) & ~31); it += GP_TH) {
+        const bool in = it < total;
+        const int q = in ? it >> 2 : 0, sub = it & 3, u = q / 6, c = q - 6 * u;
+        const double* a = v + u * n3;
+        double s0 = 0.0, s1 = 0.0;
+        if (in) {
+            if (c < 3) {
+                for (int i = sub; i < n; i += 4) s0 += a[3 * i + c];
+            } else {
+                const int w = (c - 2) % 3, z = (c - 1) % 3;   // the axes after c - 3, cyclic
+                for (int i = sub; i < n; i += 4) {
+                    s0 = fma(b[3 * i + w], a[3 * i + z], s0);
+                    s1 = fma(b[3 * i + z], a[3 * i + w], s1);
+                }
+            }
+        }
+        double s = s0 - s1;
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (in && sub == 0) store(u, c, s);
+    }
+}
+
+struct GroupArgs {   // tables the grouped kernels share
+    const int4* items;     // (template, first entry of bodies, count)
+    const int* bodies;
+    const long long* body_blob_off;
+    const int *body_tmpl, *tmpl_n, *tmpl_off;
+    const long long* mat_off;   // of a template's matrices; above a wall of each body's
+    const int *blob_gm, *body_gm;
+    const double* Rb;
+    const double* tmpl_xyz;
+};
+
+// (template or, above a wall, body; first entry of bodies; count) of the block: GB = 1 takes the
+// body of the block's index
+template <bool LAB, int GB>
+__device__ __forceinline__ int4 group_item(const GroupArgs& ga) {
+    if (GB > 1) return ga.items[blockIdx.x];
+    return make_int4(LAB ? (int)blockIdx.x : ga.body_tmpl[blockIdx.x], 0, 1, 0);
+}
+
+// the lambda part of blob i in the FP32 pair kernels' source layout (its positions are written
+// when a configuration is loaded)
+__device__ __forceinline__ void pack_lambda32(float4* sdup, long long i, const double* w) {
+    const float lx = (float)w[0], ly = (float)w[1], lz = (float)w[2];
+    reinterpret_cast<float2*>(sdup + 3 * i + 1)[1] = make_float2(lx, lx);
+    sdup[3 * i + 2] = make_float4(ly, ly, lz, lz);
+}
+
+// ---- block-diagonal preconditioner ----------------------------------------------------
 //
 // Solves [M_pp -K_p; -K_p^T 0][lam; V] = [r_lam; r_V] exactly:
 //   a = M^-1 r_lam,  V = -N (r_V + K^T a),  lam = a + G V   (N = (K^T M^-1 K)^+, G = M^-1 K)
 // in the body frame of the template.
-
+//
 // LAB = false: the template's FP64 blocks in the body frame, applied to rotated vectors.
 // LAB = true (blobs above a wall): each body's own blocks in the lab frame (set up by
-// k_wall_blocks at every configuration), blob offsets d_i = r_i - Y_p, no rotation.
-// F32: the body's M^-1 product in FP32 (the template block rounded to FP32, four interleaved
-// FP32 partial sums per row added in FP64; the rest of the block solve stays FP64), for the
-// inner cycles of the FP32-mixed mobility solve, whose operator already carries FP32 rounding:
-// the preconditioner only has to be a fixed approximation, and the FP64 product there was
-// FP64-pipe bound (1/64 of the FP32 rate).
-template <bool LAB, bool F32 = false>
-__global__ void __launch_bounds__(128) k_precond(const long long* __restrict__ body_blob_off, const int* __restrict__ body_tmpl,
-                                                 const int* __restrict__ tmpl_n, const int* __restrict__ tmpl_off,
-                                                 const long long* __restrict__ minv_off, const double* __restrict__ Minv,
-                                                 const float* __restrict__ Minv32,
-                                                 const double* __restrict__ Gt, const double* __restrict__ Nt,
-                                                 const double* __restrict__ tmpl_xyz, const int* __restrict__ blob_gm,
-                                                 const int* __restrict__ body_gm, const double* __restrict__ Rb,
-                                                 const double* __restrict__ rin, double* __restrict__ zout,
-                                                 const long long* __restrict__ blk_off, const double* __restrict__ r,
-                                                 const double* __restrict__ Yc) {
-    extern __shared__ double sh[];
-    const int p = blockIdx.x;
-    const int t = LAB ? p : body_tmpl[p];
-    const int n = LAB ? (int)(body_blob_off[p + 1] - body_blob_off[p]) : tmpl_n[t];
-    const int n3 = 3 * n;
-    double* rho = sh;          // n3
-    double* av = sh + n3;      // n3
-    double* misc = sh + 2 * n3;  // 32
-    double* bl = misc + 32;      // LAB: blob offsets d (n3)
-    float* rho32 = reinterpret_cast<float*>(misc + 32);   // F32 (never with LAB): rho in FP32 (n3)
-    const double ident[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    const double* R = LAB ? ident : Rb + 9 * p;
-    const long long i0 = body_blob_off[p];
-    if (LAB)
-        for (int e = threadIdx.x; e < n3; e += blockDim.x) bl[e] = r[3 * i0 + e] - Yc[3 * p + e % 3];
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        const long long o = blob_gm[i0 + b];
-        double v[3] = {rin[o], rin[o + 1], rin[o + 2]}, w[3];
-        rotT(R, v, w);
-        rho[3 * b] = w[0];
-        rho[3 * b + 1] = w[1];
-        rho[3 * b + 2] = w[2];
-        if (F32) {
-            rho32[3 * b] = (float)w[0];
-            rho32[3 * b + 1] = (float)w[1];
-            rho32[3 * b + 2] = (float)w[2];
-        }
-    }
-    if (threadIdx.x == 0) {
-        const long long o = body_gm[p];
-        double v[3] = {rin[o], rin[o + 1], rin[o + 2]}, w[3];
-        rotT(R, v, w);
-        misc[0] = w[0];
-        misc[1] = w[1];
-        misc[2] = w[2];
-        double v2[3] = {rin[o + 3], rin[o + 4], rin[o + 5]};
-        rotT(R, v2, w);
-        misc[3] = w[0];
-        misc[4] = w[1];
-        misc[5] = w[2];
-    }
-    __syncthreads();
-    if (F32) {
-        const float* Mi = Minv32 + minv_off[t];
-        for (int row = threadIdx.x; row < n3; row += blockDim.x) {
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            int k = 0;
-            for (; k + 3 < n3; k += 4) {   // symmetric: column-major reads are coalesced over rows
-                a0 = fmaf(Mi[(long long)k * n3 + row], rho32[k], a0);
-                a1 = fmaf(Mi[(long long)(k + 1) * n3 + row], rho32[k + 1], a1);
-                a2 = fmaf(Mi[(long long)(k + 2) * n3 + row], rho32[k + 2], a2);
-                a3 = fmaf(Mi[(long long)(k + 3) * n3 + row], rho32[k + 3], a3);
+// k_wall_blocks at every configuration), blob offsets d_i = r_i - Y_p, no rotation, one body
+// per block.
+// T = float: the M^-1 product in FP32 (the template block rounded to FP32, partial sums added
+// in FP64; the rest of the block solve stays FP64), for the inner cycles of the FP32-mixed
+// mobility solve, whose operator already carries FP32 rounding: the preconditioner only has to
+// be a fixed approximation.
+// sdup: lambda also goes there in the FP32 pair kernels' layout (the product that follows).
+template <bool LAB, int GB, typename T>
+__global__ void __launch_bounds__(GP_TH) k_precond(GroupArgs ga, const T* __restrict__ Minv, const double* __restrict__ Gt,
+                                                   const double* __restrict__ Nt, const double* __restrict__ rin,
+                                                   double* __restrict__ zout, const double* __restrict__ r,
+                                                   const double* __restrict__ Yc, float4* __restrict__ sdup) {
+    extern __shared__ __align__(16) double sh[];
+    const int4 it = group_item<LAB, GB>(ga);
+    const int t = it.x, cnt = it.z;
+    auto body = [&](int u) { return GB == 1 ? (int)blockIdx.x : ga.bodies[it.y + u]; };
+    const int n = LAB ? (int)(ga.body_blob_off[t + 1] - ga.body_blob_off[t]) : ga.tmpl_n[t], n3 = 3 * n;
+    double* av = sh;                       // [GB][n3]
+    double* misc = av + GB * n3;           // [GB][24]: r_V, K^T a, V
+    double* bl = misc + GB * 24;           // LAB: blob offsets (n3)
+    T* in = reinterpret_cast<T*>(bl + (LAB ? n3 : 0));   // [n3][GB]
+    T* part = in + GB * n3;
+    for (int e = threadIdx.x; e < GB * n; e += GP_TH) {
+        const int u = e / n, b = e - u * n;
+        double w[3] = {0.0, 0.0, 0.0};
+        if (u < cnt) {
+            const int p = body(u);
+            const long long i = ga.body_blob_off[p] + b, o = ga.blob_gm[i];
+            const double v[3] = {rin[o], rin[o + 1], rin[o + 2]};
+            if (LAB) {
+                for (int a = 0; a < 3; ++a) {
+                    w[a] = v[a];
+                    bl[3 * b + a] = r[3 * i + a] - Yc[3 * p + a];
+                }
+            } else {
+                rotT(ga.Rb + 9 * p, v, w);
             }
-            for (; k < n3; ++k) a0 = fmaf(Mi[(long long)k * n3 + row], rho32[k], a0);
-            av[row] = ((double)a0 + (double)a1) + ((double)a2 + (double)a3);
         }
-    } else {
-        const double* Mi = Minv + (LAB ? blk_off[p] : minv_off[t]);
-        for (int row = threadIdx.x; row < n3; row += blockDim.x) {
-            double acc = 0.0;
-            for (int k = 0; k < n3; ++k) acc = fma(Mi[(long long)k * n3 + row], rho[k], acc);  // symmetric
-            av[row] = acc;
-        }
+        for (int a = 0; a < 3; ++a) in[(3 * b + a) * GB + u] = (T)w[a];
+    }
+    for (int e = threadIdx.x; e < 2 * cnt; e += GP_TH) {
+        const int u = e >> 1, h = e & 1, p = body(u);
+        const long long o = ga.body_gm[p] + 3 * h;
+        const double v[3] = {rin[o], rin[o + 1], rin[o + 2]};
+        double w[3] = {v[0], v[1], v[2]};
+        if (!LAB) rotT(ga.Rb + 9 * p, v, w);
+        for (int a = 0; a < 3; ++a) misc[24 * u + 3 * h + a] = w[a];
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const double* b = LAB ? bl : tmpl_xyz + 3LL * tmpl_off[t];
-        double g[6] = {0, 0, 0, 0, 0, 0};
-        for (int i = threadIdx.x; i < n; i += 32) {
-            const double a0 = av[3 * i], a1 = av[3 * i + 1], a2 = av[3 * i + 2];
-            const double d0 = b[3 * i], d1 = b[3 * i + 1], d2 = b[3 * i + 2];
-            g[0] += a0;
-            g[1] += a1;
-            g[2] += a2;
-            g[3] += d1 * a2 - d2 * a1;
-            g[4] += d2 * a0 - d0 * a2;
-            g[5] += d0 * a1 - d1 * a0;
-        }
+    group_product<GB, GP_FULL, T>(Minv + ga.mat_off[t], n3, in, part, av);   // symmetric: coalesced over rows
+    const double* b = LAB ? bl : ga.tmpl_xyz + 3LL * ga.tmpl_off[t];
+    group_KT(cnt, n, b, av, [&](int u, int c, double s) { misc[24 * u + 8 + c] = s; });
+    __syncthreads();
+    for (int e = threadIdx.x; e < 6 * cnt; e += GP_TH) {
+        const int u = e / 6, a = e - 6 * u;
+        const double* N = Nt + 36LL * t + 6 * a;
+        const double* m = misc + 24 * u;
+        double acc = 0.0;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) g[k] = warp_sum(g[k]);
-        if (threadIdx.x == 0) {
-            const double* N = Nt + 36 * t;
-            for (int a = 0; a < 6; ++a) {
-                double acc = 0.0;
-                for (int k = 0; k < 6; ++k) acc += N[6 * a + k] * (misc[k] + g[k]);
-                misc[8 + a] = -acc;
-            }
-        }
+        for (int k = 0; k < 6; ++k) acc = fma(N[k], m[k] + m[8 + k], acc);
+        misc[24 * u + 16 + a] = -acc;
     }
     __syncthreads();
     // G is 3n x 6, blocks back to back (templates, or LAB bodies in blob order)
-    const double* Gtt = Gt + 18LL * (LAB ? body_blob_off[p] : (long long)tmpl_off[t]);
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
+    const double* Gp = Gt + 18LL * (LAB ? ga.body_blob_off[t] : (long long)ga.tmpl_off[t]);
+    for (int e = threadIdx.x; e < cnt * n; e += GP_TH) {
+        const int u = e / n, q = e - u * n, p = body(u);
         double lb[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const int row = 3 * b + a;
-            double acc = av[row];
-            for (int k = 0; k < 6; ++k) acc = fma(Gtt[6LL * row + k], misc[8 + k], acc);
+            const int row = 3 * q + a;
+            double acc = av[u * n3 + row];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) acc = fma(Gp[6 * row + k], misc[24 * u + 16 + k], acc);
             lb[a] = acc;
         }
-        double w[3];
-        rot(R, lb, w);
-        const long long o = blob_gm[i0 + b];
+        double w[3] = {lb[0], lb[1], lb[2]};
+        if (!LAB) rot(ga.Rb + 9 * p, lb, w);
+        const long long i = ga.body_blob_off[p] + q, o = ga.blob_gm[i];
         zout[o] = w[0];
         zout[o + 1] = w[1];
         zout[o + 2] = w[2];
+        if (sdup) pack_lambda32(sdup, i, w);
     }
-    if (threadIdx.x == 0) {
-        double w[3];
-        const long long o = body_gm[p];
-        rot(R, misc + 8, w);
-        zout[o] = w[0];
-        zout[o + 1] = w[1];
-        zout[o + 2] = w[2];
-        rot(R, misc + 11, w);
-        zout[o + 3] = w[0];
-        zout[o + 4] = w[1];
-        zout[o + 5] = w[2];
+    for (int e = threadIdx.x; e < 2 * cnt; e += GP_TH) {
+        const int u = e >> 1, h = e & 1, p = body(u);
+        const double* v = misc + 24 * u + 16 + 3 * h;
+        double w[3] = {v[0], v[1], v[2]};
+        if (!LAB) rot(ga.Rb + 9 * p, v, w);
+        const long long o = ga.body_gm[p] + 3 * h;
+        for (int a = 0; a < 3; ++a) zout[o + a] = w[a];
     }
 }
 
-// ---- intra-body block of the RPY product in FP64 ---------------------------------------
+// ---- same-body block of the RPY product ------------------------------------------------
 //
-// y_p += M_pp lambda_p with M_pp = R M_t R^T (M_t: the template's RPY block, FP64, built at
-// init).  The FP32 pair kernel leaves out same-body pairs, so the large near-field terms of
-// each body are added here exactly.  One block per body; x and y use the saddle layout
-// (gm = 1) or 3 doubles per blob (gm = 0).
-__global__ void __launch_bounds__(128) k_intra_body(const long long* __restrict__ body_blob_off, const int* __restrict__ body_tmpl,
-                                                    const int* __restrict__ tmpl_n, const long long* __restrict__ minv_off,
-                                                    const double* __restrict__ Mt, const int* __restrict__ blob_gm,
-                                                    const double* __restrict__ Rb, const double* __restrict__ x,
-                                                    double* __restrict__ y, int gm) {
-    extern __shared__ double sh[];
-    const int p = blockIdx.x;
-    const int t = body_tmpl[p];
-    const int n3 = 3 * tmpl_n[t];
-    double* rho = sh;
-    const double* R = Rb + 9 * p;
-    const long long i0 = body_blob_off[p];
-    for (int b = threadIdx.x; b < n3 / 3; b += blockDim.x) {
-        const long long o = gm ? (long long)blob_gm[i0 + b] : 3 * (i0 + b);
-        double v[3] = {x[o], x[o + 1], x[o + 2]}, w[3];
-        rotT(R, v, w);
-        rho[3 * b] = w[0];
-        rho[3 * b + 1] = w[1];
-        rho[3 * b + 2] = w[2];
-    }
-    __syncthreads();
-    const double* M = Mt + minv_off[t];
-    double* av = sh + n3;
-    for (int row = threadIdx.x; row < n3; row += blockDim.x) {
-        double acc = 0.0;
-        for (int q = 0; q < n3; ++q) acc = fma(M[(long long)q * n3 + row], rho[q], acc);  // symmetric
-        av[row] = acc;
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < n3 / 3; b += blockDim.x) {
-        double w[3];
-        rot(R, av + 3 * b, w);
-        const long long o = gm ? (long long)blob_gm[i0 + b] : 3 * (i0 + b);
-        y[o] += w[0];
-        y[o + 1] += w[1];
-        y[o + 2] += w[2];
-    }
-}
-
-// The same block for the FP32 products, whose other terms carry FP32 rounding: M_t in FP32
-// (tmpl_M32), rho rounded to FP32, each row sum split into four interleaved FP32 partial
-// sums that are added in FP64; the rotations stay in FP64.  Shared memory: av (n3 doubles),
-// then rho (n3 floats).
-__global__ void __launch_bounds__(128) k_intra_body32(const long long* __restrict__ body_blob_off,
-                                                      const int* __restrict__ body_tmpl, const int* __restrict__ tmpl_n,
-                                                      const long long* __restrict__ minv_off, const float* __restrict__ Mt,
-                                                      const int* __restrict__ blob_gm, const double* __restrict__ Rb,
-                                                      const double* __restrict__ x, double* __restrict__ y, int gm) {
-    extern __shared__ double sh[];
-    const int p = blockIdx.x;
-    const int t = body_tmpl[p];
-    const int n3 = 3 * tmpl_n[t];
-    double* av = sh;
-    float* rho = reinterpret_cast<float*>(sh + n3);
-    const double* R = Rb + 9 * p;
-    const long long i0 = body_blob_off[p];
-    for (int b = threadIdx.x; b < n3 / 3; b += blockDim.x) {
-        const long long o = gm ? (long long)blob_gm[i0 + b] : 3 * (i0 + b);
-        double v[3] = {x[o], x[o + 1], x[o + 2]}, w[3];
-        rotT(R, v, w);
-        rho[3 * b] = (float)w[0];
-        rho[3 * b + 1] = (float)w[1];
-        rho[3 * b + 2] = (float)w[2];
-    }
-    __syncthreads();
-    const float* M = Mt + minv_off[t];
-    for (int row = threadIdx.x; row < n3; row += blockDim.x) {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        int q = 0;
-        for (; q + 4 <= n3; q += 4) {   // M_t is symmetric: column reads, coalesced over rows
-            a0 = fmaf(M[(long long)q * n3 + row], rho[q], a0);
-            a1 = fmaf(M[(long long)(q + 1) * n3 + row], rho[q + 1], a1);
-            a2 = fmaf(M[(long long)(q + 2) * n3 + row], rho[q + 2], a2);
-            a3 = fmaf(M[(long long)(q + 3) * n3 + row], rho[q + 3], a3);
+// y_p += M_pp lambda_p with M_pp = R M_t R^T (M_t: the template's RPY block, built at init in
+// FP64).  T = double: the double-float residual product, whose pair kernel leaves same-body
+// pairs out; T = float: the FP32 products, whose other terms carry FP32 rounding (M_t and the
+// rotated lambda rounded to FP32, the rotations in FP64).  x and y use the saddle layout (gm =
+// 1) or 3 doubles per blob (gm = 0); in the saddle layout the body rows -K^T lambda of the
+// operator are formed here as well, from the rotated lambda and the template's offsets (one
+// launch instead of two, lambda read once).
+template <int GB, typename T>
+__global__ void __launch_bounds__(GP_TH) k_intra_body(GroupArgs ga, const T* __restrict__ Mt, const double* __restrict__ x,
+                                                      double* __restrict__ y, int gm) {
+    extern __shared__ __align__(16) double sh[];
+    const int4 it = group_item<false, GB>(ga);
+    const int t = it.x, cnt = it.z, n = ga.tmpl_n[t], n3 = 3 * n;
+    auto body = [&](int u) { return GB == 1 ? (int)blockIdx.x : ga.bodies[it.y + u]; };
+    double* av = sh;                 // [GB][n3]
+    double* rho = av + GB * n3;      // [GB][n3]: the rotated lambda
+    double* kt = rho + GB * n3;      // [GB][6]
+    T* in = reinterpret_cast<T*>(kt + GB * 6);
+    T* part = in + GB * n3;
+    for (int e = threadIdx.x; e < GB * n; e += GP_TH) {
+        const int u = e / n, b = e - u * n;
+        double w[3] = {0.0, 0.0, 0.0};
+        if (u < cnt) {
+            const int p = body(u);
+            const long long i = ga.body_blob_off[p] + b, o = gm ? (long long)ga.blob_gm[i] : 3 * i;
+            const double v[3] = {x[o], x[o + 1], x[o + 2]};
+            rotT(ga.Rb + 9 * p, v, w);
         }
-        for (; q < n3; ++q) a0 = fmaf(M[(long long)q * n3 + row], rho[q], a0);
-        av[row] = ((double)a0 + (double)a1) + ((double)a2 + (double)a3);
+        for (int a = 0; a < 3; ++a) {
+            rho[u * n3 + 3 * b + a] = w[a];
+            in[(3 * b + a) * GB + u] = (T)w[a];
+        }
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < n3 / 3; b += blockDim.x) {
+    group_product<GB, GP_FULL, T>(Mt + ga.mat_off[t], n3, in, part, av);
+    for (int e = threadIdx.x; e < cnt * n; e += GP_TH) {
+        const int u = e / n, b = e - u * n, p = body(u);
         double w[3];
-        rot(R, av + 3 * b, w);
-        const long long o = gm ? (long long)blob_gm[i0 + b] : 3 * (i0 + b);
+        rot(ga.Rb + 9 * p, av + u * n3 + 3 * b, w);
+        const long long i = ga.body_blob_off[p] + b, o = gm ? (long long)ga.blob_gm[i] : 3 * i;
         y[o] += w[0];
         y[o + 1] += w[1];
         y[o + 2] += w[2];
+    }
+    if (!gm) return;
+    group_KT(cnt, n, ga.tmpl_xyz + 3LL * ga.tmpl_off[t], rho, [&](int u, int c, double s) { kt[6 * u + c] = s; });
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * cnt; e += GP_TH) {
+        const int u = e >> 1, h = e & 1, p = body(u);
+        double w[3];
+        rot(ga.Rb + 9 * p, kt + 6 * u + 3 * h, w);
+        const long long o = ga.body_gm[p] + 3 * h;
+        for (int a = 0; a < 3; ++a) y[o + a] = -w[a];
     }
 }
 
 __global__ void k_round_f32(long long n, const double* __restrict__ a, float* __restrict__ b) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         b[i] = (float)a[i];
-}
-
-void launch_intra_body32(gdc_ctx* c, const double* x, double* y, int gm) {
-    const size_t smem = (size_t)(3 * c->max_body_blobs) * (sizeof(double) + sizeof(float));
-    ++c->n_launch, k_intra_body32<<<c->NB, 128, smem, c->stream>>>(c->body_blob_off, c->body_tmpl, c->tmpl_n, c->minv_off,
-                                                                   c->tmpl_M32, c->blob_gm, c->Rb, x, y, gm);
-}
-
-void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm) {
-    const size_t smem = (size_t)(2 * 3 * c->max_body_blobs) * sizeof(double);
-    ++c->n_launch, k_intra_body<<<c->NB, 128, smem, c->stream>>>(c->body_blob_off, c->body_tmpl, c->tmpl_n, c->minv_off,
-                                                                 c->tmpl_M, c->blob_gm, c->Rb, x, y, gm);
-}
-
-// The block preconditioner for several bodies of one template per block (the items of
-// k_body_tri_tb): the template's M^-1 product grouped, each element read once for all of the
-// block's bodies (FP32 when F32, one accumulator per body and row), then per body (a warp
-// each) the sums K^T (M^-1 rho), the 6 x 6 solve with N and the correction G V, as k_precond.
-template <bool F32>
-__global__ void __launch_bounds__(128) k_precond_tb(const int4* __restrict__ items, const int* __restrict__ bodies,
-                                                    const long long* __restrict__ body_blob_off,
-                                                    const int* __restrict__ tmpl_n, const int* __restrict__ tmpl_off,
-                                                    const long long* __restrict__ minv_off,
-                                                    const double* __restrict__ Minv, const float* __restrict__ Minv32,
-                                                    const double* __restrict__ Gt, const double* __restrict__ Nt,
-                                                    const double* __restrict__ tmpl_xyz, const int* __restrict__ blob_gm,
-                                                    const int* __restrict__ body_gm, const double* __restrict__ Rb,
-                                                    const double* __restrict__ rin, double* __restrict__ zout) {
-    extern __shared__ double sh[];
-    const int4 it = items[blockIdx.x];
-    const int t = it.x, cnt = it.z;
-    const int n = tmpl_n[t], n3 = 3 * n;
-    double* rho = sh;                                         // [cnt][n3]
-    double* av = rho + (long long)cnt * n3;                   // [cnt][n3]
-    double* misc = av + (long long)cnt * n3;                  // [cnt][16]: 0-5 body rows, 8-13 V
-    float* rho32 = reinterpret_cast<float*>(misc + 16 * cnt);   // [cnt][n3] (F32)
-    for (int e = threadIdx.x; e < cnt * n; e += blockDim.x) {
-        const int u = e / n, b = e - u * n;
-        const int p = bodies[it.y + u];
-        const long long o = blob_gm[body_blob_off[p] + b];
-        double v[3] = {rin[o], rin[o + 1], rin[o + 2]}, w[3];
-        rotT(Rb + 9 * p, v, w);
-        for (int a = 0; a < 3; ++a) {
-            rho[u * n3 + 3 * b + a] = w[a];
-            if (F32) rho32[u * n3 + 3 * b + a] = (float)w[a];
-        }
-    }
-    for (int e = threadIdx.x; e < 2 * cnt; e += blockDim.x) {
-        const int u = e >> 1, h = e & 1;
-        const int p = bodies[it.y + u];
-        const long long o = body_gm[p] + 3 * h;
-        double v[3] = {rin[o], rin[o + 1], rin[o + 2]}, w[3];
-        rotT(Rb + 9 * p, v, w);
-        misc[16 * u + 3 * h] = w[0];
-        misc[16 * u + 3 * h + 1] = w[1];
-        misc[16 * u + 3 * h + 2] = w[2];
-    }
-    __syncthreads();
-    const long long mo = minv_off[t];
-    for (int row = threadIdx.x; row < n3; row += blockDim.x) {   // symmetric: coalesced over rows
-        if (F32) {
-            float a[GDC_TB_MAX];
-#pragma unroll
-            for (int u = 0; u < GDC_TB_MAX; ++u) a[u] = 0.f;
-            for (int k = 0; k < n3; ++k) {
-                const float f = Minv32[mo + (long long)k * n3 + row];
-#pragma unroll
-                for (int u = 0; u < GDC_TB_MAX; ++u)
-                    if (u < cnt) a[u] = fmaf(f, rho32[u * n3 + k], a[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < GDC_TB_MAX; ++u)
-                if (u < cnt) av[u * n3 + row] = (double)a[u];
-        } else {
-            double a[GDC_TB_MAX];
-#pragma unroll
-            for (int u = 0; u < GDC_TB_MAX; ++u) a[u] = 0.0;
-            for (int k = 0; k < n3; ++k) {
-                const double f = Minv[mo + (long long)k * n3 + row];
-#pragma unroll
-                for (int u = 0; u < GDC_TB_MAX; ++u)
-                    if (u < cnt) a[u] = fma(f, rho[u * n3 + k], a[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < GDC_TB_MAX; ++u)
-                if (u < cnt) av[u * n3 + row] = a[u];
-        }
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double* bx = tmpl_xyz + 3LL * tmpl_off[t];
-    for (int u = warp; u < cnt; u += blockDim.x >> 5) {
-        double g[6] = {0, 0, 0, 0, 0, 0};
-        for (int i = lane; i < n; i += 32) {
-            const double a0 = av[u * n3 + 3 * i], a1 = av[u * n3 + 3 * i + 1], a2 = av[u * n3 + 3 * i + 2];
-            const double d0 = bx[3 * i], d1 = bx[3 * i + 1], d2 = bx[3 * i + 2];
-            g[0] += a0;
-            g[1] += a1;
-            g[2] += a2;
-            g[3] += d1 * a2 - d2 * a1;
-            g[4] += d2 * a0 - d0 * a2;
-            g[5] += d0 * a1 - d1 * a0;
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) g[k] = warp_sum(g[k]);
-        if (lane == 0) {
-            const double* N = Nt + 36 * t;
-            for (int a = 0; a < 6; ++a) {
-                double acc = 0.0;
-                for (int k = 0; k < 6; ++k) acc += N[6 * a + k] * (misc[16 * u + k] + g[k]);
-                misc[16 * u + 8 + a] = -acc;
-            }
-        }
-    }
-    __syncthreads();
-    const double* Gtt = Gt + 18LL * tmpl_off[t];   // 3n x 6
-    for (int e = threadIdx.x; e < cnt * n; e += blockDim.x) {
-        const int u = e / n, b = e - u * n;
-        const int p = bodies[it.y + u];
-        double lb[3];
-        for (int a = 0; a < 3; ++a) {
-            const int row = 3 * b + a;
-            double acc = av[u * n3 + row];
-            for (int k = 0; k < 6; ++k) acc = fma(Gtt[6LL * row + k], misc[16 * u + 8 + k], acc);
-            lb[a] = acc;
-        }
-        double w[3];
-        rot(Rb + 9 * p, lb, w);
-        const long long o = blob_gm[body_blob_off[p] + b];
-        zout[o] = w[0];
-        zout[o + 1] = w[1];
-        zout[o + 2] = w[2];
-    }
-    for (int u = threadIdx.x; u < cnt; u += blockDim.x) {
-        const int p = bodies[it.y + u];
-        double w[3];
-        const long long o = body_gm[p];
-        rot(Rb + 9 * p, misc + 16 * u + 8, w);
-        zout[o] = w[0];
-        zout[o + 1] = w[1];
-        zout[o + 2] = w[2];
-        rot(Rb + 9 * p, misc + 16 * u + 11, w);
-        zout[o + 3] = w[0];
-        zout[o + 4] = w[1];
-        zout[o + 5] = w[2];
-    }
-}
-
-void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32) {
-    const size_t smem = (size_t)(3 * 3 * c->max_body_blobs + 32) * sizeof(double);
-    if (c->p.wall)
-        ++c->n_launch, k_precond<true><<<c->NB, 128, smem, c->stream>>>(
-            c->body_blob_off, c->body_tmpl, c->tmpl_n, c->tmpl_off, c->minv_off, c->blk_Minv, nullptr, c->blk_G, c->blk_N,
-            c->tmpl_xyz, c->blob_gm, c->body_gm, c->Rb, r, z, c->blk_off, c->r, c->Yc);
-    else if (c->tb_use && fp32)   // many bodies: grouped by template
-        ++c->n_launch, k_precond_tb<true><<<c->tb_n_items, 128, c->tb_precond_smem, c->stream>>>(
-            c->tb_items, c->tb_bodies, c->body_blob_off, c->tmpl_n, c->tmpl_off, c->minv_off, c->tmpl_Minv,
-            c->tmpl_Minv32, c->tmpl_G, c->tmpl_N, c->tmpl_xyz, c->blob_gm, c->body_gm, c->Rb, r, z);
-    else if (c->tb_use)
-        ++c->n_launch, k_precond_tb<false><<<c->tb_n_items, 128, c->tb_precond_smem, c->stream>>>(
-            c->tb_items, c->tb_bodies, c->body_blob_off, c->tmpl_n, c->tmpl_off, c->minv_off, c->tmpl_Minv,
-            c->tmpl_Minv32, c->tmpl_G, c->tmpl_N, c->tmpl_xyz, c->blob_gm, c->body_gm, c->Rb, r, z);
-    else if (fp32)
-        ++c->n_launch, k_precond<false, true><<<c->NB, 128, smem, c->stream>>>(
-            c->body_blob_off, c->body_tmpl, c->tmpl_n, c->tmpl_off, c->minv_off, c->tmpl_Minv, c->tmpl_Minv32, c->tmpl_G,
-            c->tmpl_N, c->tmpl_xyz, c->blob_gm, c->body_gm, c->Rb, r, z, nullptr, nullptr, nullptr);
-    else
-        ++c->n_launch, k_precond<false><<<c->NB, 128, smem, c->stream>>>(
-            c->body_blob_off, c->body_tmpl, c->tmpl_n, c->tmpl_off, c->minv_off, c->tmpl_Minv, nullptr, c->tmpl_G,
-            c->tmpl_N, c->tmpl_xyz, c->blob_gm, c->body_gm, c->Rb, r, z, nullptr, nullptr, nullptr);
 }
 
 // ---- factors of the body blocks: block-preconditioned Lanczos (Sec. 4.1, Chow & Saad) ----
@@ -543,177 +449,143 @@ void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32) {
 //   TRI_LINV:   out_p = L_p^-1 x_p (+ add_p) = L_t^-1 (R-hat_p^T x_p) (+ add_p)
 //   TRI_L:      out_p = L_p x_p = R-hat_p (L_t x_p)
 // F is the template's factor stored so that out_i = sum_k F[k n3 + i] in_k (coalesced over
-// the rows i); the triangular structure limits k to [i, n3) (TRI_LINV_T) or [0, i].  FP64.
-// One block per body; x, add and out hold 3 doubles per blob.  Shared memory: 2 x 3n doubles.
+// the rows i); the triangular structure limits k to [i, n3) (TRI_LINV_T) or [0, i].
+// x, add and out hold 3 doubles per blob.
 // LAB (blobs above a wall): body p's own factor of its lab-frame block (L_p from
-// k_wall_blocks, at blk_off[p]), no rotation.  T: the type of the factor and of the sums
-// (float for the FP32 products of the FP32-mixed Lanczos, whose other terms carry FP32
-// rounding; the rotations and the added vector stay FP64).
-template <int MODE, bool LAB, typename T>
-__global__ void __launch_bounds__(128) k_body_tri(const long long* __restrict__ body_blob_off,
-                                                  const int* __restrict__ body_tmpl, const int* __restrict__ tmpl_n,
-                                                  const long long* __restrict__ minv_off, const T* __restrict__ F,
-                                                  const double* __restrict__ Rb, const double* __restrict__ x,
-                                                  const double* __restrict__ add, double* __restrict__ out) {
-    extern __shared__ double sh[];
-    const int p = blockIdx.x;
-    const int t = LAB ? p : body_tmpl[p];
-    const int n = LAB ? (int)(body_blob_off[p + 1] - body_blob_off[p]) : tmpl_n[t], n3 = 3 * n;
-    double* res = sh;
-    T* in = reinterpret_cast<T*>(sh + n3);
-    const double ident[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    const double* R = LAB ? ident : Rb + 9 * p;
-    const long long i0 = body_blob_off[p];
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        double v[3] = {x[3 * (i0 + b)], x[3 * (i0 + b) + 1], x[3 * (i0 + b) + 2]};
-        if (MODE == TRI_LINV) {
-            double w[3];
-            rotT(R, v, w);
-            v[0] = w[0];
-            v[1] = w[1];
-            v[2] = w[2];
-        }
-        in[3 * b] = (T)v[0];
-        in[3 * b + 1] = (T)v[1];
-        in[3 * b + 2] = (T)v[2];
-    }
-    __syncthreads();
-    const T* Ft = F + minv_off[t];
-    for (int i = threadIdx.x; i < n3; i += blockDim.x) {
-        const int k0 = MODE == TRI_LINV_T ? i : 0, k1 = MODE == TRI_LINV_T ? n3 : i + 1;
-        T a0 = T(0), a1 = T(0);
-        int k = k0;
-        for (; k + 1 < k1; k += 2) {
-            a0 = fma(Ft[(long long)k * n3 + i], in[k], a0);
-            a1 = fma(Ft[(long long)(k + 1) * n3 + i], in[k + 1], a1);
-        }
-        if (k < k1) a0 = fma(Ft[(long long)k * n3 + i], in[k], a0);
-        res[i] = (double)a0 + (double)a1;
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
-        double w[3] = {res[3 * b], res[3 * b + 1], res[3 * b + 2]};
-        if (MODE != TRI_LINV) {
-            double v[3];
-            rot(R, w, v);
-            w[0] = v[0];
-            w[1] = v[1];
-            w[2] = v[2];
-        }
-        const long long o = 3 * (i0 + b);
-        if (add) {
-            w[0] += add[o];
-            w[1] += add[o + 1];
-            w[2] += add[o + 2];
-        }
-        out[o] = w[0];
-        out[o + 1] = w[1];
-        out[o + 2] = w[2];
-    }
-}
-
-// The same products for several bodies of one template per block (the bodies of item
-// (t, first, count) in `bodies`): each element of the template's factor, read once from L2,
-// serves all of them, where a block per body re-reads the factor body after body (at 36,121
-// bodies that is hundreds of MB per launch).  One accumulator per body and row.
-template <int MODE, typename T>
-__global__ void __launch_bounds__(128) k_body_tri_tb(const int4* __restrict__ items, const int* __restrict__ bodies,
-                                                     const long long* __restrict__ body_blob_off,
-                                                     const int* __restrict__ tmpl_n,
-                                                     const long long* __restrict__ minv_off, const T* __restrict__ F,
-                                                     const double* __restrict__ Rb, const double* __restrict__ x,
-                                                     const double* __restrict__ add, double* __restrict__ out) {
-    extern __shared__ double sh[];
-    const int4 it = items[blockIdx.x];
+// k_wall_blocks, at blk_off[p]), no rotation, one body per block.  T: the type of the factor
+// and of the sums (float for the FP32 products of the FP32-mixed Lanczos, whose other terms
+// carry FP32 rounding; the rotations and the added vector stay FP64).  sdup as in k_precond.
+template <int MODE, bool LAB, int GB, typename T>
+__global__ void __launch_bounds__(GP_TH) k_body_tri(GroupArgs ga, const T* __restrict__ F, const double* __restrict__ x,
+                                                    const double* __restrict__ add, double* __restrict__ out,
+                                                    float4* __restrict__ sdup) {
+    extern __shared__ __align__(16) double sh[];
+    const int4 it = group_item<LAB, GB>(ga);
     const int t = it.x, cnt = it.z;
-    const int n = tmpl_n[t], n3 = 3 * n;
-    double* res = sh;                                    // [cnt][n3]
-    T* in = reinterpret_cast<T*>(sh + (long long)cnt * n3);   // [cnt][n3]
-    for (int e = threadIdx.x; e < cnt * n; e += blockDim.x) {
+    auto body = [&](int u) { return GB == 1 ? (int)blockIdx.x : ga.bodies[it.y + u]; };
+    const int n = LAB ? (int)(ga.body_blob_off[t + 1] - ga.body_blob_off[t]) : ga.tmpl_n[t], n3 = 3 * n;
+    double* res = sh;                                 // [GB][n3]
+    T* in = reinterpret_cast<T*>(res + GB * n3);      // [n3][GB]
+    T* part = in + GB * n3;
+    for (int e = threadIdx.x; e < GB * n; e += GP_TH) {
         const int u = e / n, b = e - u * n;
-        const int p = bodies[it.y + u];
-        const long long o = 3 * (body_blob_off[p] + b);
-        double v[3] = {x[o], x[o + 1], x[o + 2]};
-        if (MODE == TRI_LINV) {
-            double w[3];
-            rotT(Rb + 9 * p, v, w);
-            v[0] = w[0];
-            v[1] = w[1];
-            v[2] = w[2];
+        double w[3] = {0.0, 0.0, 0.0};
+        if (u < cnt) {
+            const int p = body(u);
+            const long long o = 3 * (ga.body_blob_off[p] + b);
+            const double v[3] = {x[o], x[o + 1], x[o + 2]};
+            if (MODE == TRI_LINV && !LAB) {
+                rotT(ga.Rb + 9 * p, v, w);
+            } else {
+                for (int a = 0; a < 3; ++a) w[a] = v[a];
+            }
         }
-        in[u * n3 + 3 * b] = (T)v[0];
-        in[u * n3 + 3 * b + 1] = (T)v[1];
-        in[u * n3 + 3 * b + 2] = (T)v[2];
+        for (int a = 0; a < 3; ++a) in[(3 * b + a) * GB + u] = (T)w[a];
     }
     __syncthreads();
-    const T* Ft = F + minv_off[t];
-    for (int i = threadIdx.x; i < n3; i += blockDim.x) {
-        const int k0 = MODE == TRI_LINV_T ? i : 0, k1 = MODE == TRI_LINV_T ? n3 : i + 1;
-        T a[GDC_TB_MAX];
-#pragma unroll
-        for (int u = 0; u < GDC_TB_MAX; ++u) a[u] = T(0);
-        for (int k = k0; k < k1; ++k) {
-            const T f = Ft[(long long)k * n3 + i];
-#pragma unroll
-            for (int u = 0; u < GDC_TB_MAX; ++u)
-                if (u < cnt) a[u] = fma(f, in[u * n3 + k], a[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < GDC_TB_MAX; ++u)
-            if (u < cnt) res[u * n3 + i] = (double)a[u];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < cnt * n; e += blockDim.x) {
-        const int u = e / n, b = e - u * n;
-        const int p = bodies[it.y + u];
-        double w[3] = {res[u * n3 + 3 * b], res[u * n3 + 3 * b + 1], res[u * n3 + 3 * b + 2]};
-        if (MODE != TRI_LINV) {
-            double v[3];
-            rot(Rb + 9 * p, w, v);
-            w[0] = v[0];
-            w[1] = v[1];
-            w[2] = v[2];
-        }
-        const long long o = 3 * (body_blob_off[p] + b);
-        if (add) {
-            w[0] += add[o];
-            w[1] += add[o + 1];
-            w[2] += add[o + 2];
-        }
-        out[o] = w[0];
-        out[o + 1] = w[1];
-        out[o + 2] = w[2];
+    group_product<GB, MODE == TRI_LINV_T ? GP_FROM_DIAG : GP_TO_DIAG, T>(F + ga.mat_off[t], n3, in, part, res);
+    for (int e = threadIdx.x; e < cnt * n; e += GP_TH) {
+        const int u = e / n, b = e - u * n, p = body(u);
+        const double* v = res + u * n3 + 3 * b;
+        double w[3] = {v[0], v[1], v[2]};
+        if (MODE != TRI_LINV && !LAB) rot(ga.Rb + 9 * p, v, w);
+        const long long i = ga.body_blob_off[p] + b, o = 3 * i;
+        if (add)
+            for (int a = 0; a < 3; ++a) w[a] += add[o + a];
+        for (int a = 0; a < 3; ++a) out[o + a] = w[a];
+        if (sdup) pack_lambda32(sdup, i, w);
     }
 }
 
-void launch_body_tri(gdc_ctx* c, int mode, const double* x, const double* add, double* out, bool fp32) {
-    const size_t smem = (size_t)(2 * 3 * c->max_body_blobs) * sizeof(double);
+// ---- launches of the grouped kernels ---------------------------------------------------
+
+static GroupArgs group_args(const gdc_ctx* c) {
+    return GroupArgs{c->tb_items,  c->tb_bodies, c->body_blob_off, c->body_tmpl, c->tmpl_n, c->tmpl_off,
+                     c->p.wall ? c->blk_off : c->minv_off, c->blob_gm, c->body_gm, c->Rb, c->tmpl_xyz};
+}
+
+// Shared memory of a block: the largest over the templates
+static size_t group_smem(const gdc_ctx* c, int GB, size_t t, int more_per_row, int more) {
+    size_t s = 0;
+    for (int n : c->h_tmpl_n) s = std::max(s, gp_bytes(GB, 3 * n, t) + (size_t)(more_per_row * 3 * n + more) * sizeof(double));
+    return s;
+}
+
+template <bool LAB, int GB, typename T>
+static void precond_launch(gdc_ctx* c, const T* Minv, const double* r, double* z, float4* sdup) {
+    const size_t smem = group_smem(c, GB, sizeof(T), LAB ? 1 : 0, 24 * GB);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_precond<LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ++c->n_launch, k_precond<LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
+        group_args(c), Minv, LAB ? c->blk_G : c->tmpl_G, LAB ? c->blk_N : c->tmpl_N, r, z, c->r, c->Yc, sdup);
+}
+
+void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32, bool pack) {
+    float4* sdup = pack ? c->sdup : nullptr;
+    if (c->p.wall)
+        precond_launch<true, 1, double>(c, c->blk_Minv, r, z, sdup);
+    else if (fp32 && c->tb_group == 8)
+        precond_launch<false, 8, float>(c, c->tmpl_Minv32, r, z, sdup);
+    else if (fp32 && c->tb_group == 4)
+        precond_launch<false, 4, float>(c, c->tmpl_Minv32, r, z, sdup);
+    else if (fp32)
+        precond_launch<false, 1, float>(c, c->tmpl_Minv32, r, z, sdup);
+    else
+        precond_launch<false, 1, double>(c, c->tmpl_Minv, r, z, sdup);
+}
+
+template <int GB, typename T>
+static void intra_launch(gdc_ctx* c, const T* M, const double* x, double* y, int gm) {
+    const size_t smem = group_smem(c, GB, sizeof(T), GB, 6 * GB);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_intra_body<GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    GroupArgs ga = group_args(c);
+    ga.mat_off = c->minv_off;
+    ++c->n_launch, k_intra_body<GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(ga, M, x, y, gm);
+}
+
+void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm, bool fp32) {
+    if (!fp32)
+        intra_launch<1, double>(c, c->tmpl_M, x, y, gm);
+    else if (c->tb_group == 8)
+        intra_launch<8, float>(c, c->tmpl_M32, x, y, gm);
+    else if (c->tb_group == 4)
+        intra_launch<4, float>(c, c->tmpl_M32, x, y, gm);
+    else
+        intra_launch<1, float>(c, c->tmpl_M32, x, y, gm);
+}
+
+template <int MODE, bool LAB, int GB, typename T>
+static void tri_launch(gdc_ctx* c, const T* F, const double* x, const double* add, double* out, float4* sdup) {
+    const size_t smem = group_smem(c, GB, sizeof(T), 0, 0);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(k_body_tri<MODE, LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ++c->n_launch, k_body_tri<MODE, LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
+        group_args(c), F, x, add, out, sdup);
+}
+
+template <int MODE>
+static void tri_group(gdc_ctx* c, const float* F, const double* x, const double* add, double* out, float4* sdup) {
+    if (c->tb_group == 8)
+        tri_launch<MODE, false, 8, float>(c, F, x, add, out, sdup);
+    else if (c->tb_group == 4)
+        tri_launch<MODE, false, 4, float>(c, F, x, add, out, sdup);
+    else
+        tri_launch<MODE, false, 1, float>(c, F, x, add, out, sdup);
+}
+
+void launch_body_tri(gdc_ctx* c, int mode, const double* x, const double* add, double* out, bool fp32, bool pack) {
+    float4* sdup = pack ? c->sdup : nullptr;
     const bool lab = c->p.wall != 0;
-    const long long* off = lab ? c->blk_off : c->minv_off;
-    // lab-frame factors (above a wall) and fewer bodies: one block per body; many bodies:
-    // grouped by template
-#define GDC_TRI(MODE, LAB, T, F)                                                                                  \
-    do {                                                                                                          \
-        if (LAB || !c->tb_use)                                                                                    \
-            k_body_tri<MODE, LAB, T><<<c->NB, 128, smem, c->stream>>>(c->body_blob_off, c->body_tmpl, c->tmpl_n,  \
-                                                                     off, F, c->Rb, x, add, out);                \
-        else                                                                                                      \
-            k_body_tri_tb<MODE, T><<<c->tb_n_items, 128, c->tb_smem, c->stream>>>(                               \
-                c->tb_items, c->tb_bodies, c->body_blob_off, c->tmpl_n, c->minv_off, F, c->Rb, x, add, out);     \
-    } while (0)
-    ++c->n_launch;
-    if (fp32 && !lab && mode == TRI_LINV_T)
-        GDC_TRI(TRI_LINV_T, false, float, c->tmpl_X32);
-    else if (fp32 && !lab && mode == TRI_LINV)
-        GDC_TRI(TRI_LINV, false, float, c->tmpl_XT32);
-    else if (mode == TRI_LINV_T) {
-        if (lab) GDC_TRI(TRI_LINV_T, true, double, c->blk_X); else GDC_TRI(TRI_LINV_T, false, double, c->tmpl_X);
+    if (mode == TRI_LINV_T) {
+        if (lab) tri_launch<TRI_LINV_T, true, 1, double>(c, c->blk_X, x, add, out, sdup);
+        else if (fp32) tri_group<TRI_LINV_T>(c, c->tmpl_X32, x, add, out, sdup);
+        else tri_launch<TRI_LINV_T, false, 1, double>(c, c->tmpl_X, x, add, out, sdup);
     } else if (mode == TRI_LINV) {
-        if (lab) GDC_TRI(TRI_LINV, true, double, c->blk_XT); else GDC_TRI(TRI_LINV, false, double, c->tmpl_XT);
+        if (lab) tri_launch<TRI_LINV, true, 1, double>(c, c->blk_XT, x, add, out, sdup);
+        else if (fp32) tri_group<TRI_LINV>(c, c->tmpl_XT32, x, add, out, sdup);
+        else tri_launch<TRI_LINV, false, 1, double>(c, c->tmpl_XT, x, add, out, sdup);
     } else {
-        if (lab) GDC_TRI(TRI_L, true, double, c->blk_LT); else GDC_TRI(TRI_L, false, double, c->tmpl_LT);
+        if (lab) tri_launch<TRI_L, true, 1, double>(c, c->blk_LT, x, add, out, sdup);
+        else tri_launch<TRI_L, false, 1, double>(c, c->tmpl_LT, x, add, out, sdup);
     }
-#undef GDC_TRI
 }
 
 // ---- per-template setup (once, at init) -------------------------------------------------

@@ -29,10 +29,9 @@
 #define GDC_MAX_RESTART 100
 #define GDC_MAX_LANCZOS 128
 #define GDC_MAX_TMPL_BLOBS 340   // 3n <= 1020 rows of a template block
-#define GDC_TB_MAX 8             // bodies of one template per block in the factor products
-#define GDC_ORTH_SLICE 4096      // elements per block of the fused orthogonalisation (8 blocks per suspension at most)
+#define GDC_ORTH_SLICE 4096      // elements per block of the fused orthogonalisation
+#define GDC_ORTH_MAX 32768       // and per suspension (longer: separate kernels)
 #define GDC_NEAR_CAP 32          // blobs closer than 2a listed per blob (beyond: a search of the suspension)
-#define GDC_EPI_WIDE 32768       // FP32 product epilogue: 8 threads per blob up to this many blobs, one above
 #define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
 #define GDC_NEAR_SRC_MAX 2048
 #define GDC_SYM_TILE 512         // blobs per tile of the symmetric FP32 pair kernel
@@ -123,13 +122,11 @@ struct gdc_ctx {
     // host copies of the layout
     std::vector<long long> h_body_off, h_blob_off, h_gm_off, h_body_blob_off;
     std::vector<int> h_body_tmpl, h_tmpl_n, h_tmpl_off, h_body_susp;
-    // factor products of several bodies of one template per block (body.cu k_body_tri_tb):
-    // items (template, first entry in tb_bodies, count), bodies grouped by template
+    // per-body products, bodies of one template grouped per block (body.cu): items (template,
+    // first entry in tb_bodies, count) of up to tb_group bodies, bodies grouped by template
     int4* tb_items = 0;
     int* tb_bodies = 0;
-    int tb_n_items = 0;
-    bool tb_use = false;   // the grouped products replace one block per body
-    size_t tb_smem = 0, tb_precond_smem = 0;
+    int tb_n_items = 0, tb_group = 1;
     std::vector<int4> h_tb_items;
     double* lz_qbuf = 0;     // the eigen-step's Q / refined-root scratch per suspension (global)
     bool lz_qbuf_on = false; // more suspensions than SMs: the scratch in global memory, not shared
@@ -427,14 +424,16 @@ const char* noalloc_last_error();
 // body.cu
 void launch_body_KT(gdc_ctx* c, const double* x, int x_gm, double* y, int y_gm, double scale);
 void launch_lsq(gdc_ctx* c, const double* vbrev, double* calV);
-void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32 = false);
-void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm);
-void launch_intra_body32(gdc_ctx* c, const double* x, double* y, int gm);
+// pack: lambda also into sdup, in the layout of the FP32 pair kernels (launch_pack_lambda's work)
+void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32 = false, bool pack = false);
+// y += the same-body blocks times x; in the saddle layout (gm) also the body rows -K^T lambda
+void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm, bool fp32);
 void launch_template_setup(gdc_ctx* c, const double* Mext = nullptr);   // Mext: given template blocks
 // per-body products with the template-block factors L_p = R-hat_p L_t (block-preconditioned
 // Lanczos): mode 0 out = L_p^-T x, mode 1 out = L_p^-1 x (+ add), mode 2 out = L_p x
 enum { TRI_LINV_T = 0, TRI_LINV = 1, TRI_L = 2 };
-void launch_body_tri(gdc_ctx* c, int mode, const double* x, const double* add, double* out, bool fp32 = false);
+void launch_body_tri(gdc_ctx* c, int mode, const double* x, const double* add, double* out, bool fp32 = false,
+                     bool pack = false);
 gdc_status wall_init_attributes(gdc_ctx* c);
 void launch_wall_blocks(gdc_ctx* c);   // per-body blocks above a wall (at every configuration)
 
@@ -444,7 +443,7 @@ void launch_wall_apply(gdc_ctx* c, int prec, const double* x, double* y, int gm)
 void launch_wall_forces(gdc_ctx* c, double* fblob);                                 // fblob += wall + weight
 
 // krylov.cu
-gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y);
+gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y, bool packed = false);   // packed: lambda is in sdup
 gdc_status rpy_op(gdc_ctx* c, int prec, const double* lam, double* u);
 gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* info);
 gdc_status lanczos_sqrt(gdc_ctx* c, const double* W, double* out, double scale, int fixed_iters,

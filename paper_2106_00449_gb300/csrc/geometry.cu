@@ -26,7 +26,7 @@ __global__ void k_blob_pos(int NBL, const int* __restrict__ blob_body, const int
                            const int* __restrict__ tmpl_off, const double* __restrict__ tmpl_xyz,
                            const double* __restrict__ Y, const double* __restrict__ Rb,
                            const double* __restrict__ ref, double* __restrict__ r,
-                           float4* __restrict__ spos, double4_32a* __restrict__ spos64) {
+                           float4* __restrict__ spos, double4_32a* __restrict__ spos64, float4* __restrict__ sdup) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NBL) return;
     const int p = blob_body[i];
@@ -43,7 +43,11 @@ __global__ void k_blob_pos(int NBL, const int* __restrict__ blob_body, const int
     const int s = blob_susp[i];
     const double rx = x - ref[3 * s], ry = y - ref[3 * s + 1], rz = z - ref[3 * s + 2];
     const float pb = __int_as_float(p);
-    spos[i] = make_float4((float)rx, (float)ry, (float)rz, pb);
+    const float fx = (float)rx, fy = (float)ry, fz = (float)rz;
+    spos[i] = make_float4(fx, fy, fz, pb);
+    // the position part of the FP32 pair kernels' source layout
+    sdup[3LL * i] = make_float4(fx, fx, fy, fy);
+    reinterpret_cast<float2*>(sdup + 3LL * i + 1)[0] = make_float2(fz, fz);
     spos64[i] = make_double4_32a(rx, ry, rz, (double)p);
 }
 
@@ -51,7 +55,7 @@ void load_config(gdc_ctx* c, const double* Y, const double* q, bool near) {
     ++c->n_launch, k_body_rot<<<ceil_div(c->NB, 128), 128, 0, c->stream>>>(c->NB, Y, q, c->Rb, c->Yc);
     ++c->n_launch, k_blob_pos<<<ceil_div(c->NBL, 128), 128, 0, c->stream>>>(
         c->NBL, c->blob_body, c->blob_susp, c->body_tmpl, c->body_blob_off, c->tmpl_off, c->tmpl_xyz,
-        Y, c->Rb, c->ref, c->r, c->spos, c->spos64);
+        Y, c->Rb, c->ref, c->r, c->spos, c->spos64, c->sdup);
     if (near) launch_near_build(c);   // pairs closer than 2a, corrected after every FP32 product
     if (c->p.wall) launch_wall_blocks(c);   // a wall: per-body blocks depend on the configuration
 }

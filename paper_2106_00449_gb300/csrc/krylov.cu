@@ -248,7 +248,7 @@ gdc_status rpy_op(gdc_ctx* c, int prec, const double* lam, double* u) {
     return GDC_OK;
 }
 
-gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y) {
+gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y, bool packed) {
     if (c->fcm) {   // one suspension: lambda is the first 3 N_b entries of the saddle vector
         const gdc_status st = gdc_fcm_apply(c->fcm, (int)c->NBL, c->r, x, c->fcm_u);
         if (st != GDC_OK) return fail(c, st, std::string("FCM: ") + gdc_fcm_last_error(c->fcm));
@@ -256,11 +256,11 @@ gdc_status saddle_op(gdc_ctx* c, int prec, const double* x, double* y) {
         launch_body_KT(c, x, 1, y, 1, -1.0);
         return GDC_OK;
     }
-    launch_pack_lambda(c, prec, x, 1);
+    if (!packed) launch_pack_lambda(c, prec, x, 1);
     launch_rpy(c, prec, x, 1);
-    launch_rpy_epilogue(c, prec, x, y, 1);
+    launch_rpy_epilogue(c, prec, x, y, 1);   // with same-body blocks apart, the body rows too
     if (c->p.wall) launch_wall_apply(c, prec, x, y, 1);
-    launch_body_KT(c, x, 1, y, 1, -1.0);
+    if (prec == GDC_FP64) launch_body_KT(c, x, 1, y, 1, -1.0);
     return GDC_OK;
 }
 
@@ -277,8 +277,7 @@ static void lz_operator(gdc_ctx* c, int prec, const double* x, double* w) {
     }
     if (prec == GDC_FP32_MIXED && !c->p.wall) {
         // the factor products in FP32 too: the coupling term they feed carries FP32 rounding
-        launch_body_tri(c, TRI_LINV_T, x, nullptr, c->lz_z, true);
-        launch_pack_lambda(c, prec, c->lz_z, 0);
+        launch_body_tri(c, TRI_LINV_T, x, nullptr, c->lz_z, true, true);
         launch_rpy(c, prec, c->lz_z, 0);
         launch_rpy_epilogue(c, prec, c->lz_z, c->lz_u, 0, false);
         launch_body_tri(c, TRI_LINV, c->lz_u, x, w, true);
@@ -393,15 +392,15 @@ __global__ void k_gm_backsolve(int S, int m, const double* __restrict__ H, const
 // w is orthogonalised against V_0..V_j (classical Gram-Schmidt, twice), normalised into
 // V_(j+1), and for GMRES the Hessenberg column is rotated (k_gm_arnoldi's work).  As separate
 // kernels this is eleven launches of 2 to 13 us for suspensions of a few thousand blobs,
-// each waiting for a handful of warps; here a cluster of up to 8 blocks per suspension keeps
+// each waiting for a handful of warps; here a cluster of up to 16 blocks per suspension keeps
 // its part of w in shared memory, and the partial inner products meet through distributed
 // shared memory (every block adds all of them in block order, so each holds the same sums;
 // deterministic).
 //
-// Bound by the FP64 pipes of the cluster's SMs: 4 (j + 1) n FMAs at 2 per clock per SM.  Eight
-// SMs need 8 us for n = 9,216 at j = 6 (30 us measured, 46% FP64 pipe: the rest is the latency of
-// the passes, kept down by 16 warps and 8 loads in flight per thread); at n = 32,768 (GDC_ORTH_SLICE elements per block) the
-// whole chip's separate kernels become as fast, and beyond it they are used.
+// Bound by the FP64 pipes of the cluster's SMs (4 (j + 1) n FMAs at 2 per clock per SM) and by
+// the latency of the passes, kept down by 16 warps and 8 loads in flight per thread: n = 9,216
+// at j = 6 took 30 us on 8 SMs, 46% of it FP64.  From about GDC_ORTH_MAX elements the whole
+// chip's separate kernels are as fast, and beyond it they are used.
 
 namespace cg = cooperative_groups;
 
@@ -450,6 +449,11 @@ __global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __rest
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int e = threadIdx.x; e < m; e += ORTH_TH) ws[e] = w[lo + e];
     if (threadIdx.x < k) hsum[threadIdx.x] = 0.0;
+    double gj = 0.0, bn = 1.0;   // for the rotation at the end
+    if (gm.H && rank == 0 && threadIdx.x == 0) {
+        gj = gm.g[(long long)s * (gm.m + 1) + j];
+        bn = gm.bnorm[s];
+    }
     // few columns: G warps share one, each a contiguous piece of the block's part
     const int G = k >= 9 ? 1 : (k >= 5 ? 2 : (k >= 3 ? 4 : 8));
     const int piece = (m + G - 1) / G;
@@ -474,14 +478,23 @@ __global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __rest
             if (lane == 0) part[pass][u] = acc;
         }
         cl.sync();
-        if (threadIdx.x < k) {
+        // C neighbouring lanes fetch a column's sums from the C blocks at once (one after the other
+        // the remote loads would cost 0.25 us each)
+        for (int u = threadIdx.x; u < ((k * C + 31) & ~31); u += ORTH_TH) {
+            const int i = u / C, c = u % C;
             double h = 0.0;
-            for (int c = 0; c < C; ++c) {
-                const double* p = cl.map_shared_rank(part[pass], c);
-                for (int g = 0; g < G; ++g) h += p[threadIdx.x * G + g];
+            if (i < k) {
+                const double* p = cl.map_shared_rank(part[pass], c) + i * G;
+                double g[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) g[q] = q < G ? p[q] : 0.0;
+                h = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7]));
             }
-            hs[threadIdx.x] = h;
-            hsum[threadIdx.x] += h;
+            for (int o = 1; o < C; o <<= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+            if (i < k && c == 0) {
+                hs[i] = h;
+                hsum[i] += h;
+            }
         }
         __syncthreads();
         for (int e = threadIdx.x; e < m; e += ORTH_TH) {
@@ -558,10 +571,9 @@ __global__ void __launch_bounds__(ORTH_TH) k_orth(int C, const long long* __rest
         gm.sn[(long long)s * gm.m + j] = ss;
         Hs[j * gm.m + j] = rr;
         Hs[(j + 1) * gm.m + j] = 0.0;
-        const double gj = gs[j];
         gs[j + 1] = -ss * gj;
         gs[j] = cc * gj;
-        const double e = fabs(ss * gj) / gm.bnorm[s];
+        const double e = fabs(ss * gj) / bn;
         gm.est[s] = e;
         gm.jcount[s] = j + 1;
         if (!(e > gm.inner_tol) || beta == 0.0 || j + 1 == gm.m) gm.active[s] = 0;
@@ -575,13 +587,15 @@ static long long longest_segment(const gdc::Seg& sg) {
 }
 
 // Blocks per cluster of the fused orthogonalisation of a segmented space, 0: the separate
-// kernels (a suspension longer than 8 parts).  Parts of at most 1,024 elements while the
-// cluster can grow, so that a suspension spreads over more FP64 pipes.
-static int orth_cluster(const gdc::Seg& sg) {
+// kernels (a suspension longer than GDC_ORTH_MAX).  The cluster doubles while its parts are
+// longer than GDC_ORTH_SLICE, or longer than 512 elements with fewer than two blocks per SM
+// in all, so that few suspensions spread over more FP64 pipes.
+static int orth_cluster(const gdc_ctx* c, const gdc::Seg& sg) {
     const long long n = longest_segment(sg);
-    if (n > 8LL * GDC_ORTH_SLICE) return 0;
+    if (n > GDC_ORTH_MAX) return 0;
     int C = 1;
-    while (C < 8 && n > 1024LL * C) C *= 2;
+    while (C < 16 && (n > (long long)GDC_ORTH_SLICE * C || (n > 512LL * C && (long long)c->S * C < 2LL * c->num_sms)))
+        C *= 2;
     return C;
 }
 
@@ -607,7 +621,7 @@ static void gm_orthogonalise(gdc_ctx* c, int j, const int* jd, double inner_tol,
     const gdc::Seg& sg = c->seg_gm;
     const long long n = c->ngm;
     const int m = c->m, cols = c->red_cols, cap = jd ? m : 0, k = jd ? 1 : j + 1;
-    if (const int C = orth_cluster(sg)) {
+    if (const int C = orth_cluster(c, sg)) {
         const OrthGm gm{m, c->gm_H, c->gm_cs, c->gm_sn, c->gm_g, c->gm_bnorm, inner_tol, c->gm_res + c->S, c->gm_active,
                         c->gm_j};
         launch_orth(c, sg, C, c->gm_V, n, c->gm_w, j, jd, c->gm_active, vcur, gm, OrthLz{});
@@ -682,9 +696,9 @@ gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* i
         int j = 0;
         for (; j < m; ++j) {
             double* Vj = c->gm_V + (long long)j * n;
-            launch_precond(c, Vj, c->gm_z, prec == GDC_FP32_MIXED);
+            launch_precond(c, Vj, c->gm_z, prec == GDC_FP32_MIXED, prec == GDC_FP32_MIXED);
             c->mv_active = c->gm_active;   // suspensions that have converged need no product
-            saddle_op(c, prec, c->gm_z, c->gm_w);
+            saddle_op(c, prec, c->gm_z, c->gm_w, prec == GDC_FP32_MIXED);
             c->mv_active = nullptr;
             if (prec == GDC_FP32_MIXED) inf.matvecs_fp32++; else inf.matvecs_fp64++;
             gm_orthogonalise(c, j, nullptr, inner_tol, nullptr);
@@ -701,12 +715,12 @@ gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* i
         // x += P^-1 V y
         ++c->n_launch, k_gm_backsolve<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(c->S, m, c->gm_H, c->gm_g, c->gm_j, c->gm_y, cols);
         ++c->n_launch, k_combine<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, c->gm_j, c->gm_y, cols, nullptr, c->gm_w);
-        launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED);   // the correction e of this cycle
+        launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED, prec == GDC_FP32_MIXED);   // the correction e of this cycle
         ++c->n_launch, k_axpy_chunks<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, 1.0, c->gm_z, x);
         if (prec == GDC_FP32_MIXED && rmax <= GDC_RESID_UPDATE) {
             // r <- r - A e: the residual is already small, so A e is too, and the FP32 product's
             // relative error (~3e-7) leaves r accurate to ~3e-7 * rmax, far below gmres_tol
-            saddle_op(c, GDC_FP32_MIXED, c->gm_z, c->gm_w);
+            saddle_op(c, GDC_FP32_MIXED, c->gm_z, c->gm_w, true);
             inf.matvecs_fp32++;
             ++c->n_launch, k_axpy_chunks<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, -1.0, c->gm_w, c->gm_r);
         } else {
@@ -1134,6 +1148,7 @@ __global__ void k_lz_reset(int S, int* __restrict__ lastk) {
 void krylov_init_attributes() {
     cudaFuncSetAttribute(k_lz_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)lz_tridiag_smem(GDC_MAX_LANCZOS));
+    cudaFuncSetAttribute(k_orth, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of 16
 }
 
 // A Lanczos iteration's full reorthogonalisation of lz_w against v_0..v_j, the eigen-step and
@@ -1142,7 +1157,7 @@ static void lz_orthogonalise(gdc_ctx* c, int j, const int* jd, int fixed_mode, d
     const gdc::Seg& sg = c->seg_lz;
     const long long n = 3LL * c->NBL;
     const int cols = c->red_cols, kmax = c->kmax, cap = jd ? kmax : 0, k = jd ? 1 : j + 1;
-    const int C = orth_cluster(sg);
+    const int C = orth_cluster(c, sg);
     if (C) {
         launch_orth(c, sg, C, c->lz_V, n, c->lz_w, j, jd, c->lz_active, vcur, OrthGm{},
                     OrthLz{c->lz_h, c->gm_h2, c->lz_alpha, cols, kmax, c->susp_blob_off});
@@ -1498,9 +1513,9 @@ void gmres_solve_graph(gdc_ctx* c, const double* b, double* x) {
         cap_while_begin(c, hi);
         const unsigned long long before_i = c->n_launch;
         {
-            launch_precond(c, c->gm_vcur, c->gm_z, prec == GDC_FP32_MIXED);
+            launch_precond(c, c->gm_vcur, c->gm_z, mixed, mixed);
             c->mv_active = c->gm_active;
-            saddle_op(c, prec, c->gm_z, c->gm_w);
+            saddle_op(c, prec, c->gm_z, c->gm_w, prec == GDC_FP32_MIXED);
             c->mv_active = nullptr;
             gm_orthogonalise(c, 0, jd, inner_tol, c->gm_vcur);
             ++c->n_launch, k_gm_inner_next<<<1, 32, 0, c->stream>>>(c->S, c->gm_active, c->ctl, max_iter, hi);
@@ -1511,7 +1526,7 @@ void gmres_solve_graph(gdc_ctx* c, const double* b, double* x) {
                                                                                   c->gm_y, cols);
         ++c->n_launch, k_combine<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, c->gm_j, c->gm_y, cols,
                                                                      nullptr, c->gm_w);
-        launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED);   // the correction e of this cycle
+        launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED, prec == GDC_FP32_MIXED);   // the correction e of this cycle
         ++c->n_launch, k_axpy_chunks<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, 1.0, c->gm_z, x);
         // the residual: recomputed, r = b - A x (accurate product), or updated, r <- r - A e
         // (FP32 product of the small correction), as k_gm_check decided
@@ -1523,7 +1538,7 @@ void gmres_solve_graph(gdc_ctx* c, const double* b, double* x) {
             ++c->n_launch, k_count<<<1, 1, 0, c->stream>>>(&c->rep->gm_df);
             cap_ifelse_next(c, REP_GM_DF, before_a);
             const unsigned long long before_u = c->n_launch;
-            saddle_op(c, GDC_FP32_MIXED, c->gm_z, c->gm_w);
+            saddle_op(c, GDC_FP32_MIXED, c->gm_z, c->gm_w, true);
             ++c->n_launch, k_axpy_chunks<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, -1.0, c->gm_w, c->gm_r);
             cap_ifelse_end(c, REP_GM_UPD, before_u);
         }

@@ -26,17 +26,17 @@ constexpr int MV_TILE = GDC_MV_TILE;   // sources staged in shared memory per ti
 // ---- source packing ---------------------------------------------------------
 
 // FP32 sources in the layout the pair kernel's shared-memory tiles use, three float4 per
-// blob: (x,x,y,y) (z,z,lx,lx) (ly,ly,lz,lz) -- each value twice, one per packed lane.
+// blob: (x,x,y,y) (z,z,lx,lx) (ly,ly,lz,lz) -- each value twice, one per packed lane.  The
+// positions are written when a configuration is loaded (k_blob_pos), lambda here or by the
+// per-body kernel that produced it.
 __global__ void k_pack_lam32(int NBL, const int* __restrict__ map, const double* __restrict__ x,
-                             const float4* __restrict__ spos, float4* __restrict__ sdup) {
+                             float4* __restrict__ sdup) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NBL) return;
     const long long o = map ? (long long)map[i] : 3LL * i;
     const float lx = (float)x[o], ly = (float)x[o + 1], lz = (float)x[o + 2];
-    const float4 ps = spos[i];
-    sdup[3 * i] = make_float4(ps.x, ps.x, ps.y, ps.y);
-    sdup[3 * i + 1] = make_float4(ps.z, ps.z, lx, lx);
-    sdup[3 * i + 2] = make_float4(ly, ly, lz, lz);
+    reinterpret_cast<float2*>(sdup + 3LL * i + 1)[1] = make_float2(lx, lx);
+    sdup[3LL * i + 2] = make_float4(ly, ly, lz, lz);
 }
 
 __global__ void k_pack_lam64(int NBL, const int* __restrict__ map, const double* __restrict__ x,
@@ -50,7 +50,7 @@ __global__ void k_pack_lam64(int NBL, const int* __restrict__ map, const double*
 void launch_pack_lambda(gdc_ctx* c, int prec, const double* x, int gm_layout) {
     const int* map = gm_layout ? c->blob_gm : nullptr;
     if (prec == GDC_FP32_MIXED)
-        ++c->n_launch, k_pack_lam32<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(c->NBL, map, x, c->spos, c->sdup);
+        ++c->n_launch, k_pack_lam32<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(c->NBL, map, x, c->sdup);
     else if (prec == GDC_PREC_DF64)
         ++c->n_launch, k_pack_lam64<<<ceil_div(c->NBL, 256), 256, 0, c->stream>>>(c->NBL, map, x, c->slam64);
 }
@@ -417,10 +417,11 @@ __device__ inline void same_body_subtract(const float4 pt, long long j0, long lo
 // out the pair kernel's same-body terms (the intra-body kernel adds the template's block).
 //
 // EPI neighbouring threads share a blob: they take every EPI-th slot, same-body blob and near
-// pair, joined by shuffles in a fixed order.  8 threads up to GDC_EPI_WIDE blobs, where the
-// chain of dependent loads of one thread is what the launch waits for (2,560 blobs: 12.9 us
-// at one thread per blob); one thread above it, where the FP64 tail (2 lanes per clock per
-// SM, paid per warp) would cost more than the chain.
+// pair, joined by shuffles in a fixed order.  More threads shorten the chain of dependent loads,
+// but the FP64 tail (2 lanes per clock per SM) is paid per warp.  us per launch with 1 / 2 / 4
+// / 8 threads: 2,560 blobs 13.3 / 10.6 / 8.8 / 8.1, 20,202 blobs 17.8 / 13.6 / 14.5 / 18.0,
+// 65,520 blobs 37.8 / 29.1 / 40.2 / 58.0, 161,000 blobs in 160 suspensions 67.8 / 78.1 / 100 /
+// 154: 8 threads up to 8,192 blobs, 2 up to 98,304, 1 above.
 template <typename P, int EPI>
 __global__ void __launch_bounds__(256) k_rpy_epilogue(int NBL, const P* __restrict__ part, const int* __restrict__ blob_susp,
                                const int* __restrict__ nk, double c0, const double* __restrict__ x,
@@ -554,17 +555,16 @@ static void launch_epilogue_t(gdc_ctx* c, const P* part, bool sym, double c0, co
 static void launch_epilogue(gdc_ctx* c, int prec, double c0, const double* x, double* y, int gm_layout,
                             bool near) {
     const bool sym = prec == GDC_FP32_MIXED && near && c->use_sym;   // RPY products only, not forces
-    const bool wide = c->NBL > GDC_EPI_WIDE;
     if (prec == GDC_FP32_MIXED) {
         const float4* part = sym ? c->sym_part_i : (const float4*)c->mv_part;
-        if (wide)
-            launch_epilogue_t<float4, 1>(c, part, sym, c0, x, y, gm_layout, near);
-        else
+        if (c->NBL <= 8192)
             launch_epilogue_t<float4, 8>(c, part, sym, c0, x, y, gm_layout, near);
-    } else if (wide) {
-        launch_epilogue_t<double4_32a, 1>(c, (const double4_32a*)c->mv_part, false, c0, x, y, gm_layout, false);
+        else if (c->NBL <= 98304)
+            launch_epilogue_t<float4, 2>(c, part, sym, c0, x, y, gm_layout, near);
+        else
+            launch_epilogue_t<float4, 1>(c, part, sym, c0, x, y, gm_layout, near);
     } else {
-        launch_epilogue_t<double4_32a, 8>(c, (const double4_32a*)c->mv_part, false, c0, x, y, gm_layout, false);
+        launch_epilogue_t<double4_32a, 2>(c, (const double4_32a*)c->mv_part, false, c0, x, y, gm_layout, false);
     }
 }
 
@@ -576,8 +576,8 @@ void launch_rpy_epilogue(gdc_ctx* c, int prec, const double* x, double* y, int g
     // same-body blocks from the template: the df64 pair kernel leaves those pairs out and the
     // FP32 epilogue has taken the FP32 pair kernel's same-body terms out again (so without
     // them an FP32 product is exactly the blocks between different bodies)
-    if (prec == GDC_PREC_DF64) launch_intra_body(c, x, y, gm_layout);
-    if (prec == GDC_FP32_MIXED && same_body) launch_intra_body32(c, x, y, gm_layout);
+    if (prec == GDC_PREC_DF64 || (prec == GDC_FP32_MIXED && same_body))
+        launch_intra_body(c, x, y, gm_layout, prec == GDC_FP32_MIXED);
 }
 
 // ---- pairs closer than 2a ------------------------------------------------------------
