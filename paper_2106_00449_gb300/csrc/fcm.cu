@@ -52,8 +52,9 @@ struct gdc_fcm {
     int* start = nullptr;
     int* fill = nullptr;
     int* list = nullptr;
-    float4* poff = nullptr;   // per list entry: the blob's offset from its cell's corner (FP32)
+    float4* poff = nullptr;   // per list entry: the blob's offset from its cell's corner (spreading), from its box (averaging)
     float4* plam = nullptr;   // per list entry: its lambda (FP32)
+    int4* box = nullptr;      // per blob: its box of grid points (averaging)
     int* scan = nullptr;
     bool have_field = false;
     unsigned long long n_launch = 0;
@@ -107,6 +108,7 @@ static size_t fcm_carve(gdc_fcm* f, void* base) {
     f->list = w.take<int>(f->p.max_blobs);
     f->poff = w.take<float4>(f->p.max_blobs);
     f->plam = w.take<float4>(f->p.max_blobs);
+    f->box = w.take<int4>(f->p.max_blobs);
     f->scan = w.take<int>(scan_scratch(nc3));
     return w.off + 256;
 }
@@ -204,6 +206,160 @@ __global__ void k_fcm_stage_blobs(int n, double w, int nc, const int* __restrict
 }
 
 constexpr int SP_CHUNK = 128;    // blob entries examined per round (one per thread)
+
+constexpr int SPC_KZ = 12;   // layers of a column a thread keeps
+
+// Spreading with at least 4 binning cells per side (no minimum image, as in k_fcm_spread below):
+// a block takes up to 256 columns (x, y) of a cell (blockDim.x, at least 128) and up to SPC_KZ of its
+// layers, a thread one column.
+// Per blob a thread forms dx^2 + dy^2 and its Gaussian once, and the layers' dz^2 and Gaussians
+// come from a table that the block fills once per staged blob, so a grid point costs a compare
+// and three FMAs (1.03 ms at 512^3 for 65,520 blobs; 13 instructions with the whole Gaussian per
+// point were issue-bound at 80%: 1.73 ms); the layers beyond the blob's reach are skipped (the same on
+// every thread).  Blobs out of reach of the block's points are dropped at staging; sums run in
+// list order: deterministic, no atomics on the grid.
+__global__ void __launch_bounds__(256) k_fcm_spread_col(int N, double h, double w, int nc, const int* __restrict__ cnt,
+                                                        const int* __restrict__ start, const float4* __restrict__ poff,
+                                                        const float4* __restrict__ plam, float R2, float Rt, float l2s,
+                                                        float norm, float2* __restrict__ f, long long NG, int zchunks) {
+    __shared__ float4 sp[SP_CHUNK];   // x, y of a staged blob; first and last layer in reach
+    __shared__ float4 sl[SP_CHUNK];
+    __shared__ float sz[SP_CHUNK];
+    __shared__ float2 ez[SP_CHUNK][SPC_KZ];   // dz^2 and its Gaussian per layer
+    __shared__ int wkept[SP_CHUNK / 32];
+    __shared__ int c_start[27], c_off[28];
+    __shared__ float base_off[3];   // offset of the cell's first grid point from its corner
+    const int b = blockIdx.x;
+    const int c3[3] = {b % nc, (b / nc) % nc, b / (nc * nc)};
+    int g0[3], gn[3];
+    for (int d = 0; d < 3; ++d) {
+        g0[d] = (c3[d] * N + nc - 1) / nc;                  // first i with floor(i nc / N) = c
+        gn[d] = ((c3[d] + 1) * N + nc - 1) / nc - g0[d];
+    }
+    const int ncol = gn[0] * gn[1];
+    const int col0 = (int)(blockIdx.y / zchunks) * (int)blockDim.x, k0 = (int)(blockIdx.y % zchunks) * SPC_KZ;
+    if (col0 >= ncol || k0 >= gn[2]) return;   // whole block: the cell has no points there
+    const int nz = min(SPC_KZ, gn[2] - k0);
+    if (threadIdx.x < 27) {
+        const int k = threadIdx.x;
+        const int ox = k % 3 - 1, oy = (k / 3) % 3 - 1, oz = k / 9 - 1;
+        const int id = (c3[0] + ox + nc) % nc + nc * ((c3[1] + oy + nc) % nc + nc * ((c3[2] + oz + nc) % nc));
+        c_start[k] = start[id];
+        c_off[k + 1] = cnt[id];
+    }
+    if (threadIdx.x >= 32 && threadIdx.x < 35) {
+        const int d = (int)threadIdx.x - 32;
+        base_off[d] = (float)(g0[d] * h - c3[d] * w);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {   // running sums of the 27 counts
+        int v = threadIdx.x < 27 ? c_off[threadIdx.x + 1] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, v, o);
+            if ((int)threadIdx.x >= o) v += t;
+        }
+        __syncwarp();
+        if (threadIdx.x < 27) c_off[threadIdx.x + 1] = v;
+        if (threadIdx.x == 0) c_off[0] = 0;
+    }
+    __syncthreads();
+    const int total = c_off[27];
+    const float hf = (float)h, wf = (float)w, ih = 1.0f / hf;
+    const int col = col0 + (int)threadIdx.x;
+    const bool live = col < ncol;
+    const int jx = col % gn[0], jy = col / gn[0];
+    const float gx = fmaf((float)jx, hf, base_off[0]), gy = fmaf((float)jy, hf, base_off[1]);
+    float ax[SPC_KZ], ay[SPC_KZ], az[SPC_KZ];
+#pragma unroll
+    for (int k = 0; k < SPC_KZ; ++k) ax[k] = ay[k] = az[k] = 0.f;
+    // the bounding box of this block's grid points in the frame of the cell's corner, and the
+    // squared reach beyond it, widened by 1e-4 against rounding (dropping is only ever conservative)
+    const int ylo = col0 / gn[0], yhi = (min(col0 + (int)blockDim.x, ncol) - 1) / gn[0];
+    const float bx0 = base_off[0], bx1 = fmaf((float)(gn[0] - 1), hf, base_off[0]);
+    const float by0 = fmaf((float)ylo, hf, base_off[1]), by1 = fmaf((float)yhi, hf, base_off[1]);
+    const float bz0 = fmaf((float)k0, hf, base_off[2]), bz1 = fmaf((float)(k0 + nz - 1), hf, base_off[2]);
+    const float reach2 = R2 * 1.0001f;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int s0 = 0; s0 < total; s0 += SP_CHUNK) {
+        const int e = threadIdx.x < SP_CHUNK ? s0 + (int)threadIdx.x : total;   // one entry per thread, 128 a round
+        bool keep = false;
+        float4 vp = make_float4(0.f, 0.f, 0.f, 0.f), vl = vp;
+        if (e < total) {
+            int k = 0;   // the neighbour cell of entry e: c_off[k] <= e < c_off[k + 1]
+            for (int step = 16; step > 0; step >>= 1)
+                if (k + step <= 26 && c_off[k + step] <= e) k += step;
+            const int pos = c_start[k] + (e - c_off[k]);
+            const float4 q = poff[pos];
+            const float ox = (float)(k % 3 - 1), oy = (float)((k / 3) % 3 - 1), oz = (float)(k / 9 - 1);
+            vp = make_float4(fmaf(ox, wf, q.x), fmaf(oy, wf, q.y), fmaf(oz, wf, q.z), 0.f);
+            vl = plam[pos];
+            const float ex = fmaxf(fmaxf(bx0 - vp.x, vp.x - bx1), 0.f);
+            const float ey = fmaxf(fmaxf(by0 - vp.y, vp.y - by1), 0.f);
+            const float ezd = fmaxf(fmaxf(bz0 - vp.z, vp.z - bz1), 0.f);
+            keep = fmaf(ex, ex, fmaf(ey, ey, ezd * ezd)) <= reach2;
+        }
+        __syncthreads();   // the previous round's staged blobs and tables are no longer read
+        // staged in entry order: the kept entries of lower warps, then of lower lanes
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0 && wid < SP_CHUNK / 32) wkept[wid] = __popc(bal);
+        __syncthreads();
+        int base = 0, take = 0;
+#pragma unroll
+        for (int w2 = 0; w2 < SP_CHUNK / 32; ++w2) {
+            const int c = wkept[w2];
+            base += w2 < wid ? c : 0;
+            take += c;
+        }
+        if (keep) {
+            const int at = base + __popc(bal & ((1u << lane) - 1u));
+            // the layers within reach (widened by 1% of a layer; the test per point decides)
+            const int ka = max(0, (int)ceilf((vp.z - Rt - bz0) * ih - 0.01f));
+            const int kb = min(nz - 1, (int)floorf((vp.z + Rt - bz0) * ih + 0.01f));
+            sp[at] = make_float4(vp.x, vp.y, __int_as_float(ka), __int_as_float(kb));
+            sl[at] = make_float4(vl.x * norm, vl.y * norm, vl.z * norm, 0.f);
+            sz[at] = vp.z;
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < take * SPC_KZ; q += blockDim.x) {
+            const int j = q / SPC_KZ, k = q - j * SPC_KZ;
+            const float dz = fmaf((float)k, hf, bz0) - sz[j], dz2 = dz * dz;
+            ez[j][k] = make_float2(dz2, exp2f(-dz2 * l2s));   // exp(-dz^2 / 2s^2)
+        }
+        __syncthreads();
+        if (live) {
+            for (int j = 0; j < take; ++j) {
+                const float4 pj = sp[j];
+                const float dx = gx - pj.x, dy = gy - pj.y;
+                const float dxy = fmaf(dx, dx, dy * dy), rem = R2 - dxy;
+                if (rem < 0.f) continue;
+                const float4 lj = sl[j];
+                const float e2 = exp2f(-dxy * l2s);
+                const float lx = lj.x * e2, ly = lj.y * e2, lz = lj.z * e2;
+                const int ka = __float_as_int(pj.z), kb = __float_as_int(pj.w);
+#pragma unroll
+                for (int k = 0; k < SPC_KZ; ++k) {
+                    if (k < ka || k > kb) continue;   // the same on every thread
+                    const float2 t = ez[j][k];
+                    if (t.x <= rem) {
+                        ax[k] = fmaf(lx, t.y, ax[k]);
+                        ay[k] = fmaf(ly, t.y, ay[k]);
+                        az[k] = fmaf(lz, t.y, az[k]);
+                    }
+                }
+            }
+        }
+    }
+    if (!live) return;
+    long long gi = (g0[0] + jx) + (long long)N * ((g0[1] + jy) + (long long)N * (g0[2] + k0));
+#pragma unroll
+    for (int k = 0; k < SPC_KZ; ++k) {
+        if (k >= nz) break;
+        f[gi] = make_float2(ax[k], ay[k]);      // two real fields in one complex grid
+        f[NG + gi] = make_float2(az[k], 0.f);
+        gi += (long long)N * N;
+    }
+}
 
 // f(x_g) = sum of lambda_j Delta_j(x_g).  One block per binning cell (cells at least R_t wide)
 // and chunk of 128 PT of its grid points (blockIdx.y): the cell's grid points are those with
@@ -759,90 +915,123 @@ __global__ void k_fcm_stress(long long NG, unsigned long long seed, unsigned own
 
 // ---- averaging ------------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(128) k_fcm_average(int n, const double* __restrict__ r, double L, int N, double h,
-                                                     double R_t, float l2s, double wscale,
-                                                     const float4* __restrict__ u, double* __restrict__ v) {
-    const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= n) return;
-    // the blob's box and its offset from the box's first grid point, formed by lane 0 and
-    // shared by shuffles: FP64 divisions on every lane would keep the FP64 pipe (1/64 of
-    // the FP32 rate) busier than the whole sum over the box
+// Per entry e of the blob list (order: cell-sorted, or null for index order): the box of grid
+// points around its blob and the offset from the blob to the box's first point, formed in FP64
+// with full warps (on one lane of a warp per blob these divisions took a third of the FP64
+// pipe's time beside the sum itself).
+__global__ void k_fcm_boxes(int n, const int* __restrict__ order, const double* __restrict__ r, double L, double h,
+                            double R_t, int4* __restrict__ box, float4* __restrict__ off) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int i = order ? order[e] : e;
     int lo[3], cn[3];
     float d0[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        int l = 0, c = 0;
-        float o = 0.f;
-        if (lane == 0) {
-            double x = r[3LL * i + d];
-            x -= L * floor(x / L);
-            if (!(x < L) || !(x >= 0.0)) x = 0.0;
-            l = (int)ceil((x - R_t) / h);
-            c = min(31, (int)floor((x + R_t) / h) - l + 1);
-            o = (float)(l * h - x);   // magnitude below R_t + h: FP32 keeps it to ~1e-7 R_t
-        }
-        lo[d] = __shfl_sync(0xffffffffu, l, 0);
-        cn[d] = __shfl_sync(0xffffffffu, c, 0);
-        d0[d] = __shfl_sync(0xffffffffu, o, 0);
+        double x = r[3LL * i + d];
+        x -= L * floor(x / L);
+        if (!(x < L) || !(x >= 0.0)) x = 0.0;
+        lo[d] = (int)ceil((x - R_t) / h);
+        cn[d] = min(31, (int)floor((x + R_t) / h) - lo[d] + 1);
+        d0[d] = (float)(lo[d] * h - x);   // magnitude below R_t + h: FP32 keeps it to ~1e-7 R_t
     }
-    // offsets from the blob to the grid points of its box: the first one, then steps of h
-    const float hf = (float)h, ih = 1.0f / hf, R2 = (float)(R_t * R_t);
-    const float d0x = d0[0], d0y = d0[1], d0z = d0[2];
+    box[e] = make_int4(lo[0], lo[1], lo[2], cn[0] | cn[1] << 8 | cn[2] << 16);
+    off[e] = make_float4(d0[0], d0[1], d0[2], __int_as_float(i));
+}
+
+// A sum of FP32 terms with compensation: s - c is the value.
+__device__ __forceinline__ void fcm_kahan(float& s, float& c, float v) {
+    const float y = __fsub_rn(v, c), t = __fadd_rn(s, y);
+    c = __fsub_rn(__fsub_rn(t, s), y);
+    s = t;
+}
+
+constexpr int AV_WARPS = 4;   // warps per blob
+
+// v_i = h^3 sum_g u(x_g) Delta_i(x_g): one block per blob, its warps taking every AV_WARPS-th
+// plane of the box.  Bound by the latency and traffic of the gather: blobs in cell order share
+// the lines of neighbouring boxes in L1 and L2 (in index order the field is re-read from HBM),
+// four loads are in flight per lane, and several warps per blob keep the last wave short
+// (8,190 blobs on 256^3: 373 us with one warp each in index order, 183 so; 65,520 on 512^3: 1.88 and
+// 1.29 ms).
+__global__ void __launch_bounds__(32 * AV_WARPS) k_fcm_average(const int4* __restrict__ box, const float4* __restrict__ off,
+                                                               int N, float hf, float R2, float l2s, double wscale,
+                                                               const float4* __restrict__ u, double* __restrict__ v) {
+    __shared__ float part[AV_WARPS][6];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int4 bx = box[blockIdx.x];
+    const float4 of = off[blockIdx.x];
+    const int cx = bx.w & 255, cy = (bx.w >> 8) & 255, cz = bx.w >> 16;
+    const float ih = 1.0f / hf, icx = 1.0f / (float)cx;
     const int mask = N - 1;   // N is a power of two
-    const int cx = cn[0];
-    const float icx = 1.0f / (float)cx;
     // the planes' sums added with compensation (Kahan) in FP32: as accurate as FP64 for a
-    // box's at most 31 planes, without an FP32-to-FP64 conversion and FP64 add per plane
+    // box's at most 31 planes
     float acc[3] = {0.f, 0.f, 0.f}, cmp[3] = {0.f, 0.f, 0.f};
-    float foz = 0.f;   // the plane offset also kept as a float (exact)
-    for (int oz = 0; oz < cn[2]; ++oz, foz += 1.f) {
-        const float dz = fmaf(foz, hf, d0z), dz2 = dz * dz, rem = R2 - dz2;
+    for (int oz = warp; oz < cz; oz += AV_WARPS) {
+        const float dz = fmaf((float)oz, hf, of.z), dz2 = dz * dz, rem = R2 - dz2;
         if (rem < 0.f) continue;   // the plane misses the sphere (the same on every lane)
         // the rows that can meet the sphere's disc in this plane (widened by 1% of a row
         // against rounding; the point test decides), taken as one run of points, x fastest,
         // so the lanes stay busy whatever the box width
         const float sq = sqrtf(rem);
-        const int y0 = max(0, (int)ceilf((-sq - d0y) * ih - 0.01f));
-        const int y1 = min(cn[1] - 1, (int)floorf((sq - d0y) * ih + 0.01f));
+        const int y0 = max(0, (int)ceilf((-sq - of.y) * ih - 0.01f));
+        const int y1 = min(cy - 1, (int)floorf((sq - of.y) * ih + 0.01f));
         const int npt = (y1 - y0 + 1) * cx;
         const float wz = exp2f(-dz2 * l2s);   // exp(-dz^2 / 2s^2)
-        const long long zoff = (long long)((lo[2] + oz) & mask) * N * N;
+        const float4* uz = u + (long long)((bx.z + oz) & mask) * N * N;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-#pragma unroll 4
-        for (int p = lane; p < npt; p += 32) {
-            // p = (oy - y0) cx + ox; the FP32 quotient is exact (p < 1024, and p / cx lies at
-            // least 1 / (2 cx) away from an integer)
-            const int qy = (int)(((float)p + 0.5f) * icx);
-            const int ox = p - qy * cx, oy = y0 + qy;
-            const float dx = fmaf((float)ox, hf, d0x), dy = fmaf((float)oy, hf, d0y);
-            const float dxy = fmaf(dx, dx, dy * dy);
-            if (dxy + dz2 <= R2) {
-                const float wgt = exp2f(-dxy * l2s) * wz;
-                const float4 q = __ldg(u + zoff + ((lo[1] + oy) & mask) * N + ((lo[0] + ox) & mask));
-                a0 = fmaf(q.x, wgt, a0);
-                a1 = fmaf(q.y, wgt, a1);
-                a2 = fmaf(q.z, wgt, a2);
+        for (int p0 = lane; p0 < npt; p0 += 128) {
+            float w[4];
+            float4 q[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                // p = (oy - y0) cx + ox; the FP32 quotient is exact (p < 1024, and p / cx lies at
+                // least 1 / (2 cx) away from an integer)
+                const int p = p0 + 32 * m;
+                const int qy = (int)(((float)p + 0.5f) * icx);
+                const int ox = p - qy * cx, oy = y0 + qy;
+                const float dx = fmaf((float)ox, hf, of.x), dy = fmaf((float)oy, hf, of.y);
+                const float dxy = fmaf(dx, dx, dy * dy);
+                const bool in = p < npt && dxy + dz2 <= R2;
+                w[m] = in ? exp2f(-dxy * l2s) : 0.f;
+                q[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (in) q[m] = __ldg(uz + ((bx.y + oy) & mask) * N + ((bx.x + ox) & mask));
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float wgt = w[m] * wz;
+                a0 = fmaf(q[m].x, wgt, a0);
+                a1 = fmaf(q[m].y, wgt, a1);
+                a2 = fmaf(q[m].z, wgt, a2);
             }
         }
-        const float a[3] = {a0, a1, a2};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float y = a[c] - cmp[c], t = acc[c] + y;
-            cmp[c] = (t - acc[c]) - y;
-            acc[c] = t;
-        }
+        fcm_kahan(acc[0], cmp[0], a0);
+        fcm_kahan(acc[1], cmp[1], a1);
+        fcm_kahan(acc[2], cmp[2], a2);
     }
-    double tot[3];
+    // lanes, then warps, joined by exact two-sums in a fixed order
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        tot[c] = (double)acc[c] - (double)cmp[c];
-        for (int o = 16; o > 0; o >>= 1) tot[c] += __shfl_down_sync(0xffffffffu, tot[c], o);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, acc[c], o), c2 = __shfl_xor_sync(0xffffffffu, cmp[c], o);
+            const float t = __fadd_rn(acc[c], s2), bb = __fsub_rn(t, acc[c]);
+            const float err = __fadd_rn(__fsub_rn(acc[c], __fsub_rn(t, bb)), __fsub_rn(s2, bb));
+            cmp[c] = __fsub_rn(__fadd_rn(cmp[c], c2), err);
+            acc[c] = t;
+        }
+        if (lane == 0) {
+            part[warp][c] = acc[c];
+            part[warp][3 + c] = cmp[c];
+        }
     }
-    if (lane == 0) {
-        v[3LL * i] = tot[0] * wscale;
-        v[3LL * i + 1] = tot[1] * wscale;
-        v[3LL * i + 2] = tot[2] * wscale;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int c = threadIdx.x;
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < AV_WARPS; ++w) s += (double)part[w][c] - (double)part[w][3 + c];
+        v[3LL * __float_as_int(of.w) + c] = s * wscale;
     }
 }
 
@@ -932,13 +1121,31 @@ static void zsolve_launch(gdc_fcm* f) {
 #undef GDC_ZS
 }
 
-// which = 0: the deterministic velocity, 1: the fluctuating one
-static void fcm_average_launch(gdc_fcm* f, int n, const double* r, int which, double* v) {
+// Wraps and bins the blobs: cell-sorted list, counts and starts per cell.
+static void fcm_bin_blobs(gdc_fcm* f, int n, const double* r) {
+    const long long nc3 = (long long)f->nc * f->nc * f->nc;
+    cudaMemsetAsync(f->cnt, 0, sizeof(int) * nc3, f->stream);
+    cudaMemsetAsync(f->fill, 0, sizeof(int) * nc3, f->stream);
+    ++f->n_launch, k_fcm_bin<<<ceil_div(n, 256), 256, 0, f->stream>>>(n, r, f->p.L, f->nc, f->pw, f->cell_of, f->cnt);
+    scan_exclusive(f->stream, &f->n_launch, (int)nc3, f->cnt, f->start, f->scan);
+    ++f->n_launch, k_fcm_scatter<<<ceil_div(n, 256), 256, 0, f->stream>>>(n, f->cell_of, f->start, f->fill, f->list);
+    ++f->n_launch, k_cell_sort<<<ceil_div(nc3, 256), 256, 0, f->stream>>>((int)nc3, f->cnt, f->start, f->list);
+}
+
+// which = 0: the deterministic velocity, 1: the fluctuating one; order: the cell-sorted list, or
+// null.  A packed grid of 256^3 points and more (268 MB) exceeds L2, so there the blobs are
+// taken in cell order, which is worth the binning; smaller grids stay in L2.
+static void fcm_average_launch(gdc_fcm* f, int n, const double* r, int which, double* v, const int* order) {
     const double s2 = f->p.sigma * f->p.sigma;
     const double norm = std::pow(2.0 * 3.141592653589793 * s2, -1.5);
-    ++f->n_launch, k_fcm_average<<<ceil_div(32LL * n, 128), 128, 0, f->stream>>>(
-        n, r, f->p.L, f->N, f->h, f->p.R_t, (float)(0.5 / s2 * 1.4426950408889634), norm * f->h * f->h * f->h,
-        f->packed + which * f->NG, v);
+    if (!order && f->N >= 256 && n >= 1024) {
+        fcm_bin_blobs(f, n, r);
+        order = f->list;
+    }
+    ++f->n_launch, k_fcm_boxes<<<ceil_div(n, 128), 128, 0, f->stream>>>(n, order, r, f->p.L, f->h, f->p.R_t, f->box, f->poff);
+    ++f->n_launch, k_fcm_average<<<n, 32 * AV_WARPS, 0, f->stream>>>(
+        f->box, f->poff, f->N, (float)f->h, (float)(f->p.R_t * f->p.R_t), (float)(0.5 / s2 * 1.4426950408889634),
+        norm * f->h * f->h * f->h, f->packed + which * f->NG, v);
 }
 
 // The grid of a gDC context with the FCM mobility (defaults: sigma = a/sqrt(pi), R_t = 3a).
@@ -1016,18 +1223,15 @@ gdc_status gdc_fcm_apply(gdc_fcm* f, int n, const double* r, const double* lambd
     if (const char* m = fcm_args(f, n, r, lambda)) return fcm_fail(f, GDC_ERR_INVALID_ARG, m);
     if (!u) return fcm_fail(f, GDC_ERR_INVALID_ARG, "NULL pointer");
     const long long nc3 = (long long)f->nc * f->nc * f->nc;
-    cudaMemsetAsync(f->cnt, 0, sizeof(int) * nc3, f->stream);
-    cudaMemsetAsync(f->fill, 0, sizeof(int) * nc3, f->stream);
-    ++f->n_launch, k_fcm_bin<<<ceil_div(n, 256), 256, 0, f->stream>>>(n, r, f->p.L, f->nc, f->pw, f->cell_of, f->cnt);
-    scan_exclusive(f->stream, &f->n_launch, (int)nc3, f->cnt, f->start, f->scan);
-    ++f->n_launch, k_fcm_scatter<<<ceil_div(n, 256), 256, 0, f->stream>>>(n, f->cell_of, f->start, f->fill, f->list);
-    ++f->n_launch, k_cell_sort<<<ceil_div(nc3, 256), 256, 0, f->stream>>>((int)nc3, f->cnt, f->start, f->list);
+    fcm_bin_blobs(f, n, r);
     ++f->n_launch, k_fcm_stage_blobs<<<ceil_div(n, 256), 256, 0, f->stream>>>(
         n, f->p.L / f->nc, f->nc, f->list, f->cell_of, f->pw, lambda, f->poff, f->plam);
     const double s2 = f->p.sigma * f->p.sigma;
     {
-        // 4 grid points per thread, 512 per block (2 and 256 when a cell has at most 256
-        // points, so that small cells leave fewer idle slots); the largest cell has side^3 points
+        // columns of a cell per thread from 8 points per cell side on (64 columns fill half a
+        // block) and 4 cells per side; else points: 4 per thread, 512 per block (2 and 256 when a
+        // cell has at most 256 points, so that small cells leave fewer idle slots).  The largest
+        // cell has side^3 points
         const long long side = (f->N + f->nc - 1) / f->nc;
         const int pt = side * side * side <= 256 ? 2 : 4;
         const unsigned chunks = (unsigned)((side * side * side + 128 * pt - 1) / (128 * pt));
@@ -1040,7 +1244,13 @@ gdc_status gdc_fcm_apply(gdc_fcm* f, int n, const double* r, const double* lambd
         f->N, f->h, f->p.L, 1.0 / f->p.L, f->p.L / f->nc, f->nc, f->pw, f->cnt, f->start, f->list, lambda, f->poff, \
         f->plam, R2, i2, nrm, f->grid, f->NG)
         const bool wrap = f->nc < 4;
-        if (pt == 2) {
+        if (!wrap && side >= 8) {
+            const int cols = (int)(side * side), zch = ceil_div(side, SPC_KZ);
+            const int th = std::min(256, std::max(128, (cols + 31) / 32 * 32));
+            k_fcm_spread_col<<<dim3((unsigned)nc3, (unsigned)(ceil_div(cols, th) * zch)), th, 0, f->stream>>>(
+                f->N, f->h, f->p.L / f->nc, f->nc, f->cnt, f->start, f->poff, f->plam, R2, (float)f->p.R_t, i2, nrm,
+                f->grid, f->NG, zch);
+        } else if (pt == 2) {
             if (wrap)
                 GDC_SPREAD(2, true);
             else
@@ -1060,7 +1270,7 @@ gdc_status gdc_fcm_apply(gdc_fcm* f, int n, const double* r, const double* lambd
     zsolve_launch(f);
     fft3(f, 2, 2, true, 1, 2);
     fft_x_pack(f, 2, 0);
-    fcm_average_launch(f, n, r, 0, u);
+    fcm_average_launch(f, n, r, 0, u, f->list);
     gdc_status st = fcm_check(f, cudaGetLastError(), "FCM launch");
     if (st == GDC_OK) st = fcm_check(f, cudaStreamSynchronize(f->stream), "FCM product");
     return st;
@@ -1084,7 +1294,7 @@ gdc_status gdc_fcm_brownian(gdc_fcm* f, unsigned long long seed, unsigned int ow
     fft3(f, 7, 2, true, 1, 3);
     fft_x_pack(f, 7, 1);
     f->have_field = true;
-    fcm_average_launch(f, n, r, 1, v);
+    fcm_average_launch(f, n, r, 1, v, nullptr);
     gdc_status st = fcm_check(f, cudaGetLastError(), "FCM launch");
     if (st == GDC_OK) st = fcm_check(f, cudaStreamSynchronize(f->stream), "FCM Brownian velocity");
     return st;
@@ -1094,7 +1304,7 @@ gdc_status gdc_fcm_average(gdc_fcm* f, int n, const double* r, double* v) {
     if (!f) return GDC_ERR_INVALID_ARG;
     if (const char* m = fcm_args(f, n, r, v)) return fcm_fail(f, GDC_ERR_INVALID_ARG, m);
     if (!f->have_field) return fcm_fail(f, GDC_ERR_INVALID_ARG, "no fluctuating field yet: call gdc_fcm_brownian first");
-    fcm_average_launch(f, n, r, 1, v);
+    fcm_average_launch(f, n, r, 1, v, nullptr);
     gdc_status st = fcm_check(f, cudaGetLastError(), "FCM launch");
     if (st == GDC_OK) st = fcm_check(f, cudaStreamSynchronize(f->stream), "FCM average");
     return st;
