@@ -287,9 +287,11 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->cell_H = cell_buckets(NBL);
     c->cell_xyz = w.take<int4>(NBL);
     c->cell_key = w.take<unsigned>(NBL);
-    c->cell_cnt = w.take<int>(c->cell_H);
+    c->cell_cells = w.take<int4>(NBL);
+    c->cell_pos = w.take<double4_32a>(NBL);
+    c->cell_cnt = w.take<int>(2 * c->cell_H);
+    c->cell_fill = c->cell_cnt ? c->cell_cnt + c->cell_H : nullptr;
     c->cell_start = w.take<int>(c->cell_H);
-    c->cell_fill = w.take<int>(c->cell_H);
     c->cell_list = w.take<int>(NBL);
     c->cell_scan = w.take<int>(cell_scan_ints(NBL));
     c->u3 = w.take<double>(3 * NBL);

@@ -159,7 +159,9 @@ struct gdc_ctx {
     long long cell_H = 0;         // buckets: a power of two >= 2 NBL
     int4* cell_xyz = 0;           // per blob: cell coordinates and suspension
     unsigned* cell_key = 0;       // per blob: bucket
-    int* cell_cnt = 0;            // per bucket: blobs
+    int4* cell_cells = 0;         // cell_xyz in list order
+    double4_32a* cell_pos = 0;    // positions in list order (as float4 for FP32 searches)
+    int* cell_cnt = 0;            // per bucket: blobs (cell_fill follows it)
     int* cell_start = 0;          // per bucket: first entry of cell_list
     int* cell_fill = 0;           // per bucket: scatter counter
     int* cell_list = 0;           // blob indices grouped by bucket, ascending within a bucket
