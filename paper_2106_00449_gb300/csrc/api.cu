@@ -363,7 +363,7 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->p64_part_i = w.take<double4_32a>((long long)c->p64_kmax * NBL);
     c->h_near_items.clear();
     // search blocks of 256 targets x near_src sources: as few sources as keep the list within
-    // 64 blocks per SM (2,560 blobs at 2,048 sources ran 20 blocks for 103 us)
+    // 64 blocks per SM (3,001 blobs: 144 blocks of 256 sources 20 us, 564 of 64 sources 9.0)
     int near_src = GDC_NEAR_SRC_MIN;
     for (; near_src < GDC_NEAR_SRC_MAX; near_src *= 2) {
         long long items = 0;

@@ -32,7 +32,7 @@
 #define GDC_ORTH_SLICE 4096      // elements per block of the fused orthogonalisation
 #define GDC_ORTH_MAX 32768       // and per suspension (longer: separate kernels)
 #define GDC_NEAR_CAP 32          // blobs closer than 2a listed per blob (beyond: a search of the suspension)
-#define GDC_NEAR_SRC_MIN 256     // sources per block of the near-pair search (see carve)
+#define GDC_NEAR_SRC_MIN 64      // sources per block of the near-pair search (see carve)
 #define GDC_NEAR_SRC_MAX 2048
 #define GDC_SYM_TILE 512         // blobs per tile of the symmetric FP32 pair kernel
 #define GDC_P64_EPI_WIDE 8192    // its epilogue: 16 threads per blob up to this many blobs, 4 above
@@ -349,6 +349,24 @@ __device__ __forceinline__ double rsqrt_series(double x) {
 __device__ inline double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Block sums of a[0..2] over TH threads, valid in lane 0 of warp d < 3 for component d; sh holds
+// 3 TH doubles.  Through shared memory: an FP64 add costs a warp 16 cycles whichever lanes take
+// part, and three warps adding TH / 32 values per lane need a quarter of the shuffles' adds.
+template <int TH>
+__device__ inline double block_sum3(const double* a, double* sh) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) sh[d * TH + threadIdx.x] = a[d];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v = 0.0;
+    if (warp < 3) {
+#pragma unroll
+        for (int q = 0; q < TH / 32; ++q) v += sh[warp * TH + 32 * q + lane];
+        v = warp_sum(v);
+    }
     return v;
 }
 

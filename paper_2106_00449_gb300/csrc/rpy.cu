@@ -1032,6 +1032,8 @@ gdc_status default_pair_kernel(gdc_ctx* c) {
 // of free blobs, with the same near-pair list and FP64 corrections of the self pair and of
 // the pairs closer than 2a.
 
+#include <cooperative_groups.h>
+
 #include <mutex>
 
 #define GDC_NOALLOC_SLOTS (16 * GDC_NOALLOC_MAX_BLOBS)   // partial sums: chunks x blobs of a call
@@ -1041,6 +1043,8 @@ gdc_status default_pair_kernel(gdc_ctx* c) {
 
 namespace gdc {
 
+namespace cg = cooperative_groups;
+
 struct NoallocScratch {
     float4 spos[GDC_NOALLOC_MAX_BLOBS];
     float4 sdup[3 * GDC_NOALLOC_MAX_BLOBS];
@@ -1049,41 +1053,57 @@ struct NoallocScratch {
     int near_cnt[GDC_NOALLOC_MAX_BLOBS];
     int near_idx[GDC_NOALLOC_MAX_BLOBS * GDC_NEAR_CAP];
     long long susp_blob_off[2];
-    double cen[3];   // blob centroid of the call (the FP32 positions are taken relative to it)
     int status[4];   // set by the pair kernel if a tile copy times out (u is then incomplete)
 };
 
 static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 
-// Start of a call: the blob centroid (one block; per-thread strided sums added in a fixed
-// order, so the result does not depend on timing) and the status words cleared.
-__global__ void __launch_bounds__(1024) k_noalloc_begin(NoallocScratch* __restrict__ sc, const double* __restrict__ r,
-                                                        int n) {
-    __shared__ double part[3][32];
-    double acc[3] = {0.0, 0.0, 0.0};
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += 1024)
-        for (int d = 0; d < 3; ++d) acc[d] += r[3 * i + d];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int d = 0; d < 3; ++d) {
-        const double v = warp_sum(acc[d]);
-        if (lane == 0) part[d][warp] = v;
+// Start of a call, one cluster of NOALLOC_CL blocks: the blob centroid (sums in a fixed order),
+// positions relative to it (FP32), lambda, identity body table, work list, status words.  A
+// block keeps its blobs' positions in registers between the two halves.  As a single block for
+// the centroid (bound by one SM's FP64 adds) and a second launch for the rest, 3,001 blobs took
+// 10.6 + 3.8 us; in one 9.0.
+constexpr int NOALLOC_CL = 8;
+constexpr int NOALLOC_PER = GDC_NOALLOC_MAX_BLOBS / (NOALLOC_CL * 1024);   // blobs per thread
+static_assert(NOALLOC_PER * NOALLOC_CL * 1024 == GDC_NOALLOC_MAX_BLOBS, "the cluster covers every size");
+
+__global__ void __cluster_dims__(NOALLOC_CL, 1, 1) __launch_bounds__(1024)
+    k_noalloc_prepare(NoallocScratch* __restrict__ sc, const double* __restrict__ r, const double* __restrict__ lam,
+                      int n, int nk, int csz) {
+    __shared__ double sh[3 * 1024];
+    __shared__ double part[3], cen[3];
+    cg::cluster_group cl = cg::this_cluster();
+    const int per = (n + NOALLOC_CL - 1) / NOALLOC_CL;
+    const int lo = blockIdx.x * per, hi = min(n, lo + per);
+    double p[NOALLOC_PER][3], acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < NOALLOC_PER; ++q) {
+        const int i = lo + threadIdx.x + 1024 * q;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) p[q][d] = i < hi ? r[3 * i + d] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < NOALLOC_PER; ++q)
+        if (lo + (int)threadIdx.x + 1024 * q < hi)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) acc[d] += p[q][d];
+    const double v = block_sum3<1024>(acc, sh);
+    if (threadIdx.x < 96 && (threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    cl.sync();
+    if (threadIdx.x < 3) {
+        double t = 0.0;
+#pragma unroll
+        for (int b = 0; b < NOALLOC_CL; ++b) t += *cl.map_shared_rank(&part[threadIdx.x], b);
+        cen[threadIdx.x] = t / n;
     }
     __syncthreads();
-    if (warp < 3) {
-        const double v = warp_sum(part[warp][lane]);
-        if (lane == 0) sc->cen[warp] = v / n;
-    }
-    if (threadIdx.x < 4) sc->status[threadIdx.x] = 0;
-}
-
-// Positions relative to the blob centroid (FP32), lambda, identity body table, work list.
-__global__ void k_noalloc_prepare(NoallocScratch* __restrict__ sc, const double* __restrict__ r,
-                                  const double* __restrict__ lam, int n, int nk, int csz) {
-    const double c0 = sc->cen[0], c1 = sc->cen[1], c2 = sc->cen[2];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double c0 = cen[0], c1 = cen[1], c2 = cen[2];
+#pragma unroll
+    for (int q = 0; q < NOALLOC_PER; ++q) {
+        const int i = lo + threadIdx.x + 1024 * q;
+        if (i >= hi) continue;
         sc->near_cnt[i] = 0;
-        const float x = (float)(r[3 * i] - c0), y = (float)(r[3 * i + 1] - c1), z = (float)(r[3 * i + 2] - c2);
+        const float x = (float)(p[q][0] - c0), y = (float)(p[q][1] - c1), z = (float)(p[q][2] - c2);
         const float lx = (float)lam[3 * i], ly = (float)lam[3 * i + 1], lz = (float)lam[3 * i + 2];
         sc->spos[i] = make_float4(x, y, z, __int_as_float(i));
         sc->sdup[3 * i] = make_float4(x, x, y, y);
@@ -1104,6 +1124,8 @@ __global__ void k_noalloc_prepare(NoallocScratch* __restrict__ sc, const double*
         sc->susp_blob_off[0] = 0;
         sc->susp_blob_off[1] = n;
     }
+    if (blockIdx.x == 0 && threadIdx.x < 4) sc->status[threadIdx.x] = 0;
+    cl.sync();   // no block leaves before its sums are read
 }
 
 // u_i = c0 (sum of chunk partials + self-pair and near-pair corrections), GDC_NOALLOC_EPI
@@ -1204,14 +1226,14 @@ extern "C" gdc_status gdc_rpy_apply_noalloc(const double* r, const double* lambd
     int csz = (n_blobs + nk - 1) / nk;
     csz = (csz + 31) / 32 * 32;
     nk = (n_blobs + csz - 1) / csz;
-    k_noalloc_begin<<<1, 1024, 0, st>>>(sc, r, n_blobs);
-    k_noalloc_prepare<<<std::min(1024, (n_blobs + 255) / 256 + 1), 256, 0, st>>>(sc, r, lambda, n_blobs, nk, csz);
+    k_noalloc_prepare<<<NOALLOC_CL, 1024, 0, st>>>(sc, r, lambda, n_blobs, nk, csz);
     RpyConst32 k{(float)(2.0 * a * a / 3.0), (float)(2.0 * a * a), (float)(4.0 * a * a), (float)(4.0 / (3.0 * a)),
                  (float)(9.0 / (32.0 * a)), (float)(1.0 / (8.0 * a * a))};
-    const int near_chunks = (n_blobs + GDC_NEAR_SRC_MIN - 1) / GDC_NEAR_SRC_MIN;
-    k_near_build<<<((n_blobs + 255) / 256) * near_chunks, 128, 0, st>>>(nullptr, near_chunks, GDC_NEAR_SRC_MIN,
-                                                                       sc->susp_blob_off, sc->spos, (float)(4.0 * a * a),
-                                                                       sc->near_cnt, sc->near_idx);
+    int near_src = GDC_NEAR_SRC_MIN;   // as in a context's list
+    while ((long long)ntile * ((n_blobs + near_src - 1) / near_src) > 64LL * sms) near_src *= 2;
+    const int near_chunks = (n_blobs + near_src - 1) / near_src;
+    k_near_build<<<ntile * near_chunks, 128, 0, st>>>(nullptr, near_chunks, near_src, sc->susp_blob_off, sc->spos,
+                                                      (float)(4.0 * a * a), sc->near_cnt, sc->near_idx);
     k_near_sort<<<(n_blobs + 255) / 256, 256, 0, st>>>(n_blobs, sc->near_cnt, sc->near_idx);
     k_rpy32<1, 6><<<ntile * nk, 128, 0, st>>>(sc->items, nullptr, sc->susp_blob_off, sc->spos, sc->sdup, sc->part,
                                              n_blobs, k, sc->status, first_wait_polls());

@@ -3,8 +3,8 @@
 The three x-neighbours of a blob's cell are adjacent hash buckets, read as one range; a row
 whose buckets wrap past the last one is read cell by cell.  Bodies scattered far apart in
 close pairs put their cells at arbitrary keys: of the about 250 occupied cells' nine rows each,
-2 in 1,024 wrap, so four seeds hold about 18 such rows.  Body counts 1, 2,047-2,049 are the edges
-of the reference point's four-bodies-per-thread sum."""
+2 in 1,024 wrap, so four seeds hold about 18 such rows.  Body counts 1, 256, 257 and 2,047-2,049 are the edges
+of the reference point's sum (one block or eight, four bodies per thread)."""
 import dataclasses
 
 import numpy as np
@@ -40,7 +40,7 @@ def test_scattered_pairs(lib, prec, seed):
     assert np.abs(a - b).max() <= 1500 * unit * 100 * np.abs(a).max()
 
 
-@pytest.mark.parametrize("n", [1, 2047, 2048, 2049])
+@pytest.mark.parametrize("n", [1, 256, 257, 2047, 2048, 2049])
 def test_reference_point_edges(lib, n):
     wl = _scattered(n, 7, 400.0)
     a, b = _both(lib, wl, 0)
