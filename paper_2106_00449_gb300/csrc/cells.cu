@@ -169,8 +169,10 @@ __global__ void k_cell_gather(int NBL, const int* __restrict__ list, const P4* _
 __device__ __forceinline__ long long body_of(float4 p) { return __float_as_int(p.w); }
 __device__ __forceinline__ long long body_of(double4_32a p) { return (long long)p.w; }
 
-// Calls f(e) for the list entries of the 27 cells around cell ci, cells in z, y, x order and
-// the entries of a cell in ascending blob index.  PERIODIC: nc cells per axis, neighbours wrap.
+// Calls f(e, in) for the list entries of the 27 cells around cell ci (and others that share
+// their buckets), cells in z, y, x order and the entries of a cell in ascending blob index;
+// in() tells whether entry e lies in the cells meant, and f asks it only of a blob that is close
+// enough, so that a candidate costs one load.  PERIODIC: nc cells per axis, neighbours wrap.
 template <bool PERIODIC, typename F>
 __device__ __forceinline__ void cell_neighbours(int4 ci, int nc, unsigned mask, const int* __restrict__ cnt,
                                                 const int* __restrict__ start, const int4* __restrict__ cell_s, F f) {
@@ -181,10 +183,12 @@ __device__ __forceinline__ void cell_neighbours(int4 ci, int nc, unsigned mask, 
                     const int cx = (ci.x + dx + nc) % nc, cy = (ci.y + dy + nc) % nc, cz = (ci.z + dz + nc) % nc;
                     const unsigned key = cell_hash(cx, cy, cz, ci.w, mask);
                     const int e0 = start[key], e1 = e0 + cnt[key];
-                    for (int e = e0; e < e1; ++e) {
-                        const int4 cj = cell_s[e];
-                        if (cj.x == cx && cj.y == cy && cj.z == cz && cj.w == ci.w) f(e);
-                    }
+#pragma unroll 4
+                    for (int e = e0; e < e1; ++e)
+                        f(e, [&] {
+                            const int4 cj = cell_s[e];
+                            return cj.x == cx && cj.y == cy && cj.z == cz && cj.w == ci.w;
+                        });
                 }
         return;
     }
@@ -199,22 +203,26 @@ __device__ __forceinline__ void cell_neighbours(int4 ci, int nc, unsigned mask, 
         e0[q] = start[key];
         e1[q] = start[k2] + cnt[k2];
     }
+    if (whole) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const int cy = ci.y + q % 3 - 1, cz = ci.z + q / 3 - 1;
-        if (whole) {
-            for (int e = e0[q]; e < e1[q]; ++e) {
-                const int4 cj = cell_s[e];
-                if (cj.y == cy && cj.z == cz && cj.w == ci.w && cj.x >= ci.x - 1 && cj.x <= ci.x + 1) f(e);
-            }
-        } else {
-            for (int dx = -1; dx <= 1; ++dx) {
-                const unsigned key = cell_hash(ci.x + dx, cy, cz, ci.w, mask);
-                for (int e = start[key], end = e + cnt[key]; e < end; ++e) {
+        for (int q = 0; q < 9; ++q) {
+            const int cy = ci.y + q % 3 - 1, cz = ci.z + q / 3 - 1;
+#pragma unroll 4
+            for (int e = e0[q]; e < e1[q]; ++e)
+                f(e, [&] {
                     const int4 cj = cell_s[e];
-                    if (cj.x == ci.x + dx && cj.y == cy && cj.z == cz && cj.w == ci.w) f(e);
-                }
-            }
+                    return cj.y == cy && cj.z == cz && cj.w == ci.w && cj.x >= ci.x - 1 && cj.x <= ci.x + 1;
+                });
+        }
+    } else {
+        for (int q = 0; q < 27; ++q) {
+            const int cx = ci.x + q % 3 - 1, cy = ci.y + q / 3 % 3 - 1, cz = ci.z + q / 9 - 1;
+            const unsigned key = cell_hash(cx, cy, cz, ci.w, mask);
+            for (int e = start[key], end = e + cnt[key]; e < end; ++e)
+                f(e, [&] {
+                    const int4 cj = cell_s[e];
+                    return cj.x == cx && cj.y == cy && cj.z == cz && cj.w == ci.w;
+                });
         }
     }
 }
@@ -233,7 +241,7 @@ __global__ void __launch_bounds__(128) k_forces_cell(int NBL, const P4* __restri
     const P4 pi = pos_s[t];
     const long long bi = body_of(pi);
     T fx = T(0), fy = T(0), fz = T(0);
-    cell_neighbours<PERIODIC>(cell_s[t], nc, mask, cnt, start, cell_s, [&](int e) {
+    cell_neighbours<PERIODIC>(cell_s[t], nc, mask, cnt, start, cell_s, [&](int e, auto in) {
         const P4 pj = pos_s[e];
         T ddx = pi.x - pj.x, ddy = pi.y - pj.y, ddz = pi.z - pj.z;
         if (PERIODIC) {
@@ -242,7 +250,7 @@ __global__ void __launch_bounds__(128) k_forces_cell(int NBL, const P4* __restri
             ddz -= box * rint(ddz / box);
         }
         const T r2 = fma(ddx, ddx, fma(ddy, ddy, ddz * ddz));
-        if (body_of(pj) != bi && r2 < k.rc2 && r2 > T(0)) {
+        if (r2 < k.rc2 && r2 > T(0) && body_of(pj) != bi && in()) {
             const T r = sqrt(r2);
             const T s = pair_force(r, k) / r;
             fx = fma(s, ddx, fx);
@@ -289,11 +297,11 @@ __global__ void __launch_bounds__(128) k_near_cell(int NBL, const float4* __rest
     const float4 pi = pos_s[t];
     const long long i = list[t];
     int m = 0;
-    cell_neighbours<false>(cell_s[t], 0, mask, cnt, start, cell_s, [&](int e) {
+    cell_neighbours<false>(cell_s[t], 0, mask, cnt, start, cell_s, [&](int e, auto in) {
         const float4 pj = pos_s[e];
         const float ddx = __fsub_rn(pj.x, pi.x), ddy = __fsub_rn(pj.y, pi.y), ddz = __fsub_rn(pj.z, pi.z);
         const float r2 = __fmaf_rn(ddx, ddx, __fmaf_rn(ddy, ddy, __fmul_rn(ddz, ddz)));
-        if (r2 < four_a2 && __float_as_int(pj.w) != __float_as_int(pi.w)) {
+        if (r2 < four_a2 && __float_as_int(pj.w) != __float_as_int(pi.w) && in()) {
             if (m < GDC_NEAR_CAP) near_idx[i * GDC_NEAR_CAP + m] = list[e];
             ++m;
         }
