@@ -31,6 +31,26 @@ __device__ __forceinline__ df df_mul(df x, df y) {
     e = fmaf(x.h, y.l, fmaf(x.l, y.h, e));
     return df_fast(p, e);
 }
+// x y before its closing fast two-sum: h the rounded product, l up to 1.5 ulp of h.  For a
+// consumer that adds h with a two-sum anyway.
+__device__ __forceinline__ df df_mul_open(df x, df y) {
+    const float p = __fmul_rn(x.h, y.h);
+    return {p, fmaf(x.h, y.l, fmaf(x.l, y.h, fmaf(x.h, y.h, -p)))};
+}
+// x + y of open or closed values, left open
+__device__ __forceinline__ df df_add_open(df x, df y) {
+    const df s = df_two_sum(x.h, y.h);
+    return {s.h, __fadd_rn(s.l, __fadd_rn(x.l, y.l))};
+}
+__device__ __forceinline__ df df_close(df x) { return df_fast(x.h, x.l); }
+// 1 + x, |x| < 1 (the larger term is known: three operations instead of six), left open
+__device__ __forceinline__ df df_one_plus(df x) {
+    const df s = df_fast(1.f, x.h);
+    return {s.h, __fadd_rn(s.l, x.l)};
+}
+__device__ __forceinline__ df df_dot3(df ax, df ay, df az, df bx, df by, df bz) {
+    return df_close(df_add_open(df_add_open(df_mul_open(ax, bx), df_mul_open(ay, by)), df_mul_open(az, bz)));
+}
 __device__ __forceinline__ df df_from(double v) {
     const float h = (float)v;
     return {h, (float)(v - (double)h)};

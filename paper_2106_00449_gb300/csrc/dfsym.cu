@@ -34,33 +34,41 @@ struct DfPair {   // the shared part of one pair: d = r_j - r_i, A, B
 };
 
 __device__ __forceinline__ DfPair df_pair(df xs, df ys, df zs, df xt, df yt, df zt, const RpyConstDF& k) {
-    const df one{1.f, 0.f};
     DfPair p;
     p.dx = df_sub(xs, xt);
     p.dy = df_sub(ys, yt);
     p.dz = df_sub(zs, zt);
-    const df r2 = df_add(df_add(df_mul(p.dx, p.dx), df_mul(p.dy, p.dy)), df_mul(p.dz, p.dz));
+    const df r2 = df_dot3(p.dx, p.dy, p.dz, p.dx, p.dy, p.dz);
     const df ri = df_rsqrt(r2);
     if (r2.h > k.four_a2.h || (r2.h == k.four_a2.h && r2.l >= k.four_a2.l)) {
         const df ri2 = df_mul(ri, ri);
-        const df ri3 = df_mul(ri2, ri);
-        p.A = df_add(ri, df_mul(k.c23, ri3));
-        p.B = df_mul(ri3, df_sub(one, df_mul(k.c2, ri2)));
+        // A = (1 + 2a^2/(3 r^2)) / r, B = (1 - 2a^2/r^2) / r^3; r >= 2a, so both brackets are
+        // one plus a term below one
+        const df w = df_mul_open(k.c2, ri2);
+        p.A = df_mul(ri, df_one_plus(df_mul_open(k.c23, ri2)));
+        p.B = df_mul(df_mul(ri2, ri), df_one_plus(df{-w.h, -w.l}));
     } else {   // overlapping blobs of different bodies (r > 0 for distinct blobs)
         const df r = df_mul(r2, ri);
-        p.A = df_mul(k.cA, df_sub(one, df_mul(k.c9, r)));
+        p.A = df_mul(k.cA, df_sub(df{1.f, 0.f}, df_mul(k.c9, r)));
         p.B = df_mul(k.cB, ri);
     }
     return p;
 }
 
-// u += A lambda + B (d . lambda) d
+// u += A lambda + B (d . lambda) d.  A product is closed (its low part brought below half an ulp
+// of the high part) only where it is multiplied again; sums take it open and close once per
+// component: 119 operations a side, against 158 with every product and sum closed, and fewer
+// roundings of the low parts.  The kernel is bound by FP32 issue: 65,520 blobs 30.6 -> 24.2 ms,
+// relative error of the product against FP64 2.0e-14 both; 2,560 blobs 98 -> 78 us, 1.9e-14 ->
+// 8.6e-15.
+__device__ __forceinline__ df df_accumulate(df u, df A, df l, df s, df d) {
+    return df_close(df_add_open(u, df_add_open(df_mul_open(A, l), df_mul_open(s, d))));
+}
 __device__ __forceinline__ void df_side(const DfPair& p, df lx, df ly, df lz, df& ux, df& uy, df& uz) {
-    const df dl = df_add(df_add(df_mul(p.dx, lx), df_mul(p.dy, ly)), df_mul(p.dz, lz));
-    const df s = df_mul(p.B, dl);
-    ux = df_add(ux, df_add(df_mul(p.A, lx), df_mul(s, p.dx)));
-    uy = df_add(uy, df_add(df_mul(p.A, ly), df_mul(s, p.dy)));
-    uz = df_add(uz, df_add(df_mul(p.A, lz), df_mul(s, p.dz)));
+    const df s = df_mul(p.B, df_dot3(p.dx, p.dy, p.dz, lx, ly, lz));
+    ux = df_accumulate(ux, p.A, lx, s, p.dx);
+    uy = df_accumulate(uy, p.A, ly, s, p.dy);
+    uz = df_accumulate(uz, p.A, lz, s, p.dz);
 }
 
 __device__ __forceinline__ df shfl_df(df v, int src) {
@@ -222,9 +230,10 @@ void launch_rpy_df_sym_pairs(gdc_ctx* c) {
 
 // Work list: the longest ranges (16 to 1,024 sources; longer in suspensions above 65,536
 // blobs, so that a row has at most 64 target-side slots) that give 24 items per SM.  us per
-// launch by that rule, and as items of two whole tiles before: 2,560 blobs 98 / 2,067, 7,800
-// blobs 543 / 2,159, 20,202 blobs 3,144 / 3,813, 48 suspensions of 63,702 blobs 1,196 / 2,624,
-// 65,520 blobs 30,660 / 30,640.
+// launch by that rule, and as items of two whole tiles (with every product and sum of df_side
+// closed): 2,560 blobs 98 / 2,067, 7,800 blobs 543 / 2,159, 20,202 blobs 3,144 / 3,813, 48
+// suspensions of 63,702 blobs 1,196 / 2,624, 65,520 blobs 30,660 / 30,640.  With df_side as it
+// is now: 78, 427, 2,450, 905 and 24,170, relative error against FP64 6e-15 to 2e-14.
 void build_dfs_list(gdc_ctx* c) {
     long long nmax = 1;
     for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
