@@ -70,7 +70,7 @@ def _dist():
 PAIR_KERNELS = {
     1: ("rpy.cu", "template <int P, int MINB>\n__global__ void __launch_bounds__(128, MINB) k_rpy32",
         r"#define (GDC_MV_TILE) (\S+)", "k_rpy32_c3_65k.md", "k_rpy32 (ordered FP32 RPY pair kernel)"),
-    2: ("sym.cu", "template <int MINB>\n__global__ void __launch_bounds__(128, MINB) k_rpy32_sym",
+    2: ("sym.cu", "template <int MINB, bool FULL>\n__global__ void __launch_bounds__(128, MINB) k_rpy32_sym",
         r"#define (GDC_SYM_TILE) (\S+)", "k_rpy32_sym_c3_65k.md",
         "k_rpy32_sym (symmetric FP32 RPY pair kernel)"),
 }

@@ -20,8 +20,8 @@
 // cells one contiguous range of the list (9 ranges per blob instead of 27 buckets, their bounds
 // loaded at once); a candidate's cell and position lie at its list entry (not behind an index);
 // threads take the blobs in list order, so neighbours read the same lines.  Body forces of
-// 16,384 bodies: 285 us, against 655 us with a bucket per cell and indirect candidates (the
-// search alone was 433); 20,202-blob product with its near lists: 423 us, against 448.
+// 16,384 bodies: 270 us, against 655 us with a bucket per cell and indirect candidates (the
+// search alone 125, against 433); 20,202-blob product with its near lists: 415 us, against 448.
 #include <algorithm>
 
 #include "common.cuh"

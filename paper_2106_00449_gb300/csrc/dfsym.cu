@@ -76,7 +76,7 @@ __device__ __forceinline__ df shfl_df(df v, int src) {
 }
 
 // MINB: resident blocks per SM the register allocator is asked to allow, 3 (162 registers) or
-// 4 (128); the autotuner times both against the ordered double-float kernel.
+// 4 (128, the rule below GDC_TUNE_PAIRS); above, the autotuner times both.
 // FULL: every range is whole tiles, as in the symmetric FP32 kernel.
 template <int MINB, bool FULL>
 __global__ void __launch_bounds__(128, MINB) k_rpy_df_sym(const PairItem* __restrict__ items,
