@@ -370,21 +370,38 @@ __global__ void k_gm_arnoldi(int S, int j, const int* __restrict__ jdev, int m, 
 }
 
 // y = H^-1 g (upper triangular, size jcount[s])
-__global__ void k_gm_backsolve(int S, int m, const double* __restrict__ H, const double* __restrict__ g,
-                               const int* __restrict__ jcount, double* __restrict__ y, int cols) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    const int k = jcount[s];
-    const int mp1 = m + 1;
-    const double* Hs = H + (long long)s * mp1 * m;
-    const double* gs = g + (long long)s * mp1;
+// One warp per suspension: y_i, then its column taken off the rows above by the lanes, the next
+// column loaded meanwhile.  Bound by the chain of k divisions and by latency: as one thread with
+// k^2 / 2 dependent loads, 13 columns took 16 us and 18 columns of 48 suspensions 24 us.
+static_assert(GDC_MAX_RESTART <= 128, "four rows per lane");
+
+__global__ void __launch_bounds__(32) k_gm_backsolve(int m, const double* __restrict__ H, const double* __restrict__ g,
+                                                     const int* __restrict__ jcount, double* __restrict__ y, int cols) {
+    __shared__ double acc[128];
+    const int s = blockIdx.x, lane = threadIdx.x, k = jcount[s];
+    const double* Hs = H + (long long)s * (m + 1) * m;
+    const double* gs = g + (long long)s * (m + 1);
     double* ys = y + (long long)s * cols;
+    for (int i = lane; i < k; i += 32) acc[i] = gs[i];
+    double col[4], diag = k > 0 ? Hs[(k - 1) * m + k - 1] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) col[q] = lane + 32 * q < k - 1 ? Hs[(lane + 32 * q) * m + k - 1] : 0.0;
+    __syncwarp();
     for (int i = k - 1; i >= 0; --i) {
-        double acc = gs[i];
-        for (int q = i + 1; q < k; ++q) acc -= Hs[i * m + q] * ys[q];
-        ys[i] = Hs[i * m + i] != 0.0 ? acc / Hs[i * m + i] : 0.0;
+        double next[4], ndiag = i > 0 ? Hs[(i - 1) * m + i - 1] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) next[q] = lane + 32 * q < i - 1 ? Hs[(lane + 32 * q) * m + i - 1] : 0.0;
+        const double yi = diag != 0.0 ? acc[i] / diag : 0.0;
+        if (lane == 0) ys[i] = yi;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (lane + 32 * q < i) acc[lane + 32 * q] -= col[q] * yi;
+            col[q] = next[q];
+        }
+        diag = ndiag;
+        __syncwarp();
     }
-    for (int i = k; i < cols; ++i) ys[i] = 0.0;
+    for (int i = k + lane; i < cols; i += 32) ys[i] = 0.0;
 }
 
 // ---- one iteration's orthogonalisation in one launch -----------------------------------
@@ -713,7 +730,7 @@ gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* i
         }
         inf.iterations = std::max(inf.iterations, total);
         // x += P^-1 V y
-        ++c->n_launch, k_gm_backsolve<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(c->S, m, c->gm_H, c->gm_g, c->gm_j, c->gm_y, cols);
+        ++c->n_launch, k_gm_backsolve<<<c->S, 32, 0, c->stream>>>(m, c->gm_H, c->gm_g, c->gm_j, c->gm_y, cols);
         ++c->n_launch, k_combine<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, c->gm_j, c->gm_y, cols, nullptr, c->gm_w);
         launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED, prec == GDC_FP32_MIXED);   // the correction e of this cycle
         ++c->n_launch, k_axpy_chunks<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, 1.0, c->gm_z, x);
@@ -1522,8 +1539,7 @@ void gmres_solve_graph(gdc_ctx* c, const double* b, double* x) {
         }
         cap_while_end(c, REP_GM_TOTAL, before_i);
         // x += P^-1 V y
-        ++c->n_launch, k_gm_backsolve<<<ceil_div(c->S, 128), 128, 0, c->stream>>>(c->S, m, c->gm_H, c->gm_g, c->gm_j,
-                                                                                  c->gm_y, cols);
+        ++c->n_launch, k_gm_backsolve<<<c->S, 32, 0, c->stream>>>(m, c->gm_H, c->gm_g, c->gm_j, c->gm_y, cols);
         ++c->n_launch, k_combine<<<sg.n_chunks, 256, 0, c->stream>>>(sg.chunks, c->gm_V, n, c->gm_j, c->gm_y, cols,
                                                                      nullptr, c->gm_w);
         launch_precond(c, c->gm_w, c->gm_z, prec == GDC_FP32_MIXED, prec == GDC_FP32_MIXED);   // the correction e of this cycle
