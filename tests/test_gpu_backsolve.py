@@ -1,5 +1,5 @@
 """GPU: GMRES cycles whose back substitution has the fewest columns a restart allows (2), a few, and
-as many as the solve takes (past one lane row of 32 where it takes that long).
+more than one lane row of 32 (the FP32-mixed cycle aims a decade below its tolerance).
 
 Forces without torques (a torque along a rod's axis has no solution).  Each solve is judged by its
 own residual through the FP64 saddle product: at most the solver's tolerance, plus the product's
