@@ -150,64 +150,83 @@ __host__ __device__ inline int gp_split(int n3) {
     return R >= GP_TH ? 1 : GP_TH / R;
 }
 
+// FP32 rows of more than 64 columns keep at least four chains, joined in FP64, where up to a few
+// thousand bodies share the work (GB < 8): two of them, or two joined in FP32, lose up to a third
+// of the accuracy of a body's own block (relative error of an FP32 product of single bodies, two
+// chains and four: 340 blobs 4.2e-7 and 3.2e-7, 85 blobs 2.4e-7 and 1.9e-7).  Shorter rows have
+// more chains anyway, each shorter; GB = 8 stays with two, half the FP64 additions.
+// gp_halves: the parts that a thread takes of a whole row in turn, each summed into FP64;
+// gp_parts: the chains that a thread of a split row leaves to be joined.
+template <int GB, typename T>
+__host__ __device__ inline int gp_halves(int KS) { return GB < 8 && sizeof(T) == 4 && KS == 1 ? 2 : 1; }
+template <int GB, typename T>
+__host__ __device__ inline int gp_parts(int KS) { return GB < 8 && sizeof(T) == 4 && KS == 2 ? 2 : 1; }
+
 // out[u n3 + i] = sum_k M[k n3 + i] in[k GB + u] over the columns SHAPE leaves row i, u < GB (in
-// padded with zeros): sums of type T over at most n3 / KS columns, the KS partial sums added
-// in FP64.  part: KS GB n3 values of T (unused for KS = 1).  Ends with a barrier.
+// padded with zeros): two chains of type T over each thread's columns, the threads' sums added in
+// FP64.  part: gp_parts KS GB n3 values of T (unused for KS = 1).  Ends with a barrier.
 template <int GB, int SHAPE, typename T>
 __device__ __forceinline__ void group_product(const T* __restrict__ M, int n3, const T* in_, T* part, double* out) {
     // 16-byte aligned by the callers' layouts for GB >= 4, so a column's entries are vector loads
     const T* in = GB >= 4 ? (const T*)__builtin_assume_aligned(in_, 16) : in_;
-    const int R = (n3 + 31) & ~31, KS = gp_split(n3);
+    const int R = (n3 + 31) & ~31, KS = gp_split(n3), halves = gp_halves<GB, T>(KS), NP = gp_parts<GB, T>(KS);
     const int ks = KS == 1 ? 0 : (int)threadIdx.x / R;
-    const int chunk = (n3 + KS - 1) / KS;
+    const int chunk = (n3 + KS * halves - 1) / (KS * halves);
     for (int row = KS == 1 ? (int)threadIdx.x : (int)threadIdx.x % R; row < n3 && ks < KS; row += GP_TH) {
-        int k0 = ks * chunk, k1 = min(n3, k0 + chunk);
-        if (SHAPE == GP_FROM_DIAG) k0 = max(k0, row);
-        if (SHAPE == GP_TO_DIAG) k1 = min(k1, row + 1);
-        T a[GB], b[GB];
+        for (int h = 0; h < halves; ++h) {
+            int k0 = (ks + h) * chunk, k1 = min(n3, k0 + chunk);
+            if (SHAPE == GP_FROM_DIAG) k0 = max(k0, row);
+            if (SHAPE == GP_TO_DIAG) k1 = min(k1, row + 1);
+            T a[GB], b[GB];
 #pragma unroll
-        for (int u = 0; u < GB; ++u) a[u] = b[u] = T(0);
-        int k = k0;
-        const T* Mr = M + row;
-        for (; k + 7 < k1; k += 8) {   // eight elements in flight: the matrix comes from L2
-            T f[8];
+            for (int u = 0; u < GB; ++u) a[u] = b[u] = T(0);
+            int k = k0;
+            const T* Mr = M + row;
+            for (; k + 7 < k1; k += 8) {   // eight elements in flight: the matrix comes from L2
+                T f[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) f[q] = Mr[(long long)(k + q) * n3];
+                for (int q = 0; q < 8; ++q) f[q] = Mr[(long long)(k + q) * n3];
 #pragma unroll
-            for (int q = 0; q < 8; q += 2)
+                for (int q = 0; q < 8; q += 2)
+#pragma unroll
+                    for (int u = 0; u < GB; ++u) {
+                        a[u] = fma(f[q], in[(k + q) * GB + u], a[u]);
+                        b[u] = fma(f[q + 1], in[(k + q + 1) * GB + u], b[u]);
+                    }
+            }
+#pragma unroll 2
+            for (; k + 1 < k1; k += 2) {
+                const T f = Mr[(long long)k * n3], g = Mr[(long long)(k + 1) * n3];
 #pragma unroll
                 for (int u = 0; u < GB; ++u) {
-                    a[u] = fma(f[q], in[(k + q) * GB + u], a[u]);
-                    b[u] = fma(f[q + 1], in[(k + q + 1) * GB + u], b[u]);
+                    a[u] = fma(f, in[k * GB + u], a[u]);
+                    b[u] = fma(g, in[(k + 1) * GB + u], b[u]);
                 }
-        }
-#pragma unroll 2
-        for (; k + 1 < k1; k += 2) {
-            const T f = Mr[(long long)k * n3], g = Mr[(long long)(k + 1) * n3];
+            }
+            if (k < k1) {
+                const T f = M[(long long)k * n3 + row];
+#pragma unroll
+                for (int u = 0; u < GB; ++u) a[u] = fma(f, in[k * GB + u], a[u]);
+            }
 #pragma unroll
             for (int u = 0; u < GB; ++u) {
-                a[u] = fma(f, in[k * GB + u], a[u]);
-                b[u] = fma(g, in[(k + 1) * GB + u], b[u]);
+                if (KS == 1) {
+                    const double s = (double)a[u] + (double)b[u];
+                    out[u * n3 + row] = h == 0 ? s : out[u * n3 + row] + s;
+                } else if (NP == 2) {
+                    part[(2 * ks * GB + u) * n3 + row] = a[u];
+                    part[((2 * ks + 1) * GB + u) * n3 + row] = b[u];
+                } else {
+                    part[(ks * GB + u) * n3 + row] = a[u] + b[u];
+                }
             }
-        }
-        if (k < k1) {
-            const T f = M[(long long)k * n3 + row];
-#pragma unroll
-            for (int u = 0; u < GB; ++u) a[u] = fma(f, in[k * GB + u], a[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < GB; ++u) {
-            if (KS == 1)
-                out[u * n3 + row] = (double)a[u] + (double)b[u];
-            else
-                part[(ks * GB + u) * n3 + row] = a[u] + b[u];
         }
     }
     __syncthreads();
     if (KS > 1) {
         for (int e = threadIdx.x; e < GB * n3; e += GP_TH) {
             double s = (double)part[e];
-            for (int q = 1; q < KS; ++q) s += (double)part[q * GB * n3 + e];
+            for (int q = 1; q < NP * KS; ++q) s += (double)part[q * GB * n3 + e];
             out[e] = s;
         }
         __syncthreads();
@@ -215,9 +234,10 @@ __device__ __forceinline__ void group_product(const T* __restrict__ M, int n3, c
 }
 
 // Bytes of group_product's arrays: in (T), part (T), out (double)
-static size_t gp_bytes(int GB, int n3, size_t t) {
+template <int GB, typename T>
+static size_t gp_bytes(int n3) {
     const int KS = gp_split(n3);
-    return (size_t)GB * n3 * (sizeof(double) + t + (KS > 1 ? KS * t : 0));
+    return (size_t)GB * n3 * (sizeof(double) + sizeof(T) * (1 + (KS > 1 ? KS * gp_parts<GB, T>(KS) : 0)));
 }
 
 // K^T of the group's body-frame vectors v (double, [u][n3]) with blob offsets b: four threads per
@@ -385,9 +405,10 @@ __global__ void __launch_bounds__(GP_TH) k_precond(GroupArgs ga, const T* __rest
 // rotated lambda rounded to FP32, the rotations in FP64).  x and y use the saddle layout (gm =
 // 1) or 3 doubles per blob (gm = 0); in the saddle layout the body rows -K^T lambda of the
 // operator are formed here as well, from the rotated lambda and the template's offsets (one
-// launch instead of two, lambda read once).
+// launch instead of two, lambda read once).  GB = 4 is held to 48 registers, five blocks per SM:
+// with 63 the 816 blocks of 48 suspensions took a wave and a third (their solve 5.44 ms, 5.33 so).
 template <int GB, typename T>
-__global__ void __launch_bounds__(GP_TH) k_intra_body(GroupArgs ga, const T* __restrict__ Mt, const double* __restrict__ x,
+__global__ void __launch_bounds__(GP_TH, GB == 4 ? 5 : 0) k_intra_body(GroupArgs ga, const T* __restrict__ Mt, const double* __restrict__ x,
                                                       double* __restrict__ y, int gm) {
     extern __shared__ __align__(16) double sh[];
     const int4 it = group_item<false, GB>(ga);
@@ -505,15 +526,16 @@ static GroupArgs group_args(const gdc_ctx* c) {
 }
 
 // Shared memory of a block: the largest over the templates
-static size_t group_smem(const gdc_ctx* c, int GB, size_t t, int more_per_row, int more) {
+template <int GB, typename T>
+static size_t group_smem(const gdc_ctx* c, int more_per_row, int more) {
     size_t s = 0;
-    for (int n : c->h_tmpl_n) s = std::max(s, gp_bytes(GB, 3 * n, t) + (size_t)(more_per_row * 3 * n + more) * sizeof(double));
+    for (int n : c->h_tmpl_n) s = std::max(s, gp_bytes<GB, T>(3 * n) + (size_t)(more_per_row * 3 * n + more) * sizeof(double));
     return s;
 }
 
 template <bool LAB, int GB, typename T>
 static void precond_launch(gdc_ctx* c, const T* Minv, const double* r, double* z, float4* sdup) {
-    const size_t smem = group_smem(c, GB, sizeof(T), LAB ? 1 : 0, 24 * GB);
+    const size_t smem = group_smem<GB, T>(c, LAB ? 1 : 0, 24 * GB);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_precond<LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_precond<LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), Minv, LAB ? c->blk_G : c->tmpl_G, LAB ? c->blk_N : c->tmpl_N, r, z, c->r, c->Yc, sdup);
@@ -535,7 +557,7 @@ void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32, bool pack
 
 template <int GB, typename T>
 static void intra_launch(gdc_ctx* c, const T* M, const double* x, double* y, int gm) {
-    const size_t smem = group_smem(c, GB, sizeof(T), GB, 6 * GB);
+    const size_t smem = group_smem<GB, T>(c, GB, 6 * GB);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_intra_body<GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     GroupArgs ga = group_args(c);
     ga.mat_off = c->minv_off;
@@ -555,7 +577,7 @@ void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm, bool fp32
 
 template <int MODE, bool LAB, int GB, typename T>
 static void tri_launch(gdc_ctx* c, const T* F, const double* x, const double* add, double* out, float4* sdup) {
-    const size_t smem = group_smem(c, GB, sizeof(T), 0, 0);
+    const size_t smem = group_smem<GB, T>(c, 0, 0);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_body_tri<MODE, LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_body_tri<MODE, LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), F, x, add, out, sdup);
