@@ -26,7 +26,24 @@ int first_wait_polls() {
     return v == 0 ? GDC_WAIT_POLLS : (v < 0 ? 0 : v);
 }
 
+// A cluster launch can be refused although the kernel is sound (a device or partition that cannot
+// place the cluster); the stream then simply lacks the kernel, and nothing that is waited for
+// later fails.  So its result is kept and reported by the call's next check, before anything
+// read back is used.
+void note_launch(gdc_ctx* c, cudaError_t e) {
+    if (e == cudaSuccess) return;
+    cudaGetLastError();   // reported through the context, not by an unrelated later call
+    if (c->launch_err == cudaSuccess) c->launch_err = e;
+}
+
 gdc_status cuda_check(gdc_ctx* c, cudaError_t e, const char* what) {
+    if (c && c->launch_err != cudaSuccess) {
+        if (e == cudaSuccess) {
+            e = c->launch_err;
+            what = "kernel launch";
+        }
+        c->launch_err = cudaSuccess;
+    }
     if (e == cudaSuccess) return GDC_OK;
     return fail(c, GDC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
@@ -489,7 +506,7 @@ static gdc_status read_status(gdc_ctx* c) {
     int st[4] = {0, 0, 0, 0};
     cudaError_t e = cudaMemcpyAsync(st, c->dev_status, sizeof(st), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_check(c, e, "status read");
+    if (const gdc_status s = cuda_check(c, e, "status read")) return s;
     if ((st[0] != 0 || st[1] != 0 || st[2] != 0) && clear_status(c) != GDC_OK) return GDC_ERR_CUDA;
     // a timed-out tile copy first: an incomplete product explains any later failure
     if (st[1] != 0) return fail(c, GDC_ERR_TIMEOUT, "a pair-kernel tile copy did not complete in time");
@@ -838,9 +855,9 @@ static gdc_status build_graph(gdc_ctx* c) {
     c->n_launch = n0;
     if (e == cudaSuccess && c->cap_err != cudaSuccess) e = c->cap_err;
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) {
+    if ((st = cuda_check(c, e, "step graph capture")) != GDC_OK) {
         if (g) cudaGraphDestroy(g);
-        return cuda_check(c, e, "step graph capture");
+        return st;
     }
     c->graph = g;
     if ((st = cuda_check(c, cudaGraphInstantiate(&c->graph_exec, g, 0), "step graph instantiate")) != GDC_OK) {

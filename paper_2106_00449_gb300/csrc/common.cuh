@@ -283,6 +283,7 @@ struct gdc_ctx {
     cudaGraph_t cap_bodies[2] = {0, 0};        // the two bodies of the IF/ELSE node being captured
     int cap_depth = 0;
     cudaError_t cap_err = cudaSuccess;
+    cudaError_t launch_err = cudaSuccess;   // the first refused cluster launch (note_launch)
     unsigned long long graph_base_launches = 0;               // kernels outside the loops
     std::vector<std::pair<int, unsigned long long>> graph_loops;   // (report slot, kernels per iteration)
     unsigned long long d_step_mirror = ~0ull;                 // value last written to ctl->step
@@ -375,7 +376,8 @@ inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 // ---- host-side helpers (defined in api.cu) --------------------------------
 int first_wait_polls();   // poll bound of the pair kernels' waits for a tile copy (gdc_debug_wait_polls)
 gdc_status fail(gdc_ctx* c, gdc_status s, const std::string& msg);
-gdc_status cuda_check(gdc_ctx* c, cudaError_t e, const char* what);
+gdc_status cuda_check(gdc_ctx* c, cudaError_t e, const char* what);   // refused cluster launches too
+void note_launch(gdc_ctx* c, cudaError_t e);   // keeps a cluster launch's result for the next cuda_check
 int prof_begin(gdc_ctx* c, int kind);     // records a start event when timing is on (-1 otherwise)
 void prof_end(gdc_ctx* c, int idx);
 void prof_flush(gdc_ctx* c);

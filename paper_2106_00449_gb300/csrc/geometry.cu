@@ -329,7 +329,7 @@ void launch_ref(gdc_ctx* c, const double* Y) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     ++c->n_launch;
-    cudaLaunchKernelEx(&cfg, k_ref, C, c->susp_body_off, Y, c->ref);
+    note_launch(c, cudaLaunchKernelEx(&cfg, k_ref, C, c->susp_body_off, Y, c->ref));
 }
 
 }  // namespace gdc

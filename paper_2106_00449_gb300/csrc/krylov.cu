@@ -630,7 +630,7 @@ static void launch_orth(gdc_ctx* c, const gdc::Seg& sg, int C, double* V, long l
     cfg.attrs = at;
     cfg.numAttrs = 1;
     ++c->n_launch;
-    cudaLaunchKernelEx(&cfg, k_orth, C, sg.off, V, ld, w, j, jdev, active, vcur, gm, lz);
+    note_launch(c, cudaLaunchKernelEx(&cfg, k_orth, C, sg.off, V, ld, w, j, jdev, active, vcur, gm, lz));
 }
 
 // A GMRES iteration's orthogonalisation of gm_w against V_0..V_j, and its column of H
