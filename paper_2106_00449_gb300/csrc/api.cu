@@ -1000,7 +1000,7 @@ gdc_status gdc_init(gdc_ctx** out, const gdc_params* params, int n_templates, co
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if ((st = cuda_check(c, e, "state read")) != GDC_OK) return st;
     if ((st = check_state_host(c, hY.data(), hq.data())) != GDC_OK) return st;
-    krylov_init_attributes();
+    if ((st = krylov_init_attributes(c)) != GDC_OK) return st;
     if (c->p.mobility == GDC_MOB_FCM) {
         // the FCM grid first: the preconditioner's template blocks are FCM blocks
         const gdc_fcm_params fp = fcm_params_of(c->p, c->NBL);

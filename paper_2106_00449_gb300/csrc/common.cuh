@@ -284,6 +284,7 @@ struct gdc_ctx {
     int cap_depth = 0;
     cudaError_t cap_err = cudaSuccess;
     cudaError_t launch_err = cudaSuccess;   // the first refused cluster launch (note_launch)
+    int orth_cluster_max = 1;               // blocks per cluster that the device grants k_orth
     unsigned long long graph_base_launches = 0;               // kernels outside the loops
     std::vector<std::pair<int, unsigned long long>> graph_loops;   // (report slot, kernels per iteration)
     unsigned long long d_step_mirror = ~0ull;                 // value last written to ctl->step
@@ -471,7 +472,7 @@ gdc_status gmres_solve(gdc_ctx* c, const double* b, double* x, gdc_solve_info* i
 gdc_status lanczos_sqrt(gdc_ctx* c, const double* W, double* out, double scale, int fixed_iters,
                         int* iters_out, double* err_out);
 void setup_segments(gdc_ctx* c);
-void krylov_init_attributes();
+gdc_status krylov_init_attributes(gdc_ctx* c);
 // graph mode (capture helpers and the device-driven loops)
 cudaGraphConditionalHandle cap_cond(gdc_ctx* c);
 void cap_while_begin(gdc_ctx* c, cudaGraphConditionalHandle h);

@@ -604,31 +604,39 @@ static long long longest_segment(const gdc::Seg& sg) {
 }
 
 // Blocks per cluster of the fused orthogonalisation of a segmented space, 0: the separate
-// kernels (a suspension longer than GDC_ORTH_MAX).  The cluster doubles while its parts are
-// longer than GDC_ORTH_SLICE, or longer than 512 elements with fewer than two blocks per SM
-// in all, so that few suspensions spread over more FP64 pipes.
+// kernels (a suspension longer than GDC_ORTH_MAX, or than what the largest cluster of the device
+// holds).  The cluster doubles while its parts are longer than GDC_ORTH_SLICE, or longer than
+// 512 elements with fewer than two blocks per SM in all, so that few suspensions spread over
+// more FP64 pipes.
 static int orth_cluster(const gdc_ctx* c, const gdc::Seg& sg) {
     const long long n = longest_segment(sg);
     if (n > GDC_ORTH_MAX) return 0;
     int C = 1;
-    while (C < 16 && (n > (long long)GDC_ORTH_SLICE * C || (n > 512LL * C && (long long)c->S * C < 2LL * c->num_sms)))
+    while (C < c->orth_cluster_max &&
+           (n > (long long)GDC_ORTH_SLICE * C || (n > 512LL * C && (long long)c->S * C < 2LL * c->num_sms)))
         C *= 2;
-    return C;
+    return n > (long long)GDC_ORTH_SLICE * C ? 0 : C;
 }
 
-static void launch_orth(gdc_ctx* c, const gdc::Seg& sg, int C, double* V, long long ld, const double* w, int j,
-                        const int* jdev, const int* active, double* vcur, const OrthGm& gm, const OrthLz& lz) {
+// C blocks per suspension, a part of `part` elements each
+static cudaLaunchConfig_t orth_config(const gdc_ctx* c, int C, long long part, cudaLaunchAttribute* at) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(c->S * C));
     cfg.blockDim = dim3(ORTH_TH);
-    cfg.dynamicSmemBytes = sizeof(double) * (size_t)((longest_segment(sg) + C - 1) / C);
+    cfg.dynamicSmemBytes = sizeof(double) * (size_t)part;
     cfg.stream = c->stream;
-    cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)C;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+static void launch_orth(gdc_ctx* c, const gdc::Seg& sg, int C, double* V, long long ld, const double* w, int j,
+                        const int* jdev, const int* active, double* vcur, const OrthGm& gm, const OrthLz& lz) {
+    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = orth_config(c, C, (longest_segment(sg) + C - 1) / C, at);
     ++c->n_launch;
     note_launch(c, cudaLaunchKernelEx(&cfg, k_orth, C, sg.off, V, ld, w, j, jdev, active, vcur, gm, lz));
 }
@@ -1162,10 +1170,29 @@ __global__ void k_lz_reset(int S, int* __restrict__ lastk) {
     }
 }
 
-void krylov_init_attributes() {
-    cudaFuncSetAttribute(k_lz_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)lz_tridiag_smem(GDC_MAX_LANCZOS));
-    cudaFuncSetAttribute(k_orth, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of 16
+// Launch attributes, and the largest cluster of k_orth that the device can place: 16 blocks are more
+// than the portable 8, and a device or partition may have no group of SMs for them.
+gdc_status krylov_init_attributes(gdc_ctx* c) {
+    const gdc_status st = cuda_check(c, cudaFuncSetAttribute(k_lz_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                             (int)lz_tridiag_smem(GDC_MAX_LANCZOS)),
+                                     "eigen-step attributes");
+    if (st != GDC_OK) return st;
+    int C = 16;
+    if (cudaFuncSetAttribute(k_orth, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();   // a refusal, here and below, is an answer
+        C = 8;
+    }
+    for (; C > 1; C /= 2) {
+        cudaLaunchAttribute at[1];
+        cudaLaunchConfig_t cfg = orth_config(c, C, std::min(GDC_ORTH_SLICE, GDC_ORTH_MAX / C), at);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_orth, &cfg) != cudaSuccess)
+            cudaGetLastError();
+        else if (n > 0)
+            break;
+    }
+    c->orth_cluster_max = C;
+    return GDC_OK;
 }
 
 // A Lanczos iteration's full reorthogonalisation of lz_w against v_0..v_j, the eigen-step and

@@ -116,3 +116,15 @@ c.step(1)
 print("stepped", c.get_state()[2] == s0 + 1)
 """ % graph)
     assert out.split("\n")[:6] == ["status 2 True"] * 3 + ["state True", "again True", "stepped True"], out
+
+
+@pytest.mark.parametrize("largest", [8, 2, 1])
+def test_smaller_clusters_where_the_device_refuses_16(child, largest):
+    """8 and 2 blocks, and the separate kernels where no cluster holds a suspension."""
+    _, f = child("np.save(os.environ['OUT'], results(context()))")
+    full = np.load(f)
+    _, f = child("fake.fake_limit(%d, 1)\nnp.save(os.environ['OUT'], results(context()))" % largest)
+    # converged to 1e-9 of the right-hand side and of the root; the block-preconditioned operators'
+    # condition numbers are below 1e3
+    few = np.load(f)
+    assert np.linalg.norm(few - full) < 1e-6 * np.linalg.norm(full)
