@@ -338,14 +338,17 @@ __device__ inline void quat_exp_mul(const double* u, const double* q, double* ou
     out[3] = e0 * q3 + q0 * e3 + (e1 * q2 - e2 * q1);
 }
 
-// 1/sqrt(x) for positive normal x in 5 FP64 instructions: the hardware's approximation y times
-// the series 1 + e/2 + 3 e^2/8, e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2) cut
-// after e^2: with |e| below 4e-6 the next term is below 2e-17).
+// 1/sqrt(x) for positive normal x, and 0 for +inf (distances whose square overflows), in 5 FP64
+// instructions: the hardware's approximation y times the series 1 + e/2 + 3 e^2/8, e = 1 - x y^2
+// (the binomial series of (1 - e)^(-1/2) cut after e^2: with |e| below 4e-6 the next term is
+// below 2e-17).  At x = +inf y is 0 and the series a NaN; the test is on integers, which cost
+// nothing beside the FP64 pipe.
 __device__ __forceinline__ double rsqrt_series(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-(x * y), y, 1.0);
-    return fma(fma(0.375, e, 0.5), y * e, y);
+    const double v = fma(fma(0.375, e, 0.5), y * e, y);
+    return __double2hiint(y) == 0 ? y : v;
 }
 
 __device__ inline double warp_sum(double v) {
