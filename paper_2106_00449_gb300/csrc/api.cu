@@ -358,26 +358,30 @@ static size_t carve(gdc_ctx* c, void* base) {
     c->red_part = w.take<double>((long long)std::max(c->seg_gm.n_chunks, c->seg_lz.n_chunks) * cols);
     c->mv_items = w.take<MvItem>(c->mv_cap_items);
     c->mv_nk = w.take<int>(S);
-    c->mv_part = (void*)w.take<double4_32a>((long long)c->mv_cap_kmax * NBL);
+    // Partial sums, target side ([slot][blob]) and source side ([slot][tile]): one array each
+    // for all pair kernels, whose epilogue takes a kernel's sums before the next kernel starts
+    // (one stream, one product or force evaluation at a time).
+    const long long part_i = std::max(std::max<long long>(c->mv_cap_kmax, (c->sym_cap_kmax + 1) / 2),
+                                      std::max<long long>(c->dfs_kmax, c->p64_kmax)) * NBL;
+    const long long part_j = std::max(c->sym_n_jslots * GDC_SYM_TILE, c->h_p64_jbase.back() * c->p64_tile);
+    double4_32a* const parts = w.take<double4_32a>(part_i);
+    double4_32a* const parts_j = w.take<double4_32a>(part_j);
+    c->mv_part = (void*)parts;
+    c->sym_part_i = (float4*)parts;
+    c->dfs_part_i = c->p64_part_i = parts;
+    c->sym_part_j = (float4*)parts_j;
+    c->dfs_part_j = c->p64_part_j = parts_j;
     c->dev_status = w.take<int>(4);
     c->sym_items = w.take<PairItem>(c->sym_cap_items);
     c->sym_row_nk = w.take<int>(std::max<long long>(1, c->sym_n_tiles));
     c->sym_tile_base = w.take<long long>(S + 1);
     c->sym_jbase = w.take<long long>(S + 1);
-    c->sym_part_i = w.take<float4>((long long)c->sym_cap_kmax * NBL);
-    c->sym_part_j = w.take<float4>(std::max<long long>(1, c->sym_n_jslots) * GDC_SYM_TILE);
     c->dfs_items = w.take<PairItem>(c->dfs_n_items);
     c->dfs_row_nk = w.take<int>(std::max<long long>(1, c->sym_n_tiles));
-    c->dfs_part_i = w.take<double4_32a>((long long)c->dfs_kmax * NBL);
-    // source-side slots of the double-float and the FP64 kernel: one product at a time uses them
-    c->dfs_part_j = w.take<double4_32a>(std::max<long long>(
-        1, std::max(c->sym_n_jslots * GDC_SYM_TILE, c->h_p64_jbase.back() * c->p64_tile)));
-    c->p64_part_j = c->dfs_part_j;
     c->p64_items = w.take<PairItem>((long long)c->h_p64_items.size());
     c->p64_row_nk = w.take<int>((long long)c->h_p64_row_nk.size());
     c->p64_tile_base = w.take<long long>(S + 1);
     c->p64_jbase = w.take<long long>(S + 1);
-    c->p64_part_i = w.take<double4_32a>((long long)c->p64_kmax * NBL);
     c->h_near_items.clear();
     // search blocks of 256 targets x near_src sources: as few sources as keep the list within
     // 64 blocks per SM (3,001 blobs: 144 blocks of 256 sources 20 us, 564 of 64 sources 9.0)
