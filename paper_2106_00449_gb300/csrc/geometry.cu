@@ -278,8 +278,10 @@ namespace gdc {
 // positions relative to it, which keeps FP32 coordinates small.  A cluster of C blocks per
 // suspension, four bodies in flight per thread.  Bound by load latency and, in one block, by its
 // SM's FP64 adds (3 per body at 2 per clock): 8 blocks from REF_SPLIT bodies on.  16,384 bodies:
-// 21 us in one block, 8.2 us in eight.
-constexpr int REF_TH = 512, REF_SPLIT = 256;
+// 21 us in one block, 8.2 us in eight.  More than REF_SUSP suspensions fill the chip with one
+// block each, and idle blocks then cost: 750 bodies beside 2,000 single ones took 190 us in
+// clusters of eight.
+constexpr int REF_TH = 512, REF_SPLIT = 256, REF_SUSP = 38;
 
 __global__ void __launch_bounds__(REF_TH) k_ref(int C, const long long* __restrict__ susp_body_off,
                                                 const double* __restrict__ Y, double* __restrict__ ref) {
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(REF_TH) k_ref(int C, const long long* __restri
 void launch_ref(gdc_ctx* c, const double* Y) {
     long long nb = 0;
     for (int s = 0; s < c->S; ++s) nb = std::max(nb, c->h_body_off[s + 1] - c->h_body_off[s]);
-    const int C = nb > REF_SPLIT ? 8 : 1;
+    const int C = nb > REF_SPLIT && c->S <= REF_SUSP ? 8 : 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(c->S * C));
     cfg.blockDim = dim3(REF_TH);
