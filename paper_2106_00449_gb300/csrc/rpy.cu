@@ -850,10 +850,12 @@ static const int kMvMinBlocks[2] = {4, 6};       // resident blocks per SM of th
 static const int kDfsMinBlocks[2] = {3, 4};      // resident blocks per SM of the symmetric double-float kernel
 
 // Sources per item of the symmetric FP32 kernel: the longest range (a power of two, 32 to
-// 2,048) that gives at least 6 items per SM and is at most 1/48 of the largest suspension, or
-// gives at least 16 items per SM whatever its length.  Short ranges spread few pairs over the
+// 2,048) that gives at least 6 full items per SM and is at most 1/48 of the largest suspension, or
+// gives at least 16 full items per SM whatever its length.  Short ranges spread few pairs over the
 // chip and leave more partial sums to add; long ones end in a ragged last wave, which 16 items
-// per SM make short.  us per product (positions, near lists, pair kernel, epilogue) at 3 resident
+// per SM make short.  Full items, the sources of all rows over the width: thousands of tiny
+// suspensions have as many items but hardly any work to hide a long one behind (one of 2,040
+// blobs and 4,000 of 12: 407 us with 2,048 sources, 278 with 32).  us per product (positions, near lists, pair kernel, epilogue) at 3 resident
 // blocks per SM, by this rule (its width) and at 32 / 128 / 512 / 1,024 / 2,048 sources:
 //   one suspension of 2,556 blobs 121 (32): 124 / 134 / 164 / 217 / 295
 //   8,400 blobs 190 (64): 204 / 189 / 205 / 269 / 398
@@ -861,14 +863,15 @@ static const int kDfsMinBlocks[2] = {3, 4};      // resident blocks per SM of th
 //   65,520 blobs 2,538 (1,024): 3,392 / 2,624 / 2,553 / 2,539 / 2,623
 //   24 of 2,700 blobs 304 (64): 308 / 296 / 320 / 336 / 414
 //   24 of 9,000 blobs 1,346 (512): 1,661 / 1,400 / 1,346 / 1,343 / 1,393
-//   310 of 2,700 blobs 1,853 (2,048): 2,164 / 1,933 / 1,868 / 1,853 / 1,853
-//   512 of 8 to 128 bodies, 746,060 blobs, 1,333 (1,024): 1,534 / 1,384 / 1,331 / 1,333 / 1,335
+//   310 of 2,700 blobs 1,853 (1,024): 2,164 / 1,933 / 1,868 / 1,853 / 1,853
+//   512 of 8 to 128 bodies, 746,060 blobs, 1,331 (512): 1,534 / 1,384 / 1,331 / 1,333 / 1,335
 static int sym_default_width(const gdc_ctx* c) {
     long long nmax = 1;
     for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
+    const long long sources = pair_list_items(c, GDC_SYM_TILE, 1);   // over all rows of tiles
     int w = 2048;
     for (; w > 32; w /= 2) {
-        const long long items = pair_list_items(c, GDC_SYM_TILE, w);
+        const long long items = sources / w;
         if (items >= 16LL * c->num_sms || (w <= nmax / 48 && items >= 6LL * c->num_sms)) break;
     }
     return w;
