@@ -150,17 +150,18 @@ __host__ __device__ inline int gp_split(int n3) {
     return R >= GP_TH ? 1 : GP_TH / R;
 }
 
-// FP32 rows of more than 64 columns keep at least four chains, joined in FP64, where up to a few
-// thousand bodies share the work (GB < 8): two of them, or two joined in FP32, lose up to a third
-// of the accuracy of a body's own block (relative error of an FP32 product of single bodies, two
-// chains and four: 340 blobs 4.2e-7 and 3.2e-7, 85 blobs 2.4e-7 and 1.9e-7).  Shorter rows have
-// more chains anyway, each shorter; GB = 8 stays with two, half the FP64 additions.
+// FP32 rows of more than 64 columns of a body's own block or its inverse keep at least four
+// chains, joined in FP64, where up to a few thousand bodies share the work (GB < 8): two of them,
+// or two joined in FP32, lose up to a third of the accuracy (relative error of an FP32 product of
+// single bodies, two chains and four: 340 blobs 4.2e-7 and 3.2e-7, 85 blobs 2.4e-7 and 1.9e-7).
+// Shorter rows have more chains anyway, each shorter; GB = 8 stays with two, half the FP64
+// additions, and so do the factors, whose sums enter beside the pair kernel's.
 // gp_halves: the parts that a thread takes of a whole row in turn, each summed into FP64;
 // gp_parts: the chains that a thread of a split row leaves to be joined.
-template <int GB, typename T>
-__host__ __device__ inline int gp_halves(int KS) { return GB < 8 && sizeof(T) == 4 && KS == 1 ? 2 : 1; }
-template <int GB, typename T>
-__host__ __device__ inline int gp_parts(int KS) { return GB < 8 && sizeof(T) == 4 && KS == 2 ? 2 : 1; }
+template <int GB, int SHAPE, typename T>
+__host__ __device__ inline int gp_halves(int KS) { return SHAPE == GP_FULL && GB < 8 && sizeof(T) == 4 && KS == 1 ? 2 : 1; }
+template <int GB, int SHAPE, typename T>
+__host__ __device__ inline int gp_parts(int KS) { return SHAPE == GP_FULL && GB < 8 && sizeof(T) == 4 && KS == 2 ? 2 : 1; }
 
 // out[u n3 + i] = sum_k M[k n3 + i] in[k GB + u] over the columns SHAPE leaves row i, u < GB (in
 // padded with zeros): two chains of type T over each thread's columns, the threads' sums added in
@@ -169,7 +170,8 @@ template <int GB, int SHAPE, typename T>
 __device__ __forceinline__ void group_product(const T* __restrict__ M, int n3, const T* in_, T* part, double* out) {
     // 16-byte aligned by the callers' layouts for GB >= 4, so a column's entries are vector loads
     const T* in = GB >= 4 ? (const T*)__builtin_assume_aligned(in_, 16) : in_;
-    const int R = (n3 + 31) & ~31, KS = gp_split(n3), halves = gp_halves<GB, T>(KS), NP = gp_parts<GB, T>(KS);
+    const int R = (n3 + 31) & ~31, KS = gp_split(n3);
+    const int halves = gp_halves<GB, SHAPE, T>(KS), NP = gp_parts<GB, SHAPE, T>(KS);
     const int ks = KS == 1 ? 0 : (int)threadIdx.x / R;
     const int chunk = (n3 + KS * halves - 1) / (KS * halves);
     for (int row = KS == 1 ? (int)threadIdx.x : (int)threadIdx.x % R; row < n3 && ks < KS; row += GP_TH) {
@@ -234,10 +236,10 @@ __device__ __forceinline__ void group_product(const T* __restrict__ M, int n3, c
 }
 
 // Bytes of group_product's arrays: in (T), part (T), out (double)
-template <int GB, typename T>
+template <int GB, int SHAPE, typename T>
 static size_t gp_bytes(int n3) {
     const int KS = gp_split(n3);
-    return (size_t)GB * n3 * (sizeof(double) + sizeof(T) * (1 + (KS > 1 ? KS * gp_parts<GB, T>(KS) : 0)));
+    return (size_t)GB * n3 * (sizeof(double) + sizeof(T) * (1 + (KS > 1 ? KS * gp_parts<GB, SHAPE, T>(KS) : 0)));
 }
 
 // K^T of the group's body-frame vectors v (double, [u][n3]) with blob offsets b: four threads per
@@ -526,16 +528,16 @@ static GroupArgs group_args(const gdc_ctx* c) {
 }
 
 // Shared memory of a block: the largest over the templates
-template <int GB, typename T>
+template <int GB, int SHAPE, typename T>
 static size_t group_smem(const gdc_ctx* c, int more_per_row, int more) {
     size_t s = 0;
-    for (int n : c->h_tmpl_n) s = std::max(s, gp_bytes<GB, T>(3 * n) + (size_t)(more_per_row * 3 * n + more) * sizeof(double));
+    for (int n : c->h_tmpl_n) s = std::max(s, gp_bytes<GB, SHAPE, T>(3 * n) + (size_t)(more_per_row * 3 * n + more) * sizeof(double));
     return s;
 }
 
 template <bool LAB, int GB, typename T>
 static void precond_launch(gdc_ctx* c, const T* Minv, const double* r, double* z, float4* sdup) {
-    const size_t smem = group_smem<GB, T>(c, LAB ? 1 : 0, 24 * GB);
+    const size_t smem = group_smem<GB, GP_FULL, T>(c, LAB ? 1 : 0, 24 * GB);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_precond<LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_precond<LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), Minv, LAB ? c->blk_G : c->tmpl_G, LAB ? c->blk_N : c->tmpl_N, r, z, c->r, c->Yc, sdup);
@@ -557,7 +559,7 @@ void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32, bool pack
 
 template <int GB, typename T>
 static void intra_launch(gdc_ctx* c, const T* M, const double* x, double* y, int gm) {
-    const size_t smem = group_smem<GB, T>(c, GB, 6 * GB);
+    const size_t smem = group_smem<GB, GP_FULL, T>(c, GB, 6 * GB);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_intra_body<GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     GroupArgs ga = group_args(c);
     ga.mat_off = c->minv_off;
@@ -577,7 +579,7 @@ void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm, bool fp32
 
 template <int MODE, bool LAB, int GB, typename T>
 static void tri_launch(gdc_ctx* c, const T* F, const double* x, const double* add, double* out, float4* sdup) {
-    const size_t smem = group_smem<GB, T>(c, 0, 0);
+    const size_t smem = group_smem<GB, GP_TO_DIAG, T>(c, 0, 0);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_body_tri<MODE, LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_body_tri<MODE, LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), F, x, add, out, sdup);
