@@ -131,13 +131,18 @@ void launch_lsq(gdc_ctx* c, const double* vbrev, double* calV) {
 // lanes idle.  One 128-thread block per body spent 200 FP64 warp instructions per body in the
 // preconditioner (68% of the pipe), mostly on one lane's 6 x 6 product and 30 shuffle adds.
 //
-// GB, the bodies per block, in FP32: 8 from 40 bodies per SM on, 4 from 512 bodies on, 1 below and
-// with templates above 85 blobs.  us per launch with GB = 1 / 4 / 8 (preconditioner; same-body
+// GB, the bodies per block, in FP32: 8 from 40 bodies per SM on, 4 from 512 bodies on, 1 below and,
+// for all templates of a context, with one above 85 blobs (a thread per row then ends).  us per launch with GB = 1 / 4 / 8 (preconditioner; same-body
 // block with K^T; factor products): 777 bodies 16.6 / 14.2 / 18.5; 15.1 / 12.3 / 16.3; 23.8 /
 // 27.5 / 24.8.  2,520 bodies 39.9 / 21.1 / 22.8; 40.2 / 18.1 / 20.7; 50.2 / 40.0 / 32.6.  12,082
 // bodies 140 / 70 / 60; 129 / 57 / 66; 154 / 95 / 77.  One block per body took 40.0, 36.0
 // (two launches) and 34.8 at 2,520 bodies.  In FP64 one body per block is as fast or faster up
 // to 3,000 bodies (same-body block 57.6 / 54.1 / 65.1, factor 34.9 / 36.6 / 46.3) and always used.
+// Against the earlier kernels, which grouped whatever the template and FP64 products too from 4,864
+// bodies on, neither rule loses (us per call, before and now): the FP64 preconditioner of 6,000
+// bodies 280 / 147, of 36,121 723 / 510; with a 162-blob body among 12,081 of 12 blobs a solve 196,600
+// / 164,900 and a Brownian velocity 204,800 / 199,300, among 35,839 in 512 suspensions 9,950 / 8,370
+// and 8,430 / 5,960.
 
 constexpr int GP_TH = 256;
 
@@ -527,7 +532,8 @@ static GroupArgs group_args(const gdc_ctx* c) {
                      c->p.wall ? c->blk_off : c->minv_off, c->blob_gm, c->body_gm, c->Rb, c->tmpl_xyz};
 }
 
-// Shared memory of a block: the largest over the templates
+// Shared memory of a block: the largest over the templates.  At most 41 KB (eight bodies of 85 blobs),
+// so no launch needs the attribute that 48 KB and more take.
 template <int GB, int SHAPE, typename T>
 static size_t group_smem(const gdc_ctx* c, int more_per_row, int more) {
     size_t s = 0;
@@ -538,7 +544,6 @@ static size_t group_smem(const gdc_ctx* c, int more_per_row, int more) {
 template <bool LAB, int GB, typename T>
 static void precond_launch(gdc_ctx* c, const T* Minv, const double* r, double* z, float4* sdup) {
     const size_t smem = group_smem<GB, GP_FULL, T>(c, LAB ? 1 : 0, 24 * GB);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_precond<LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_precond<LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), Minv, LAB ? c->blk_G : c->tmpl_G, LAB ? c->blk_N : c->tmpl_N, r, z, c->r, c->Yc, sdup);
 }
@@ -560,7 +565,6 @@ void launch_precond(gdc_ctx* c, const double* r, double* z, bool fp32, bool pack
 template <int GB, typename T>
 static void intra_launch(gdc_ctx* c, const T* M, const double* x, double* y, int gm) {
     const size_t smem = group_smem<GB, GP_FULL, T>(c, GB, 6 * GB);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_intra_body<GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     GroupArgs ga = group_args(c);
     ga.mat_off = c->minv_off;
     ++c->n_launch, k_intra_body<GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(ga, M, x, y, gm);
@@ -580,7 +584,6 @@ void launch_intra_body(gdc_ctx* c, const double* x, double* y, int gm, bool fp32
 template <int MODE, bool LAB, int GB, typename T>
 static void tri_launch(gdc_ctx* c, const T* F, const double* x, const double* add, double* out, float4* sdup) {
     const size_t smem = group_smem<GB, GP_TO_DIAG, T>(c, 0, 0);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_body_tri<MODE, LAB, GB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     ++c->n_launch, k_body_tri<MODE, LAB, GB, T><<<GB == 1 ? c->NB : c->tb_n_items, GP_TH, smem, c->stream>>>(
         group_args(c), F, x, add, out, sdup);
 }

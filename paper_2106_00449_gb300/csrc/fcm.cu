@@ -22,11 +22,12 @@
 //     of the inverse transform): for M_FCM lambda it runs between the forward and inverse z
 //     passes in one launch (a block takes pencils with their mirrors, whose modes -k the split
 //     of the two real fields needs), for v-breve it is one pass over the modes;
-//   * averaging reads the packed velocity (one 16-byte load per point) and takes one warp per
-//     blob; in each z-plane of the blob's box (at most 31 points per side) the rows that can
-//     meet the sphere are one run of points, x fastest, dealt to the lanes in turn; each lane
-//     sums its points of a plane in FP32 and the planes with FP32 compensation, and the lanes
-//     are added in FP64 in a fixed order.
+//   * averaging reads the packed velocity (one 16-byte load per point) and takes four warps per
+//     blob, each every fourth z-plane of the blob's box (at most 31 points per side); the rows
+//     of a plane that can meet the sphere are one run of points, x fastest, dealt to the lanes
+//     in turn; each lane sums its points of a plane in FP32 and the planes with FP32
+//     compensation, the lanes are joined as compensated FP32 pairs (exact two-sums, so to
+//     about 2^-48) and the four warps in FP64, all in a fixed order.
 #include <algorithm>
 #include <cmath>
 #include <new>
@@ -226,8 +227,9 @@ __device__ __forceinline__ float exp2_series(float x) {
 constexpr int SPC_KZ = 12;   // layers of a column a thread keeps
 
 // Spreading with at least 4 binning cells per side (no minimum image, as in k_fcm_spread below):
-// a block takes up to 256 columns (x, y) of a cell (blockDim.x, at least 128) and up to SPC_KZ of its
-// layers, a thread one column.
+// a block takes the columns (x, y) of a cell (at most 16 x 16: R_t spans at most 15 spacings and N is
+// a power of two; blockDim.x of them, at least 128) and up to SPC_KZ of its layers, a thread one
+// column.
 // Per blob a thread forms dx^2 + dy^2 and its Gaussian once, and the layers' dz^2 and Gaussians
 // come from a table that the block fills once per staged blob, so a grid point costs a compare
 // and three FMAs (1.03 ms at 512^3 for 65,520 blobs; 13 instructions with the whole Gaussian per
@@ -240,7 +242,7 @@ constexpr int SPC_KZ = 12;   // layers of a column a thread keeps
 __global__ void __launch_bounds__(256) k_fcm_spread_col(int N, double h, double w, int nc, const int* __restrict__ cnt,
                                                         const int* __restrict__ start, const float4* __restrict__ poff,
                                                         const float4* __restrict__ plam, float R2, float Rt, float l2s,
-                                                        float norm, float2* __restrict__ f, long long NG, int zchunks) {
+                                                        float norm, float2* __restrict__ f, long long NG) {
     __shared__ float4 sp[SP_CHUNK];   // x, y of a staged blob; first and last layer in reach
     __shared__ float4 sl[SP_CHUNK];
     __shared__ float sz[SP_CHUNK];
@@ -256,8 +258,8 @@ __global__ void __launch_bounds__(256) k_fcm_spread_col(int N, double h, double 
         gn[d] = ((c3[d] + 1) * N + nc - 1) / nc - g0[d];
     }
     const int ncol = gn[0] * gn[1];
-    const int col0 = (int)(blockIdx.y / zchunks) * (int)blockDim.x, k0 = (int)(blockIdx.y % zchunks) * SPC_KZ;
-    if (col0 >= ncol || k0 >= gn[2]) return;   // whole block: the cell has no points there
+    const int k0 = (int)blockIdx.y * SPC_KZ;
+    if (k0 >= gn[2]) return;   // whole block: the cell has no points there
     const int nz = min(SPC_KZ, gn[2] - k0);
     if (threadIdx.x < 27) {
         const int k = threadIdx.x;
@@ -285,7 +287,7 @@ __global__ void __launch_bounds__(256) k_fcm_spread_col(int N, double h, double 
     __syncthreads();
     const int total = c_off[27];
     const float hf = (float)h, wf = (float)w, ih = 1.0f / hf;
-    const int col = col0 + (int)threadIdx.x;
+    const int col = threadIdx.x;
     const bool live = col < ncol;
     const int jx = col % gn[0], jy = col / gn[0];
     const float gx = fmaf((float)jx, hf, base_off[0]), gy = fmaf((float)jy, hf, base_off[1]);
@@ -294,9 +296,8 @@ __global__ void __launch_bounds__(256) k_fcm_spread_col(int N, double h, double 
     for (int k = 0; k < SPC_KZ; ++k) ax[k] = ay[k] = az[k] = 0.f;
     // the bounding box of this block's grid points in the frame of the cell's corner, and the
     // squared reach beyond it, widened by 1e-4 against rounding (dropping is only ever conservative)
-    const int ylo = col0 / gn[0], yhi = (min(col0 + (int)blockDim.x, ncol) - 1) / gn[0];
     const float bx0 = base_off[0], bx1 = fmaf((float)(gn[0] - 1), hf, base_off[0]);
-    const float by0 = fmaf((float)ylo, hf, base_off[1]), by1 = fmaf((float)yhi, hf, base_off[1]);
+    const float by0 = base_off[1], by1 = fmaf((float)(gn[1] - 1), hf, base_off[1]);
     const float bz0 = fmaf((float)k0, hf, base_off[2]), bz1 = fmaf((float)(k0 + nz - 1), hf, base_off[2]);
     const float reach2 = R2 * 1.0001f;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1252,10 +1253,11 @@ gdc_status gdc_fcm_apply(gdc_fcm* f, int n, const double* r, const double* lambd
         n, f->p.L / f->nc, f->nc, f->list, f->cell_of, f->pw, lambda, f->poff, f->plam);
     const double s2 = f->p.sigma * f->p.sigma;
     {
-        // columns of a cell per thread from 8 points per cell side on (64 columns fill half a
+        // a column of a cell per thread from 8 points per cell side on (64 columns fill half a
         // block) and 4 cells per side; else points: 4 per thread, 512 per block (2 and 256 when a
-        // cell has at most 256 points, so that small cells leave fewer idle slots).  The largest
-        // cell has side^3 points
+        // cell has at most 256 points, so that small cells leave fewer idle slots; beside columns
+        // that leaves 4 to cells of 7 points a side and to fewer than 4 cells).  The largest cell
+        // has side^3 points
         const long long side = (f->N + f->nc - 1) / f->nc;
         const int pt = side * side * side <= 256 ? 2 : 4;
         const unsigned chunks = (unsigned)((side * side * side + 128 * pt - 1) / (128 * pt));
@@ -1269,11 +1271,10 @@ gdc_status gdc_fcm_apply(gdc_fcm* f, int n, const double* r, const double* lambd
         f->plam, R2, i2, nrm, f->grid, f->NG)
         const bool wrap = f->nc < 4;
         if (!wrap && side >= 8) {
-            const int cols = (int)(side * side), zch = ceil_div(side, SPC_KZ);
-            const int th = std::min(256, std::max(128, (cols + 31) / 32 * 32));
-            k_fcm_spread_col<<<dim3((unsigned)nc3, (unsigned)(ceil_div(cols, th) * zch)), th, 0, f->stream>>>(
+            const int th = std::max(128, ((int)(side * side) + 31) / 32 * 32);   // a thread per column: at most 256
+            k_fcm_spread_col<<<dim3((unsigned)nc3, (unsigned)ceil_div(side, SPC_KZ)), th, 0, f->stream>>>(
                 f->N, f->h, f->p.L / f->nc, f->nc, f->cnt, f->start, f->poff, f->plam, R2, (float)f->p.R_t, i2, nrm,
-                f->grid, f->NG, zch);
+                f->grid, f->NG);
         } else if (pt == 2) {
             if (wrap)
                 GDC_SPREAD(2, true);

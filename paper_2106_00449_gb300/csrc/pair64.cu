@@ -18,7 +18,7 @@
 // warps' sums of a source meet in shared memory, are added in warp order and go to the one
 // slot of (I, J): every slot is written once, all sums run in a fixed order (deterministic).
 // Because the pipe is so slow one target per lane already hides every latency, and short
-// ranges spread a small suspension over all SMs: 1,560 blobs take 1,360 items of 8 sources.
+// ranges spread a small suspension over all SMs: 1,560 blobs take 1,287 items of 8 sources.
 // Above GDC_P64_WIDE blobs TPL = 4 keeps the slot arrays at n^2/1024 entries.
 //
 // Measured against the ordered kernel that it replaced (128 or 256 or 512 targets per block
@@ -256,8 +256,9 @@ __global__ void __launch_bounds__(128) k_p64_epilogue(
 }
 
 // Work list: tiles of 128 blobs, or 512 when a suspension is larger than GDC_P64_WIDE; source
-// ranges as long as possible while a launch still has 8 items per SM (all of them resident
-// together, so an SM's share differs from the mean by at most an eighth), longest first.
+// ranges as long as possible while a launch still has 8 items per SM (7 resident with one target
+// per lane, at 71 registers; 3 with four, at 142), so that an SM's share differs from the mean by
+// about an eighth; longest first.
 void build_p64_list(gdc_ctx* c) {
     long long nmax = 0;
     for (int s = 0; s < c->S; ++s) nmax = std::max(nmax, c->h_blob_off[s + 1] - c->h_blob_off[s]);
