@@ -540,9 +540,10 @@ def main(argv=None) -> int:
     ap.add_argument("--op", default=None, help="time one building block instead of the step (see the module doc)")
     ap.add_argument("--bodies", type=int, default=0, help="--op: only the first N bodies of the workload (0 = all)")
     ap.add_argument("--reps", type=int, default=5, help="--op: timed calls")
-    ap.add_argument("--pair-kernel", type=int, default=0, help="--op: 0 autotuned, 1 ordered, 2 symmetric")
+    ap.add_argument("--pair-kernel", type=int, default=0, help="--op: 0 or 2 symmetric, 1 ordered")
     ap.add_argument("--df-kernel", type=int, default=0,
-                    help="--op: double-float kernel, 0 autotuned, 1 ordered, 3/4 symmetric at 3/4 blocks per SM")
+                    help="--op: double-float kernel, 0 as --pair-kernel (blocks per SM tuned from 2^28 pairs on), "
+                         "1 ordered, 3/4 symmetric at 3/4 blocks per SM")
     ap.add_argument("--graph", type=int, default=1, help="--op step32: 1 graph replay, 0 host-driven")
     ap.add_argument("--force-method", type=int, default=0, help="--op: 0 choose, 1 all pairs, 2 cell list")
     ap.add_argument("--potential", type=int, default=0, help="--op: 0 soft sphere, 1 and 2 the Sec. 6.4 wells")
