@@ -136,7 +136,8 @@ void launch_lsq(gdc_ctx* c, const double* vbrev, double* calV) {
 // block with K^T; factor products): 777 bodies 16.6 / 14.2 / 18.5; 15.1 / 12.3 / 16.3; 23.8 /
 // 27.5 / 24.8.  2,520 bodies 39.9 / 21.1 / 22.8; 40.2 / 18.1 / 20.7; 50.2 / 40.0 / 32.6.  12,082
 // bodies 140 / 70 / 60; 129 / 57 / 66; 154 / 95 / 77.  One block per body took 40.0, 36.0
-// (two launches) and 34.8 at 2,520 bodies.  In FP64 one body per block is as fast or faster up
+// (two launches) and 34.8 at 2,520 bodies.  (With GB = 4 in two chains a row; in four, see gp_parts,
+// the first two take 15.7 and 12.7 at 777 bodies, 23.1 and 19.3 at 2,520.)  In FP64 one body per block is as fast or faster up
 // to 3,000 bodies (same-body block 57.6 / 54.1 / 65.1, factor 34.9 / 36.6 / 46.3) and always used.
 // Against the earlier kernels, which grouped whatever the template and FP64 products too from 4,864
 // bodies on, neither rule loses (us per call, before and now): the FP64 preconditioner of 6,000
